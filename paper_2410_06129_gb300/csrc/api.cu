@@ -76,6 +76,17 @@ pinv_status build_gram(pinv_plan* p, cudaStream_t s, bool main_gram) {
     if (main_gram) {
         if (p->precision == PINV_FP64) {
             CK(launch_gram64(p->enc, p->lambda_abs, p->G, ld, s));
+        } else if (p->Gx) {
+            // plans that keep the exact Gram for their residual factor it too: its
+            // Toeplitz table needs (2 n - 1) offsets per axis times M_k products where the
+            // tensor-core Gram needs N^2 / 2 times M_k (64x64, 8192 samples: 1.72 ms with
+            // the split-BF16 Gram and its table; 128x128, 32768 samples: 103 ms), and it is
+            // exact to 2^-45 where the split products are to 2^-24
+            float4* work = nullptr;
+            CK(work_alloc((void**)&work, toeplitz_work_bytes(p->enc), s));
+            CK(launch_toeplitz(p->enc, work, p->Ttab, s));
+            CK(cudaFreeAsync(work, s));
+            CK(launch_gram_exact(p->enc, p->Ttab, p->lambda_abs, p->Gx, (float4*)p->G, s));
         } else {
             // bulk-fed Gram from a split operand table; without room for the table
             // (or with PINV_GRAM_BULK=0) the kernel generates its operands itself
@@ -104,21 +115,16 @@ pinv_status build_gram(pinv_plan* p, cudaStream_t s, bool main_gram) {
     // one (below, beside the Cholesky), else from G before the Cholesky overwrites it
     if (!p->Gx) CK(launch_gram_norm1(gdf ? nullptr : p->G, gdf ? (const float4*)p->G : nullptr, nullptr, N, ld, p->st, s));
     if (p->Gx) {
-        // exact Gram for the refinement residual (Toeplitz table, then coil products,
-        // then its digit tiles). Only applies and the condition check read it, so mixed
-        // plans form it on their lowest-priority stream beside the Cholesky and the
-        // inverse, in the SMs their launches leave free (build_factor joins that stream).
+        // the exact Gram's norm and digit tiles, and the digit table of conj(A). Only
+        // applies and the condition check read them, so mixed plans form them on their
+        // lowest-priority stream beside the Cholesky and the inverse, in the SMs their
+        // launches leave free (build_factor joins that stream).
         cudaStream_t sx = s;
         if (p->s_x) {
             CK(cudaEventRecord(p->ev_xfork, s));
             CK(cudaStreamWaitEvent(p->s_x, p->ev_xfork, 0));
             sx = p->s_x;
         }
-        float4* work = nullptr;
-        CK(work_alloc((void**)&work, toeplitz_work_bytes(p->enc), sx));
-        CK(launch_toeplitz(p->enc, work, p->Ttab, sx));
-        CK(cudaFreeAsync(work, sx));
-        CK(launch_gram_exact(p->enc, p->Ttab, p->lambda_abs, p->Gx, sx));
         CK(launch_gram_norm1(nullptr, nullptr, p->Gx, N, N, p->st, sx));
         if (p->Gd) CK(launch_gram_digits(p->Gx, N, p->eG, p->Gd, sx));
         if (p->Ad) CK(launch_adj_digits(p->enc, p->Ad, sx));

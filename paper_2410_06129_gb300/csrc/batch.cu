@@ -2,7 +2,8 @@
 //
 // A batch groups existing plans (many slices, time series or trajectories).
 // Its build runs the dominant tensor-core work of all plans as shared
-// persistent launches: one launch forms every plan's Gram, and per chunk of
+// persistent launches: one launch forms the Gram of every plan that keeps no
+// exact one (those form theirs on their own streams), and per chunk of
 // samples one launch forms every plan's T = W E^H and one every plan's
 // Recon = W^H T (all bulk-fed from per-plan operand tables); the sequential
 // Cholesky and triangular inverse of each plan run concurrently on per-plan
@@ -103,16 +104,15 @@ pinv_status build_sequence(pinv_batch* b, cudaStream_t s) {
     for (auto* p : b->plans) STB(build_begin(p, s));
     if (b->mixed) {
         const size_t n = b->plans.size();
-        for (size_t i = 0; i < n; ++i) CKB(gram_bulk_table(b->plans[i]->enc, b->slices, b->pwork[i], s));
-        CKB(tc_multi_launch(b->gram, b->slices, b->st, s));  // every plan's Gram
-        for (size_t i = 0; i < n; ++i) {
-            pinv_plan* p = b->plans[i];
-            CKB(gram_bulk_finish(p->enc, p->lambda_abs, b->slices, (float4*)p->G, p->N, b->pwork[i], s));
-            STB(build_gram(p, s, false));
-        }
+        for (size_t i = 0; i < n; ++i)
+            if (!b->plans[i]->Gx) CKB(gram_bulk_table(b->plans[i]->enc, b->slices, b->pwork[i], s));
+        CKB(tc_multi_launch(b->gram, b->slices, b->st, s));  // the Gram of every plan without an exact one
         STB(fork_all(b, s));
         for (size_t i = 0; i < n; ++i) {
             pinv_plan* p = b->plans[i];
+            if (!p->Gx)
+                CKB(gram_bulk_finish(p->enc, p->lambda_abs, b->slices, (float4*)p->G, p->N, b->pwork[i], b->side[i]));
+            STB(build_gram(p, b->side[i], p->Gx != nullptr));
             STB(build_factor(p, b->side[i], false));
             if (p->recon) CKB(recon_bulk_wtables(p->enc, p->W32, b->slices, b->pwork[i], b->side[i]));
         }
@@ -225,7 +225,7 @@ pinv_status pinv_batch_create(pinv_plan* const* plans, int n, int flags, pinv_ba
         int64_t chunks = 0;
         for (int i = 0; i < n; ++i) {
             const pinv_plan* p = b->plans[i];
-            size_t need = gram_bulk_bytes(p->enc, b->slices);
+            size_t need = p->Gx ? 0 : gram_bulk_bytes(p->enc, b->slices);
             if (p->recon) {
                 need = std::max(need, recon_bulk_bytes(p->enc, b->slices));
                 chunks = std::max(chunks, recon_bulk_chunks(p->enc, b->slices));
@@ -233,14 +233,14 @@ pinv_status pinv_batch_create(pinv_plan* const* plans, int n, int flags, pinv_ba
             off[i] = bytes;
             bytes += (need + 255) & ~(size_t)255;
         }
-        cudaError_t e = cudaMalloc(&b->work, bytes);
+        cudaError_t e = bytes ? cudaMalloc(&b->work, bytes) : cudaSuccess;
         if (e != cudaSuccess) return bad(cuda_err(e, "batch workspace"));
         std::vector<TcPlanArgs> all, rec;
         for (int i = 0; i < n; ++i) {
             pinv_plan* p = b->plans[i];
             b->pwork.push_back((unsigned char*)b->work + off[i]);
             const TcPlanArgs a{&p->enc, p->lambda_abs, (float4*)p->G, p->W32, (float2*)p->R, b->pwork[i]};
-            all.push_back(a);
+            if (!p->Gx) all.push_back(a);
             if (p->recon) rec.push_back(a);
         }
         e = tc_multi_create(TC_MULTI_GRAM, all.data(), (int)all.size(), b->slices, 0, &b->gram);

@@ -300,41 +300,87 @@ cudaError_t launch_adjoint_df(const EncodeDev& e, const double2* U, int64_t F, d
 // n' <= n also writes the conjugate to G[n'][n], so G is Hermitian to the bit).
 // The residual of the normal equations is then r = E^H d - G x with E^H d formed
 // once per apply.
-__global__ void k_gram_exact(EncodeDev e, const double2* T, double lam, float4* G) {
-    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;  // n'
-    const int64_t i = blockIdx.y;                                         // n
-    if (j > i) return;
-    const int* gi = e.vox_ijk + 3 * i;
-    const int* gj = e.vox_ijk + 3 * j;
+//
+// One CTA per 32 x 32 tile of the lower triangle: the coil values of the tile's rows
+// and columns are staged in shared memory (8 coils at a time), each thread forms four
+// entries, and the mirrored tile leaves through a transposed copy in shared memory, so
+// every store covers whole 512-byte row pieces. A mixed TOEPLITZ plan's Cholesky starts
+// from this Gram: Gl (or null) receives its lower triangle in the same pass. HBM-bound
+// but for the coil products (C x 48 FP32 instructions per entry).
+constexpr int GXT = 32;  // tile side
+constexpr int GXC = 8;   // coils staged at a time
+__global__ void __launch_bounds__(256) k_gram_exact(EncodeDev e, const double2* T, double lam, float4* G, float4* Gl) {
+    __shared__ float4 Si[GXC][GXT], Sj[GXC][GXT];
+    __shared__ float4 Vt[GXT][GXT + 1];
+    const int64_t t = blockIdx.x;
+    int64_t ti = (int64_t)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
+    while (ti * (ti + 1) / 2 > t) --ti;
+    while ((ti + 1) * (ti + 2) / 2 <= t) ++ti;
+    const int64_t tj = t - ti * (ti + 1) / 2;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int64_t i0 = ti * GXT, j0 = tj * GXT, j = j0 + tx;
     const int64_t Tx = 2 * e.nx - 1, Ty = 2 * e.ny - 1;
-    const int64_t t = ((int64_t)(gi[2] - gj[2] + e.nz - 1) * Ty + (gi[1] - gj[1] + e.ny - 1)) * Tx +
-                      (gi[0] - gj[0] + e.nx - 1);
-    float4 v = to_df_i(T[t]);
+    float4 v[4], sc[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int64_t i = i0 + ty + 8 * r;
+        v[r] = sc[r] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (i >= e.N || j > i) continue;
+        const int* gi = e.vox_ijk + 3 * i;
+        const int* gj = e.vox_ijk + 3 * j;
+        const int64_t at = ((int64_t)(gi[2] - gj[2] + e.nz - 1) * Ty + (gi[1] - gj[1] + e.ny - 1)) * Tx +
+                           (gi[0] - gj[0] + e.nx - 1);
+        v[r] = to_df_i(T[at]);
+    }
     if (e.coilsdf) {
-        float4 sc = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int c = 0; c < e.C; ++c)
-            cacc(sc, cdf_conj(e.coilsdf[(int64_t)c * e.N + i]), e.coilsdf[(int64_t)c * e.N + j]);
-        v = cdf_mul(v, sc);
-    } else if (e.coils) {
-        double2 sc = make_double2(0.0, 0.0);
-        for (int c = 0; c < e.C; ++c)
-            zfma(sc, zconj(e.coils[(int64_t)c * e.N + i]), e.coils[(int64_t)c * e.N + j]);
-        v = to_df_i(zmul(T[t], sc));
+        for (int c0 = 0; c0 < e.C; c0 += GXC) {
+            {
+                const int c = c0 + ty;
+                const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+                Si[ty][tx] = c < e.C && i0 + tx < e.N ? cdf_conj(e.coilsdf[(int64_t)c * e.N + i0 + tx]) : z;
+                Sj[ty][tx] = c < e.C && j < e.N ? e.coilsdf[(int64_t)c * e.N + j] : z;
+            }
+            __syncthreads();
+            const int nc = e.C - c0 < GXC ? e.C - c0 : GXC;
+            for (int c = 0; c < nc; ++c) {
+                const float4 b = Sj[c][tx];
+#pragma unroll
+                for (int r = 0; r < 4; ++r) cacc(sc[r], Si[c][ty + 8 * r], b);
+            }
+            __syncthreads();
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) v[r] = cdf_mul(v[r], sc[r]);
     }
-    if (i == j) {
-        const float2 l = f64_to_df_rn(lam);
-        float rh, rl;
-        df_add(v.x, v.y, l.x, l.y, rh, rl);
-        v.x = rh;
-        v.y = rl;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int64_t i = i0 + ty + 8 * r;
+        if (i == j) {
+            const float2 l = f64_to_df_rn(lam);
+            float rh, rl;
+            df_add(v[r].x, v[r].y, l.x, l.y, rh, rl);
+            v[r].x = rh;
+            v[r].y = rl;
+        }
+        Vt[tx][ty + 8 * r] = v[r];
+        if (i < e.N && j <= i) {
+            G[i * e.N + j] = v[r];
+            if (Gl) Gl[i * e.N + j] = v[r];
+        }
     }
-    G[i * e.N + j] = v;
-    if (j != i) G[j * e.N + i] = cdf_conj(v);
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {  // row j0 + ty + 8 r of the mirrored tile, column i0 + tx
+        const int64_t row = j0 + ty + 8 * r, col = i0 + tx;
+        if (col < e.N && row < col) G[row * e.N + col] = cdf_conj(Vt[ty + 8 * r][tx]);
+    }
 }
 
-cudaError_t launch_gram_exact(const EncodeDev& e, const double2* T, double lam, float4* G, cudaStream_t s) {
-    dim3 grid((unsigned)((e.N + 255) / 256), (unsigned)e.N);
-    k_gram_exact<<<grid, 256, 0, s>>>(e, T, lam, G);
+cudaError_t launch_gram_exact(const EncodeDev& e, const double2* T, double lam, float4* G, float4* Gl,
+                              cudaStream_t s) {
+    if (e.coils && !e.coilsdf) return cudaErrorInvalidValue;
+    const int64_t nt = (e.N + GXT - 1) / GXT;
+    k_gram_exact<<<(unsigned)(nt * (nt + 1) / 2), 256, 0, s>>>(e, T, lam, G, Gl);
     note_launch();
     return cudaGetLastError();
 }

@@ -388,7 +388,9 @@ cudaError_t launch_gram_resid_exact(const uint8_t* Gd, const int* eG, int64_t N,
 // double-float phase tables (exdf, eydf, ezdf).
 size_t toeplitz_work_bytes(const EncodeDev& e);
 cudaError_t launch_toeplitz(const EncodeDev& e, float4* work, double2* T, cudaStream_t s);
-cudaError_t launch_gram_exact(const EncodeDev& e, const double2* T, double lam, float4* G, cudaStream_t s);
+// (Gl, or null, receives the lower triangle again: the matrix the Cholesky factors)
+cudaError_t launch_gram_exact(const EncodeDev& e, const double2* T, double lam, float4* G, float4* Gl,
+                              cudaStream_t s);
 cudaError_t launch_gram_resid_df(const float4* G, int64_t N, const double2* B, const double2* X, int64_t F,
                                  double2* R, cudaStream_t s, float4* work);
 cudaError_t launch_from_df(const float4* a, int64_t n, double2* b, cudaStream_t s);
