@@ -22,6 +22,9 @@
 #include "df.cuh"
 
 namespace pinv {
+namespace tc {
+int sm_count();
+}
 
 // ------------------------------------------------------------------ double-float tile engine
 // C[i][j] = sum_k a(i,k) b(k,j) over rows i, frames j. With a split of the k
@@ -267,12 +270,18 @@ cudaError_t launch_toeplitz(const EncodeDev& e, float4* work, double2* T, cudaSt
     if (!e.exdf || !e.eydf || !e.ezdf) return cudaErrorInvalidValue;
     const int64_t Tx = 2 * e.nx - 1, Ty = 2 * e.ny - 1, Tyz = Ty * (2 * e.nz - 1), jm = (Tyz - 1) / 2;
     const int64_t rows = Tx, F = Tyz - jm, K = e.Mk;
-    // sample splits of about 128 samples (short CTAs: the table forms beside the
-    // Cholesky, whose launches need the SMs back quickly), at most 64
+    // sample splits of about 128 samples, at most 64 (the partial tables), and the largest
+    // tile that still gives every SM two CTAs: the build waits for this table, and a CTA of
+    // 64 x 64 entries and 128 samples takes 100 us, one of 16 x 16 takes 8 (issue-bound
+    // double-float MACs)
     const int sp = (int)std::max<int64_t>(1, std::min<int64_t>(64, (K + 127) / 128));
     const int64_t chunk = ((K + sp - 1) / sp + 15) / 16 * 16;
     const ToeplitzDF p{e, T, Tx, Ty, Tyz, jm};
-    cudaError_t err = df_shape<64, 64, 4, 4>(p, rows, F, sp, chunk, work, s);
+    auto ctas = [&](int64_t t) { return ((rows + t - 1) / t) * ((F + t - 1) / t) * sp; };
+    const int64_t want = 2 * tc::sm_count();
+    cudaError_t err = ctas(64) >= want   ? df_shape<64, 64, 4, 4>(p, rows, F, sp, chunk, work, s)
+                      : ctas(32) >= want ? df_shape<32, 32, 2, 2>(p, rows, F, sp, chunk, work, s)
+                                         : df_shape<16, 16, 1, 1>(p, rows, F, sp, chunk, work, s);
     if (err != cudaSuccess || sp == 1) return err;
     const int64_t n = rows * F;
     k_df_reduce<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(p, work, sp, rows, F);
@@ -359,8 +368,7 @@ __global__ void __launch_bounds__(256) k_gram_exact(EncodeDev e, const double2* 
             const float2 l = f64_to_df_rn(lam);
             float rh, rl;
             df_add(v[r].x, v[r].y, l.x, l.y, rh, rl);
-            v[r].x = rh;
-            v[r].y = rl;
+            v[r] = make_float4(rh, rl, 0.f, 0.f);  // |s_c|^2 sums: real
         }
         Vt[tx][ty + 8 * r] = v[r];
         if (i < e.N && j <= i) {
