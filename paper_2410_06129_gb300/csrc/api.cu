@@ -31,6 +31,55 @@ pinv_status cuda_fail(cudaError_t e, const char* where) {
     g_err = std::string(where) + ": " + cudaGetErrorString(e);
     return e == cudaErrorMemoryAllocation ? PINV_ERR_OOM : PINV_ERR_CUDA;
 }
+
+// Pairs (n, m) of voxels at opposite positions, m = -1 where the plan has no voxel at -r.
+// Voxel index i of an axis lies at (i - dims / 2) / dims fov, so its mirror is dims - i; the
+// y and z tables are not applied on axes of one voxel (every index mirrors itself there).
+// Each voxel of ijk ([N][3], a voxel may be listed twice) is in exactly one pair; full: the
+// voxels are the whole grid in flat order.
+std::vector<int> mirror_pairs(const int* dims, const std::vector<int>& ijk, bool full) {
+    const int N = (int)(ijk.size() / 3);
+    auto key = [&](const int* g) { return ((int64_t)g[2] * dims[1] + g[1]) * dims[0] + g[0]; };
+    std::vector<std::pair<int64_t, int>> at;  // (flat index, voxel), sorted
+    if (!full) {
+        at.resize(N);
+        for (int n = 0; n < N; ++n) at[n] = {key(&ijk[3 * n]), n};
+        std::sort(at.begin(), at.end());
+    }
+    std::vector<char> used(N, 0);
+    std::vector<int> out;
+    out.reserve(N + 64);
+    for (int n = 0; n < N; ++n) {
+        if (used[n]) continue;
+        used[n] = 1;
+        int m = -1, g[3];
+        bool inside = true;
+        for (int d = 0; d < 3; ++d) {
+            const int i = ijk[3 * n + d];
+            g[d] = d > 0 && dims[d] == 1 ? i : dims[d] - i;
+            inside = inside && g[d] < dims[d];
+        }
+        if (inside && full) {
+            const int k = (int)key(g);
+            if (!used[k]) {
+                m = k;
+                used[m] = 1;
+            }
+        } else if (inside) {
+            const int64_t k = key(g);
+            for (auto it = std::lower_bound(at.begin(), at.end(), std::make_pair(k, INT_MIN));
+                 it != at.end() && it->first == k; ++it)
+                if (!used[it->second]) {
+                    m = it->second;
+                    used[m] = 1;
+                    break;
+                }
+        }
+        out.push_back(n);
+        out.push_back(m);
+    }
+    return out;
+}
 #define CK(call)                                              \
     do {                                                      \
         cudaError_t e_ = (call);                              \
@@ -379,6 +428,7 @@ pinv_status pinv_plan_create(const pinv_plan_desc* d, void* stream, pinv_plan** 
     const bool toeplitz = p->refine_residual == PINV_RESIDUAL_TOEPLITZ;
     p->lean = d->lean != 0;
 
+    std::vector<int> pairs;  // copied to the device below, asynchronously
     // voxel grid coordinates
     std::vector<int> ijk(3 * p->N);
     for (int64_t n = 0; n < p->N; ++n) {
@@ -543,6 +593,13 @@ pinv_status pinv_plan_create(const pinv_plan_desc* d, void* stream, pinv_plan** 
             e.extdf = xt;
             e.eytdf = yt;
             e.eztdf = zt;
+            // mirror pairs for the exact E^H d
+            pairs = mirror_pairs(p->dims, ijk, !d->voxel_index);
+            int2* pd;
+            AL(pd, sizeof(int) * pairs.size(), "mirror pairs");
+            CKC(cudaMemcpyAsync(pd, pairs.data(), sizeof(int) * pairs.size(), cudaMemcpyHostToDevice, s));
+            e.pair = pd;
+            e.U = (int64_t)pairs.size() / 2;
         }
         if (e.b0tab) {
             const int64_t nt = (int64_t)tuniq.size() * p->N;

@@ -64,7 +64,10 @@ size_t apply_scratch_layout(const pinv_plan* p, int64_t F, int dtype, void* base
     // residuals and the FP64 factor-only temporary), image-space residual,
     // E^H d, the mixed path's c64 data / image / correction temporaries, and
     // the per-frame norms of the stopping rule
-    const bool need_d128 = dtype == PINV_C64 && (!md.mixed || !p->recon || md.refine);
+    const bool xadj = md.need_b && exact_adjoint_ok(p->enc, F, p->Ad != nullptr);
+    // c64 data that only the exact E^H d reads need no FP64 copy
+    const bool d32 = dtype == PINV_C64 && xadj && !(md.dfres && md.refine);
+    const bool need_d128 = dtype == PINV_C64 && !d32 && (!md.mixed || !p->recon || md.refine);
     const bool need_x128 = dtype == PINV_C64;
     const bool need_u128 = (md.refine && !md.toep) || (md.fpres && !p->recon);
     const bool need_r128 = md.refine || !p->recon;
@@ -86,27 +89,22 @@ size_t apply_scratch_layout(const pinv_plan* p, int64_t F, int dtype, void* base
     if (ctc) s.cw = cv.take<float2>(correct_tc_work_elems(N, F));
     if (atc || ctc) s.sched = cv.take<DevStatus>(1);
     if (md.dfres || md.toep || md.need_b) {
-        // E^H u (rows N, length M), E x (rows M, length N), G x (rows N, length N),
-        // and the exact tensor-core E^H d
-        size_t w = std::max(df_work_elems(N, F, M), std::max(df_work_elems(M, F, N), df_work_elems(N, F, N)));
-        const bool xadj = md.need_b && exact_adjoint_ok(p->enc, F, p->Ad != nullptr);
+        // E^H u (rows N, length M), E x (rows M, length N), G x (rows N, length N) one
+        // after another: the largest scratch of any
+        size_t w = sizeof(float4) *
+                   std::max(df_work_elems(N, F, M), std::max(df_work_elems(M, F, N), df_work_elems(N, F, N)));
         const bool xres = md.toep && md.refine && p->Gd;
         // plans with B0 and the digit tables: E x and E^H u of every residual exactly
         const bool xfwd = md.dfres && md.refine && p->Af && p->Ad && exact_adjoint_ok(p->enc, F, true);
-        if (xadj || xfwd) w = std::max(w, exact_work_elems(p->enc, F));
-        if (xres) w = std::max(w, resid_exact_work_elems(N, F));
-        if (xfwd) w = std::max(w, exact_fwd_work_elems(p->enc, F));
-        if (xadj || xres || xfwd) {
-            s.fexp = cv.take<int>((size_t)F);
-            size_t bd = std::max(xadj || xfwd ? exact_bdigit_bytes(p->enc, F) : 0,
-                                 xres ? resid_bdigit_bytes(N, F) : 0);
-            if (xfwd) bd = std::max(bd, exact_fwd_bdigit_bytes(p->enc, F));
-            s.xbd = cv.take<uint8_t>(bd);
-        }
+        if (xadj) w = std::max(w, exact_scratch_bytes(p->enc, F, d32));
+        if (xfwd) w = std::max(w, std::max(exact_scratch_bytes(p->enc, F, false), exact_fwd_scratch_bytes(p->enc, F)));
+        if (xres) w = std::max(w, resid_scratch_bytes(N, F));
+        if (xadj || xres || xfwd) s.fexp = cv.take<int>((size_t)F);
         if (xfwd) s.y128 = cv.take<double2>(exact_fwd_y_elems(p->enc, F));
         s.xadj = xadj;
+        s.d32 = d32;
         s.xfwd = xfwd;
-        s.dfw = w ? cv.take<float4>(w) : nullptr;
+        s.dfw = w ? (float4*)cv.take<uint8_t>(w) : nullptr;
     }
     if (sc) *sc = s;
     return cv.used;
@@ -147,7 +145,9 @@ pinv_status apply_impl(pinv_plan* p, const void* d_data, void* d_image, int64_t 
     };
 
     if (md.need_b) {  // b = E^H d, exactly on the tensor cores where possible
-        if (sc.xadj) CKA(launch_adjoint_exact(p->enc, D, F, sc.fexp, sc.xbd, sc.b128, sc.dfw, p->st, s, p->Ad));
+        if (sc.xadj && sc.d32)
+            CKA(launch_adjoint_exact32(p->enc, (const float2*)d_data, F, sc.fexp, sc.dfw, sc.b128, p->st, s, p->Ad));
+        else if (sc.xadj) CKA(launch_adjoint_exact(p->enc, D, F, sc.fexp, sc.dfw, sc.b128, p->st, s, p->Ad));
         else CKA(launch_adjoint_df(p->enc, D, F, 0.0, nullptr, sc.b128, s, sc.dfw));
     }
     if (!md.mixed) {
@@ -198,15 +198,14 @@ pinv_status apply_impl(pinv_plan* p, const void* d_data, void* d_image, int64_t 
         auto residual = [&]() -> cudaError_t {
             cudaError_t e;
             if (md.toep && p->Gd)  // r = b - G x, exactly on the tensor cores
-                return launch_gram_resid_exact(p->Gd, p->eG, N, sc.b128, X, F, sc.fexp, sc.xbd, sc.r128, sc.dfw,
-                                               p->st, s);
+                return launch_gram_resid_exact(p->Gd, p->eG, N, sc.b128, X, F, sc.fexp, sc.dfw, sc.r128, p->st, s);
             if (md.toep) return launch_gram_resid_df(p->Gx, N, sc.b128, X, F, sc.r128, s, sc.dfw);  // r = b - G x
             if (md.dfres && sc.xfwd) {  // u = d - E x, r = E^H u - lambda x, exact digit products
-                if ((e = launch_forward_exact(p->enc, X, F, D, sc.u128, p->Af, sc.y128, sc.fexp, sc.xbd, sc.dfw,
-                                              p->st, s)) != cudaSuccess)
+                if ((e = launch_forward_exact(p->enc, X, F, D, sc.u128, p->Af, sc.y128, sc.fexp, sc.dfw, p->st, s)) !=
+                    cudaSuccess)
                     return e;
-                if ((e = launch_adjoint_exact(p->enc, sc.u128, F, sc.fexp, sc.xbd, sc.r128, sc.dfw, p->st, s,
-                                              p->Ad)) != cudaSuccess)
+                if ((e = launch_adjoint_exact(p->enc, sc.u128, F, sc.fexp, sc.dfw, sc.r128, p->st, s, p->Ad)) !=
+                    cudaSuccess)
                     return e;
                 return launch_minus_lambda(sc.r128, X, p->lambda_abs, F * N, s);
             }

@@ -539,26 +539,21 @@ pinv_status build_condition(pinv_plan* p, cudaStream_t s) {
     // double-float products at two right-hand sides
     const bool xb0 = !toep && p->Af && p->Ad;
     float4* work = nullptr;
-    uint8_t* bd = nullptr;
     int* fexp = nullptr;
     double2* Yb = nullptr;
     CKC(take((void**)&zero, sizeof(double2) * 2 * (toep ? N : M)));
     CKC(cudaMemsetAsync(zero, 0, sizeof(double2) * 2 * (toep ? N : M), s));
     if (toep && p->Gd) {
-        const size_t wel = resid_exact_work_elems(N, 2);
         CKC(take((void**)&fexp, sizeof(int) * 2));
-        CKC(take((void**)&bd, resid_bdigit_bytes(N, 2)));
-        if (wel) CKC(take((void**)&work, sizeof(float4) * wel));
+        CKC(take((void**)&work, resid_scratch_bytes(N, 2)));
     } else if (toep) {
         const size_t wel = df_work_elems(N, 2, N);
         if (wel) CKC(take((void**)&work, sizeof(float4) * wel));
     } else if (xb0) {
-        const size_t wel = std::max(exact_work_elems(p->enc, 2), exact_fwd_work_elems(p->enc, 2));
         CKC(take((void**)&U2, sizeof(double2) * 2 * M));
         CKC(take((void**)&fexp, sizeof(int) * 2));
-        CKC(take((void**)&bd, std::max(exact_bdigit_bytes(p->enc, 2), exact_fwd_bdigit_bytes(p->enc, 2))));
         CKC(take((void**)&Yb, sizeof(double2) * exact_fwd_y_elems(p->enc, 2)));
-        if (wel) CKC(take((void**)&work, sizeof(float4) * wel));
+        CKC(take((void**)&work, std::max(exact_scratch_bytes(p->enc, 2, false), exact_fwd_scratch_bytes(p->enc, 2))));
     } else {
         const size_t wel = std::max(df_work_elems(M, 2, N), df_work_elems(N, 2, M));
         CKC(take((void**)&U2, sizeof(double2) * 2 * M));
@@ -567,14 +562,14 @@ pinv_status build_condition(pinv_plan* p, cudaStream_t s) {
     // R = B - G X by the refinement's residual operator (B = nullptr: R = -G X)
     auto resid = [&](const double2* B, const double2* X, double2* R) -> cudaError_t {
         cudaError_t e;
-        if (toep && p->Gd) return launch_gram_resid_exact(p->Gd, p->eG, N, B ? B : zero, X, 2, fexp, bd, R, work,
+        if (toep && p->Gd) return launch_gram_resid_exact(p->Gd, p->eG, N, B ? B : zero, X, 2, fexp, work, R,
                                                           p->st, s);
         if (toep) return launch_gram_resid_df(p->Gx, N, B ? B : zero, X, 2, R, s, work);
         if (xb0) {
-            if ((e = launch_forward_exact(p->enc, X, 2, nullptr, U2, p->Af, Yb, fexp, bd, work, p->st, s)) !=
+            if ((e = launch_forward_exact(p->enc, X, 2, nullptr, U2, p->Af, Yb, fexp, work, p->st, s)) !=
                 cudaSuccess)  // U = -E X
                 return e;
-            if ((e = launch_adjoint_exact(p->enc, U2, 2, fexp, bd, R, work, p->st, s, p->Ad)) != cudaSuccess)
+            if ((e = launch_adjoint_exact(p->enc, U2, 2, fexp, work, R, p->st, s, p->Ad)) != cudaSuccess)
                 return e;  // R = E^H U
             if ((e = launch_minus_lambda(R, X, p->lambda_abs, 2 * N, s)) != cudaSuccess) return e;
         } else if (p->refine_residual == PINV_RESIDUAL_DOUBLE_FLOAT) {

@@ -54,6 +54,10 @@ struct EncodeDev {
     const double2* ey;      // [Mk][ny]
     const double2* ez;      // [Mk][nz]
     const int* vox_ijk;     // [N][3] grid coordinates of voxel n
+    // mirror pairs (plans without B0 whose E^H d is exact): voxel .x and the voxel at -r of
+    // its position (.y, or -1 if the plan has none), each voxel in one pair
+    const int2* pair;
+    int64_t U;              // their number
     const double2* b0tab;   // [T][N] exp(-i2pi df_n t_u) or nullptr
     const int* tidx;        // [Mk] index u of t_m in b0tab, or nullptr
     const double2* coils;   // [C][N] s_c(n) or nullptr (C == 1, s = 1)
@@ -333,36 +337,34 @@ cudaError_t launch_gram_norm1(const double2* G, const float4* Gdf, const float4*
 // df_work_elems() partials (float4) when the split count is above one
 size_t df_work_elems(int64_t rows, int64_t F, int64_t K);
 
-// E^H d exactly on the tensor cores (fixed-point digits; F >= 16; plans with B0
-// only with the per-build table of conj(A), table = true).
-// fexp: [F] per-frame exponents (written here); Bd: exact_bdigit_bytes() for the
-// data's digit tiles (written here); work: partials.
+// E^H d exactly on the tensor cores (fixed-point digits; plans with B0 only with the
+// per-build table of conj(A), table = true). fexp: [F] per-frame exponents (written
+// here); scratch: exact_scratch_bytes() for the data's digit tiles and the partials.
 bool exact_adjoint_ok(const EncodeDev& e, int64_t F, bool table);
-size_t exact_work_elems(const EncodeDev& e, int64_t F);
-size_t exact_bdigit_bytes(const EncodeDev& e, int64_t F);
-// Ad (or nullptr): the digits of conj(A) in tile layout (adj_digit_bytes(), written
+// f32: for launch_adjoint_exact32 (c64 data)
+size_t exact_scratch_bytes(const EncodeDev& e, int64_t F, bool f32);
+// Ad (or nullptr): the digits of the A operand in tile layout (adj_digit_bytes(), written
 // by launch_adj_digits), copied instead of formed in every CTA.
 size_t adj_digit_bytes(const EncodeDev& e);
 cudaError_t launch_adj_digits(const EncodeDev& e, uint8_t* Ad, cudaStream_t s);
-cudaError_t launch_adjoint_exact(const EncodeDev& e, const double2* D, int64_t F, int* fexp, uint8_t* Bd,
-                                 double2* B, float4* work, DevStatus* st, cudaStream_t s,
-                                 const uint8_t* Ad = nullptr);
+cudaError_t launch_adjoint_exact(const EncodeDev& e, const double2* D, int64_t F, int* fexp, void* scratch,
+                                 double2* B, DevStatus* st, cudaStream_t s, const uint8_t* Ad = nullptr);
+cudaError_t launch_adjoint_exact32(const EncodeDev& e, const float2* D, int64_t F, int* fexp, void* scratch,
+                                   double2* B, DevStatus* st, cudaStream_t s, const uint8_t* Ad = nullptr);
 cudaError_t launch_transpose_df(const float4* src, int64_t rows, int64_t cols, float4* dst, int64_t ldd,
                                 cudaStream_t s);
 
 // U = D - E X exactly on the tensor cores (D may be null: U = -E X), from the
 // per-build digit table of A (fwd_digit_bytes(), launch_fwd_digits; rows of 128
 // samples, k = voxels); Y: exact_fwd_y_elems() FP64 scratch for s_c o x, fexp [F],
-// Bd: exact_fwd_bdigit_bytes(), work: exact_fwd_work_elems() partials (F >= 16,
-// as exact_adjoint_ok).
+// scratch: exact_fwd_scratch_bytes().
 size_t fwd_digit_bytes(const EncodeDev& e);
 cudaError_t launch_fwd_digits(const EncodeDev& e, uint8_t* Af, cudaStream_t s);
-size_t exact_fwd_work_elems(const EncodeDev& e, int64_t F);
-size_t exact_fwd_bdigit_bytes(const EncodeDev& e, int64_t F);
+size_t exact_fwd_scratch_bytes(const EncodeDev& e, int64_t F);
 size_t exact_fwd_y_elems(const EncodeDev& e, int64_t F);
 cudaError_t launch_forward_exact(const EncodeDev& e, const double2* X, int64_t F, const double2* D, double2* U,
-                                 const uint8_t* Af, double2* Y, int* fexp, uint8_t* Bd, float4* work,
-                                 DevStatus* st, cudaStream_t s);
+                                 const uint8_t* Af, double2* Y, int* fexp, void* scratch, DevStatus* st,
+                                 cudaStream_t s);
 // R -= lam X over n entries (FP64)
 cudaError_t launch_minus_lambda(double2* R, const double2* X, double lam, int64_t n, cudaStream_t s);
 
@@ -377,11 +379,10 @@ cudaError_t launch_apply_tc(const float2* R, int64_t N, int64_t M, const float2*
 // (gram_digit_bytes(N) bytes, written by launch_gram_digits at build time)
 size_t gram_digit_bytes(int64_t N);
 cudaError_t launch_gram_digits(const float4* G, int64_t N, int* eG, uint8_t* Gd, cudaStream_t s);
-size_t resid_exact_work_elems(int64_t N, int64_t F);
-size_t resid_bdigit_bytes(int64_t N, int64_t F);  // Bd of launch_gram_resid_exact
+size_t resid_scratch_bytes(int64_t N, int64_t F);
 cudaError_t launch_gram_resid_exact(const uint8_t* Gd, const int* eG, int64_t N, const double2* Bv,
-                                    const double2* X, int64_t F, int* fexp, uint8_t* Bd, double2* R,
-                                    float4* work, DevStatus* st, cudaStream_t s);
+                                    const double2* X, int64_t F, int* fexp, void* scratch, double2* R,
+                                    DevStatus* st, cudaStream_t s);
 
 // exact Gram of B0-free grid plans (Toeplitz table summed in double-float, kept
 // FP64; the Gram itself stored double-float). launch_toeplitz needs the

@@ -23,10 +23,11 @@ struct ApplyScratch {
     float2* d64;    // c64 copy of c128 data [F][M]
     float2* x64;    // c64 image / FP32 correction temporary [F][N]
     double* norms;  // per-frame squared norms [2F]
-    float4* dfw;    // partial sums of the split double-float products
+    float4* dfw;    // partial sums of the split double-float products, or (one product at a
+                    // time) the digit tiles and partials of the exact tensor-core ones
     int* fexp;      // per-frame exponents of the data / image [F] (exact tensor-core products)
-    uint8_t* xbd;   // digit tiles of their B operand
     bool xadj;      // E^H d by the exact tensor-core kernel
+    bool d32;       // ... which reads c64 data as they are (no FP64 copy)
     bool xfwd;      // the residual's E x and E^H u by the exact tensor-core kernels (plans with B0)
     double2* y128;  // s_c o x [F][C][N] for the exact E x
     float2* apw;    // partials of the tensor-core Recon x data

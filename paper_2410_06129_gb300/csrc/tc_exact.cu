@@ -6,10 +6,10 @@
 // instructions per complex MAC; this kernel reaches it with bf16 MMAs whose
 // every product and partial sum is an exact integer:
 //
-//  * The coil factor is taken out: the sample range is split at coil
-//    boundaries, each CTA forms sum_m conj(A[m][n]) d_c[f][m] with the
-//    coil-free |A| = 1, and multiplies its double-float partial by
-//    conj(s_c(n)) before the ordered reduction over all splits.
+//  * The coil factor is taken out: the columns of the product are the (frame, coil)
+//    pairs, each column forms sum_m conj(A[m][n]) d_c[f][m] with the coil-free
+//    |A| = 1, and its double-float partial is multiplied by conj(s_c(n)) before the
+//    ordered reduction over coils and splits. All columns share one read of A.
 //  * Each real operand value x, scaled by a power of two so |x| <= 1 (A needs
 //    none; data by the largest component of its frame), is written as
 //    x = sum_i x_i 2^(-6-7i), i = 0..5, with integer digits |x_i| <= 64
@@ -19,34 +19,44 @@
 //    weight class w = i + j accumulate in one TMEM region (six regions of 64
 //    columns); the 21 pairs with w <= 5 are kept (dropped pairs weigh below
 //    2^-42 relative).
-//  * Every DRAIN stages (each class sum then stays below 2^24) the producer
-//    warps read the six regions, scale class w by 2^(-12-7w) (exact) and add
-//    it into double-float accumulators held in registers.
+//  * Every XDRAIN stages the producer warps read the regions of classes 3 to 5, and
+//    every second time those of classes 0 to 2 (fewer pairs, so their sums stay
+//    below 2^24 twice as long), scale class w by 2^(-12-7w) (exact) and add it into
+//    double-float accumulators held in registers.
 //
-// Tiles are 128 voxels x 32 frames (64 output columns, real and imaginary side
-// by side, as in the split-BF16 engine), or 128 x 8 for calls of at most eight
-// frames (the condition estimate's two vectors, small requests: the MMAs of a
-// 32-frame tile would be mostly padding); the sample range is split over CTAs
-// and the double-float partials reduced in a fixed order. One MMA takes an A
-// digit against up to four B digits stacked along N (N <= 256, or 64 for the
-// narrow tile), so a stage's 21 digit pairs cost 8 MMAs per 16-deep k half. Every
-// entry's digit products, class sums and drains are the same whatever the tile. The producers form conj(A) from the
-// separable phase tables of plans without B0; plans with B0 copy the digits of
-// conj(A) (with its B0 factor) from a per-build table.
+// Mirror pairs (plans without B0). Voxels sit at r = (i - dims/2)/dims fov, so voxel
+// dims - i is at -r and A there is the complex conjugate. The A operand is then real:
+// each pair (n, its mirror) owns two rows, cos and sin of 2 pi k . r over 32 samples a
+// stage, the B columns hold the data's real and imaginary parts once each, and with
+// P = sum cos d, Q = sum sin d the pair's results are P + iQ and P - iQ, combined after
+// the last drain. A 128-row tile covers 128 voxels and 32 samples a stage where the
+// complex embedding covers 16: half the MMAs, half the digit table and half the data
+// digits. A voxel without a mirror in the plan (grid edge, mask) is a pair of one, which
+// costs what the complex embedding would. Measured with folded columns and the longer
+// drain groups: see k_exact.
+//
+// Tiles are 128 rows x 32 columns (64 output columns, real and imaginary parts side
+// by side, as in the split-BF16 engine), or narrower (16, 8) where there are fewer
+// columns: the MMAs of a 32-column tile would be mostly padding. The k range is split
+// over CTAs and the double-float partials reduced in a fixed order. One MMA takes an A
+// digit against up to four B digits stacked along N (N <= 256), so a stage's 21 digit
+// pairs cost 8 MMAs per 16-deep k half. Every entry's digit products, class sums and
+// drains are the same whatever the tile. The producers form the cos and sin rows from
+// the separable phase tables; plans with B0 copy the digits of conj(A) (with its B0
+// factor) from a per-build table.
 //
 // The forward product E x (XFWD) runs the same way with the roles of samples and
 // voxels exchanged: the A operand is a per-build table of the digits of A itself
-// (rows of 128 samples, k = voxels), the B operand the digits of s_c(n) x[f][n]
-// per coil, and each coil's samples get their own partial sums, reduced into
-// u = d - E x. With both, the refinement residual r = E^H (d - E x) - lambda x of
+// (rows of 128 samples, k = voxels), the B operand the digits of s_c(n) x[f][n], one
+// column per frame and coil, reduced into u = d - E x. With both, the refinement residual r = E^H (d - E x) - lambda x of
 // plans with B0 runs on the tensor cores too.
 //
 // The digits of the B operand (data, or x) are written once per call by
 // k_b_digits. The digits of the A operand either come from the producer warps
 // (XGEN) or are copied with one bulk copy per stage from a table in the stage layout:
-// the exact Gram's digit tiles for the refinement residual (XGRAM), or the
-// digits of conj(A) written once per build (XADJT; the same digits XGEN
-// forms, which it would otherwise form again for every coil and frame tile).
+// the exact Gram's digit tiles for the refinement residual (XGRAM), the cos and sin
+// digits written once per build (XADJP; the same digits XGEN forms, which it would
+// otherwise form again for every column tile), or with B0 those of conj(A) (XADJT).
 #include <algorithm>
 #include <cstdlib>
 
@@ -59,16 +69,16 @@ namespace tcx {
 using namespace tc;
 
 constexpr int XM = 128;        // voxels per tile
-constexpr int XN = 32;         // frames per tile (MMA N = 64 per B digit)
-constexpr int XNN = 8;         // frames per tile of the narrow variant (MMA N = 16 per B digit)
-constexpr int XKC = 16;        // complex samples per stage
+constexpr int XN = 32;         // columns per tile (MMA N = 64 per B digit); 16 and 8: narrow tiles
+constexpr int XKC = 16;        // complex k per stage
+constexpr int XKP = 32;        // samples per stage with mirror pairs (real operands)
 constexpr int NDIG = 6;        // digits per real value
 constexpr int NCLS = 6;        // weight classes kept (i + j <= 5)
-constexpr int XDRAIN = 16;     // stages per exact accumulation group
+constexpr int XDRAIN = 21;     // stages per exact accumulation group (classes 0 to 2: two groups)
 constexpr int XSTAGES = 3;
 constexpr int XA_SL = XM * 64;         // one digit slice of A: 128 rows x 32 bf16 = 8 KiB
-// per frame-tile width XNT: one digit slice of B (2 XNT stacked rows x 32 bf16: 4 KiB
-// for 32 frames), a stage (72 KiB for 32 frames) and the dynamic shared memory
+// per column-tile width XNT: one digit slice of B (2 XNT stacked rows x 32 bf16: 4 KiB
+// for 32 columns), a stage (72 KiB for 32 columns) and the dynamic shared memory
 template <int XNT>
 struct XS {
     static constexpr int B_SL = 2 * XNT * 64;
@@ -83,17 +93,19 @@ __host__ __device__ constexpr uint32_t xidesc(int n) {
 // throughout), so slices j0 .. j0 + nd - 1 form one operand of 2 XNT nd rows, and
 // the classes i + j of A digit i are adjacent TMEM regions of 2 XNT columns: one
 // MMA covers several digit pairs. Per A digit i: (first B slice, B slices) of its
-// MMAs, at most four slices.
+// MMAs, at most four slices; digit 0's runs part at class 3, whose sums restart with
+// every group, those below with every second one.
 struct XPairRun {
     int i, j0, nd;
 };
 __device__ __forceinline__ XPairRun xrun(int r) {
-    constexpr XPairRun t[8] = {{0, 0, 4}, {0, 4, 2}, {1, 0, 4}, {1, 4, 1},
+    constexpr XPairRun t[8] = {{0, 0, 3}, {0, 3, 3}, {1, 0, 4}, {1, 4, 1},
                                {2, 0, 4}, {3, 0, 3}, {4, 0, 2}, {5, 0, 1}};
     return t[r];
 }
-// Per class and group: at most 6 pairs x 32 products x XDRAIN stages, each below 2^12.
-static_assert(NCLS * 32 * XDRAIN * 4096 < (1 << 24), "exact class sums");
+// Per class and group: w + 1 pairs x 32 products x XDRAIN stages, each at most 2^12;
+// classes 0 to 2 over two groups.
+static_assert(NCLS * 32 * XDRAIN * 4096 < (1 << 24) && 3 * 32 * 2 * XDRAIN * 4096 < (1 << 24), "exact class sums");
 
 __device__ inline float rint_f(float x) { return rintf(x); }
 
@@ -131,18 +143,16 @@ struct Digits8 {
 
 struct XArgs {
     EncodeDev e;
-    const double2* D;   // adjoint: data [F][M]; Gram residual: x [F][N] (FP64)
     const int* fexp;    // per-frame exponent: |D_f| <= 2^fexp
-    int64_t F, M;
-    int64_t chunk;      // k per split (multiple of XKC); adjoint splits never cross a coil
-    int sub;            // splits per coil (Gram residual: splits)
-    float4* part;       // [splits][F][N] double-float partials, or null (one split, no coil maps)
-    double2* B;         // output [F][N] when part is null
-    const uint8_t* Gd;  // Gram residual: digit tiles of G ([row block][k block][digit] x 8 KiB)
-    const int* eG;      // Gram residual: |G| <= 2^eG
-    int64_t KB;         // k blocks of 16 per row block (per coil for the adjoint)
-    const uint8_t* Bd;  // digit tiles of the B operand (k_b_digits)
+    int64_t Q;          // columns: frames x coils (column q = frame q / C, coil q % C)
     int C;              // coils (Gram residual: 1)
+    int64_t chunk;      // k per split (a multiple of the stage's k)
+    float4* part;       // [splits][Q][rows] double-float partials, or null (one split, no coil maps)
+    double2* B;         // output [Q][rows] when part is null
+    const uint8_t* At;  // A operand digit tiles ([row block][k block][digit] x 8 KiB); XGEN: null
+    const int* eG;      // Gram residual: |G| <= 2^eG
+    int64_t KB;         // k blocks (stages) of the whole k range
+    const uint8_t* Bd;  // digit tiles of the B operand (k_b_digits)
 };
 
 // conj(A[m][n]) for 8 consecutive samples m (< mend) of voxel n, double-float,
@@ -183,7 +193,36 @@ __device__ inline void gen_ah8(const EncodeDev& e, int64_t n, int64_t m, int64_t
 }
 
 // A operand of the exact kernel
-enum XMode { XGEN = 0, XGRAM = 1, XADJT = 2, XFWD = 3 };
+enum XMode { XGEN = 0, XGRAM = 1, XADJT = 2, XFWD = 3, XADJP = 4 };
+
+// cos (re) and sin (im) of 2 pi k_m . r for 8 consecutive samples of mirror pair p
+// (zeros past the last pair or sample): conj(A) of the pair's first voxel
+__device__ inline void gen_pair8(const EncodeDev& e, int64_t p, int64_t m, int64_t mend, float (&reh)[8],
+                                 float (&rel)[8], float (&imh)[8], float (&iml)[8]) {
+    gen_ah8(e, p < e.U ? (int64_t)e.pair[p].x : e.N, m, mend, reh, rel, imh, iml);
+}
+
+// Digits of the cos and sin rows of one (64 mirror pairs, 32-sample chunk): pair p owns
+// rows 2 p and 2 p + 1 of its tile. NDIG slices of 8 KiB in the stage layout, exactly as
+// the XGEN producers write them to shared memory.
+__global__ void __launch_bounds__(256) k_pair_digits(EncodeDev e, int64_t KB, uint8_t* Ad) {
+    const int64_t kb = blockIdx.x, rb = blockIdx.y;
+    const int ra = threadIdx.x & (XM / 2 - 1), ga = threadIdx.x >> 6;
+    float reh[8], rel[8], imh[8], iml[8];
+    gen_pair8(e, rb * (XM / 2) + ra, kb * XKP + 8 * ga, e.Mk, reh, rel, imh, iml);
+    Digits8 dr, di;
+    dr.init(reh, rel, 1.f);
+    di.init(imh, iml, 1.f);
+    uint8_t* blk = Ad + (rb * KB + kb) * (int64_t)(NDIG * XA_SL);
+#pragma unroll
+    for (int dg = 0; dg < NDIG; ++dg) {
+        uint32_t w[4];
+        dr.next(w, 0u);
+        *reinterpret_cast<uint4*>(blk + dg * XA_SL + koff(2 * ra, ga)) = make_uint4(w[0], w[1], w[2], w[3]);
+        di.next(w, 0u);
+        *reinterpret_cast<uint4*>(blk + dg * XA_SL + koff(2 * ra + 1, ga)) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+}
 
 // Digits of conj(A) for one (voxel tile, 16-sample chunk): NDIG slices of 8 KiB in
 // the stage layout, exactly as the XGEN producers write them to shared memory.
@@ -249,35 +288,41 @@ __global__ void k_coil_times(EncodeDev e, const double2* X, int64_t F, double2* 
     Y[idx] = from_df(v);
 }
 
-// Digits of the B operand (data d, or x for the Gram residual) for one (XNT-frame
-// tile, coil, 16-sample chunk): NDIG slices of B_SL bytes in the stage layout.
-// Frame f of the tile owns row f, [Br | -Bi], and row XNT + f, [Bi | Br], each value
-// scaled by 2^-fexp[f]; samples at or past Kc (the coil's end) and frames at or past
-// F are zero. Value (f, c, m) is D[f * ld + c * Kc + m]. 256 / (2 XNT) chunks per
-// 256-thread block, one (frame, 8 samples) unit per thread.
-template <int XNT>
-__global__ void __launch_bounds__(256) k_b_digits(const double2* D, int64_t ld, int64_t F, int C, int64_t Kc,
-                                                  int64_t KB, const int* fexp, uint8_t* Bd) {
-    constexpr int TPT = 2 * XNT;  // threads per chunk
-    const int64_t FT = (F + XNT - 1) / XNT;
+// Values of a B operand in double-float: FP64 (x of a residual, c128 data) or FP32 (c64
+// data, exact as it is)
+__device__ inline float4 b_value(double2 v) { return to_df_i(v); }
+__device__ inline float4 b_value(float2 v) { return make_float4(v.x, 0.f, v.y, 0.f); }
+
+// Digits of the B operand (data d, or x for the Gram residual) for one (XNT-column
+// tile, k chunk): NDIG slices of B_SL bytes in the stage layout, each value scaled by
+// 2^-fexp[frame]; k at or past Kc and columns at or past Q are zero. Column q is the row
+// D + q Kc. Complex embedding (PAIR = false, 16 k per chunk): column c of the tile owns
+// row c, [Br | -Bi], and row XNT + c, [Bi | Br]. Real operands (PAIR, 32 k per chunk):
+// row c holds Br, row XNT + c holds Bi. One (column, 8 k) unit per thread, consecutive
+// threads along the column's k groups (their reads are contiguous).
+template <int XNT, bool PAIR, class T>
+__global__ void __launch_bounds__(256) k_b_digits(const T* D, int64_t Q, int C, int64_t Kc, int64_t KB,
+                                                  const int* fexp, uint8_t* Bd) {
+    constexpr int GPC = PAIR ? 4 : 2;    // groups of 8 k per chunk
+    constexpr int TPT = GPC * XNT;       // threads per chunk
+    const int64_t CT = (Q + XNT - 1) / XNT;
     const int64_t tile = (int64_t)blockIdx.x * (256 / TPT) + threadIdx.x / TPT;
-    if (tile >= FT * C * KB) return;
-    const int64_t kb = tile % KB, fc = tile / KB;
-    const int c = (int)(fc % C);
-    const int cb = (int)(threadIdx.x % XNT), gb = (int)((threadIdx.x / XNT) & 1);
-    const int64_t f = (fc / C) * XNT + cb;
-    const int64_t mk0 = kb * XKC + 8 * gb;
+    if (tile >= CT * KB) return;
+    const int64_t kb = tile % KB;
+    const int u = (int)(threadIdx.x % TPT), cb = u / GPC, gb = u % GPC;
+    const int64_t q = (tile / KB) * XNT + cb;
+    const int64_t mk0 = kb * (8 * GPC) + 8 * gb;
     float reh[8], rel[8], imh[8], iml[8];
 #pragma unroll
     for (int t = 0; t < 8; ++t) {
         const int64_t m = mk0 + t;
-        const float4 v = to_df_i((f < F && m < Kc) ? D[f * ld + (int64_t)c * Kc + m] : make_double2(0.0, 0.0));
+        const float4 v = q < Q && m < Kc ? b_value(D[q * Kc + m]) : make_float4(0.f, 0.f, 0.f, 0.f);
         reh[t] = v.x;
         rel[t] = v.y;
         imh[t] = v.z;
         iml[t] = v.w;
     }
-    const float scale = f < F ? __int_as_float((127 - fexp[f]) << 23) : 1.f;
+    const float scale = q < Q ? __int_as_float((127 - fexp[q / C]) << 23) : 1.f;
     Digits8 dr, di;
     dr.init(reh, rel, scale);
     di.init(imh, iml, scale);
@@ -288,26 +333,30 @@ __global__ void __launch_bounds__(256) k_b_digits(const double2* D, int64_t ld, 
         dr.next(wr, 0u);
         di.next(wi, 0u);
         uint8_t* sl = bb + dg * XS<XNT>::B_SL;
-        *reinterpret_cast<uint4*>(sl + koff(cb, gb)) = make_uint4(wr[0], wr[1], wr[2], wr[3]);  // [Br|-Bi]
-        *reinterpret_cast<uint4*>(sl + koff(cb, gb + 2)) =
-            make_uint4(wi[0] ^ 0x80008000u, wi[1] ^ 0x80008000u, wi[2] ^ 0x80008000u, wi[3] ^ 0x80008000u);
-        *reinterpret_cast<uint4*>(sl + koff(XNT + cb, gb)) = make_uint4(wi[0], wi[1], wi[2], wi[3]);  // [Bi|Br]
-        *reinterpret_cast<uint4*>(sl + koff(XNT + cb, gb + 2)) = make_uint4(wr[0], wr[1], wr[2], wr[3]);
+        *reinterpret_cast<uint4*>(sl + koff(cb, gb)) = make_uint4(wr[0], wr[1], wr[2], wr[3]);
+        *reinterpret_cast<uint4*>(sl + koff(XNT + cb, gb)) = make_uint4(wi[0], wi[1], wi[2], wi[3]);
+        if constexpr (!PAIR) {
+            *reinterpret_cast<uint4*>(sl + koff(cb, gb + 2)) =
+                make_uint4(wi[0] ^ 0x80008000u, wi[1] ^ 0x80008000u, wi[2] ^ 0x80008000u, wi[3] ^ 0x80008000u);
+            *reinterpret_cast<uint4*>(sl + koff(XNT + cb, gb + 2)) = make_uint4(wr[0], wr[1], wr[2], wr[3]);
+        }
     }
 }
 
-// XGEN / XADJT: b = E^H d; XGRAM: G x with the digits of G in tile layout and x as
-// the B operand. The B operand's digit tiles (k_b_digits) are copied per stage.
+// XGEN / XADJP / XADJT: b = E^H d; XGRAM: G x with the digits of G in tile layout and x
+// as the B operand; XFWD: E x. The B operand's digit tiles (k_b_digits) are copied per stage.
 //
-// One-dimensional grid, frame tile fastest, then coil, row block and split: the
-// CTAs that read one A tile (all frame tiles and coils of a row block and split)
-// run side by side and share it in L2.
+// One-dimensional grid, column tile fastest, then row block and split: the CTAs that
+// read one A tile (all column tiles of a row block and split) run side by side and
+// share it in L2.
 template <int MODE, int XNT>
 __global__ void __launch_bounds__(NTHREADS, 1) k_exact(XArgs a, DevStatus* st) {
     constexpr bool GRAM = MODE == XGRAM;
     constexpr bool FWD = MODE == XFWD;
+    constexpr bool PAIR = MODE == XGEN || MODE == XADJP;
+    constexpr int KS = PAIR ? XKP : XKC;     // k per stage
     constexpr int B_SL = XS<XNT>::B_SL, XSTAGE = XS<XNT>::STAGE;
-    constexpr int FPT = XNT / 2;  // frames per drain thread (two halves of the tile)
+    constexpr int FPT = XNT / 2;  // columns per drain thread (two halves of the tile)
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t full_bar[XSTAGES], empty_bar[XSTAGES];
     __shared__ uint64_t abar[XSTAGES];  // the stage's bulk copies (their bytes)
@@ -317,24 +366,20 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_exact(XArgs a, DevStatus* st) {
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long wlim = st->wait_limit > 0 ? st->wait_limit : WAIT_LIMIT;  // pipeline waits
-    // output rows (voxels; samples of one coil for the forward product)
+    // output rows (voxels; samples for the forward product), tile rows (pairs: two each)
     const int64_t N = FWD ? a.e.Mk : a.e.N;
-    const int64_t FT = (a.F + XNT - 1) / XNT, RB = (N + XM - 1) / XM;
+    const int64_t CT = (a.Q + XNT - 1) / XNT, RB = ((PAIR ? 2 * a.e.U : N) + XM - 1) / XM;
     int64_t lin = blockIdx.x;
-    const int64_t ft = lin % FT;
-    lin /= FT;
-    const int coil = (int)(lin % a.C);
-    lin /= a.C;
+    const int64_t ct = lin % CT;
+    lin /= CT;
     const int64_t rb = lin % RB;
     const int split = (int)(lin / RB);
-    const int64_t zpart = (int64_t)coil * a.sub + split;  // partial slot
-    const int64_t n0 = rb * XM, f0 = ft * XNT;
-    // k range [mb, me): adjoint samples inside coil `coil`, Gram columns, or the
-    // voxels of the forward product
+    const int64_t q0 = ct * XNT;
+    // k range [mb, me): samples, Gram columns, or the voxels of the forward product
     const int64_t Mk = GRAM ? N : (FWD ? a.e.N : a.e.Mk);
     const int64_t mb = (int64_t)split * a.chunk;
     const int64_t me = mb + a.chunk < Mk ? mb + a.chunk : Mk;
-    const int nk = me > mb ? (int)((me - mb + XKC - 1) / XKC) : 0;
+    const int nk = me > mb ? (int)((me - mb + KS - 1) / KS) : 0;
     const int ngroups = (nk + XDRAIN - 1) / XDRAIN;
 
     if (threadIdx.x == 0) {
@@ -365,18 +410,30 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_exact(XArgs a, DevStatus* st) {
         bool ok = true;
         int drained = 0;
         auto drain = [&](int g) -> bool {
-            if (!mbar_wait(&tfull, (uint32_t)g & 1u, &abort_flag, wlim)) return false;
+            // the warp decides together: its TMEM loads need every lane
+            if (!__all_sync(0xffffffffu, mbar_wait(&tfull, (uint32_t)g & 1u, &abort_flag, wlim))) return false;
             tc_fence_after();
+            // classes 0 to 2 gather two groups
 #pragma unroll 1
-            for (int w = 0; w < NCLS; ++w) {
-                // region w: columns 2 XNT w .. (real parts of the tile's frames, then imaginary)
+            for (int w = (g & 1) || g == ngroups - 1 ? 0 : 3; w < NCLS; ++w) {
+                // region w: columns 2 XNT w .. (real parts of the tile's columns, then imaginary)
                 uint32_t vr[FPT], vi[FPT];
                 if constexpr (XNT == 32) {
                     tmem_ld16(trow + (uint32_t)(64 * w + 16 * h), vr);
                     tmem_ld16(trow + (uint32_t)(64 * w + XNT + 16 * h), vi);
                     tmem_wait_ld();
+                } else if constexpr (XNT == 16) {
+                    uint32_t v[16], z[16];
+                    tmem_ld16(trow + (uint32_t)(32 * w), v);
+                    tmem_ld16(trow + (uint32_t)(32 * w + XNT), z);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int u = 0; u < FPT; ++u) {  // constant indices: v, z stay in registers
+                        vr[u] = h ? v[FPT + u] : v[u];
+                        vi[u] = h ? z[FPT + u] : z[u];
+                    }
                 } else {
-                    static_assert(XNT == 8, "tile widths 32 and 8");
+                    static_assert(XNT == 8, "tile widths 32, 16 and 8");
                     uint32_t v[16];
                     tmem_ld16(trow + (uint32_t)(16 * w), v);
                     tmem_wait_ld();
@@ -402,25 +459,26 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_exact(XArgs a, DevStatus* st) {
             mbar_arrive(&tempty);
             return true;
         };
-        // A unit (XGEN): voxel row ua & 127, 8 samples of k-group ua >> 7
-        const int ua = threadIdx.x, ra = ua & (XM - 1), ga = ua >> 7;
-        const int64_t nrow = n0 + ra;
+        // A unit (XGEN): mirror pair ua & 63, 8 samples of k-group ua >> 6
+        const int ua = threadIdx.x, ra = ua & (XM / 2 - 1), ga = ua >> 6;
         int a_issued = 0;  // stages whose tiles this thread (thread 0) has started copying
         constexpr uint32_t kTx = (MODE != XGEN ? NDIG * XA_SL : 0) + NDIG * B_SL;
-        const uint8_t* bsrc = a.Bd + ((ft * a.C + coil) * a.KB) * (int64_t)(NDIG * B_SL);
+        const uint8_t* bsrc = a.Bd + ct * a.KB * (int64_t)(NDIG * B_SL);
         for (int kt = 0; kt < nk && ok; ++kt) {
             const int s = kt % XSTAGES;
             const uint32_t ph = (uint32_t)(kt / XSTAGES) & 1u;
-            if (kt >= XSTAGES && !(ok = mbar_wait(&empty_bar[s], ph ^ 1u, &abort_flag, wlim))) break;
+            if (kt >= XSTAGES &&
+                !(ok = __all_sync(0xffffffffu, mbar_wait(&empty_bar[s], ph ^ 1u, &abort_flag, wlim))))
+                break;
             uint8_t* base = smem + s * XSTAGE;
-            const int64_t m0 = mb + (int64_t)kt * XKC;  // k index (sample inside the coil, or Gram column)
-            const int64_t kb = m0 / XKC;
+            const int64_t m0 = mb + (int64_t)kt * KS;  // first k of the stage
+            const int64_t kb = m0 / KS;
             if (threadIdx.x == 0) {
                 // the stage's digit tiles: A (NDIG x 8 KiB, unless formed below) and
-                // B (NDIG x 4 KiB), counted in bytes on abar
+                // B (NDIG x B_SL), counted in bytes on abar
                 mbar_arrive_expect_tx(&abar[s], kTx);
                 if (MODE != XGEN)
-                    bulk_g2s(base, a.Gd + (rb * a.KB + kb) * (int64_t)(NDIG * XA_SL), (uint32_t)(NDIG * XA_SL),
+                    bulk_g2s(base, a.At + (rb * a.KB + kb) * (int64_t)(NDIG * XA_SL), (uint32_t)(NDIG * XA_SL),
                              &abar[s]);
                 bulk_g2s(base + NDIG * XA_SL, bsrc + kb * (int64_t)(NDIG * B_SL), (uint32_t)(NDIG * B_SL),
                          &abar[s]);
@@ -428,7 +486,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_exact(XArgs a, DevStatus* st) {
             }
             if constexpr (MODE == XGEN) {
                 float reh[8], rel[8], imh[8], iml[8];
-                gen_ah8(a.e, nrow, m0 + 8 * ga, me, reh, rel, imh, iml);
+                gen_pair8(a.e, rb * (XM / 2) + ra, m0 + 8 * ga, me, reh, rel, imh, iml);
                 Digits8 dr, di;
                 dr.init(reh, rel, 1.f);
                 di.init(imh, iml, 1.f);
@@ -436,9 +494,10 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_exact(XArgs a, DevStatus* st) {
                 for (int dg = 0; dg < NDIG; ++dg) {
                     uint32_t w[4];
                     dr.next(w, 0u);
-                    *reinterpret_cast<uint4*>(base + dg * XA_SL + koff(ra, ga)) = make_uint4(w[0], w[1], w[2], w[3]);
+                    *reinterpret_cast<uint4*>(base + dg * XA_SL + koff(2 * ra, ga)) =
+                        make_uint4(w[0], w[1], w[2], w[3]);
                     di.next(w, 0u);
-                    *reinterpret_cast<uint4*>(base + dg * XA_SL + koff(ra, ga + 2)) =
+                    *reinterpret_cast<uint4*>(base + dg * XA_SL + koff(2 * ra + 1, ga)) =
                         make_uint4(w[0], w[1], w[2], w[3]);
                 }
                 fence_proxy_async();
@@ -455,25 +514,46 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_exact(XArgs a, DevStatus* st) {
             ok = drain(drained);
             ++drained;
         }
-        if (ok && !abort_flag) {
-            // this thread: voxel n0 + q*32 + lane, frames f0 + FPT h .. + FPT - 1
-            const int64_t n = n0 + q * 32 + lane;
-            if (n < N) {
-                float4 cs = make_float4(1.f, 0.f, 0.f, 0.f);
-                if (!GRAM && !FWD && a.e.coilsdf) cs = cdf_conj(a.e.coilsdf[(int64_t)coil * N + n]);
-                const int eA = GRAM ? *a.eG : 0;
+        // (the flag may rise at any time: the decision to write is the warp's)
+        if (__all_sync(0xffffffffu, ok && !abort_flag)) {
+            // this thread: tile row q * 32 + lane, columns q0 + FPT h .. + FPT - 1
+            const int64_t row = rb * XM + q * 32 + lane;
+            int64_t n = row;  // output row, or out of range
+            if constexpr (PAIR) {
+                // even rows hold P = sum cos d, odd rows Q = sum sin d of the pair: its
+                // first voxel takes P + iQ (written by the even lane), its mirror P - iQ
+                const int2 pr = (row >> 1) < a.e.U ? a.e.pair[row >> 1] : make_int2(-1, -1);
+                n = (lane & 1) ? pr.y : pr.x;
+                if (n < 0) n = N;
+            }
+            const int eA = GRAM ? *a.eG : 0;
 #pragma unroll
-                for (int u = 0; u < FPT; ++u) {
-                    const int64_t f = f0 + FPT * h + u;
-                    if (f >= a.F) continue;
-                    const float sc = __int_as_float((127 + eA + a.fexp[f]) << 23);
-                    float4 v = make_float4(acc[0][u] * sc, acc[1][u] * sc, acc[2][u] * sc, acc[3][u] * sc);
-                    if (!GRAM && !FWD && a.e.coilsdf) v = cdf_mul(v, cs);
-                    if (a.part)
-                        a.part[(zpart * a.F + f) * N + n] = v;
-                    else
-                        a.B[f * N + n] = from_df(v);
+            for (int u = 0; u < FPT; ++u) {
+                float4 v = make_float4(acc[0][u], acc[1][u], acc[2][u], acc[3][u]);
+                if constexpr (PAIR) {
+                    const float4 o = make_float4(__shfl_xor_sync(0xffffffffu, v.x, 1), __shfl_xor_sync(0xffffffffu, v.y, 1),
+                                                 __shfl_xor_sync(0xffffffffu, v.z, 1), __shfl_xor_sync(0xffffffffu, v.w, 1));
+                    float rh, rl, ih, il;
+                    if (lane & 1) {  // P in o, Q in v: (Pr + Qi) + i (Pi - Qr)
+                        df_add(o.x, o.y, v.z, v.w, rh, rl);
+                        df_add(o.z, o.w, -v.x, -v.y, ih, il);
+                    } else {         // P in v, Q in o: (Pr - Qi) + i (Pi + Qr)
+                        df_add(v.x, v.y, -o.z, -o.w, rh, rl);
+                        df_add(v.z, v.w, o.x, o.y, ih, il);
+                    }
+                    v = make_float4(rh, rl, ih, il);
                 }
+                const int64_t qc = q0 + FPT * h + u;
+                if (qc >= a.Q || n >= N) continue;
+                const int64_t f = qc / a.C;
+                const float sc = __int_as_float((127 + eA + a.fexp[f]) << 23);
+                v = make_float4(v.x * sc, v.y * sc, v.z * sc, v.w * sc);
+                if (!GRAM && !FWD && a.e.coilsdf)
+                    v = cdf_mul(v, cdf_conj(a.e.coilsdf[(qc - f * a.C) * N + n]));
+                if (a.part)
+                    a.part[((int64_t)split * a.Q + qc) * N + n] = v;
+                else
+                    a.B[qc * N + n] = from_df(v);
             }
         }
         if (threadIdx.x == 0) {
@@ -499,12 +579,14 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_exact(XArgs a, DevStatus* st) {
             for (int kk = 0; kk < 2; ++kk) {
 #pragma unroll
                 for (int r = 0; r < 8; ++r) {
-                    // the runs of A digit 0 cover all six regions: they start each group
+                    // the runs of A digit 0 cover all six regions: they start each group,
+                    // the first (classes 0 to 2) every second one
                     const XPairRun u = xrun(r);
+                    const bool fresh = first && u.i == 0 && kk == 0 && (u.j0 > 0 || (g & 1) == 0);
                     const uint64_t da = sdesc(abase + u.i * XA_SL + kk * 256, 128, 512);
                     const uint64_t db = sdesc(bbase + u.j0 * B_SL + kk * 256, 128, 512);
                     mma_bf16(tmem + (uint32_t)(2 * XNT * (u.i + u.j0)), da, db, xidesc(2 * XNT * u.nd),
-                             (first && u.i == 0 && kk == 0) ? 0u : 1u);
+                             fresh ? 0u : 1u);
                 }
             }
             mma_commit(&empty_bar[s]);
@@ -523,26 +605,21 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_exact(XArgs a, DevStatus* st) {
     if (threadIdx.x == 0 && abort_flag) atomicMax(&st->timeout_site, 20);
 }
 
-// store functor for the ordered reduction of the partials
-struct BStore {
-    double2* B;
-    int64_t N;
-    __device__ void store(int64_t i, int64_t j, double2 v) const { B[j * N + i] = v; }
-};
-
-__global__ void k_exact_reduce(BStore o, const float4* part, int splits, int64_t rows, int64_t F) {
+// B[f][i] = the partials of frame f's columns (coils) and splits, coil by coil in split order
+__global__ void k_exact_reduce(double2* B, const float4* part, int splits, int C, int64_t rows, int64_t F) {
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= rows * F) return;
-    const int64_t i = idx % rows, j = idx / rows;
-    float4 a = part[j * rows + i];
-    for (int z = 1; z < splits; ++z) {
-        const float4 b = part[((int64_t)z * F + j) * rows + i];
-        float rh, rl, ih, il;
-        df_add(a.x, a.y, b.x, b.y, rh, rl);
-        df_add(a.z, a.w, b.z, b.w, ih, il);
-        a = make_float4(rh, rl, ih, il);
-    }
-    o.store(i, j, from_df(a));
+    const int64_t i = idx % rows, f = idx / rows, Q = F * C;
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int c = 0; c < C; ++c)
+        for (int z = 0; z < splits; ++z) {
+            const float4 b = part[((int64_t)z * Q + f * C + c) * rows + i];
+            float rh, rl, ih, il;
+            df_add(a.x, a.y, b.x, b.y, rh, rl);
+            df_add(a.z, a.w, b.z, b.w, ih, il);
+            a = make_float4(rh, rl, ih, il);
+        }
+    B[idx] = from_df(a);
 }
 
 // r[f][n] = b[f][n] - sum_z part[z][f][n], partials added in order
@@ -562,19 +639,14 @@ __global__ void k_resid_reduce(const double2* b, const float4* part, int splits,
     r[idx] = make_double2(bb.x - g.x, bb.y - g.y);
 }
 
-// u[f][c Mk + m] = d[f][c Mk + m] - sum_s part[c sub + s][f][m] (d may be null:
-// u = -E x), the splits of each coil added in order
-__global__ void k_fwd_reduce(const double2* d, const float4* part, int sub, int C, int64_t Mk, int64_t F,
-                             double2* u) {
+// u[q][m] = d[q][m] - sum_s part[s][q][m] for every column q = (frame, coil) (d may be
+// null: u = -E x), the splits added in order
+__global__ void k_fwd_reduce(const double2* d, const float4* part, int splits, int64_t n, double2* u) {
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t M = Mk * C;
-    if (idx >= M * F) return;
-    const int64_t f = idx / M, cm = idx % M;
-    const int c = (int)(cm / Mk);
-    const int64_t m = cm % Mk;
-    float4 a = part[(((int64_t)c * sub) * F + f) * Mk + m];
-    for (int z = 1; z < sub; ++z) {
-        const float4 b = part[(((int64_t)c * sub + z) * F + f) * Mk + m];
+    if (idx >= n) return;
+    float4 a = part[idx];
+    for (int z = 1; z < splits; ++z) {
+        const float4 b = part[(int64_t)z * n + idx];
         float rh, rl, ih, il;
         df_add(a.x, a.y, b.x, b.y, rh, rl);
         df_add(a.z, a.w, b.z, b.w, ih, il);
@@ -613,16 +685,15 @@ __global__ void k_gram_exp(const float4* G, int64_t N, int* eG) {
     }
 }
 
-// Digit tiles of G: one thread per (row n, 8 columns); every position of the
-// padded [RB * 128][KB * 16] array is written (zeros outside N x N).
-__global__ void k_gram_digits(const float4* G, int64_t N, int64_t KB, const int* eG, uint8_t* Gd) {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t RB = (N + XM - 1) / XM;
-    if (idx >= RB * XM * KB * 2) return;
-    const int64_t n = idx / (KB * 2), rem = idx % (KB * 2);
-    const int64_t kb = rem / 2;
-    const int g = (int)(rem % 2);
-    const int64_t c0 = kb * XKC + 8 * g;
+// Digit tiles of G, one CTA per (row block, 16-column block), zeros outside N x N:
+// thread (row, 8 columns), consecutive threads along the rows, so a warp's 16-byte
+// stores cover whole 128-byte core-matrix rows (one thread per row and k group in row
+// order stored 16 bytes to a different tile each: 10.1 ms at N = 16384).
+__global__ void __launch_bounds__(256) k_gram_digits(const float4* G, int64_t N, int64_t KB, const int* eG,
+                                                     uint8_t* Gd) {
+    const int64_t kb = blockIdx.x, rb = blockIdx.y;
+    const int r = threadIdx.x & (XM - 1), g = threadIdx.x >> 7;
+    const int64_t n = rb * XM + r, c0 = kb * XKC + 8 * g;
     float reh[8], rel[8], imh[8], iml[8];
 #pragma unroll
     for (int t = 0; t < 8; ++t) {
@@ -637,8 +708,7 @@ __global__ void k_gram_digits(const float4* G, int64_t N, int64_t KB, const int*
     Digits8 dr, di;
     dr.init(reh, rel, scale);
     di.init(imh, iml, scale);
-    uint8_t* tile = Gd + ((n / XM) * KB + kb) * (int64_t)(NDIG * XA_SL);
-    const int r = (int)(n % XM);
+    uint8_t* tile = Gd + (rb * KB + kb) * (int64_t)(NDIG * XA_SL);
 #pragma unroll
     for (int dg = 0; dg < NDIG; ++dg) {
         uint32_t w[4];
@@ -653,22 +723,31 @@ __global__ void k_gram_digits(const float4* G, int64_t N, int64_t KB, const int*
 // fexp[f] = the least e with max_j |D[f][j]| <= 2^e (0 for a zero frame). The
 // maximum is taken over the bit patterns with the sign cleared, whose order is the
 // order of the magnitudes (NaN and infinity left out), on the integer pipe.
+constexpr int FEXP_THREADS = 512;
 __device__ inline unsigned long long mag_bits(double x) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
     return (b >> 52) == 0x7ffull ? 0ull : b;
 }
-__global__ void __launch_bounds__(256) k_frame_exp(const double2* D, int64_t M, int* fexp) {
-    __shared__ unsigned long long red[256];
+__device__ inline unsigned long long mag_bits(float x) {
+    const unsigned b = __float_as_uint(x) & 0x7fffffffu;
+    return (b >> 23) == 0xffu ? 0ull : (unsigned long long)b;
+}
+template <class T>
+__global__ void __launch_bounds__(FEXP_THREADS) k_frame_exp(const T* D, int64_t M, int* fexp) {
+    constexpr int W = FEXP_THREADS, FB = sizeof(T) == 8 ? 23 : 52, BIAS = sizeof(T) == 8 ? 127 : 1023;
+    __shared__ unsigned long long red[W];
     const int64_t f = blockIdx.x;
     unsigned long long m = 0ull;
-    const double2* row = D + f * M;
+    const T* row = D + f * M;
     int64_t j = threadIdx.x;
-    for (; j + 768 < M; j += 1024) {  // four loads in flight
-        const double2 a = row[j], b = row[j + 256], c = row[j + 512], d = row[j + 768];
-        m = max(m, max(max(mag_bits(a.x), mag_bits(a.y)), max(mag_bits(b.x), mag_bits(b.y))));
-        m = max(m, max(max(mag_bits(c.x), mag_bits(c.y)), max(mag_bits(d.x), mag_bits(d.y))));
+    for (; j + 7 * W < M; j += 8 * W) {  // eight loads in flight
+        T v[8];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) v[t] = row[j + t * W];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) m = max(m, max(mag_bits(v[t].x), mag_bits(v[t].y)));
     }
-    for (; j < M; j += 256) m = max(m, max(mag_bits(row[j].x), mag_bits(row[j].y)));
+    for (; j < M; j += W) m = max(m, max(mag_bits(row[j].x), mag_bits(row[j].y)));
     red[threadIdx.x] = m;
     __syncthreads();
     for (int w = blockDim.x / 2; w > 0; w >>= 1) {
@@ -677,88 +756,136 @@ __global__ void __launch_bounds__(256) k_frame_exp(const double2* D, int64_t M, 
     }
     if (threadIdx.x == 0) {
         const unsigned long long B = red[0];
-        const int eb = (int)(B >> 52);
-        const unsigned long long mf = B & ((1ull << 52) - 1ull);
+        const int eb = (int)(B >> FB);
+        const unsigned long long mf = B & ((1ull << FB) - 1ull);
         int e = 0;
         if (B == 0ull)
             e = 0;
-        else if (eb == 0)  // subnormal: B = mf 2^-1074
-            e = (64 - __clzll((long long)mf)) - 1074 - ((mf & (mf - 1ull)) == 0ull ? 1 : 0);
-        else  // (1 + mf 2^-52) 2^(eb - 1023): one more bit unless a power of two
-            e = eb - 1023 + (mf != 0ull ? 1 : 0);
+        else if (eb == 0)  // subnormal: B = mf 2^(1 - BIAS - FB)
+            e = (64 - __clzll((long long)mf)) + 1 - BIAS - FB - ((mf & (mf - 1ull)) == 0ull ? 1 : 0);
+        else  // (1 + mf 2^-FB) 2^(eb - BIAS): one more bit unless a power of two
+            e = eb - BIAS + (mf != 0ull ? 1 : 0);
         fexp[f] = e;
     }
 }
 
 }  // namespace tcx
 
-// frame-tile width of a call of F frames (the narrow tile for at most eight), and
-// the number of frame tiles
-static int exact_xn(int64_t F) { return F <= tcx::XNN ? tcx::XNN : tcx::XN; }
-static int64_t exact_ft(int64_t F) { return (F + exact_xn(F) - 1) / exact_xn(F); }
+// ------------------------------------------------------------------ shapes of a call
+// A product has Q columns (frames x coils) and k blocks; its scratch holds the digit
+// tiles of the B operand, then the partials. Both are bounded by what the same call
+// took before columns were folded (every coil its own 8- or 32-frame tiles, `sub`
+// splits per coil), so that no call needs more scratch than it did:
+// the tile width and the splits are chosen within it.
+namespace {
+constexpr int64_t COL_BYTES = tcx::NDIG * 2 * 64;  // digit bytes of one column and k block
+
+struct XShape {
+    int xn, sub;               // columns per tile, splits of the k range
+    int64_t ct, rb, kb, ks;    // column tiles, row blocks, k blocks, k per block
+    int64_t chunk;             // k per split
+    size_t bd, part;           // bytes of the digit tiles, and of the partials (0: none)
+};
+
+int64_t cdiv64(int64_t a, int64_t b) { return (a + b - 1) / b; }
+size_t align256(size_t n) { return (n + 255) & ~(size_t)255; }
+
+// rows: output rows; trows: tile rows (twice the mirror pairs); K: length of the sum;
+// partials: needed even with one split; slack: bytes the call saves elsewhere
+XShape x_shape(int64_t rows, int64_t trows, int64_t K, bool pair, int64_t F, int64_t C, bool partials, size_t slack) {
+    XShape x;
+    const int64_t Q = F * C, kb16 = cdiv64(K, tcx::XKC);
+    x.ks = pair ? tcx::XKP : tcx::XKC;
+    x.kb = cdiv64(K, x.ks);
+    x.rb = cdiv64(trows, tcx::XM);
+    // the bound: per coil, tiles of 8 (up to 8 frames) or 32 frames, and their splits
+    const int64_t ow = F <= 8 ? 8 : 32, oft = cdiv64(F, ow);
+    const int hi = (int)std::max<int64_t>(1, std::min<int64_t>(32, K / 512));
+    const int osub = tc::wave_splits(cdiv64(rows, tcx::XM) * oft * C, K, 1, hi, 256);
+    const size_t obd = (size_t)(oft * ow * C * kb16 * COL_BYTES);
+    const size_t slot = (size_t)(Q * rows) * sizeof(float4);
+    const size_t opart = osub * C > 1 || partials ? (size_t)osub * slot : 0;
+    const size_t bound = align256(obd) + opart + slack;
+    // the width and the splits within the bound that take the least time: waves of CTAs x
+    // (k per split + fill, drain and epilogue in k) x tensor cycles of a stage (its 16 MMAs
+    // take at least 32 cycles each, however narrow)
+    double best = 0.0;
+    for (int xn : {tcx::XN, 16, 8}) {
+        const int64_t ct = cdiv64(Q, xn);
+        const size_t bd = align256((size_t)(ct * xn * x.kb * COL_BYTES));
+        if (xn > 8 && (2 * Q <= xn || bd + slot > bound)) continue;
+        const int64_t room = bd < bound ? (int64_t)((bound - bd) / slot) : 0;
+        const int sub = room < 1 ? 1 : tc::wave_splits(x.rb * ct, K, 1, (int)std::min<int64_t>(hi, room), 256);
+        const double t = (double)cdiv64(x.rb * ct * sub, tc::sm_count()) * ((double)K / sub + 256.0) *
+                         (xn == 8 ? 512.0 : xn == 16 ? 736.0 : 1344.0);
+        if (best == 0.0 || t < best) {
+            best = t;
+            x.xn = xn;
+            x.ct = ct;
+            x.bd = bd;
+            x.sub = sub;
+        }
+    }
+    x.chunk = cdiv64(cdiv64(K, x.sub), x.ks) * x.ks;
+    x.part = x.sub > 1 || partials ? (size_t)x.sub * slot : 0;
+    return x;
+}
+
+bool paired(const EncodeDev& e) { return e.pair && !e.b0df && !e.b0tab; }
+// E^H d; f32: c64 data are read as they are (their FP64 copy is not made)
+XShape adj_shape(const EncodeDev& e, int64_t F, bool f32) {
+    const bool pr = paired(e);
+    return x_shape(e.N, pr ? 2 * e.U : e.N, e.Mk, pr, F, e.C, e.coilsdf != nullptr || e.C > 1,
+                   f32 ? (size_t)(16 * F * e.C * e.Mk) : 0);
+}
+XShape fwd_shape(const EncodeDev& e, int64_t F) { return x_shape(e.Mk, e.Mk, e.N, false, F, e.C, true, 0); }
+XShape gram_shape(int64_t N, int64_t F) { return x_shape(N, N, N, false, F, 1, true, 0); }
+}  // namespace
 
 template <int MODE, int XNT>
-static cudaError_t exact_attr() {
+static cudaError_t exact_run(const tcx::XArgs& a, unsigned grid, DevStatus* st, cudaStream_t s) {
     static bool attr = false;
-    if (attr) return cudaSuccess;
-    cudaError_t err = cudaFuncSetAttribute(tcx::k_exact<MODE, XNT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           tcx::XS<XNT>::SMEM);
-    if (err == cudaSuccess) attr = true;
-    return err;
-}
-// the exact kernel for a call of F frames, `grid` CTAs
-template <int MODE>
-static cudaError_t launch_exact(const tcx::XArgs& a, int64_t F, unsigned grid, DevStatus* st, cudaStream_t s) {
-    cudaError_t err;
-    if (exact_xn(F) == tcx::XNN) {
-        if ((err = exact_attr<MODE, tcx::XNN>()) != cudaSuccess) return err;
-        tcx::k_exact<MODE, tcx::XNN><<<grid, tc::NTHREADS, tcx::XS<tcx::XNN>::SMEM, s>>>(a, st);
-    } else {
-        if ((err = exact_attr<MODE, tcx::XN>()) != cudaSuccess) return err;
-        tcx::k_exact<MODE, tcx::XN><<<grid, tc::NTHREADS, tcx::XS<tcx::XN>::SMEM, s>>>(a, st);
+    if (!attr) {
+        cudaError_t err = cudaFuncSetAttribute(tcx::k_exact<MODE, XNT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               tcx::XS<XNT>::SMEM);
+        if (err != cudaSuccess) return err;
+        attr = true;
     }
+    tcx::k_exact<MODE, XNT><<<grid, tc::NTHREADS, tcx::XS<XNT>::SMEM, s>>>(a, st);
     note_launch();
     return cudaGetLastError();
 }
-
-// splits per coil: whole waves of CTAs over all coils, chunks of at least two
-// accumulation groups
-static int exact_sub(const EncodeDev& e, int64_t F) {
-    const int64_t tiles = ((e.N + tcx::XM - 1) / tcx::XM) * exact_ft(F) * e.C;
-    const int hi = (int)std::max<int64_t>(1, std::min<int64_t>(32, e.Mk / (tcx::XKC * tcx::XDRAIN * 2)));
-    return tc::wave_splits(tiles, e.Mk, 1, hi, 256);
+template <int MODE>
+static cudaError_t launch_exact(const tcx::XArgs& a, const XShape& x, DevStatus* st, cudaStream_t s) {
+    const unsigned grid = (unsigned)(x.ct * x.rb * x.sub);
+    return x.xn == 8 ? exact_run<MODE, 8>(a, grid, st, s)
+                     : x.xn == 16 ? exact_run<MODE, 16>(a, grid, st, s) : exact_run<MODE, tcx::XN>(a, grid, st, s);
 }
 
-size_t exact_work_elems(const EncodeDev& e, int64_t F) {
-    const int64_t splits = (int64_t)exact_sub(e, F) * e.C;
-    return splits > 1 || e.coilsdf ? (size_t)splits * (size_t)e.N * (size_t)F : 0;
+template <int XNT, bool PAIR, class T>
+static void b_digits_run(const T* D, int64_t Q, int C, int64_t Kc, int64_t KB, const int* fexp, uint8_t* Bd,
+                         cudaStream_t s) {
+    const int64_t per = 256 / ((PAIR ? 4 : 2) * XNT);  // chunks per block
+    tcx::k_b_digits<XNT, PAIR, T>
+        <<<(unsigned)cdiv64(cdiv64(Q, XNT) * KB, per), 256, 0, s>>>(D, Q, C, Kc, KB, fexp, Bd);
 }
-
-// digit tiles of the B operand: frame tiles x coils x 16-sample chunks per coil
-static size_t b_digit_bytes(int64_t F, int64_t C, int64_t Kc) {
-    return (size_t)exact_ft(F) * (size_t)C * (size_t)((Kc + tcx::XKC - 1) / tcx::XKC) *
-           (size_t)(tcx::NDIG * 2 * exact_xn(F) * 64);
-}
-
-static cudaError_t launch_b_digits(const double2* D, int64_t ld, int64_t F, int C, int64_t Kc, const int* fexp,
-                                   uint8_t* Bd, cudaStream_t s) {
-    const int64_t KB = (Kc + tcx::XKC - 1) / tcx::XKC;
-    const int64_t tiles = exact_ft(F) * C * KB;
-    const int64_t per = 256 / (2 * exact_xn(F));  // chunks per block
-    if (exact_xn(F) == tcx::XNN)
-        tcx::k_b_digits<tcx::XNN><<<(unsigned)((tiles + per - 1) / per), 256, 0, s>>>(D, ld, F, C, Kc, KB, fexp, Bd);
-    else
-        tcx::k_b_digits<tcx::XN><<<(unsigned)((tiles + per - 1) / per), 256, 0, s>>>(D, ld, F, C, Kc, KB, fexp, Bd);
-    note_launch();
+// frame exponents of D [F][C][Kc], then its digit tiles
+template <bool PAIR, class T>
+static cudaError_t launch_b_digits(const T* D, int64_t F, int C, int64_t Kc, const XShape& x, int* fexp, uint8_t* Bd,
+                                   cudaStream_t s) {
+    tcx::k_frame_exp<T><<<(unsigned)F, tcx::FEXP_THREADS, 0, s>>>(D, C * Kc, fexp);
+    const int64_t Q = F * C;
+    if (x.xn == 8) b_digits_run<8, PAIR, T>(D, Q, C, Kc, x.kb, fexp, Bd, s);
+    else if (x.xn == 16) b_digits_run<16, PAIR, T>(D, Q, C, Kc, x.kb, fexp, Bd, s);
+    else b_digits_run<tcx::XN, PAIR, T>(D, Q, C, Kc, x.kb, fexp, Bd, s);
+    note_launch(2);
     return cudaGetLastError();
 }
 
-size_t exact_bdigit_bytes(const EncodeDev& e, int64_t F) { return b_digit_bytes(F, e.C, e.Mk); }
-
+// ------------------------------------------------------------------ E^H d
 // the fewest frames for which the exact products replace the double-float ones:
-// every count since calls of up to eight frames take the 8-frame tile (a 64x64
-// apply of 1-12 frames: 11.5-14 ms with the double-float products, 1.8-2.1 ms with
-// these and the tensor-core correction). PINV_EXACT_MIN_FRAMES: another count.
+// every count since small calls take narrow tiles (a 64x64 apply of 1-12 frames:
+// 11.5-14 ms with the double-float products). PINV_EXACT_MIN_FRAMES: another count.
 static int64_t exact_min_frames() {
     static const int64_t v = [] {
         const char* s = std::getenv("PINV_EXACT_MIN_FRAMES");
@@ -770,148 +897,146 @@ static int64_t exact_min_frames() {
 bool exact_adjoint_ok(const EncodeDev& e, int64_t F, bool table) {
     // plans with B0 only from the per-build table of conj(A) (the producers form
     // A from the separable tables of plans without B0)
-    const bool gen = e.extdf && !e.b0df && !e.b0tab;
+    const bool gen = e.extdf && paired(e);
     const bool tab = table && e.b0df && e.exdf;
     return (gen || tab) && F >= exact_min_frames() && tc_available();
 }
 
+// with B0: [N / 128][M_k / 16] tiles of conj(A); without: [pairs / 64][M_k / 32] tiles of
+// the mirror pairs, half as many on a grid and as many where no voxel has a mirror (the
+// allocation is the same in both cases)
 size_t adj_digit_bytes(const EncodeDev& e) {
-    const int64_t RB = (e.N + tcx::XM - 1) / tcx::XM, KB = (e.Mk + tcx::XKC - 1) / tcx::XKC;
-    return (size_t)RB * (size_t)KB * (size_t)(tcx::NDIG * tcx::XA_SL);
+    const int64_t full = cdiv64(e.N, tcx::XM) * cdiv64(e.Mk, tcx::XKC);
+    const int64_t tiles = paired(e) ? std::max(full, cdiv64(2 * e.U, tcx::XM) * cdiv64(e.Mk, tcx::XKP)) : full;
+    return (size_t)tiles * (size_t)(tcx::NDIG * tcx::XA_SL);
 }
 
 cudaError_t launch_adj_digits(const EncodeDev& e, uint8_t* Ad, cudaStream_t s) {
-    const int64_t RB = (e.N + tcx::XM - 1) / tcx::XM, KB = (e.Mk + tcx::XKC - 1) / tcx::XKC;
-    tcx::k_adj_digits<<<dim3((unsigned)KB, (unsigned)RB), 256, 0, s>>>(e, KB, Ad);
+    if (paired(e)) {
+        const int64_t KB = cdiv64(e.Mk, tcx::XKP);
+        tcx::k_pair_digits<<<dim3((unsigned)KB, (unsigned)cdiv64(2 * e.U, tcx::XM)), 256, 0, s>>>(e, KB, Ad);
+    } else {
+        const int64_t KB = cdiv64(e.Mk, tcx::XKC);
+        tcx::k_adj_digits<<<dim3((unsigned)KB, (unsigned)cdiv64(e.N, tcx::XM)), 256, 0, s>>>(e, KB, Ad);
+    }
     note_launch();
     return cudaGetLastError();
 }
 
-cudaError_t launch_adjoint_exact(const EncodeDev& e, const double2* D, int64_t F, int* fexp, uint8_t* Bd,
-                                 double2* B, float4* work, DevStatus* st, cudaStream_t s, const uint8_t* Ad) {
+size_t exact_scratch_bytes(const EncodeDev& e, int64_t F, bool f32) {
+    const XShape x = adj_shape(e, F, f32);
+    return x.bd + x.part;
+}
+
+template <class T>
+static cudaError_t adjoint_exact(const EncodeDev& e, const T* D, int64_t F, int* fexp, void* scratch, double2* B,
+                                 DevStatus* st, cudaStream_t s, const uint8_t* Ad) {
     if (F == 0) return cudaSuccess;
-    if (!Bd) return cudaErrorInvalidValue;
-    const int64_t M = e.Mk * e.C;
-    tcx::k_frame_exp<<<(unsigned)F, 256, 0, s>>>(D, M, fexp);
-    note_launch();
-    cudaError_t berr = launch_b_digits(D, M, F, (int)e.C, e.Mk, fexp, Bd, s);
-    if (berr != cudaSuccess) return berr;
-    const int sub = exact_sub(e, F);
-    const int64_t splits = (int64_t)sub * e.C;
-    const bool partials = splits > 1 || e.coilsdf;
-    if (partials && !work) return cudaErrorInvalidValue;
-    const int64_t chunk = ((e.Mk + sub - 1) / sub + tcx::XKC - 1) / tcx::XKC * tcx::XKC;
-    const int64_t KB = (e.Mk + tcx::XKC - 1) / tcx::XKC;
-    tcx::XArgs a{e, D, fexp, F, M, chunk, sub, partials ? work : nullptr, B, Ad, nullptr, KB, Bd, (int)e.C};
-    const unsigned grid = (unsigned)(exact_ft(F) * ((e.N + tcx::XM - 1) / tcx::XM) * splits);
-    cudaError_t err = Ad ? launch_exact<tcx::XADJT>(a, F, grid, st, s) : launch_exact<tcx::XGEN>(a, F, grid, st, s);
-    if (err != cudaSuccess || !partials) return err;
-    const int64_t n = e.N * F;
-    tcx::k_exact_reduce<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(tcx::BStore{B, e.N}, work, (int)splits, e.N, F);
+    if (!scratch || !fexp) return cudaErrorInvalidValue;
+    const XShape x = adj_shape(e, F, sizeof(T) == sizeof(float2));
+    const bool pr = paired(e);
+    uint8_t* Bd = (uint8_t*)scratch;
+    float4* part = x.part ? (float4*)(Bd + x.bd) : nullptr;
+    cudaError_t err = pr ? launch_b_digits<true, T>(D, F, e.C, e.Mk, x, fexp, Bd, s)
+                         : launch_b_digits<false, T>(D, F, e.C, e.Mk, x, fexp, Bd, s);
+    if (err != cudaSuccess) return err;
+    tcx::XArgs a{e, fexp, F * e.C, e.C, x.chunk, part, B, Ad, nullptr, x.kb, Bd};
+    err = !pr ? launch_exact<tcx::XADJT>(a, x, st, s)
+              : Ad ? launch_exact<tcx::XADJP>(a, x, st, s) : launch_exact<tcx::XGEN>(a, x, st, s);
+    if (err != cudaSuccess || !part) return err;
+    tcx::k_exact_reduce<<<(unsigned)cdiv64(e.N * F, 256), 256, 0, s>>>(B, part, x.sub, e.C, e.N, F);
     note_launch();
     return cudaGetLastError();
+}
+cudaError_t launch_adjoint_exact(const EncodeDev& e, const double2* D, int64_t F, int* fexp, void* scratch,
+                                 double2* B, DevStatus* st, cudaStream_t s, const uint8_t* Ad) {
+    return adjoint_exact(e, D, F, fexp, scratch, B, st, s, Ad);
+}
+cudaError_t launch_adjoint_exact32(const EncodeDev& e, const float2* D, int64_t F, int* fexp, void* scratch,
+                                   double2* B, DevStatus* st, cudaStream_t s, const uint8_t* Ad) {
+    return adjoint_exact(e, D, F, fexp, scratch, B, st, s, Ad);
 }
 
 // ------------------------------------------------------------------ exact forward product
-// splits of the voxel range per coil: whole waves of CTAs over all coils
-static int fwd_sub(const EncodeDev& e, int64_t F) {
-    const int64_t tiles = ((e.Mk + tcx::XM - 1) / tcx::XM) * exact_ft(F) * e.C;
-    const int hi = (int)std::max<int64_t>(1, std::min<int64_t>(32, e.N / (tcx::XKC * tcx::XDRAIN * 2)));
-    return tc::wave_splits(tiles, e.N, 1, hi, 256);
-}
-
 size_t fwd_digit_bytes(const EncodeDev& e) {
-    const int64_t RB = (e.Mk + tcx::XM - 1) / tcx::XM, KB = (e.N + tcx::XKC - 1) / tcx::XKC;
-    return (size_t)RB * (size_t)KB * (size_t)(tcx::NDIG * tcx::XA_SL);
+    return (size_t)(cdiv64(e.Mk, tcx::XM) * cdiv64(e.N, tcx::XKC)) * (size_t)(tcx::NDIG * tcx::XA_SL);
 }
 
 cudaError_t launch_fwd_digits(const EncodeDev& e, uint8_t* Af, cudaStream_t s) {
-    const int64_t RB = (e.Mk + tcx::XM - 1) / tcx::XM, KB = (e.N + tcx::XKC - 1) / tcx::XKC;
+    const int64_t RB = cdiv64(e.Mk, tcx::XM), KB = cdiv64(e.N, tcx::XKC);
     tcx::k_fwd_digits<<<dim3((unsigned)KB, (unsigned)RB), 256, 0, s>>>(e, KB, Af);
     note_launch();
     return cudaGetLastError();
 }
 
-size_t exact_fwd_work_elems(const EncodeDev& e, int64_t F) {
-    return (size_t)fwd_sub(e, F) * (size_t)e.C * (size_t)F * (size_t)e.Mk;
+size_t exact_fwd_scratch_bytes(const EncodeDev& e, int64_t F) {
+    const XShape x = fwd_shape(e, F);
+    return x.bd + x.part;
 }
-size_t exact_fwd_bdigit_bytes(const EncodeDev& e, int64_t F) { return b_digit_bytes(F, e.C, e.N); }
 size_t exact_fwd_y_elems(const EncodeDev& e, int64_t F) { return (size_t)F * (size_t)e.C * (size_t)e.N; }
 
 cudaError_t launch_forward_exact(const EncodeDev& e, const double2* X, int64_t F, const double2* D, double2* U,
-                                 const uint8_t* Af, double2* Y, int* fexp, uint8_t* Bd, float4* work,
-                                 DevStatus* st, cudaStream_t s) {
+                                 const uint8_t* Af, double2* Y, int* fexp, void* scratch, DevStatus* st,
+                                 cudaStream_t s) {
     if (F == 0) return cudaSuccess;
-    if (!Af || !Y || !Bd || !work) return cudaErrorInvalidValue;
-    cudaError_t err;
+    if (!Af || !Y || !scratch || !fexp) return cudaErrorInvalidValue;
     const int64_t ny = F * e.C * e.N;
-    tcx::k_coil_times<<<(unsigned)((ny + 255) / 256), 256, 0, s>>>(e, X, F, Y);  // Y[f][c] = s_c o x_f
-    tcx::k_frame_exp<<<(unsigned)F, 256, 0, s>>>(Y, e.C * e.N, fexp);
-    note_launch(2);
-    if ((err = launch_b_digits(Y, e.C * e.N, F, (int)e.C, e.N, fexp, Bd, s)) != cudaSuccess) return err;
-    const int sub = fwd_sub(e, F);
-    const int64_t chunk = ((e.N + sub - 1) / sub + tcx::XKC - 1) / tcx::XKC * tcx::XKC;
-    const int64_t KB = (e.N + tcx::XKC - 1) / tcx::XKC;
-    tcx::XArgs a{e, Y, fexp, F, e.C * e.N, chunk, sub, work, nullptr, Af, nullptr, KB, Bd, (int)e.C};
-    const unsigned grid = (unsigned)(exact_ft(F) * ((e.Mk + tcx::XM - 1) / tcx::XM) * e.C * sub);
-    if ((err = launch_exact<tcx::XFWD>(a, F, grid, st, s)) != cudaSuccess) return err;
+    tcx::k_coil_times<<<(unsigned)cdiv64(ny, 256), 256, 0, s>>>(e, X, F, Y);  // Y[f][c] = s_c o x_f
+    note_launch();
+    const XShape x = fwd_shape(e, F);
+    uint8_t* Bd = (uint8_t*)scratch;
+    float4* part = (float4*)(Bd + x.bd);
+    cudaError_t err = launch_b_digits<false, double2>(Y, F, e.C, e.N, x, fexp, Bd, s);
+    if (err != cudaSuccess) return err;
+    tcx::XArgs a{e, fexp, F * e.C, e.C, x.chunk, part, nullptr, Af, nullptr, x.kb, Bd};
+    if ((err = launch_exact<tcx::XFWD>(a, x, st, s)) != cudaSuccess) return err;
     const int64_t n = e.Mk * e.C * F;
-    tcx::k_fwd_reduce<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(D, work, sub, (int)e.C, e.Mk, F, U);
+    tcx::k_fwd_reduce<<<(unsigned)cdiv64(n, 256), 256, 0, s>>>(D, part, x.sub, n, U);
     note_launch();
     return cudaGetLastError();
 }
 
 cudaError_t launch_minus_lambda(double2* R, const double2* X, double lam, int64_t n, cudaStream_t s) {
-    tcx::k_minus_lam<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(R, X, lam, n);
+    tcx::k_minus_lam<<<(unsigned)cdiv64(n, 256), 256, 0, s>>>(R, X, lam, n);
     note_launch();
     return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------ exact Gram residual
 size_t gram_digit_bytes(int64_t N) {
-    const int64_t RB = (N + tcx::XM - 1) / tcx::XM, KB = (N + tcx::XKC - 1) / tcx::XKC;
-    return (size_t)RB * (size_t)KB * (size_t)(tcx::NDIG * tcx::XA_SL);
+    return (size_t)(cdiv64(N, tcx::XM) * cdiv64(N, tcx::XKC)) * (size_t)(tcx::NDIG * tcx::XA_SL);
 }
 
 cudaError_t launch_gram_digits(const float4* G, int64_t N, int* eG, uint8_t* Gd, cudaStream_t s) {
     tcx::k_gram_exp<<<1, 256, 0, s>>>(G, N, eG);
     note_launch();
-    const int64_t KB = (N + tcx::XKC - 1) / tcx::XKC, RB = (N + tcx::XM - 1) / tcx::XM;
-    const int64_t n = RB * tcx::XM * KB * 2;
-    tcx::k_gram_digits<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(G, N, KB, eG, Gd);
+    const int64_t KB = cdiv64(N, tcx::XKC), RB = cdiv64(N, tcx::XM);
+    tcx::k_gram_digits<<<dim3((unsigned)KB, (unsigned)RB), 256, 0, s>>>(G, N, KB, eG, Gd);
     note_launch();
     return cudaGetLastError();
 }
 
-static int resid_splits(int64_t N, int64_t F) {
-    const int64_t tiles = ((N + tcx::XM - 1) / tcx::XM) * exact_ft(F);
-    const int hi = (int)std::max<int64_t>(1, std::min<int64_t>(32, N / (tcx::XKC * tcx::XDRAIN * 2)));
-    return tc::wave_splits(tiles, N, 1, hi, 256);
+size_t resid_scratch_bytes(int64_t N, int64_t F) {
+    const XShape x = gram_shape(N, F);
+    return x.bd + x.part;
 }
 
-size_t resid_exact_work_elems(int64_t N, int64_t F) { return (size_t)resid_splits(N, F) * (size_t)N * (size_t)F; }
-
-size_t resid_bdigit_bytes(int64_t N, int64_t F) { return b_digit_bytes(F, 1, N); }
-
 cudaError_t launch_gram_resid_exact(const uint8_t* Gd, const int* eG, int64_t N, const double2* Bv,
-                                    const double2* X, int64_t F, int* fexp, uint8_t* Bd, double2* R,
-                                    float4* work, DevStatus* st, cudaStream_t s) {
+                                    const double2* X, int64_t F, int* fexp, void* scratch, double2* R,
+                                    DevStatus* st, cudaStream_t s) {
     if (F == 0) return cudaSuccess;
-    if (!Bd) return cudaErrorInvalidValue;
-    cudaError_t err;
-    tcx::k_frame_exp<<<(unsigned)F, 256, 0, s>>>(X, N, fexp);
-    note_launch();
-    if ((err = launch_b_digits(X, N, F, 1, N, fexp, Bd, s)) != cudaSuccess) return err;
-    const int sp = resid_splits(N, F);
-    const int64_t chunk = ((N + sp - 1) / sp + tcx::XKC - 1) / tcx::XKC * tcx::XKC;
+    if (!scratch || !fexp) return cudaErrorInvalidValue;
+    const XShape x = gram_shape(N, F);
+    uint8_t* Bd = (uint8_t*)scratch;
+    float4* part = (float4*)(Bd + x.bd);
+    cudaError_t err = launch_b_digits<false, double2>(X, F, 1, N, x, fexp, Bd, s);
+    if (err != cudaSuccess) return err;
     EncodeDev e{};
     e.N = N;
-    const int64_t KB = (N + tcx::XKC - 1) / tcx::XKC;
-    tcx::XArgs a{e, X, fexp, F, N, chunk, sp, work, nullptr, Gd, eG, KB, Bd, 1};
-    const unsigned grid = (unsigned)(exact_ft(F) * ((N + tcx::XM - 1) / tcx::XM) * sp);
-    if ((err = launch_exact<tcx::XGRAM>(a, F, grid, st, s)) != cudaSuccess) return err;
+    tcx::XArgs a{e, fexp, F, 1, x.chunk, part, nullptr, Gd, eG, x.kb, Bd};
+    if ((err = launch_exact<tcx::XGRAM>(a, x, st, s)) != cudaSuccess) return err;
     const int64_t n = N * F;
-    tcx::k_resid_reduce<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(Bv, work, sp, N, F, R);
+    tcx::k_resid_reduce<<<(unsigned)cdiv64(n, 256), 256, 0, s>>>(Bv, part, x.sub, N, F, R);
     note_launch();
     return cudaGetLastError();
 }
