@@ -230,8 +230,10 @@ pinv_status pinv_plan_sync(pinv_plan* plan);
 /*
  * image = Recon x data for n_frames frames (Eq. 3), or G^-1 E^H data for
  * factor-only plans (Section 3.3). d_data: device [F][C][M_k], d_image:
- * device [F][N], both of `dtype` (pinv_dtype). Mixed-precision plans refine
- * each frame with FP64 residuals r = E^H (d - E x) - lambda x up to
+ * device [F][N], both of `dtype` (pinv_dtype). Mixed plans that refine with the
+ * TOEPLITZ residual start from G^-1 E^H data whether or not they hold Recon (E^H data is
+ * formed exactly either way; the images agree to the refinement's accuracy).
+ * Mixed-precision plans refine each frame with FP64 residuals r = E^H (d - E x) - lambda x up to
  * refine_max_iters times. n_frames == 0 is a no-op. With the stopping rule
  * (refine_tol > 0) a residual or image that is not finite (NaN or Inf in the
  * data) ends the call with PINV_ERR_INVALID_ARG naming the frame. Uses plan-owned
