@@ -89,9 +89,11 @@ size_t apply_scratch_layout(const pinv_plan* p, int64_t F, int dtype, void* base
     s.x64 = need_x64 ? cv.take<float2>((size_t)(F * N)) : nullptr;
     s.norms = md.stop_rule ? cv.take<double>((size_t)(3 * F)) : nullptr;
     const bool atc = md.use_recon && apply_tc_ok(F);
-    const bool ctc = md.mixed && (md.dfres || md.toep || !p->recon) && correct_tc_ok(F);
+    const bool corr = md.mixed && (md.dfres || md.toep || !p->recon) && correct_tc_ok(F);
+    const bool crows = corr && correct_rows_ok(N, F), ctc = corr && !crows;
     if (atc) s.apw = cv.take<float2>(apply_tc_work_elems(N, M, F));
     if (ctc) s.cw = cv.take<float2>(correct_tc_work_elems(N, F));
+    if (crows) s.r32 = cv.take<float2>((size_t)(F * N));
     if (atc || ctc) s.sched = cv.take<DevStatus>(1);
     if (md.dfres || md.toep || md.need_b) {
         // E^H u (rows N, length M), E x (rows M, length N), G x (rows N, length N) one
@@ -143,8 +145,10 @@ pinv_status apply_impl(pinv_plan* p, const void* d_data, void* d_image, int64_t 
     }
     double2* X = dtype == PINV_C128 ? (double2*)d_image : sc.x128;
     if (sc.sched) CKA(cudaMemsetAsync(sc.sched, 0, sizeof(DevStatus), s));
-    // x += W^H (W r) with the FP32 W: on the tensor cores (correct_tc_ok), else SIMT
+    // x += W^H (W r) with the FP32 W: one pass over W per product for few frames
+    // (correct_rows_ok), else on the tensor cores (correct_tc_ok), else SIMT
     auto correct = [&](const double2* r) -> cudaError_t {
+        if (sc.r32) return launch_correct_rows(p->W32, N, r, F, sc.x64, X, sc.r32, s);
         if (sc.cw) return launch_correct_tc(p->W32, N, r, F, sc.x64, X, sc.cw, p->slices(), sc.sched, s);
         return launch_correct32(p->W32, N, r, F, sc.x64, X, s);
     };

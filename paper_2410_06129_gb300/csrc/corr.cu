@@ -1,0 +1,236 @@
+// The refinement's correction x += W^H (W r) in plain FP32 for few frames.
+//
+// W = L^-1 (FP32, lower, row-major) is read once per product, N^2 / 2 entries of 8 bytes:
+// with few frames that traffic is the cost, and the tensor-core form (CorrW / CorrWH)
+// spends its time splitting W into BF16 slices for 128-frame tiles that are mostly
+// padding. Here each product is one pass over W with FP32 FMAs and no partial sums in
+// memory:
+//   k_corr_rows   T[f][i] = sum_{k <= i} W[i][k] r[f][k]: a CTA owns CR rows, its eight
+//                 warps take the columns in turn, lane l the entry pair 2 l, 2 l + 1 of a
+//                 warp's 64 (one 16-byte load per row), so one load of r serves CR rows; the
+//                 sums meet in shuffles and shared memory.
+//   k_corr_cols   X[f][n] += sum_{k >= n} conj(W[k][n]) T[f][k]: a CTA owns 32 columns (256
+//                 contiguous bytes of each row), its half-warps take the rows in turn, and
+//                 their sums meet in shared memory, added in order.
+// Frames go in blocks of CF = 1, 2, 4 or 8, without a branch per frame in the loops (a
+// ragged block repeats its last frame and stores nothing for it), so the loads of several
+// steps are in flight together.
+#include <algorithm>
+#include <cstdlib>
+
+#include "df.cuh"
+
+namespace pinv {
+namespace {
+
+constexpr int CR = 4;          // rows per CTA of k_corr_rows
+constexpr int CC = 32;         // columns per CTA of k_corr_cols
+constexpr int CW = 16;         // its warps
+constexpr int CFMAX = 8;       // frames per launch
+
+__global__ void k_corr_f32(const double2* a, float2* b, int64_t n) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) b[i] = make_float2(f64_to_f32_rn(a[i].x), f64_to_f32_rn(a[i].y));
+}
+
+__device__ inline void cmacf(float2& acc, float2 a, float2 b) {  // acc += a b
+    acc.x = fmaf(a.x, b.x, fmaf(-a.y, b.y, acc.x));
+    acc.y = fmaf(a.x, b.y, fmaf(a.y, b.x, acc.y));
+}
+__device__ inline void cmacf_conj(float2& acc, float2 a, float2 b) {  // acc += conj(a) b
+    acc.x = fmaf(a.x, b.x, fmaf(a.y, b.y, acc.x));
+    acc.y = fmaf(a.x, b.y, fmaf(-a.y, b.x, acc.y));
+}
+
+// entries p[0], p[1]; one 16-byte load when the address allows (every row of an even N)
+template <bool EVEN>
+__device__ inline float4 ld2(const float2* p, bool second) {
+    if (EVEN) return __ldg(reinterpret_cast<const float4*>(p));
+    const float2 a = __ldg(p), b = second ? __ldg(p + 1) : make_float2(0.f, 0.f);
+    return make_float4(a.x, a.y, b.x, b.y);
+}
+
+// rows from the last (longest) to the first; W is zero above its diagonal, so the pair
+// that straddles it needs no care, and entries past N are never read
+template <int CF, bool EVEN>
+__global__ void __launch_bounds__(256) k_corr_rows(const float2* __restrict__ W, int64_t N, int F,
+                                                   const float2* __restrict__ r, float2* __restrict__ T) {
+    __shared__ float2 red[8][CR * CF];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t i0 = ((int64_t)gridDim.x - 1 - blockIdx.x) * CR;
+    const int64_t end = i0 + CR < N ? i0 + CR : N;  // columns 0 .. end - 1
+    float2 acc[CR][CF];
+    const float2 *row[CR], *rf[CF];
+#pragma unroll
+    for (int a = 0; a < CR; ++a) {
+        row[a] = W + (i0 + a < N ? i0 + a : N - 1) * N;
+#pragma unroll
+        for (int f = 0; f < CF; ++f) acc[a][f] = make_float2(0.f, 0.f);
+    }
+#pragma unroll
+    for (int f = 0; f < CF; ++f) rf[f] = r + (int64_t)(f < F ? f : F - 1) * N;
+#pragma unroll 2
+    for (int64_t k = 64 * warp + 2 * lane; k < end; k += 512) {
+        const bool second = k + 1 < N;
+        float4 w[CR], v[CF];
+#pragma unroll
+        for (int a = 0; a < CR; ++a) w[a] = ld2<EVEN>(row[a] + k, second);
+#pragma unroll
+        for (int f = 0; f < CF; ++f) v[f] = ld2<EVEN>(rf[f] + k, second);
+#pragma unroll
+        for (int f = 0; f < CF; ++f)
+#pragma unroll
+            for (int a = 0; a < CR; ++a) {
+                cmacf(acc[a][f], make_float2(w[a].x, w[a].y), make_float2(v[f].x, v[f].y));
+                cmacf(acc[a][f], make_float2(w[a].z, w[a].w), make_float2(v[f].z, v[f].w));
+            }
+    }
+#pragma unroll
+    for (int a = 0; a < CR; ++a) {
+#pragma unroll
+        for (int f = 0; f < CF; ++f) {
+            float2 s = acc[a][f];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
+                s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
+            }
+            if (lane == 0) red[warp][a * CF + f] = s;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < CR * CF) {
+        const int a = threadIdx.x / CF, f = threadIdx.x % CF;
+        float2 s = red[0][threadIdx.x];
+#pragma unroll
+        for (int g = 1; g < 8; ++g) {
+            s.x += red[g][threadIdx.x].x;
+            s.y += red[g][threadIdx.x].y;
+        }
+        if (f < F && i0 + a < N) T[(int64_t)f * N + i0 + a] = s;
+    }
+}
+
+template <int CF, bool EVEN>
+__global__ void __launch_bounds__(CW * 32) k_corr_cols(const float2* __restrict__ W, int64_t N, int F,
+                                                       const float2* __restrict__ T, double2* __restrict__ X) {
+    __shared__ float2 red[CF][CW][CC + 1];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int half = lane >> 4, c2 = 2 * (lane & 15);
+    const int64_t n0 = (int64_t)blockIdx.x * CC, n = n0 + c2;
+    float2 acc[2][CF];
+    const float2* tf[CF];
+#pragma unroll
+    for (int f = 0; f < CF; ++f) {
+        acc[0][f] = acc[1][f] = make_float2(0.f, 0.f);
+        tf[f] = T + (int64_t)(f < F ? f : F - 1) * N;
+    }
+    const bool in = n < N, second = n + 1 < N;
+    const float2* col = W + (in ? n : 0);  // a lane past N reads column 0 (aligned as n is), unstored
+    // rows k >= n0; above the diagonal of the CTA's first rows W is zero
+    constexpr int U = CF <= 2 ? 8 : CF == 4 ? 4 : 2;
+    int64_t k = n0 + 2 * warp + half;
+    for (; k + 2 * CW * (U - 1) < N; k += 2 * CW * U) {
+        float4 w[U];
+        float2 t[U][CF];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            w[u] = ld2<EVEN>(col + (k + 2 * CW * u) * N, second);
+#pragma unroll
+            for (int f = 0; f < CF; ++f) t[u][f] = __ldg(tf[f] + k + 2 * CW * u);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int f = 0; f < CF; ++f) {
+                cmacf_conj(acc[0][f], make_float2(w[u].x, w[u].y), t[u][f]);
+                cmacf_conj(acc[1][f], make_float2(w[u].z, w[u].w), t[u][f]);
+            }
+    }
+    for (; k < N; k += 2 * CW) {
+        const float4 w = ld2<EVEN>(col + k * N, second);
+#pragma unroll
+        for (int f = 0; f < CF; ++f) {
+            const float2 t = __ldg(tf[f] + k);
+            cmacf_conj(acc[0][f], make_float2(w.x, w.y), t);
+            cmacf_conj(acc[1][f], make_float2(w.z, w.w), t);
+        }
+    }
+#pragma unroll
+    for (int f = 0; f < CF; ++f) {
+        float2 a = acc[0][f], b = acc[1][f];
+        a.x += __shfl_xor_sync(0xffffffffu, a.x, 16);
+        a.y += __shfl_xor_sync(0xffffffffu, a.y, 16);
+        b.x += __shfl_xor_sync(0xffffffffu, b.x, 16);
+        b.y += __shfl_xor_sync(0xffffffffu, b.y, 16);
+        if (half == 0) {
+            red[f][warp][c2] = a;
+            red[f][warp][c2 + 1] = b;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < CF * CC) {
+        const int f = threadIdx.x >> 5;
+        float2 s = red[f][0][lane];
+#pragma unroll
+        for (int g = 1; g < CW; ++g) {
+            s.x += red[f][g][lane].x;
+            s.y += red[f][g][lane].y;
+        }
+        if (f < F && n0 + lane < N) {
+            double2* x = X + (int64_t)f * N + n0 + lane;
+            *x = make_double2(x->x + (double)s.x, x->y + (double)s.y);
+        }
+    }
+}
+
+template <int CF>
+cudaError_t corr_block(const float2* W, int64_t N, int F, const float2* r, float2* T, double2* X, cudaStream_t s) {
+    const unsigned rb = (unsigned)((N + CR - 1) / CR), cb = (unsigned)((N + CC - 1) / CC);
+    if ((N & 1) == 0) {
+        k_corr_rows<CF, true><<<rb, 256, 0, s>>>(W, N, F, r, T);
+        k_corr_cols<CF, true><<<cb, CW * 32, 0, s>>>(W, N, F, T, X);
+    } else {
+        k_corr_rows<CF, false><<<rb, 256, 0, s>>>(W, N, F, r, T);
+        k_corr_cols<CF, false><<<cb, CW * 32, 0, s>>>(W, N, F, T, X);
+    }
+    note_launch(2);
+    return cudaGetLastError();
+}
+}  // namespace
+
+// Which frame counts take these kernels: each block of eight frames reads W again, the
+// tensor-core form pays for 128 frames at any count. Whole applies (three refinement
+// steps, one coil), tensor cores / here: N = 400, 8 / 32 / 64 frames 633 / 647 / 670 us
+// against 244 / 421 / 654; N = 1024, 8 / 16 / 32: 556 / 558 / 563 against 308 / 407 / 604;
+// N = 2025, 8 / 16 / 32: 718 / 731 / 806 against 435 / 602 / 995; N = 4096, 1 / 8 / 16:
+// 1025 / 1044 / 1072 against 500 / 784 / 1155; N = 10 000, 1 / 8: 5039 / 5114 against
+// 2003 / 3108. PINV_CORR_ROWS_MAX: another count (0: none).
+bool correct_rows_ok(int64_t N, int64_t F) {
+    static const int64_t v = [] {
+        const char* e = std::getenv("PINV_CORR_ROWS_MAX");
+        return e ? std::max<int64_t>(0, std::atoll(e)) : (int64_t)-1;
+    }();
+    if (v >= 0) return F <= v;
+    return F <= 8 || (F <= 16 && N <= 3072) || (F <= 48 && N <= 512);
+}
+
+cudaError_t launch_correct_rows(const float2* W32, int64_t N, const double2* R, int64_t F, float2* T, double2* X,
+                                float2* r32, cudaStream_t s) {
+    if (F == 0) return cudaSuccess;
+    k_corr_f32<<<(unsigned)((N * F + 255) / 256), 256, 0, s>>>(R, r32, N * F);
+    note_launch();
+    cudaError_t e = cudaGetLastError();
+    for (int64_t f0 = 0; f0 < F && e == cudaSuccess; f0 += CFMAX) {
+        const int Fc = (int)std::min<int64_t>(CFMAX, F - f0);
+        const float2* r = r32 + f0 * N;
+        float2* t = T + f0 * N;
+        double2* x = X + f0 * N;
+        e = Fc <= 1   ? corr_block<1>(W32, N, Fc, r, t, x, s)
+            : Fc <= 2 ? corr_block<2>(W32, N, Fc, r, t, x, s)
+            : Fc <= 4 ? corr_block<4>(W32, N, Fc, r, t, x, s) : corr_block<8>(W32, N, Fc, r, t, x, s);
+    }
+    return e;
+}
+
+}  // namespace pinv

@@ -403,8 +403,12 @@ cudaError_t launch_adjoint_df(const EncodeDev& e, const double2* U, int64_t F, d
 // X[f] += W^H (W R[f]) in FP32 with scratch T [F][N]
 cudaError_t launch_correct32(const float2* W32, int64_t N, const double2* R, int64_t F, float2* T, double2* X,
                              cudaStream_t s);
-// The same correction on the tensor cores (split-BF16, split-K with ordered
-// partial sums; `work` of correct_tc_work_elems() float2), for 16 or more frames.
+// The same for few frames, one pass over W per product (corr.cu); r32: scratch [F][N]
+bool correct_rows_ok(int64_t N, int64_t F);
+cudaError_t launch_correct_rows(const float2* W32, int64_t N, const double2* R, int64_t F, float2* T, double2* X,
+                                float2* r32, cudaStream_t s);
+// The same on the tensor cores (split-BF16, split-K with ordered partial sums; `work` of
+// correct_tc_work_elems() float2).
 bool correct_tc_ok(int64_t F);
 size_t correct_tc_work_elems(int64_t N, int64_t F);
 cudaError_t launch_correct_tc(const float2* W32, int64_t N, const double2* R, int64_t F, float2* T, double2* X,

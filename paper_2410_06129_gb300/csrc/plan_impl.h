@@ -32,6 +32,7 @@ struct ApplyScratch {
     double2* y128;  // s_c o x [F][C][N] for the exact E x
     float2* apw;    // partials of the tensor-core Recon x data
     float2* cw;     // partials of the tensor-core correction x += W^H (W r)
+    float2* r32;    // FP32 copy of r for the correction of few frames [F][N]
     DevStatus* sched;  // tile counter of those launches: one per scratch region, since
                        // applies of one plan may run concurrently on several streams
 };

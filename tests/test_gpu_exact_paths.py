@@ -102,3 +102,25 @@ def test_exact_adjoint_mirror_pairs(dims, keep, coils, frames, samples):
     assert torch.equal(x64.cpu(), torch.from_numpy(x128).to(torch.complex64))
     lean = _plan(dims, k, maps, lean=True, **kw).build()
     assert torch.equal(lean.apply(dd), x64)
+
+
+@pytest.mark.parametrize("dims,frames", [((1,), 1), ((31,), 2), ((32,), 3), ((33,), 4), ((8, 8), 5), ((13, 5), 8),
+                                         ((10, 20), 9), ((27, 19), 17), ((30, 20), 1)])
+def test_correction_of_few_frames(dims, frames):
+    """x = W^H (W b) in FP32, one pass over W per product: N = 1 to 600 around the 4-row and
+    32-column tiles and the 512-column strips, odd (8-byte loads) and even, frames in ragged
+    blocks of 1, 2, 4 and 8. Against the plan's own W in FP64: sums of at most N terms of
+    FP32 products in the two passes, each off by at most 4 sqrt(N) 2^-24 of its magnitudes."""
+    rng = np.random.default_rng(43)
+    N, D = int(np.prod(dims)), len(dims)
+    k = rng.uniform(-0.5 * max(dims), 0.5 * max(dims), size=(3 * N + 5, D))
+    d = rng.standard_normal((frames, 1, len(k))) + 1j * rng.standard_normal((frames, 1, len(k)))
+    E = O.encode(k, O.voxel_positions(dims))
+    pl = _plan(dims, k, lam=0.1, recon_mode=L.RECON_NONE, refine_max_iters=0).build()
+    x = pl.apply(torch.from_numpy(d).cuda()).cpu().numpy()
+    W = pl.export(L.EXPORT_LINV).cpu().numpy()
+    b = (E.conj().T @ d[:, 0].T)
+    want = (W.conj().T @ (W @ b)).T
+    amp = np.linalg.norm(np.abs(W).T @ (np.abs(W) @ np.abs(b))) / np.linalg.norm(want)
+    # two FP32 passes, and W and b rounded to FP32
+    assert rel(x, want) < (2 * 4 * np.sqrt(N) + 4) * 2.0 ** -24 * amp
