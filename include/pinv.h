@@ -427,18 +427,18 @@ pinv_status pinv_plan_map(pinv_plan* plan, int what, const double* psi, double* 
 
 /* Eigenvalue decomposition of the Gram matrix (Section 2.1: the eigenvalues of
  * E^H E are the squared singular values of Encode, and their spectrum shows the
- * conditioning): E^H E + lambda I = P diag(mu + lambda) P^H, by parallel cyclic
- * Jacobi in FP64 on the plan's kept Gram (pinv_plan_keep_gram before the build;
- * a mixed plan's Gram carries its split-precision rounding).
+ * conditioning): E^H E + lambda I = P diag(mu + lambda) P^H, in FP64 on the plan's kept
+ * Gram (pinv_plan_keep_gram before the build; a mixed plan's Gram carries its own
+ * rounding): Householder reduction to a real symmetric tridiagonal, then divide and
+ * conquer, or bisection for the eigenvalues alone.
  *   d_mu  [N] doubles, device: eigenvalues of E^H E (lambda removed), decreasing.
  *   d_P   [N][N] c128, device, row-major, column i the eigenvector of mu[i];
- *         may be NULL: eigenvalues only, by Householder reduction to a real
- *         symmetric tridiagonal and bisection instead (sweeps_out = 0).
- *   sweeps_out  Jacobi sweeps taken (may be NULL).
- * Synchronises with the device once per sweep. Sweeps stop at an off-diagonal
- * Frobenius norm of 4 N eps of the whole, or once a sweep no longer halves it
- * below 1e-10. UNSUPPORTED without a kept Gram, or for eigenvectors with N > 8192;
- * PINV_ERR_INTERNAL if 30 sweeps do not converge (the outputs are still written). */
+ *         may be NULL: eigenvalues only (sweeps_out = 0).
+ *   sweeps_out  passes over the eigenvectors: the leaves' solves and the levels of
+ *         merges after them, at least 1 (may be NULL).
+ * Waits for the device once, at its end. UNSUPPORTED without a kept Gram, or for
+ * eigenvectors with N > 8192; PINV_ERR_INTERNAL if a leaf does not converge, TIMEOUT if a
+ * bounded wait of the reduction gave up. */
 pinv_status pinv_plan_eig(pinv_plan* plan, double* d_mu, void* d_P, int* sweeps_out, void* cuda_stream);
 
 /* Truncated eigen (tSVD) reconstruction (Section 2.1): image = P_r diag(1 / (mu_r

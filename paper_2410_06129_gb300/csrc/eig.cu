@@ -2,19 +2,21 @@
 // (Section 2.1: the SVD spectrum of Encode, truncated SVD, and the eigenvalue
 // decomposition E^H E + lambda I = P Lambda P^H of the normal equations).
 //
-// Parallel cyclic Jacobi, two-sided, in FP64 on a copy of the plan's kept Gram.
-// A sweep is np - 1 rounds (np = n rounded up to even; an odd n leaves one index
-// idle per round). Round r pairs every index once by the circle method: index
-// np - 1 with r, and (r + k) mod (np - 1) with (r - k) mod (np - 1). Pair (p, q)
-// gets the rotation J = diag(1, e^{-i phi}) R(theta) that zeroes G[p][q] (phi the
-// phase of G[p][q], theta the real Jacobi angle of the phase-corrected 2 x 2
-// block). The rotations of a round touch disjoint rows and columns, so they apply
-// together and in place: G <- G J (each row mixes its entries p and q; a CTA
-// rotates a row staged in shared memory), G <- J^H G (a CTA mixes rows p and q),
-// and V <- V J. The rounds of a sweep are captured once into a CUDA graph and
-// replayed. Sweeps stop when the off-diagonal Frobenius norm is below 4 n eps of
-// the whole (the rounding floor of the rotations grows with n), or when a sweep
-// no longer halves it once it is below 1e-10 of the whole, or after 30.
+// Three steps, all in FP64 on a copy of the plan's kept Gram, on the caller's stream:
+//  1. Householder reduction to a real symmetric tridiagonal T (the reflectors kept);
+//  2. the eigenvalues of T alone by bisection with Sturm counts, or with eigenvectors by
+//     divide and conquer (J. J. M. Cuppen, Numer. Math. 36, 1981): T is torn into leaves of
+//     at most 32 rows (each solved by one warp with cyclic Jacobi), and neighbours are
+//     merged level by level. A merge is a rank-one update D + rho z z^T: entries of z that
+//     vanish and poles that coincide are deflated, the other eigenvalues are the roots of
+//     the secular equation, each found by one warp as an offset from its nearest pole, and
+//     z is then recomputed from the roots (M. Gu and S. Eisenstat, SIAM J. Matrix Anal.
+//     Appl. 16, 1995), which keeps the eigenvectors orthogonal to working precision;
+//  3. the reflectors applied to T's eigenvectors.
+// Gram matrices of trajectories have most eigenvalues in clusters, so most of a merge's
+// columns deflate. (The two-sided Jacobi iteration this replaced stayed linear on such
+// spectra: 18-28 sweeps of 3 (n - 1) launches, 21 us a round at n = 400; the whole call
+// took 155 ms there.)
 #include <algorithm>
 #include <cmath>
 #include <climits>
@@ -32,92 +34,11 @@ pinv_status eig_err(cudaError_t e, const char* where) {
                      std::string(where) + ": " + cudaGetErrorString(e));
 }
 
-constexpr int EIG_MAX_N = 8192;   // Jacobi path: the sort stages all eigenvalues in one CTA
-constexpr int EIG_MAX_SWEEPS = 30;
+constexpr int EIG_MAX_N = 8192;   // eigenvectors: a merge stages its poles in one CTA's shared memory
 
 __device__ inline double2 cmul(double2 a, double2 b) { return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
 __device__ inline double2 cconj(double2 a) { return make_double2(a.x, -a.y); }
 __device__ inline double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
-
-// pair k of round r (circle method over np indices), p < q
-__device__ inline void round_pair(int np, int r, int k, int& p, int& q) {
-    if (k == 0) {
-        p = r;
-        q = np - 1;
-    } else {
-        p = (r + k) % (np - 1);
-        q = (r - k + np - 1) % (np - 1);
-    }
-    if (p > q) {
-        const int t = p;
-        p = q;
-        q = t;
-    }
-}
-
-// One rotation per pair: new column j = column j * ca[j] + column part[j] * cb[j].
-__global__ void k_jac_rot(const double2* __restrict__ A, int n, int np, int r, double2* ca, double2* cb, int* part) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= np / 2) return;
-    int p, q;
-    round_pair(np, r, k, p, q);
-    if (q >= n) {  // p is paired with the idle index
-        ca[p] = make_double2(1.0, 0.0);
-        cb[p] = make_double2(0.0, 0.0);
-        part[p] = p;
-        return;
-    }
-    const double a = A[(int64_t)p * n + p].x, d = A[(int64_t)q * n + q].x;
-    const double2 b = A[(int64_t)p * n + q];
-    const double babs = hypot(b.x, b.y);
-    double2 jpp = make_double2(1.0, 0.0), jpq = make_double2(0.0, 0.0), jqp = make_double2(0.0, 0.0),
-            jqq = make_double2(1.0, 0.0);
-    if (babs > 0.0) {
-        const double2 ph = make_double2(b.x / babs, b.y / babs);  // G[p][q] = |G[p][q]| e^{i phi}
-        const double zeta = (d - a) / (2.0 * babs);
-        const double t = fabs(zeta) > 1e150 ? 0.5 / zeta
-                                            : (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-        const double c = 1.0 / sqrt(1.0 + t * t), s = c * t;
-        // J = diag(1, e^{-i phi}) [[c, s], [-s, c]]
-        jpp = make_double2(c, 0.0);
-        jpq = make_double2(s, 0.0);
-        jqp = make_double2(-s * ph.x, s * ph.y);  // -s conj(ph)
-        jqq = make_double2(c * ph.x, -c * ph.y);  // c conj(ph)
-    }
-    ca[p] = jpp;
-    cb[p] = jqp;
-    part[p] = q;
-    ca[q] = jqq;
-    cb[q] = jpq;
-    part[q] = p;
-}
-
-// M <- M J for G and V (blockIdx.y: row, blockIdx.z: 0 = G, 1 = V), in place through shared memory
-__global__ void __launch_bounds__(256) k_jac_cols(double2* G, double2* V, int n, const double2* __restrict__ ca,
-                                                 const double2* __restrict__ cb, const int* __restrict__ part) {
-    extern __shared__ double2 row[];
-    double2* M = blockIdx.z ? V : G;
-    double2* m = M + (int64_t)blockIdx.y * n;
-    for (int j = threadIdx.x; j < n; j += blockDim.x) row[j] = m[j];
-    __syncthreads();
-    for (int j = threadIdx.x; j < n; j += blockDim.x) m[j] = cadd(cmul(row[j], ca[j]), cmul(row[part[j]], cb[j]));
-}
-
-// G <- J^H G: row j becomes conj(ca[j]) row j + conj(cb[j]) row part[j] (one CTA per pair)
-__global__ void __launch_bounds__(256) k_jac_rows(double2* G, int n, int np, int r, const double2* __restrict__ ca,
-                                                 const double2* __restrict__ cb) {
-    int p, q;
-    round_pair(np, r, blockIdx.x, p, q);
-    if (q >= n) return;
-    double2* gp = G + (int64_t)p * n;
-    double2* gq = G + (int64_t)q * n;
-    const double2 app = cconj(ca[p]), apq = cconj(cb[p]), aqq = cconj(ca[q]), aqp = cconj(cb[q]);
-    for (int c = threadIdx.x; c < n; c += blockDim.x) {
-        const double2 x = gp[c], y = gq[c];
-        gp[c] = cadd(cmul(app, x), cmul(apq, y));
-        gq[c] = cadd(cmul(aqq, y), cmul(aqp, x));
-    }
-}
 
 // the upper triangle from the lower (the Gram kernels write only the lower part)
 __global__ void k_hermitian_fill(double2* A, int n) {
@@ -126,110 +47,6 @@ __global__ void k_hermitian_fill(double2* A, int n) {
     const int i = (int)(idx / n), j = (int)(idx % n);
     if (j > i) A[idx] = cconj(A[(int64_t)j * n + i]);
     if (j == i) A[idx].y = 0.0;
-}
-
-__global__ void k_identity(double2* V, int n) {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx < (int64_t)n * n) V[idx] = make_double2(idx / n == idx % n ? 1.0 : 0.0, 0.0);
-}
-
-// per-row sums of |A_ij|^2: off-diagonal in part[i], the diagonal in part[n + i]
-__global__ void __launch_bounds__(256) k_row_norms(const double2* __restrict__ A, int n, double* part) {
-    __shared__ double s_off[256], s_dia[256];
-    const int i = blockIdx.x;
-    double off = 0.0, dia = 0.0;
-    for (int j = threadIdx.x; j < n; j += blockDim.x) {
-        const double2 v = A[(int64_t)i * n + j];
-        const double m = v.x * v.x + v.y * v.y;
-        if (j == i) dia += m;
-        else off += m;
-    }
-    s_off[threadIdx.x] = off;
-    s_dia[threadIdx.x] = dia;
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) {
-            s_off[threadIdx.x] += s_off[threadIdx.x + w];
-            s_dia[threadIdx.x] += s_dia[threadIdx.x + w];
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        part[i] = s_off[0];
-        part[n + i] = s_dia[0];
-    }
-}
-// out[0] = off-diagonal, out[1] = whole squared Frobenius norm (fixed summation order)
-__global__ void __launch_bounds__(256) k_sum_norms(const double* part, int n, double* out) {
-    __shared__ double s_off[256], s_all[256];
-    double off = 0.0, all = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        off += part[i];
-        all += part[i] + part[n + i];
-    }
-    s_off[threadIdx.x] = off;
-    s_all[threadIdx.x] = all;
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) {
-            s_off[threadIdx.x] += s_off[threadIdx.x + w];
-            s_all[threadIdx.x] += s_all[threadIdx.x + w];
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        out[0] = s_off[0];
-        out[1] = s_all[0];
-    }
-}
-
-// Eigenvalues (diag(A) - lam) in decreasing order, ties by index: bitonic sort of
-// (value, index) in one CTA over a power-of-two padding; order[i] = index of mu[i].
-__global__ void __launch_bounds__(1024) k_eig_sort(const double2* __restrict__ A, int n, int npow, double lam,
-                                                  double* mu, int* order) {
-    extern __shared__ double sv[];
-    int* si = reinterpret_cast<int*>(sv + npow);
-    for (int i = threadIdx.x; i < npow; i += blockDim.x) {
-        sv[i] = i < n ? A[(int64_t)i * n + i].x - lam : -INFINITY;
-        si[i] = i;
-    }
-    __syncthreads();
-    for (int size = 2; size <= npow; size <<= 1) {
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int i = threadIdx.x; i < npow; i += blockDim.x) {
-                const int j = i ^ stride;
-                if (j > i) {
-                    // descending by value, ascending by index: "before" means larger value or same value, smaller index
-                    const bool i_before = sv[i] > sv[j] || (sv[i] == sv[j] && si[i] < si[j]);
-                    const bool want_i_before = (i & size) == 0;
-                    if (i_before != want_i_before) {
-                        const double tv = sv[i];
-                        sv[i] = sv[j];
-                        sv[j] = tv;
-                        const int ti = si[i];
-                        si[i] = si[j];
-                        si[j] = ti;
-                    }
-                }
-            }
-            __syncthreads();
-        }
-    }
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        mu[i] = sv[i];
-        order[i] = si[i];
-    }
-}
-
-// P[row][i] = V[row][order[i]] (conj = 0), or Ph[i][row] = conj(V[row][order[i]]) (conj = 1)
-__global__ void k_eig_gather(const double2* __restrict__ V, int n, const int* __restrict__ order, int conj_t,
-                             double2* out) {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (int64_t)n * n) return;
-    const int row = (int)(idx / n), i = (int)(idx % n);
-    const double2 v = V[(int64_t)row * n + order[i]];
-    if (conj_t) out[(int64_t)i * n + row] = cconj(v);
-    else out[idx] = v;
 }
 
 // rank r: the fewest leading eigenvalues holding `energy` of their (non-negative)
@@ -274,37 +91,73 @@ __global__ void k_scale_rows(double2* C, int64_t F, int n, const double* __restr
     C[idx].y *= s;
 }
 
-// ------------------------------------------------------------------ eigenvalues only
-// Householder reduction of the Hermitian A to a real symmetric tridiagonal, one
-// column k at a time (the reflector's scalar tau is chosen so that the subdiagonal
-// entry beta is real), then bisection with Sturm counts, one eigenvalue per thread.
-// Column k below the diagonal is read as the conjugate of row k to the right of it.
-// With H = I - tau v v^H: p = tau A v, c = -Re(conj(tau) v^H p) / 2,
-// w = p + c v, A <- H^H A H = A - w v^H - v w^H on the trailing block.
-struct HhScalars {
-    double2 tau;
-    double beta;
-    double c;
-};
+// ------------------------------------------------------------------ Householder reduction
+// A to a real symmetric tridiagonal, one column k at a time (the reflector's scalar tau
+// is chosen so that the subdiagonal entry beta is real). Column k below the diagonal is
+// read as the conjugate of row k to the right of it. With H = I - tau v v^H: p = tau A v,
+// c = -Re(conj(tau) v^H p) / 2, w = p + c v, A <- H^H A H = A - w v^H - v w^H on the
+// trailing block. v (v[0] = 1) is kept in V's row k from column k + 1, tau in taus[k].
+//
+// One cooperative launch up to n = 4096 (v, w and the next v in shared memory): in step k
+// every CTA forms w of step k - 1 from p, then row k and its reflector, redundantly and
+// alike, and its warps take the rows below in turn, applying step k - 1's update and
+// multiplying by the new v in one pass over A. One grid barrier per column, when p is
+// complete; rows pass from warp to warp through L2 (no load is served by L1). The 4 (n - 2)
+// launches this replaced took 10 us a column at n = 400.
+constexpr int HH_THREADS = 256;
+constexpr int HH_COOP_MAX = 4096;
+constexpr long long HH_WAIT_LIMIT = 4000000000LL;  // clock64 cycles, about 2 s
 
-// reflector of x = A[k + 1 ..][k]: v (v[0] = 1), tau, beta; d[k] and e[k] recorded
-__global__ void __launch_bounds__(256) k_hh_reflector(const double2* __restrict__ A, int n, int k, double2* v,
-                                                     HhScalars* hs, double* d, double* e) {
-    __shared__ double red[256];
-    const int m = n - k - 1;
-    const double2* row = A + (int64_t)k * n + k + 1;  // conj(x_j) = row[j]
-    double s = 0.0;
-    for (int j = 1 + threadIdx.x; j < m; j += blockDim.x) s += row[j].x * row[j].x + row[j].y * row[j].y;
-    red[threadIdx.x] = s;
+struct GridBar {
+    unsigned arrived;  // counts up over the whole launch
+    int failed;        // a wait ran out
+};
+// every thread of the CTA calls it; false once any CTA's wait ran out
+__device__ inline bool grid_barrier(GridBar* gb, unsigned target) {
+    __shared__ int ok;
+    __threadfence();
     __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-        __syncthreads();
+    if (threadIdx.x == 0) {
+        atomicAdd(&gb->arrived, 1u);
+        const long long t0 = clock64();
+        ok = 1;
+        while (*(volatile unsigned*)&gb->arrived < target) {
+            if (*(volatile int*)&gb->failed || clock64() - t0 > HH_WAIT_LIMIT) {
+                atomicExch(&gb->failed, 1);
+                ok = 0;
+                break;
+            }
+        }
+        __threadfence();
     }
-    const double xnorm2 = red[0];
-    const double2 alpha = cconj(row[0]);
-    double2 tau = make_double2(0.0, 0.0), scale = make_double2(0.0, 0.0);
-    double beta = alpha.x;
+    __syncthreads();
+    return ok != 0;
+}
+// sum over the CTA, the same value in every thread
+__device__ inline double block_sum(double v) {
+    __shared__ double red[HH_THREADS / 32];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    double t = 0.0;
+#pragma unroll
+    for (int w = 0; w < HH_THREADS / 32; ++w) t += red[w];
+    return t;
+}
+__device__ inline double2 ld_cg(const double2* p) {
+    double2 v;
+    asm volatile("ld.global.cg.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p) : "memory");
+    return v;
+}
+__device__ inline void st_cg(double2* p, double2 v) {
+    asm volatile("st.global.cg.v2.f64 [%0], {%1, %2};" ::"l"(p), "d"(v.x), "d"(v.y) : "memory");
+}
+// reflector of (alpha; x), xnorm2 = |x|^2: tau, beta (real) and the scale of v = x * scale
+__device__ inline void reflector(double2 alpha, double xnorm2, double2& tau, double& beta, double2& scale) {
+    tau = scale = make_double2(0.0, 0.0);
+    beta = alpha.x;
     if (xnorm2 > 0.0 || alpha.y != 0.0) {
         const double nrm = sqrt(alpha.x * alpha.x + alpha.y * alpha.y + xnorm2);
         beta = alpha.x >= 0.0 ? -nrm : nrm;
@@ -314,11 +167,142 @@ __global__ void __launch_bounds__(256) k_hh_reflector(const double2* __restrict_
         const double dd = den.x * den.x + den.y * den.y;
         scale = make_double2(den.x / dd, -den.y / dd);
     }
+}
+
+// pb: [2][n] products p, alternating; ph: the phase that makes the last subdiagonal real
+__global__ void __launch_bounds__(HH_THREADS) k_hh_reduce(double2* A, int n, double2* V, double2* taus, double* d,
+                                                          double* e, double2* ph, double2* pb, GridBar* gb) {
+    extern __shared__ double2 hsm[];
+    double2* v = hsm;           // v of the last step, entries k .. n - 1 at their own index
+    double2* w = hsm + n;
+    double2* vn = hsm + 2 * n;  // v of this step
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int gw = blockIdx.x * (HH_THREADS / 32) + (tid >> 5), nw = gridDim.x * (HH_THREADS / 32);
+    double2 tau = make_double2(0.0, 0.0);
+    for (int k = 0;; ++k) {
+        if (k > 0) {  // w of step k - 1
+            const double2* p = pb + (size_t)((k - 1) & 1) * n;
+            double t = 0.0;
+            for (int j = k + tid; j < n; j += HH_THREADS) {
+                const double2 q = ld_cg(p + j);
+                w[j] = q;
+                const double2 a = cmul(cconj(v[j]), q);
+                t += tau.x * a.x + tau.y * a.y;  // Re(conj(tau) v^H p)
+            }
+            const double c = -0.5 * block_sum(t);
+            for (int j = k + tid; j < n; j += HH_THREADS) {
+                const double2 q = w[j], u = v[j];
+                w[j] = make_double2(q.x + c * u.x, q.y + c * u.y);
+            }
+            __syncthreads();
+        }
+        auto updated = [&](int i, int j, double2 a) {  // A[i][j] after step k - 1
+            if (k == 0) return a;
+            const double2 t = cadd(cmul(w[i], cconj(v[j])), cmul(v[i], cconj(w[j])));
+            return make_double2(a.x - t.x, a.y - t.y);
+        };
+        if (k >= n - 2) {  // the last 2 x 2 block
+            if (blockIdx.x == 0 && tid == 0) {
+                for (int i = k; i < n; ++i) d[i] = updated(i, i, ld_cg(A + (size_t)i * n + i)).x;
+                ph[0] = make_double2(1.0, 0.0);
+                if (n >= 2) {
+                    const double2 b = updated(n - 1, n - 2, ld_cg(A + (size_t)(n - 1) * n + n - 2));
+                    const double m = hypot(b.x, b.y);
+                    e[n - 2] = m;
+                    if (m > 0.0) ph[0] = make_double2(b.x / m, b.y / m);
+                }
+            }
+            return;
+        }
+        // row k: conj(x), its reflector
+        const double2* row = A + (size_t)k * n;
+        double xn = 0.0;
+        for (int j = k + 1 + tid; j < n; j += HH_THREADS) {
+            const double2 x = cconj(updated(k, j, ld_cg(row + j)));
+            vn[j] = x;
+            if (j > k + 1) xn += x.x * x.x + x.y * x.y;
+        }
+        xn = block_sum(xn);  // its barriers also complete vn
+        double2 scale;
+        double beta;
+        const double2 alpha = vn[k + 1];
+        double2 tn;
+        reflector(alpha, xn, tn, beta, scale);
+        if (blockIdx.x == 0 && tid == 0) {
+            d[k] = updated(k, k, ld_cg(row + k)).x;
+            e[k] = beta;
+            taus[k] = tn;
+        }
+        __syncthreads();  // alpha read before vn[k + 1] becomes 1
+        for (int j = k + 1 + tid; j < n; j += HH_THREADS) {
+            const double2 x = j == k + 1 ? make_double2(1.0, 0.0) : cmul(vn[j], scale);
+            vn[j] = x;
+            if (blockIdx.x == 0) V[(size_t)k * n + j] = x;
+        }
+        __syncthreads();
+        // rows below: step k - 1's update and the product with v
+        double2* p = pb + (size_t)(k & 1) * n;
+        for (int i = k + 1 + gw; i < n; i += nw) {
+            double2* ar = A + (size_t)i * n;
+            double2 acc = make_double2(0.0, 0.0);
+            const double2 wi = k > 0 ? w[i] : make_double2(0.0, 0.0), vi = k > 0 ? v[i] : wi;
+            // four entries at a time: their loads are in flight together
+            for (int j = k + 1 + lane; j < n; j += 128) {
+                double2 a[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    a[u] = j + 32 * u < n ? ld_cg(ar + j + 32 * u) : make_double2(0.0, 0.0);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int ju = j + 32 * u;
+                    if (ju >= n) continue;
+                    if (k > 0) {
+                        const double2 t = cadd(cmul(wi, cconj(v[ju])), cmul(vi, cconj(w[ju])));
+                        a[u] = make_double2(a[u].x - t.x, a[u].y - t.y);
+                        st_cg(ar + ju, a[u]);
+                    }
+                    acc = cadd(acc, cmul(a[u], vn[ju]));
+                }
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
+                acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
+            }
+            if (lane == 0) st_cg(p + i, cmul(tn, acc));
+        }
+        if (!grid_barrier(gb, (unsigned)(k + 1) * gridDim.x)) return;
+        double2* t = v;
+        v = vn;
+        vn = t;
+        tau = tn;
+    }
+}
+
+// The same reduction above n = 4096, four launches a column.
+struct HhScalars {
+    double2 tau;
+    double beta;
+    double c;
+};
+
+// reflector of x = A[k + 1 ..][k]: v (v[0] = 1), tau, beta; d[k] and e[k] recorded
+__global__ void __launch_bounds__(HH_THREADS) k_hh_reflector(const double2* __restrict__ A, int n, int k, double2* v,
+                                                            HhScalars* hs, double2* taus, double* d, double* e) {
+    const int m = n - k - 1;
+    const double2* row = A + (int64_t)k * n + k + 1;  // conj(x_j) = row[j]
+    double s = 0.0;
+    for (int j = 1 + threadIdx.x; j < m; j += blockDim.x) s += row[j].x * row[j].x + row[j].y * row[j].y;
+    s = block_sum(s);
+    double2 tau, scale;
+    double beta;
+    reflector(cconj(row[0]), s, tau, beta, scale);
     for (int j = threadIdx.x; j < m; j += blockDim.x)
         v[j] = j == 0 ? make_double2(1.0, 0.0) : cmul(cconj(row[j]), scale);
     if (threadIdx.x == 0) {
         hs->tau = tau;
         hs->beta = beta;
+        taus[k] = tau;
         d[k] = A[(int64_t)k * n + k].x;
         e[k] = beta;
     }
@@ -373,12 +357,15 @@ __global__ void __launch_bounds__(256) k_hh_update(double2* A, int n, int k, con
     }
 }
 
-// last 2 x 2 block: d[n-2], d[n-1], e[n-2] = |A[n-1][n-2]|
-__global__ void k_hh_tail(const double2* __restrict__ A, int n, double* d, double* e) {
+// last 2 x 2 block: d[n-2], d[n-1], e[n-2] = |A[n-1][n-2]| and its phase
+__global__ void k_hh_tail(const double2* __restrict__ A, int n, double* d, double* e, double2* ph) {
+    ph[0] = make_double2(1.0, 0.0);
     if (n >= 2) {
         d[n - 2] = A[(int64_t)(n - 2) * n + n - 2].x;
         const double2 b = A[(int64_t)(n - 1) * n + n - 2];
-        e[n - 2] = hypot(b.x, b.y);
+        const double m = hypot(b.x, b.y);
+        e[n - 2] = m;
+        if (m > 0.0) ph[0] = make_double2(b.x / m, b.y / m);
     }
     d[n - 1] = A[(int64_t)(n - 1) * n + n - 1].x;
 }
@@ -414,6 +401,448 @@ __global__ void k_tridiag_bisect(const double* __restrict__ d, const double* __r
     mu[n - 1 - i] = 0.5 * (lo + hi) - lam;
 }
 
+// ------------------------------------------------------------------ divide and conquer
+// Leaf i of nl covers rows b(i) .. b(i + 1) - 1, b(i) = i n / nl; a merge of width w at
+// node t joins leaves 2 w t .. 2 w t + w - 1 with the next w. Q holds the eigenvectors of
+// the blocks formed so far (block diagonal, row-major n x n), D their eigenvalues.
+constexpr int DC_LEAF = 32;
+constexpr double DC_EPS = 2.220446049250313e-16;
+__host__ __device__ inline int dc_bound(int i, int n, int nl) { return (int)((int64_t)i * n / nl); }
+struct DcNode {
+    int lo, mid, hi;
+};
+__device__ inline DcNode dc_node(int t, int w, int n, int nl) {
+    return {dc_bound(2 * w * t, n, nl), dc_bound(2 * w * t + w, n, nl), dc_bound(2 * w * (t + 1), n, nl)};
+}
+// what a merge's set-up leaves for the other kernels of its level (arrays indexed from lo)
+struct DcWork {
+    double *kd, *kz;    // kept poles in increasing order, and z; then the deflated eigenvalues
+    int* kcol;          // their columns of Q
+    double *rc, *rs;    // column rotations of the deflation, in order
+    int2* rcol;
+    int *org;           // per root: the pole it is measured from
+    double *mu, *zh;    // ... its offset, and the recomputed z
+    int *K, *nrot;      // per node
+    double* rho;
+    int* failed;
+};
+
+// The leaf's tridiagonal (its corners less |e| of the torn couplings) by cyclic Jacobi, one
+// warp: the pairs of a round are disjoint, lane l mixes row l's columns, then column l's rows.
+__global__ void __launch_bounds__(32) k_dc_leaf(const double* __restrict__ d, const double* __restrict__ e, int n,
+                                               int nl, double* D, double* Q, int* failed) {
+    __shared__ double A[DC_LEAF][DC_LEAF + 1], Z[DC_LEAF][DC_LEAF + 1];
+    __shared__ double cs[DC_LEAF / 2], sn[DC_LEAF / 2];
+    const int lane = threadIdx.x;
+    const int lo = dc_bound(blockIdx.x, n, nl), hi = dc_bound(blockIdx.x + 1, n, nl), m = hi - lo;
+    const int mp = m + (m & 1);
+    for (int j = 0; j < m; ++j) {
+        if (lane < m) {
+            double a = 0.0;
+            if (lane == j) {
+                a = d[lo + j];
+                if (j == 0 && lo > 0) a -= fabs(e[lo - 1]);
+                if (j == m - 1 && hi < n) a -= fabs(e[hi - 1]);
+            } else if (lane == j + 1) {
+                a = e[lo + j];
+            } else if (lane == j - 1) {
+                a = e[lo + j - 1];
+            }
+            A[lane][j] = a;
+            Z[lane][j] = lane == j ? 1.0 : 0.0;
+        }
+    }
+    __syncwarp();
+    double nrm = 0.0;
+    if (lane < m)
+        for (int j = 0; j < m; ++j) nrm = fmax(nrm, fabs(A[lane][j]));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) nrm = fmax(nrm, __shfl_xor_sync(0xffffffffu, nrm, o));
+    const double tiny = nrm * (DC_EPS / 16.0);  // an off-diagonal entry below it changes no eigenvalue
+    bool again = m > 1;
+    int sweep = 0;
+    for (; again && sweep < 40; ++sweep) {
+        again = false;
+        for (int r = 0; r < mp - 1; ++r) {
+            // circle method: pair 0 is (mp - 1, r), pair k is (r + k, r - k) mod (mp - 1)
+            if (lane < mp / 2) {
+                int p = lane ? (r + lane) % (mp - 1) : r, q = lane ? (r - lane + mp - 1) % (mp - 1) : mp - 1;
+                if (p > q) {
+                    const int t = p;
+                    p = q;
+                    q = t;
+                }
+                double c = 1.0, s = 0.0;
+                if (q < m) {
+                    const double b = A[p][q];
+                    if (fabs(b) > tiny) {
+                        const double th = (A[q][q] - A[p][p]) / (2.0 * b);
+                        const double t = fabs(th) > 1e150 ? 0.5 / th
+                                                          : (th >= 0.0 ? 1.0 : -1.0) / (fabs(th) + sqrt(1.0 + th * th));
+                        c = 1.0 / sqrt(1.0 + t * t);
+                        s = c * t;
+                    }
+                }
+                cs[lane] = c;
+                sn[lane] = s;
+            }
+            __syncwarp();
+            bool any = false;
+            for (int k = 0; k < mp / 2; ++k) {
+                const double c = cs[k], s = sn[k];
+                if (s == 0.0) continue;
+                any = true;
+                int p = k ? (r + k) % (mp - 1) : r, q = k ? (r - k + mp - 1) % (mp - 1) : mp - 1;
+                if (p > q) {
+                    const int t = p;
+                    p = q;
+                    q = t;
+                }
+                if (lane < m) {
+                    const double x = A[lane][p], y = A[lane][q], u = Z[lane][p], v = Z[lane][q];
+                    A[lane][p] = c * x - s * y;
+                    A[lane][q] = s * x + c * y;
+                    Z[lane][p] = c * u - s * v;
+                    Z[lane][q] = s * u + c * v;
+                }
+            }
+            __syncwarp();
+            for (int k = 0; k < mp / 2; ++k) {
+                const double c = cs[k], s = sn[k];
+                if (s == 0.0) continue;
+                int p = k ? (r + k) % (mp - 1) : r, q = k ? (r - k + mp - 1) % (mp - 1) : mp - 1;
+                if (p > q) {
+                    const int t = p;
+                    p = q;
+                    q = t;
+                }
+                if (lane < m) {
+                    const double x = A[p][lane], y = A[q][lane];
+                    A[p][lane] = c * x - s * y;
+                    A[q][lane] = s * x + c * y;
+                }
+            }
+            __syncwarp();
+            again = again || any;
+        }
+    }
+    if (again && lane == 0) atomicExch(failed, 1);
+    if (lane < m) {
+        D[lo + lane] = A[lane][lane];
+        for (int j = 0; j < m; ++j) Q[(size_t)(lo + lane) * n + lo + j] = Z[lane][j];
+    }
+}
+
+// z, the sorted poles, and the deflation, one CTA per merge. The scan over the sorted poles
+// is one thread's: a pole whose rho |z| is negligible is an eigenvalue as it is, and of two
+// poles so close that a rotation of their columns moves all of z to the second at the cost
+// of a negligible off-diagonal entry, the first is.
+__global__ void __launch_bounds__(512) k_dc_setup(const double* __restrict__ D, const double* __restrict__ e,
+                                                 const double* __restrict__ Q, int n, int nl, int wd, DcWork k) {
+    extern __shared__ double dsm[];
+    const DcNode nd = dc_node(blockIdx.x, wd, n, nl);
+    const int m = nd.hi - nd.lo, tid = threadIdx.x;
+    double *ds = dsm, *zs = dsm + m;
+    int* pm = reinterpret_cast<int*>(dsm + 2 * m);
+    const double em = e[nd.mid - 1], rho = 2.0 * fabs(em), sg = em < 0.0 ? -1.0 : 1.0;
+    for (int i = tid; i < m; i += blockDim.x) {  // (a NaN has no rank: every slot holds a column of the block)
+        ds[i] = zs[i] = 0.0;
+        pm[i] = nd.lo + i;
+    }
+    __syncthreads();
+    for (int i = tid; i < m; i += blockDim.x) {
+        const double di = D[nd.lo + i];
+        int r = 0;  // rank among the poles, ties by index
+        for (int j = 0; j < m; ++j) {
+            const double dj = D[nd.lo + j];
+            r += dj < di || (dj == di && j < i);
+        }
+        const int c = nd.lo + i;
+        const double z = c < nd.mid ? Q[(size_t)(nd.mid - 1) * n + c] : sg * Q[(size_t)nd.mid * n + c];
+        ds[r] = di;
+        zs[r] = z * 0.70710678118654752440;  // |z| = 1
+        pm[r] = c;
+    }
+    __syncthreads();
+    if (tid != 0) return;
+    const double tol = 8.0 * DC_EPS * fmax(fmax(fabs(ds[0]), fabs(ds[m - 1])), rho);
+    int K = 0, nd2 = 0, nr = 0, pj = -1;
+    double* kd = k.kd + nd.lo;
+    double* kz = k.kz + nd.lo;
+    int* kc = k.kcol + nd.lo;
+    auto deflate = [&](int j) {
+        ++nd2;
+        kd[m - nd2] = ds[j];
+        kc[m - nd2] = pm[j];
+    };
+    auto keep = [&](int j) {
+        kd[K] = ds[j];
+        kz[K] = zs[j];
+        kc[K] = pm[j];
+        ++K;
+    };
+    for (int j = 0; j < m; ++j) {
+        if (rho * fabs(zs[j]) <= tol) {
+            deflate(j);
+            continue;
+        }
+        if (pj < 0) {
+            pj = j;
+            continue;
+        }
+        const double gap = ds[j] - ds[pj], tau = hypot(zs[j], zs[pj]);
+        const double c = zs[j] / tau, s = zs[pj] / tau;
+        if (fabs(gap * c * s) <= tol) {
+            // columns (pj, j) <- (c pj - s j, s pj + c j)
+            k.rcol[nd.lo + nr] = make_int2(pm[pj], pm[j]);
+            k.rc[nd.lo + nr] = c;
+            k.rs[nd.lo + nr] = s;
+            ++nr;
+            const double a = ds[pj], b = ds[j];
+            ds[pj] = a * c * c + b * s * s;
+            ds[j] = a * s * s + b * c * c;
+            zs[j] = tau;
+            deflate(pj);
+            pj = j;
+        } else {
+            keep(pj);
+            pj = j;
+        }
+    }
+    if (pj >= 0) keep(pj);
+    k.K[blockIdx.x] = K;
+    k.nrot[blockIdx.x] = nr;
+    k.rho[blockIdx.x] = rho;
+}
+
+// the deflation's column rotations, a thread per row
+__global__ void k_dc_rotate(double* Q, int n, int nl, int wd, DcWork k) {
+    const DcNode nd = dc_node(blockIdx.y, wd, n, nl);
+    const int i = nd.lo + blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= nd.hi) return;
+    double* row = Q + (size_t)i * n;
+    for (int r = 0; r < k.nrot[blockIdx.y]; ++r) {
+        const int2 c2 = k.rcol[nd.lo + r];
+        const double c = k.rc[nd.lo + r], s = k.rs[nd.lo + r], x = row[c2.x], y = row[c2.y];
+        row[c2.x] = c * x - s * y;
+        row[c2.y] = s * x + c * y;
+    }
+}
+
+__device__ inline double warp_sum_d(double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// Root i of 1 + rho sum_j z_j^2 / (d_j - lambda) in (d_i, d_{i+1}) (the last in (d_K,
+// d_K + rho |z|^2)), one warp: lambda = d_o + mu with o the nearer pole (the sign at the
+// midpoint tells). Each step fits psi and phi (the sums left and right of the root) by
+// one pole each with their values and slopes matched, and falls back to shrinking the
+// bracket, so it always ends; it stops when the sum is rounding, or the bracket a last place.
+__global__ void __launch_bounds__(256) k_dc_secular(int n, int nl, int wd, DcWork k, double* Dn) {
+    const DcNode nd = dc_node(blockIdx.y, wd, n, nl);
+    const int K = k.K[blockIdx.y], i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (i >= K) return;
+    const double rho = k.rho[blockIdx.y];
+    const double* d = k.kd + nd.lo;
+    const double* z = k.kz + nd.lo;
+    const bool last = i == K - 1;
+    double zz = 0.0;
+    if (last) {
+        for (int j = lane; j < K; j += 32) zz = fma(z[j], z[j], zz);
+        zz = warp_sum_d(zz);
+    }
+    const double gap = last ? rho * zz : d[i + 1] - d[i], mid = 0.5 * gap;
+    // sums at d_o + mu: psi, phi and their slopes
+    auto eval = [&](double base, double mu, double& psi, double& phi, double& dpsi, double& dphi) {
+        psi = phi = dpsi = dphi = 0.0;
+        for (int j = lane; j < K; j += 32) {
+            const double w = (d[j] - base) - mu, zj = z[j], t = rho * zj * zj / w, u = t / w;
+            if (j <= i) {
+                psi += t;
+                dpsi += u;
+            } else {
+                phi += t;
+                dphi += u;
+            }
+        }
+        psi = warp_sum_d(psi);
+        phi = warp_sum_d(phi);
+        dpsi = warp_sum_d(dpsi);
+        dphi = warp_sum_d(dphi);
+    };
+    double psi, phi, dpsi, dphi;
+    eval(d[i], mid, psi, phi, dpsi, dphi);
+    int o = i;
+    double lo, hi;
+    if (1.0 + psi + phi < 0.0) {  // the root lies right of the midpoint
+        if (last) {
+            lo = mid;
+            hi = gap;
+        } else {
+            o = i + 1;
+            lo = -mid;
+            hi = 0.0;
+        }
+    } else {
+        lo = 0.0;
+        hi = mid;
+    }
+    const double base = d[o], p0 = d[i] - base, p1 = last ? gap : d[i + 1] - base;
+    double mu = 0.5 * (lo + hi);
+    for (int it = 0; it < 120; ++it) {
+        eval(base, mu, psi, phi, dpsi, dphi);
+        const double f = 1.0 + psi + phi;
+        if (fabs(f) <= 2.0 * DC_EPS * (1.0 + fabs(psi) + fabs(phi))) break;
+        if (f < 0.0) lo = mu;
+        else hi = mu;
+        if (hi - lo <= DC_EPS * fmin(fabs(lo), fabs(hi)) && lo * hi > 0.0) break;
+        const double D0 = p0 - mu, D1 = p1 - mu;
+        const double c = f - D0 * dpsi - D1 * dphi, a = (D0 + D1) * f - D0 * D1 * (dpsi + dphi), b = D0 * D1 * f;
+        const double q = sqrt(fmax(a * a - 4.0 * b * c, 0.0));
+        double eta = a <= 0.0 ? (a - q) / (2.0 * c) : 2.0 * b / (a + q);
+        if (!(f * eta < 0.0)) eta = -f / (dpsi + dphi);
+        double nx = mu + eta;
+        if (!(nx > lo && nx < hi)) {
+            nx = lo == 0.0 ? 0.125 * hi : hi == 0.0 ? 0.125 * lo : 0.5 * (lo + hi);
+            if (!(nx > lo && nx < hi)) nx = 0.5 * (lo + hi);
+        }
+        if (nx == mu) break;
+        mu = nx;
+    }
+    if (lane == 0) {
+        k.org[nd.lo + i] = o;
+        k.mu[nd.lo + i] = mu;
+        Dn[nd.lo + i] = base + mu;
+    }
+}
+
+// z_j^2 = prod_k (lambda_k - d_j) / (the poles other than d_j, and rho), with z's sign; one warp per j
+__global__ void __launch_bounds__(256) k_dc_zhat(int n, int nl, int wd, DcWork k) {
+    const DcNode nd = dc_node(blockIdx.y, wd, n, nl);
+    const int K = k.K[blockIdx.y], j = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (j >= K) return;
+    const double* d = k.kd + nd.lo;
+    const double dj = d[j];
+    double p = 1.0;
+    for (int t = lane; t < K; t += 32) {
+        const double num = (d[k.org[nd.lo + t]] - dj) + k.mu[nd.lo + t];
+        const double den = t < j ? d[t] - dj : t < K - 1 ? d[t + 1] - dj : k.rho[blockIdx.y];
+        p *= num / den;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) p *= __shfl_xor_sync(0xffffffffu, p, o);
+    if (lane == 0) k.zh[nd.lo + j] = copysign(sqrt(fabs(p)), k.kz[nd.lo + j]);
+}
+
+// U[lo + i][lo + j] = z_j / (d_j - lambda_i), normalised: eigenvector i of D + rho z z^T in
+// row i; one warp per eigenvector
+__global__ void __launch_bounds__(256) k_dc_vectors(int n, int nl, int wd, DcWork k, double* U) {
+    const DcNode nd = dc_node(blockIdx.y, wd, n, nl);
+    const int K = k.K[blockIdx.y], i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (i >= K) return;
+    const double* d = k.kd + nd.lo;
+    const double base = d[k.org[nd.lo + i]], mu = k.mu[nd.lo + i];
+    double* u = U + (size_t)(nd.lo + i) * n + nd.lo;
+    double s = 0.0;
+    for (int j = lane; j < K; j += 32) {
+        const double x = k.zh[nd.lo + j] / ((d[j] - base) - mu);
+        u[j] = x;
+        s = fma(x, x, s);
+    }
+    const double r = 1.0 / sqrt(warp_sum_d(s));
+    for (int j = lane; j < K; j += 32) u[j] *= r;
+}
+
+// Qn's columns lo .. lo + K - 1 = Q's kept columns times U^T; the columns after them are
+// Q's deflated ones. 32 x 32 tile, four outputs a thread.
+__global__ void __launch_bounds__(256) k_dc_update(const double* __restrict__ Q, const double* __restrict__ U, int n,
+                                                  int nl, int wd, DcWork k, double* Qn, double* Dn) {
+    __shared__ double As[32][33], Bs[32][33];
+    const DcNode nd = dc_node(blockIdx.z, wd, n, nl);
+    const int K = k.K[blockIdx.z], m = nd.hi - nd.lo;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int c0 = blockIdx.x * 32, r0 = nd.lo + blockIdx.y * 32;
+    if (c0 >= m || r0 >= nd.hi) return;
+    const int c = c0 + tx;
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    if (c0 < K) {
+        for (int j0 = 0; j0 < K; j0 += 32) {
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const int row = r0 + ty + 8 * r, uc = c0 + ty + 8 * r, j = j0 + tx;
+                As[ty + 8 * r][tx] = row < nd.hi && j < K ? Q[(size_t)row * n + k.kcol[nd.lo + j]] : 0.0;
+                Bs[ty + 8 * r][tx] = uc < K && j < K ? U[(size_t)(nd.lo + uc) * n + nd.lo + j] : 0.0;
+            }
+            __syncthreads();
+#pragma unroll 8
+            for (int j = 0; j < 32; ++j) {
+                const double b = Bs[tx][j];
+#pragma unroll
+                for (int r = 0; r < 4; ++r) acc[r] = fma(As[ty + 8 * r][j], b, acc[r]);
+            }
+            __syncthreads();
+        }
+    }
+    if (c >= m) return;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int row = r0 + ty + 8 * r;
+        if (row < nd.hi) Qn[(size_t)row * n + nd.lo + c] = c < K ? acc[r] : Q[(size_t)row * n + k.kcol[nd.lo + c]];
+    }
+    if (c >= K && blockIdx.y == 0 && ty == 0) Dn[nd.lo + c] = k.kd[nd.lo + c];
+}
+
+// mu (decreasing, ties by index, lam removed) and the column of Q each comes from
+__global__ void k_dc_order(const double* __restrict__ D, int n, double lam, double* mu, int* order) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const double di = D[i];
+    int r = 0;
+    for (int j = 0; j < n; ++j) {
+        const double dj = D[j];
+        r += dj > di || (dj == di && j < i);
+    }
+    mu[r] = di - lam;
+    order[r] = i;
+}
+
+// P[:, i] = H_0 .. H_{n-3} (phase) Q[:, order[i]], H_k = I - tau_k v_k v_k^H: a warp per
+// column, which it holds in shared memory
+__global__ void k_hh_back(const double2* __restrict__ V, const double2* __restrict__ taus,
+                          const double2* __restrict__ ph, const double* __restrict__ Q, int n,
+                          const int* __restrict__ order, double2* P) {
+    extern __shared__ double2 zsm[];
+    const int wpb = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int i = blockIdx.x * wpb + warp;
+    if (i >= n) return;
+    double2* z = zsm + (size_t)warp * n;
+    const int col = order[i];
+    for (int j = lane; j < n; j += 32) {
+        const double q = Q[(size_t)j * n + col];
+        const double2 f = j == n - 1 ? ph[0] : make_double2(1.0, 0.0);
+        z[j] = make_double2(q * f.x, q * f.y);
+    }
+    __syncwarp();
+    for (int k = n - 3; k >= 0; --k) {
+        const double2* v = V + (size_t)k * n;
+        double2 s = make_double2(0.0, 0.0);
+#pragma unroll 4
+        for (int j = k + 1 + lane; j < n; j += 32) s = cadd(s, cmul(cconj(v[j]), z[j]));
+        s.x = warp_sum_d(s.x);
+        s.y = warp_sum_d(s.y);
+        s = cmul(taus[k], s);
+#pragma unroll 4
+        for (int j = k + 1 + lane; j < n; j += 32) {
+            const double2 t = cmul(v[j], s);
+            z[j] = make_double2(z[j].x - t.x, z[j].y - t.y);
+        }
+        __syncwarp();
+    }
+    for (int j = lane; j < n; j += 32) P[(size_t)j * n + i] = z[j];
+}
+
 inline unsigned blocks(int64_t n, int t = 256) { return (unsigned)((n + t - 1) / t); }
 
 }  // namespace
@@ -428,26 +857,13 @@ extern "C" pinv_status pinv_plan_eig(pinv_plan* p, double* d_mu, void* d_P, int*
     if (d_P && p->N > EIG_MAX_N)
         return set_error(PINV_ERR_UNSUPPORTED, "eigenvectors limited to N <= 8192 (eigenvalues alone are not)");
     if (p->N > INT_MAX / 2) return set_error(PINV_ERR_UNSUPPORTED, "N too large");
-    const int n = (int)p->N, np = n + (n & 1);
-    cudaStream_t us = (cudaStream_t)stream;
+    const int n = (int)p->N;
+    cudaStream_t s = (cudaStream_t)stream;
     const size_t nn = (size_t)n * n;
-    double2 *A = nullptr, *V = nullptr, *ca = nullptr, *cb = nullptr;
-    int *part = nullptr, *order = nullptr;
-    double *norms = nullptr, *hn = nullptr;
-    cudaStream_t s = nullptr;
-    cudaEvent_t ev = nullptr;
-    cudaGraphExec_t sweep = nullptr;
-    pinv_status result = PINV_OK;
+    // every buffer goes back to the pool in stream order when this returns
+    std::vector<void*> bufs;
     auto done = [&](pinv_status st) {
-        if (sweep) cudaGraphExecDestroy(sweep);
-        if (s) {
-            cudaStreamSynchronize(s);
-            cudaStreamDestroy(s);
-        }
-        if (ev) cudaEventDestroy(ev);
-        for (void* ptr : {(void*)A, (void*)V, (void*)ca, (void*)cb, (void*)part, (void*)order, (void*)norms})
-            if (ptr) cudaFree(ptr);
-        if (hn) cudaFreeHost(hn);
+        for (void* b : bufs) cudaFreeAsync(b, s);
         return st;
     };
 #define CKE(call)                                                \
@@ -455,118 +871,140 @@ extern "C" pinv_status pinv_plan_eig(pinv_plan* p, double* d_mu, void* d_P, int*
         cudaError_t e_ = (call);                                 \
         if (e_ != cudaSuccess) return done(eig_err(e_, #call));  \
     } while (0)
-    CKE(cudaMalloc(&A, sizeof(double2) * nn));
-    CKE(cudaMalloc(&V, sizeof(double2) * nn));
-    CKE(cudaMalloc(&ca, sizeof(double2) * np));
-    CKE(cudaMalloc(&cb, sizeof(double2) * np));
-    CKE(cudaMalloc(&part, sizeof(int) * np));
-    CKE(cudaMalloc(&order, sizeof(int) * np));
-    CKE(cudaMalloc(&norms, sizeof(double) * (2 * (size_t)n + 2)));
-    CKE(cudaMallocHost(&hn, sizeof(double) * 2));
-    // a private stream (graph capture needs one), ordered after the caller's work
-    CKE(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
-    CKE(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
-    CKE(cudaEventRecord(ev, us));
-    CKE(cudaStreamWaitEvent(s, ev, 0));
-
+    auto take = [&](void** q, size_t bytes) -> cudaError_t {
+        cudaError_t e = work_alloc(q, bytes, s);
+        if (e == cudaSuccess) bufs.push_back(*q);
+        return e;
+    };
+    struct Flags {
+        GridBar bar;
+        int leaf_failed;
+    };
+    double2 *A = nullptr, *V = nullptr, *taus = nullptr, *ph = nullptr, *pb = nullptr;
+    double *dd = nullptr, *ee = nullptr;
+    Flags* fl = nullptr;
+    HhScalars* hs = nullptr;
+    CKE(take((void**)&A, sizeof(double2) * nn));
+    CKE(take((void**)&V, sizeof(double2) * nn));
+    CKE(take((void**)&taus, sizeof(double2) * n));
+    CKE(take((void**)&ph, sizeof(double2)));
+    CKE(take((void**)&pb, sizeof(double2) * 2 * n));
+    CKE(take((void**)&dd, sizeof(double) * n));
+    CKE(take((void**)&ee, sizeof(double) * n));
+    CKE(take((void**)&fl, sizeof(Flags)));
+    CKE(take((void**)&hs, sizeof(HhScalars)));
+    CKE(cudaMemsetAsync(fl, 0, sizeof(Flags), s));
     CKE(cudaMemcpyAsync(A, p->Gkeep, sizeof(double2) * nn, cudaMemcpyDeviceToDevice, s));
     k_hermitian_fill<<<blocks((int64_t)nn), 256, 0, s>>>(A, n);
     note_launch();
     CKE(cudaGetLastError());
-    if (!d_P) {
-        // eigenvalues only: Householder tridiagonalisation, then bisection; the
-        // 4 (n - 2) launches of the reduction run from one graph
-        double2 *v = V, *pv = V + n;  // V is not needed on this path: its first 2n entries hold v and p
-        double *dd = norms, *ee = norms + n;
-        HhScalars* hs = reinterpret_cast<HhScalars*>(ca);
-        cudaGraph_t g = nullptr;
-        CKE(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
+    if (n <= HH_COOP_MAX) {
+        const size_t smem = sizeof(double2) * 3 * n;
+        CKE(cudaFuncSetAttribute(k_hh_reduce, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        int dev = 0, sms = 0, per = 0;
+        CKE(cudaGetDevice(&dev));
+        CKE(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        CKE(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_hh_reduce, HH_THREADS, smem));
+        if (per < 1) return done(set_error(PINV_ERR_INTERNAL, "the reduction does not fit an SM"));
+        // a warp per row of the first columns, at most one CTA per SM
+        const unsigned grid = std::max(1u, std::min((unsigned)sms, blocks(n, HH_THREADS / 32)));
+        int nv = n;
+        GridBar* gb = &fl->bar;
+        void* args[] = {&A, &nv, &V, &taus, &dd, &ee, &ph, &pb, &gb};
+        CKE(cudaLaunchCooperativeKernel((const void*)k_hh_reduce, dim3(grid), dim3(HH_THREADS), args, smem, s));
+        note_launch();
+    } else {
         for (int k = 0; k + 2 < n; ++k) {
             const int m = n - k - 1;
-            k_hh_reflector<<<1, 256, 0, s>>>(A, n, k, v, hs, dd, ee);
-            k_hh_matvec<<<blocks(m, 8), 256, 0, s>>>(A, n, k, v, hs, pv);
-            k_hh_coef<<<1, 256, 0, s>>>(n, k, v, pv, hs);
-            k_hh_update<<<dim3(blocks(m), m), 256, 0, s>>>(A, n, k, v, pv, hs);
+            double2* v = V + (size_t)k * n + k + 1;
+            k_hh_reflector<<<1, HH_THREADS, 0, s>>>(A, n, k, v, hs, taus, dd, ee);
+            k_hh_matvec<<<blocks(m, 8), 256, 0, s>>>(A, n, k, v, hs, pb);
+            k_hh_coef<<<1, 256, 0, s>>>(n, k, v, pb, hs);
+            k_hh_update<<<dim3(blocks(m), m), 256, 0, s>>>(A, n, k, v, pb, hs);
         }
-        k_hh_tail<<<1, 1, 0, s>>>(A, n, dd, ee);
+        k_hh_tail<<<1, 1, 0, s>>>(A, n, dd, ee, ph);
+        note_launch((unsigned long long)4 * (n - 2) + 1);
+        CKE(cudaGetLastError());
+    }
+    int levels = 0;
+    if (!d_P) {
         k_tridiag_bisect<<<blocks(n, 128), 128, 0, s>>>(dd, ee, n, p->lambda_abs, d_mu);
-        const cudaError_t ec = cudaStreamEndCapture(s, &g);
-        if (ec != cudaSuccess) {
-            if (g) cudaGraphDestroy(g);
-            return done(eig_err(ec, "cudaStreamEndCapture"));
-        }
-        const cudaError_t ei = cudaGraphInstantiate(&sweep, g, 0);
-        cudaGraphDestroy(g);
-        CKE(ei);
-        CKE(cudaGraphLaunch(sweep, s));
-        note_launch((unsigned long long)4 * (n > 2 ? n - 2 : 0) + 2);
-        CKE(cudaEventRecord(ev, s));
-        CKE(cudaStreamWaitEvent(us, ev, 0));
-        if (sweeps_out) *sweeps_out = 0;
-        return done(PINV_OK);
-    }
-    k_identity<<<blocks((int64_t)nn), 256, 0, s>>>(V, n);
-    note_launch();
-    CKE(cudaGetLastError());
-    const size_t row_smem = sizeof(double2) * n;
-    CKE(cudaFuncSetAttribute(k_jac_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)row_smem));
-
-    // one sweep as a graph: np - 1 rounds of (rotations, G J and V J, J^H G)
-    {
-        cudaGraph_t g = nullptr;
-        CKE(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
-        for (int r = 0; r < np - 1; ++r) {
-            k_jac_rot<<<blocks(np / 2), 256, 0, s>>>(A, n, np, r, ca, cb, part);
-            k_jac_cols<<<dim3(1, n, 2), 256, row_smem, s>>>(A, V, n, ca, cb, part);
-            k_jac_rows<<<np / 2, 256, 0, s>>>(A, n, np, r, ca, cb);
-        }
-        const cudaError_t ec = cudaStreamEndCapture(s, &g);
-        if (ec != cudaSuccess) {
-            if (g) cudaGraphDestroy(g);
-            return done(eig_err(ec, "cudaStreamEndCapture"));
-        }
-        const cudaError_t ei = cudaGraphInstantiate(&sweep, g, 0);
-        cudaGraphDestroy(g);
-        CKE(ei);
-    }
-    const double tol = 4.0 * n * 2.220446049250313e-16;  // relative off-diagonal norm
-    int sweeps = 0;
-    double prev = INFINITY;
-    bool converged = false;
-    for (;; ++sweeps) {
-        k_row_norms<<<n, 256, 0, s>>>(A, n, norms);
-        k_sum_norms<<<1, 256, 0, s>>>(norms, n, norms + 2 * n);
-        note_launch(2);
-        CKE(cudaMemcpyAsync(hn, norms + 2 * n, sizeof(double) * 2, cudaMemcpyDeviceToHost, s));
-        CKE(cudaStreamSynchronize(s));
-        const double off = hn[1] > 0.0 ? sqrt(hn[0] / hn[1]) : 0.0;
-        if (off <= tol || (off <= 1e-10 && off > 0.5 * prev)) {
-            converged = true;
-            break;
-        }
-        if (sweeps == EIG_MAX_SWEEPS) break;
-        prev = off;
-        CKE(cudaGraphLaunch(sweep, s));
-        note_launch((unsigned long long)3 * (np - 1));
-    }
-    if (!converged) result = set_error(PINV_ERR_INTERNAL, "Jacobi sweeps did not converge");
-    int npow = 1;
-    while (npow < n) npow <<= 1;
-    const size_t sort_smem = (sizeof(double) + sizeof(int)) * npow;
-    CKE(cudaFuncSetAttribute(k_eig_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sort_smem));
-    k_eig_sort<<<1, 1024, sort_smem, s>>>(A, n, npow, p->lambda_abs, d_mu, order);
-    note_launch();
-    if (d_P) {
-        k_eig_gather<<<blocks((int64_t)nn), 256, 0, s>>>(V, n, order, 0, (double2*)d_P);
         note_launch();
+        CKE(cudaGetLastError());
+    } else {
+        int nl = 1;
+        while ((n + nl - 1) / nl > DC_LEAF) nl <<= 1;
+        double *Q = nullptr, *Qn = nullptr, *U = nullptr, *D = nullptr, *Dn = nullptr;
+        int* order = nullptr;
+        DcWork w{};
+        CKE(take((void**)&Q, sizeof(double) * nn));
+        CKE(take((void**)&D, sizeof(double) * n));
+        CKE(take((void**)&order, sizeof(int) * n));
+        w.failed = &fl->leaf_failed;
+        // merges read whole blocks of Q and Qn: zeros outside the smaller blocks written so far
+        CKE(cudaMemsetAsync(Q, 0, sizeof(double) * nn, s));
+        k_dc_leaf<<<nl, 32, 0, s>>>(dd, ee, n, nl, D, Q, w.failed);
+        note_launch();
+        CKE(cudaGetLastError());
+        if (nl > 1) {
+            double* db = nullptr;
+            int* ib = nullptr;
+            CKE(take((void**)&Qn, sizeof(double) * nn));
+            CKE(cudaMemsetAsync(Qn, 0, sizeof(double) * nn, s));
+            CKE(take((void**)&U, sizeof(double) * nn));
+            CKE(take((void**)&Dn, sizeof(double) * n));
+            CKE(take((void**)&db, sizeof(double) * ((size_t)6 * n + nl)));
+            CKE(take((void**)&ib, sizeof(int) * ((size_t)4 * n + 2 * nl)));
+            w.kd = db;
+            w.kz = db + n;
+            w.rc = db + 2 * (size_t)n;
+            w.rs = db + 3 * (size_t)n;
+            w.mu = db + 4 * (size_t)n;
+            w.zh = db + 5 * (size_t)n;
+            w.rho = db + 6 * (size_t)n;
+            w.rcol = (int2*)ib;
+            w.kcol = ib + 2 * (size_t)n;
+            w.org = ib + 3 * (size_t)n;
+            w.K = ib + 4 * (size_t)n;
+            w.nrot = w.K + nl;
+            const size_t ssm = (2 * sizeof(double) + sizeof(int)) * (size_t)n;
+            CKE(cudaFuncSetAttribute(k_dc_setup, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssm));
+            for (int wd = 1; wd < nl; wd <<= 1, ++levels) {
+                const unsigned nodes = (unsigned)(nl / (2 * wd));
+                int mm = 0;
+                for (unsigned t = 0; t < nodes; ++t)
+                    mm = std::max(mm, dc_bound(2 * wd * (int)(t + 1), n, nl) - dc_bound(2 * wd * (int)t, n, nl));
+                const size_t sm = (2 * sizeof(double) + sizeof(int)) * (size_t)mm;
+                const dim3 wg(blocks(mm, 8), nodes);
+                k_dc_setup<<<nodes, 512, sm, s>>>(D, ee, Q, n, nl, wd, w);
+                k_dc_rotate<<<dim3(blocks(mm, 128), nodes), 128, 0, s>>>(Q, n, nl, wd, w);
+                k_dc_secular<<<wg, 256, 0, s>>>(n, nl, wd, w, Dn);
+                k_dc_zhat<<<wg, 256, 0, s>>>(n, nl, wd, w);
+                k_dc_vectors<<<wg, 256, 0, s>>>(n, nl, wd, w, U);
+                k_dc_update<<<dim3(blocks(mm, 32), blocks(mm, 32), nodes), 256, 0, s>>>(Q, U, n, nl, wd, w, Qn, Dn);
+                note_launch(6);
+                CKE(cudaGetLastError());
+                std::swap(Q, Qn);
+                std::swap(D, Dn);
+            }
+        }
+        k_dc_order<<<blocks(n, 128), 128, 0, s>>>(D, n, p->lambda_abs, d_mu, order);
+        // a warp per column, as many warps as hold their column in shared memory
+        const int wpb = (int)std::max<int64_t>(1, std::min<int64_t>(8, (int64_t)(200 << 10) / (16 * (int64_t)n)));
+        const size_t bsm = sizeof(double2) * (size_t)n * wpb;
+        CKE(cudaFuncSetAttribute(k_hh_back, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bsm));
+        k_hh_back<<<blocks(n, wpb), wpb * 32, bsm, s>>>(V, taus, ph, Q, n, order, (double2*)d_P);
+        note_launch(2);
+        CKE(cudaGetLastError());
     }
-    CKE(cudaGetLastError());
-    // the caller's stream sees the results
-    CKE(cudaEventRecord(ev, s));
-    CKE(cudaStreamWaitEvent(us, ev, 0));
-    if (sweeps_out) *sweeps_out = sweeps;
+    Flags hf{};
+    CKE(cudaMemcpyAsync(&hf, fl, sizeof(Flags), cudaMemcpyDeviceToHost, s));
+    CKE(cudaStreamSynchronize(s));
+    if (sweeps_out) *sweeps_out = d_P ? levels + 1 : 0;
+    if (hf.bar.failed) return done(set_error(PINV_ERR_TIMEOUT, "a bounded device wait gave up (tridiagonal reduction)"));
+    if (hf.leaf_failed) return done(set_error(PINV_ERR_INTERNAL, "a leaf's Jacobi sweeps did not converge"));
 #undef CKE
-    return done(result);
+    return done(PINV_OK);
 }
 
 extern "C" pinv_status pinv_tsvd_apply(pinv_plan* p, const double* d_mu, const void* d_P, double energy,

@@ -133,3 +133,36 @@ def test_eig_mixed_plan_split_precision_bound():
     # Weyl: |d mu| <= ||dG||_2 <= ||dG||_F, and the split-BF16 Gram's entries carry a
     # relative error below about 2e-6 (3 x DRAIN x 2^-24 from the accumulation groups)
     assert np.max(np.abs(mu.cpu().numpy() - mu_ref)) < 4e-6 * np.linalg.norm(E.conj().T @ E)
+
+
+# N = 1, 2, 3 (no reflector, one, two), at and past a 32-row leaf, with odd splits of the
+# leaves, and spectra that deflate: the full Cartesian grid (all eigenvalues equal) and fewer
+# samples than voxels (a null space)
+@pytest.mark.parametrize("dims,samples", [((1,), 3), ((2,), 5), ((3,), 4), ((31,), 90), ((32,), 64), ((33,), 80),
+                                          ((65,), 200), ((12, 11), 400), ((8, 8), None), ((14, 14), 90)])
+def test_eig_sizes_and_clusters(dims, samples):
+    from paper_2410_06129_gb300.plan import Plan
+    rng = np.random.default_rng(2611)
+    N, D = int(np.prod(dims)), len(dims)
+    if samples is None:
+        g = [np.arange(n) - n // 2 for n in dims]
+        k = np.stack([a.ravel() for a in np.meshgrid(*g, indexing="ij")], axis=1).astype(float)
+    else:
+        k = rng.uniform(-0.5 * max(dims), 0.5 * max(dims), size=(samples, D))
+    E = O.encode(k, O.voxel_positions(dims))
+    pl = Plan(dims, k, lam=1e-3, precision=L.FP64, keep_gram=True).build()
+    mu, P, sweeps = pl.eig()
+    mu, P = mu.cpu().numpy(), P.cpu().numpy()
+    G0 = E.conj().T @ E
+    ref = np.linalg.eigvalsh(G0)[::-1]
+    scale = ref[0]
+    # backward stable: a small multiple of N eps of the largest eigenvalue
+    tol = (40 + 4 * N) * 2.0 ** -52
+    assert np.max(np.abs(mu - ref)) < tol * scale
+    assert np.all(np.diff(mu) <= 0)
+    assert np.max(np.abs(P.conj().T @ P - np.eye(N))) < tol
+    assert np.max(np.abs(P @ np.diag(mu) @ P.conj().T - G0)) < tol * scale
+    assert 1 <= sweeps <= 30
+    only, none, zero = pl.eig(vectors=False)
+    assert none is None and zero == 0
+    assert np.max(np.abs(only.cpu().numpy() - ref)) < tol * scale
