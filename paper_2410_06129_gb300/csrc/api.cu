@@ -124,7 +124,13 @@ pinv_status build_gram(pinv_plan* p, cudaStream_t s, bool main_gram) {
     CK(cudaEventRecord(p->ev[6], s));
     if (main_gram) {
         if (p->precision == PINV_FP64) {
-            CK(launch_gram64(p->enc, p->lambda_abs, p->G, ld, s));
+            cudaError_t e = cudaErrorMemoryAllocation;
+            if (gram64_table_ok(p->enc)) e = launch_gram64_table(p->enc, p->lambda_abs, p->G, ld, s);
+            if (e == cudaErrorMemoryAllocation) {
+                cudaGetLastError();
+                e = launch_gram64(p->enc, p->lambda_abs, p->G, ld, s);
+            }
+            CK(e);
         } else if (p->Gx) {
             // plans that keep the exact Gram for their residual factor it too: its
             // Toeplitz table needs (2 n - 1) offsets per axis times M_k products where the
@@ -292,13 +298,28 @@ pinv_status build_factor(pinv_plan* p, cudaStream_t s, bool events) {
         CK(cudaFreeAsync(D32, s));
         CK(cudaFreeAsync(L32, s));
     } else {
-        CK(launch_potrf64(p->G, N, ld, p->Dinv, p->st, s));
+        // trailing updates and G^-1 = W^H W as exact digit products on the tensor cores; on
+        // other GPUs, or without room for their tables, on the FP64 pipe
+        double2 *W = nullptr, *T = nullptr;
+        void* work = nullptr;
+        const bool oz = tc_available() && work_alloc(&work, oz_panel_bytes(N), s) == cudaSuccess &&
+                        work_alloc((void**)&T, sizeof(double2) * N * 32, s) == cudaSuccess;
+        if (!oz) cudaGetLastError();
+        if (oz) CK(launch_potrf64_oz(p->G, N, p->Dinv, T, work, p->st, s));
+        else CK(launch_potrf64(p->G, N, ld, p->Dinv, p->st, s));
         CK(launch_pivot_stats(p->G, N, ld, p->st, s));
         if (events) CK(cudaEventRecord(p->ev[3], s));
-        double2* W = nullptr;
         CK(work_alloc((void**)&W, sizeof(double2) * N * N, s));
-        CK(launch_trtri64(p->G, N, ld, p->Dinv, W, s));
-        CK(launch_lauum64(W, N, ld, p->Ginv, s));
+        if (oz) CK(launch_trtri64_oz(p->G, N, p->Dinv, W, work, p->st, s));
+        else CK(launch_trtri64(p->G, N, ld, p->Dinv, W, s));
+        if (work) CK(cudaFreeAsync(work, s));
+        if (T) CK(cudaFreeAsync(T, s));
+        cudaError_t e = oz ? launch_lauum64_oz(W, N, p->Ginv, p->st, s) : cudaErrorMemoryAllocation;
+        if (e == cudaErrorMemoryAllocation) {
+            cudaGetLastError();
+            e = launch_lauum64(W, N, ld, p->Ginv, s);
+        }
+        CK(e);
         CK(cudaFreeAsync(W, s));
     }
     if (p->x_pending) {  // the exact Gram and digit tables formed beside the factor
@@ -337,7 +358,13 @@ pinv_status build_recon(pinv_plan* p, cudaStream_t s) {
             CK(cudaFreeAsync(T, s));
         }
     } else {
-        CK(launch_recon64(p->enc, p->Ginv, N, (double2*)p->R, s));
+        cudaError_t e = tc_available() ? launch_recon64_oz(p->enc, p->eexp, p->Ginv, (double2*)p->R, p->st, s)
+                                       : cudaErrorMemoryAllocation;
+        if (e == cudaErrorMemoryAllocation) {
+            cudaGetLastError();
+            e = launch_recon64(p->enc, p->Ginv, N, (double2*)p->R, s);
+        }
+        CK(e);
     }
     return PINV_OK;
 }

@@ -1,0 +1,656 @@
+// FP64 products on the tensor cores through exact integer digits.
+//
+// GB300 issues about 2 DFMA per clock and SM (1.2 TFLOP/s over the chip) and its tensor
+// cores have no FP64 kind, so the FP64 path's contractions were bound by the FP64 pipe. Here
+// each operand row (A) or column (B) is scaled by a power of two so that its components are
+// at most 1, rounded to a 55-bit fixed-point integer and cut into eight balanced 7-bit
+// digits, |x_i| <= 64, x = sum_i x_i 2^(-6-7i) within 2^-56 (error-free splitting: K. Ozaki,
+// T. Ogita, S. Oishi, S. M. Rump, Numer. Algorithms 59, 2012). bf16 holds a digit exactly, a
+// product of two digits has at most 12 bits, and the FP32 accumulator is exact below 2^24,
+// so every class sum (pairs i + j = w, one TMEM region of 64 columns each, w <= 7) is an
+// exact integer. Dropped pairs weigh below 2^-56 of the largest products. The drains add
+// the class sums, scaled, into two double-float accumulators per value (classes 0-3, whose
+// 2^-33 grid a pair holds exactly, and 4-7), joined in FP64 at the end: the result carries
+// the operands' 2^-56 roundings and one FP64 rounding, no more than an FP64 FMA chain's.
+//
+// Tile: 128 rows x 32 complex columns, the real embedding of tc_engine.cuh; a stage holds
+// 8 complex k (A 32 KiB, B 16 KiB), four stages in flight. A stage's 36 digit pairs are 12
+// MMAs of N <= 256: 1152 tensor cycles for 32 768 complex MACs, 28 a cycle and SM where
+// the FP64 pipe makes half a one. Operands come from digit tables in the stage layout, one
+// bulk copy each per stage. Rows or columns with a NaN or an infinity give NaN.
+//
+// Roles, waits and aborts follow k_exact: warps 0-7 drain and store (thread 0 also starts
+// the copies), warp 8 issues the MMAs.
+#include <algorithm>
+#include <climits>
+
+#include "df.cuh"
+#include "tc_engine.cuh"
+
+namespace pinv {
+namespace oz {
+
+using namespace tc;
+
+constexpr int OM = 128;         // rows per tile (MMA M)
+constexpr int ON = 32;          // complex columns per tile (64 MMA columns per B digit)
+constexpr int OKC = 8;          // complex k per stage (MMA K = 16)
+constexpr int OD = 8;           // digits
+constexpr int OCLS = 8;         // weight classes kept
+constexpr int ODRAIN = 31;      // stages per accumulation group (classes 0-3: two groups)
+constexpr int OST = 4;          // stages in flight
+constexpr int OA_SL = OM * 32;  // one digit slice of A: 128 rows x 16 bf16
+constexpr int OB_SL = 2 * ON * 32;
+constexpr int OA_ST = OD * OA_SL, OB_ST = OD * OB_SL, OSTAGE = OA_ST + OB_ST;
+constexpr int OSMEM = OST * OSTAGE + 1024;
+static_assert(OCLS * 16 * ODRAIN * 4096 < (1 << 24) && 4 * 16 * 2 * ODRAIN * 4096 < (1 << 24), "exact class sums");
+constexpr int PKB = 8;          // k blocks of a panel (K <= 64)
+constexpr int NONFINITE = INT_MAX;  // exponent of a row or column that holds a NaN or an infinity
+
+__host__ __device__ constexpr uint32_t oidesc(int n) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(OM >> 4) << 24);
+}
+// (A digit, first B digit, B digits) of a stage's MMAs; digit 0's two runs cover all classes
+struct Run {
+    int i, j0, nd;
+};
+__device__ __forceinline__ Run orun(int r) {
+    constexpr Run t[12] = {{0, 0, 4}, {0, 4, 4}, {1, 0, 4}, {1, 4, 3}, {2, 0, 4}, {2, 4, 2},
+                           {3, 0, 4}, {3, 4, 1}, {4, 0, 4}, {5, 0, 3}, {6, 0, 2}, {7, 0, 1}};
+    return t[r];
+}
+// byte offset of (row, 8-wide k' group 0 or 1) in a [rows][16] K-major no-swizzle tile
+__device__ inline uint32_t koff16(int r, int g) { return (uint32_t)((r >> 3) * 256 + g * 128 + (r & 7) * 16); }
+
+// x 2^e on the integer pipe (the FP64 pipe where an exponent leaves the normal range)
+__device__ inline double scale2(double x, int e) {
+    const long long b = __double_as_longlong(x);
+    const int ex = (int)((b >> 52) & 0x7ff), ne = ex + e;
+    if (ex == 0 || ex == 0x7ff || ne <= 0 || ne >= 0x7ff) return ldexp(x, e);
+    return __longlong_as_double(b + ((long long)e << 52));
+}
+
+// ------------------------------------------------------------------ exponents
+// bits of the largest |component|; NaN and infinity order above every finite value
+__device__ inline unsigned long long abs_bits(double x) {
+    return (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
+}
+__device__ inline unsigned long long max_bits(double2 v) { return max(abs_bits(v.x), abs_bits(v.y)); }
+// the least e with |x| <= 2^e from the bits of the largest |x|
+__device__ inline int bits_exp(unsigned long long b) {
+    if (b == 0ull) return 0;
+    const int eb = (int)(b >> 52);
+    const unsigned long long mf = b & ((1ull << 52) - 1ull);
+    if (eb == 0x7ff) return NONFINITE;
+    if (eb == 0) return (64 - __clzll((long long)mf)) - 1074 - ((mf & (mf - 1ull)) == 0ull ? 1 : 0);
+    return eb - 1023 + (mf != 0ull ? 1 : 0);
+}
+// exponents of the rows of a [rows][K] matrix, one CTA per row
+__global__ void __launch_bounds__(256) k_row_exp(const double2* __restrict__ A, int64_t ld, int64_t K, int* ex) {
+    __shared__ unsigned long long red[8];
+    const double2* row = A + (int64_t)blockIdx.x * ld;
+    unsigned long long m = 0ull;
+#pragma unroll 4
+    for (int64_t k = threadIdx.x; k < K; k += 256) m = max(m, max_bits(row[k]));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) m = max(m, red[w]);
+        ex[blockIdx.x] = bits_exp(m);
+    }
+}
+// exponents of the columns of a [K][cols] matrix: 32 columns per CTA, its 8 warps take the rows
+__global__ void __launch_bounds__(256) k_col_exp(const double2* __restrict__ A, int64_t ld, int64_t K, int64_t cols,
+                                                 int* ex) {
+    __shared__ unsigned long long red[8][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t c = (int64_t)blockIdx.x * 32 + lane;
+    unsigned long long m = 0ull;
+    if (c < cols)
+#pragma unroll 4
+        for (int64_t k = w; k < K; k += 8) m = max(m, max_bits(A[k * ld + c]));
+    red[w][lane] = m;
+    __syncthreads();
+    if (w == 0 && c < cols) {
+        for (int t = 1; t < 8; ++t) m = max(m, red[t][lane]);
+        ex[c] = bits_exp(m);
+    }
+}
+
+// ------------------------------------------------------------------ digit tables
+// eight 55-bit fixed-point integers, written digit by digit from the last: word t of
+// digit slice dg packs values 2t, 2t + 1 as bf16
+struct Fix8 {
+    long long x[8];
+    __device__ void set(int t, double v, int e) { x[t] = __double2ll_rn(scale2(v, 55 - e)); }
+    __device__ void next(uint32_t (&w)[4], bool top) {
+        float d[8];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            int q;
+            if (top) {
+                q = (int)x[t];
+            } else {
+                q = (((int)x[t] + 64) & 127) - 64;
+                x[t] = (x[t] - q) >> 7;
+            }
+            d[t] = __int_as_float(0x4b400000 + q) - 12582912.f;  // exact for |q| < 2^22
+        }
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            __nv_bfloat162 v = __floats2bfloat162_rn(d[2 * t], d[2 * t + 1]);  // exact: |d| <= 64
+            w[t] = *reinterpret_cast<uint32_t*>(&v);
+        }
+    }
+};
+
+// Operand element (row or column i, k). Mat: a stored matrix, [i][k] or ([k][i], trans),
+// conjugated on request; EncRow: conj(E[j][k]), j = j_off + i, generated from the FP64 tables.
+struct Mat {
+    const double2* p;
+    int64_t ld, n, K;  // n rows (columns) i, sum length K
+    int trans, cj;
+    const int* ex;
+    __device__ int exponent(int64_t i) const { return ex[i]; }
+    __device__ double2 get(int64_t i, int64_t k) const {
+        double2 v = trans ? p[k * ld + i] : p[i * ld + k];
+        if (cj) v.y = -v.y;
+        return v;
+    }
+};
+struct EncRow {
+    EncodeDev e;
+    int64_t j_off, n, K;
+    int ex;
+    __device__ int exponent(int64_t) const { return ex; }
+    __device__ double2 get(int64_t i, int64_t k) const {
+        const int64_t j = j_off + i, c = j / e.Mk;
+        return zconj(gen_e64(e, (int)c, j - c * e.Mk, k));
+    }
+};
+
+// the 8 values k0 .. k0 + 7 of row i as fixed-point integers (zeros out of range, and for a
+// row that is not finite, whose results the product replaces by NaN)
+template <class P>
+__device__ inline void load_fix(const P& p, int64_t i, int64_t k0, Fix8& re, Fix8& im) {
+    const int e = i < p.n ? p.exponent(i) : NONFINITE;
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+        const bool in = e != NONFINITE && k0 + t < p.K;
+        const double2 v = in ? p.get(i, k0 + t) : make_double2(0.0, 0.0);
+        re.set(t, v.x, in ? e : 0);
+        im.set(t, v.y, in ? e : 0);
+    }
+}
+// A tiles [row tile][k block][digit]: rows [re | im]; CTA per (k block, row tile)
+template <class P>
+__global__ void __launch_bounds__(OM) k_oz_a(P p, int64_t KB, uint8_t* At) {
+    const int64_t kb = blockIdx.x, rt = blockIdx.y;
+    const int r = threadIdx.x;
+    Fix8 re, im;
+    load_fix(p, rt * OM + r, kb * OKC, re, im);
+    uint8_t* blk = At + (rt * KB + kb) * (int64_t)OA_ST;
+#pragma unroll
+    for (int dg = OD - 1; dg >= 0; --dg) {
+        uint32_t w[4];
+        re.next(w, dg == 0);
+        *reinterpret_cast<uint4*>(blk + dg * OA_SL + koff16(r, 0)) = make_uint4(w[0], w[1], w[2], w[3]);
+        im.next(w, dg == 0);
+        *reinterpret_cast<uint4*>(blk + dg * OA_SL + koff16(r, 1)) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+}
+// B tiles [column tile][k block][digit]: column c owns row c, [re | -im], and row ON + c,
+// [im | re]; four k blocks per CTA
+template <class P>
+__global__ void __launch_bounds__(4 * ON) k_oz_b(P p, int64_t KB, uint8_t* Bt) {
+    const int64_t kb = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5), ct = blockIdx.y;
+    if (kb >= KB) return;
+    const int c = threadIdx.x & 31;
+    Fix8 re, im;
+    load_fix(p, ct * ON + c, kb * OKC, re, im);
+    uint8_t* blk = Bt + (ct * KB + kb) * (int64_t)OB_ST;
+#pragma unroll
+    for (int dg = OD - 1; dg >= 0; --dg) {
+        uint32_t wr[4], wi[4];
+        re.next(wr, dg == 0);
+        im.next(wi, dg == 0);
+        uint8_t* sl = blk + dg * OB_SL;
+        *reinterpret_cast<uint4*>(sl + koff16(c, 0)) = make_uint4(wr[0], wr[1], wr[2], wr[3]);
+        *reinterpret_cast<uint4*>(sl + koff16(c, 1)) =
+            make_uint4(wi[0] ^ 0x80008000u, wi[1] ^ 0x80008000u, wi[2] ^ 0x80008000u, wi[3] ^ 0x80008000u);
+        *reinterpret_cast<uint4*>(sl + koff16(ON + c, 0)) = make_uint4(wi[0], wi[1], wi[2], wi[3]);
+        *reinterpret_cast<uint4*>(sl + koff16(ON + c, 1)) = make_uint4(wr[0], wr[1], wr[2], wr[3]);
+    }
+}
+
+// ------------------------------------------------------------------ the product
+struct Args {
+    const uint8_t *At, *Bt;
+    int64_t KB;          // k blocks of the tables
+    const int *ra, *cb;  // exponents of the rows (null: ea) and of the columns
+    int ea;
+};
+
+// P: tile(bid, rt, ct, kb, ke) (tile coordinates and k blocks; false: nothing to do),
+// rows(), cols(), and store(bid, i, j, v) of element (i, j) of tile bid
+template <class P>
+__global__ void __launch_bounds__(NTHREADS, 1) k_oz(P p, Args a, DevStatus* st) {
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ uint64_t empty_bar[OST], abar[OST];
+    __shared__ uint64_t tfull, tempty, done_bar;
+    __shared__ uint32_t tmem_base_sh;
+    __shared__ int abort_flag;
+    int64_t rt, ct, kb, ke;
+    if (!p.tile(blockIdx.x, rt, ct, kb, ke)) return;  // the same in every thread
+    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const long long wlim = st->wait_limit > 0 ? st->wait_limit : WAIT_LIMIT;  // pipeline waits
+    const int nk = ke > kb ? (int)(ke - kb) : 0;
+    const int ngroups = (nk + ODRAIN - 1) / ODRAIN;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < OST; ++s) {
+            mbar_init(&empty_bar[s], 1);
+            mbar_init(&abar[s], 1);
+        }
+        mbar_init(&tfull, 1);
+        mbar_init(&tempty, NPW * 32);
+        mbar_init(&done_bar, 1);
+        abort_flag = 0;
+        fence_barrier_init();
+    }
+    if (warp == NPW) tmem_alloc(&tmem_base_sh, 512);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tmem_base_sh;
+
+    if (warp < NPW) {
+        // ---------------- copies (thread 0), drains, epilogue
+        const int q = warp & 3, h = warp >> 2;  // TMEM lane quarter, half of the tile's columns
+        const uint32_t trow = tmem + ((uint32_t)(q * 32) << 16);
+        float hi[4][16], lo[4][16];  // re.hi, re.lo, im.hi, im.lo of classes 0-3, and of 4-7
+#pragma unroll
+        for (int u = 0; u < 16; ++u)
+#pragma unroll
+            for (int t = 0; t < 4; ++t) hi[t][u] = lo[t][u] = 0.f;
+        // four classes from w0 into acc, renormalised once
+        auto add = [&](int w0, float(&acc)[4][16]) {
+#pragma unroll 1
+            for (int w = w0; w < w0 + 4; ++w) {
+                uint32_t vr[16], vi[16];
+                tmem_ld16(trow + (uint32_t)(64 * w + 16 * h), vr);
+                tmem_ld16(trow + (uint32_t)(64 * w + ON + 16 * h), vi);
+                tmem_wait_ld();
+                const float sc = __int_as_float((127 - 12 - 7 * w) << 23);  // 2^(-12-7w)
+#pragma unroll
+                for (int u = 0; u < 16; ++u) {
+                    float s, e;
+                    two_sum(acc[0][u], __uint_as_float(vr[u]) * sc, s, e);
+                    acc[0][u] = s;
+                    acc[1][u] += e;
+                    two_sum(acc[2][u], __uint_as_float(vi[u]) * sc, s, e);
+                    acc[2][u] = s;
+                    acc[3][u] += e;
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 16; ++u) {
+                fast_two_sum(acc[0][u], acc[1][u], acc[0][u], acc[1][u]);
+                fast_two_sum(acc[2][u], acc[3][u], acc[2][u], acc[3][u]);
+            }
+        };
+        auto drain = [&](int g) -> bool {
+            // the warp decides together: its TMEM loads need every lane
+            if (!__all_sync(0xffffffffu, mbar_wait(&tfull, (uint32_t)g & 1u, &abort_flag, wlim))) return false;
+            tc_fence_after();
+            add(4, lo);
+            if ((g & 1) || g == ngroups - 1) add(0, hi);  // classes 0-3 gather two groups
+            tc_fence_before();
+            mbar_arrive(&tempty);
+            return true;
+        };
+        bool ok = true;
+        int drained = 0, issued = 0;  // issued: stages whose copies thread 0 has started
+        for (int kt = 0; kt < nk && ok; ++kt) {
+            const int s = kt % OST;
+            if (kt >= OST &&
+                !(ok = __all_sync(0xffffffffu,
+                                  mbar_wait(&empty_bar[s], ((uint32_t)(kt / OST) & 1u) ^ 1u, &abort_flag, wlim))))
+                break;
+            if (threadIdx.x == 0) {
+                uint8_t* base = smem + s * OSTAGE;
+                mbar_arrive_expect_tx(&abar[s], (uint32_t)OSTAGE);
+                bulk_g2s(base, a.At + (rt * a.KB + kb + kt) * (int64_t)OA_ST, (uint32_t)OA_ST, &abar[s]);
+                bulk_g2s(base + OA_ST, a.Bt + (ct * a.KB + kb + kt) * (int64_t)OB_ST, (uint32_t)OB_ST, &abar[s]);
+                issued = kt + 1;
+            }
+            // a group is drained once the stages after it are in flight: its last
+            // stage's slot came back at this stage's empty wait
+            while (drained < ngroups && (drained + 1) * ODRAIN + OST - 1 <= kt) {
+                if (!(ok = drain(drained))) break;
+                ++drained;
+            }
+        }
+        while (ok && drained < ngroups) {
+            ok = drain(drained);
+            ++drained;
+        }
+        if (__all_sync(0xffffffffu, ok && !abort_flag)) {
+            const int64_t i = rt * OM + q * 32 + lane;
+            if (i < p.rows()) {
+                const int ea = a.ra ? a.ra[i] : a.ea;
+#pragma unroll
+                for (int u = 0; u < 16; ++u) {
+                    const int64_t j = ct * ON + 16 * h + u;
+                    if (j >= p.cols()) continue;
+                    const int eb = a.cb[j];
+                    double2 v;
+                    if (ea == NONFINITE || eb == NONFINITE) {
+                        v = make_double2(nan(""), nan(""));
+                    } else {
+                        v = make_double2(join_f64(hi[0][u], hi[1][u]) + join_f64(lo[0][u], lo[1][u]),
+                                         join_f64(hi[2][u], hi[3][u]) + join_f64(lo[2][u], lo[3][u]));
+                        v.x = scale2(v.x, ea + eb);
+                        v.y = scale2(v.y, ea + eb);
+                    }
+                    p.store(blockIdx.x, i, j, v);
+                }
+            }
+        }
+        if (threadIdx.x == 0) {
+            // copies still in flight (only after an abort): wait, bounded, for their bytes
+            for (int kg = issued > OST ? issued - OST : 0; kg < issued; ++kg)
+                mbar_wait(&abar[kg % OST], (uint32_t)(kg / OST) & 1u, nullptr);
+        }
+    } else if (lane == 0) {
+        // ---------------- MMA issuer: 36 digit pairs per stage in 12 MMAs
+        for (int kt = 0; kt < nk; ++kt) {
+            const int g = kt / ODRAIN;
+            const bool first = (kt % ODRAIN) == 0;
+            if (first && g >= 1 && !mbar_wait(&tempty, (uint32_t)(g - 1) & 1u, &abort_flag, wlim)) break;
+            const int s = kt % OST;
+            if (!mbar_wait(&abar[s], (uint32_t)(kt / OST) & 1u, &abort_flag, wlim)) break;
+            tc_fence_after();
+            const uint32_t abase = smem_u32(smem + s * OSTAGE), bbase = abase + OA_ST;
+#pragma unroll
+            for (int r = 0; r < 12; ++r) {
+                const Run u = orun(r);
+                const bool fresh = first && u.i == 0 && (u.j0 > 0 || (g & 1) == 0);
+                mma_bf16(tmem + (uint32_t)(2 * ON * (u.i + u.j0)), sdesc(abase + u.i * OA_SL, 128, 256),
+                         sdesc(bbase + u.j0 * OB_SL, 128, 256), oidesc(2 * ON * u.nd), fresh ? 0u : 1u);
+            }
+            mma_commit(&empty_bar[s]);
+            if ((kt % ODRAIN) == ODRAIN - 1 || kt == nk - 1) mma_commit(&tfull);
+        }
+        mma_commit(&done_bar);
+    }
+
+    tc_fence_before();
+    __syncthreads();
+    if (warp == NPW) {
+        mbar_wait(&done_bar, 0, nullptr);
+        tc_fence_after();
+        tmem_dealloc(tmem, 512);
+    }
+    if (threadIdx.x == 0 && abort_flag) atomicMax(&st->timeout_site, 21);
+}
+
+// ------------------------------------------------------------------ problems
+// Recon^T: rows j (samples of this chunk), columns n
+struct ReconOz {
+    double2* R;
+    int64_t M, j_off, mrows, N, KB, ctn;
+    __device__ int64_t rows() const { return mrows; }
+    __device__ int64_t cols() const { return N; }
+    // bands of 8 row tiles, column-major inside a band, so the tiles running at one time
+    // share few operand tiles
+    __device__ bool tile(int64_t b, int64_t& rt, int64_t& ct, int64_t& kb, int64_t& ke) const {
+        const int64_t rtn = (mrows + OM - 1) / OM, band = b / (8 * ctn), l = b - band * 8 * ctn;
+        const int64_t hgt = rtn - band * 8 < 8 ? rtn - band * 8 : 8;
+        ct = l / hgt;
+        rt = band * 8 + l % hgt;
+        kb = 0;
+        ke = KB;
+        return true;
+    }
+    __device__ void store(int64_t, int64_t i, int64_t j, double2 v) const { R[j * M + j_off + i] = v; }
+};
+// Ginv = W^H W, lower tiles mirrored; the sum starts at the row tile (W is lower triangular)
+struct LauumOz {
+    double2* Gi;
+    int64_t N, KB, ctn;
+    __device__ int64_t rows() const { return N; }
+    __device__ int64_t cols() const { return N; }
+    __device__ bool tile(int64_t b, int64_t& rt, int64_t& ct, int64_t& kb, int64_t& ke) const {
+        rt = b / ctn;
+        ct = b % ctn;
+        kb = rt * (OM / OKC);
+        ke = KB;
+        return ct * ON <= rt * OM + OM - 1;
+    }
+    __device__ void store(int64_t, int64_t i, int64_t j, double2 v) const {
+        if (j > i) return;
+        Gi[i * N + j] = v;
+        Gi[j * N + i] = zconj(v);
+    }
+};
+
+// Trailing updates of the FP64 factorisation, K <= 64: C[i][j] -= the product, rows and
+// columns at their offsets. Herk: the lower triangle from t0; Trtri: all columns below t0.
+struct UpdateOz {
+    double2* C;
+    int64_t ld, N, t0, c0, ncols, ctn;
+    int lower;
+    __device__ int64_t rows() const { return N - t0; }
+    __device__ int64_t cols() const { return ncols; }
+    __device__ bool tile(int64_t b, int64_t& rt, int64_t& ct, int64_t& kb, int64_t& ke) const {
+        rt = b / ctn;
+        ct = b % ctn;
+        kb = 0;
+        ke = PKB;
+        return !lower || ct * ON <= rt * OM + OM - 1;
+    }
+    __device__ void store(int64_t, int64_t i, int64_t j, double2 v) const {
+        if (lower && j > i) return;
+        double2* c = C + (t0 + i) * ld + c0 + j;
+        *c = zsub(*c, v);
+    }
+};
+
+// Digit tables of a panel of K <= 64 in one launch: 32 rows (or columns, trans) i per CTA,
+// thread (i, 8 k); the row's exponent from the block's maxima. Writes the A tiles, the B
+// tiles (of the conjugate, cj) or both, and the exponents.
+__global__ void __launch_bounds__(256) k_oz_panel(const double2* __restrict__ p, int64_t ld, int trans, int64_t n,
+                                                  int K, int cj, int* ex, uint8_t* At, uint8_t* Bt) {
+    __shared__ unsigned long long red[PKB][32];
+    const int r = threadIdx.x & 31, g = threadIdx.x >> 5;
+    const int64_t i = (int64_t)blockIdx.x * 32 + r;
+    double2 v[8];
+    unsigned long long m = 0ull;
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+        const int k = 8 * g + t;
+        v[t] = i < n && k < K ? (trans ? p[k * ld + i] : p[i * ld + k]) : make_double2(0.0, 0.0);
+        m = max(m, max_bits(v[t]));
+    }
+    red[g][r] = m;
+    __syncthreads();
+#pragma unroll
+    for (int t = 0; t < PKB; ++t) m = max(m, red[t][r]);
+    const int e = bits_exp(m);
+    if (g == 0 && i < n) ex[i] = e;
+    Fix8 re, im;
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+        re.set(t, e == NONFINITE ? 0.0 : v[t].x, e == NONFINITE ? 0 : e);
+        im.set(t, e == NONFINITE ? 0.0 : v[t].y, e == NONFINITE ? 0 : e);
+    }
+    uint8_t* ab = At ? At + ((i / OM) * PKB + g) * (int64_t)OA_ST : nullptr;
+    uint8_t* bb = Bt ? Bt + ((int64_t)blockIdx.x * PKB + g) * (int64_t)OB_ST : nullptr;
+    const int ra = (int)(i % OM);
+    const uint32_t fa = cj ? 0u : 0x80008000u, fb = cj ? 0x80008000u : 0u;  // signs of im in [re | -im], [im | re]
+#pragma unroll
+    for (int dg = OD - 1; dg >= 0; --dg) {
+        uint32_t wr[4], wi[4];
+        re.next(wr, dg == 0);
+        im.next(wi, dg == 0);
+        if (ab) {
+            *reinterpret_cast<uint4*>(ab + dg * OA_SL + koff16(ra, 0)) = make_uint4(wr[0], wr[1], wr[2], wr[3]);
+            *reinterpret_cast<uint4*>(ab + dg * OA_SL + koff16(ra, 1)) = make_uint4(wi[0], wi[1], wi[2], wi[3]);
+        }
+        if (bb) {
+            uint8_t* sl = bb + dg * OB_SL;
+            *reinterpret_cast<uint4*>(sl + koff16(r, 0)) = make_uint4(wr[0], wr[1], wr[2], wr[3]);
+            *reinterpret_cast<uint4*>(sl + koff16(r, 1)) = make_uint4(wi[0] ^ fa, wi[1] ^ fa, wi[2] ^ fa, wi[3] ^ fa);
+            *reinterpret_cast<uint4*>(sl + koff16(ON + r, 0)) =
+                make_uint4(wi[0] ^ fb, wi[1] ^ fb, wi[2] ^ fb, wi[3] ^ fb);
+            *reinterpret_cast<uint4*>(sl + koff16(ON + r, 1)) = make_uint4(wr[0], wr[1], wr[2], wr[3]);
+        }
+    }
+}
+
+template <class P>
+cudaError_t run(const P& p, int64_t tiles, const Args& a, DevStatus* st, cudaStream_t s) {
+    static bool attr = false;
+    if (!attr) {
+        cudaError_t e = cudaFuncSetAttribute(k_oz<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, OSMEM);
+        if (e != cudaSuccess) return e;
+        attr = true;
+    }
+    k_oz<P><<<(unsigned)tiles, NTHREADS, OSMEM, s>>>(p, a, st);
+    note_launch();
+    return cudaGetLastError();
+}
+template <class P>
+cudaError_t tab_a(const P& p, int64_t KB, uint8_t* At, cudaStream_t s) {
+    k_oz_a<P><<<dim3((unsigned)KB, (unsigned)((p.n + OM - 1) / OM)), OM, 0, s>>>(p, KB, At);
+    note_launch();
+    return cudaGetLastError();
+}
+template <class P>
+cudaError_t tab_b(const P& p, int64_t KB, uint8_t* Bt, cudaStream_t s) {
+    k_oz_b<P><<<dim3((unsigned)((KB + 3) / 4), (unsigned)((p.n + ON - 1) / ON)), 4 * ON, 0, s>>>(p, KB, Bt);
+    note_launch();
+    return cudaGetLastError();
+}
+
+// stream-ordered temporaries, given back when the scope ends
+struct Temp {
+    cudaStream_t s;
+    void* q[8];
+    int n = 0;
+    explicit Temp(cudaStream_t st) : s(st) {}
+    ~Temp() {
+        while (n > 0) cudaFreeAsync(q[--n], s);
+    }
+    template <class T>
+    cudaError_t take(T** p, size_t bytes) {
+        cudaError_t e = work_alloc((void**)p, bytes, s);
+        if (e == cudaSuccess) q[n++] = *p;
+        return e;
+    }
+};
+#define OZ(call)                              \
+    do {                                      \
+        cudaError_t e_ = (call);              \
+        if (e_ != cudaSuccess) return e_;     \
+    } while (0)
+
+}  // namespace oz
+
+// Recon[n][j] = sum_k Ginv[n][k] conj(E[j][k]) over chunks of samples whose tables stay
+// within 1 GiB
+cudaError_t launch_recon64_oz(const EncodeDev& e, int eexp, const double2* Ginv, double2* R, DevStatus* st,
+                              cudaStream_t s) {
+    using namespace oz;
+    const int64_t N = e.N, M = e.Mk * e.C, KB = (N + OKC - 1) / OKC, ctn = (N + ON - 1) / ON;
+    const int64_t rtn = (M + OM - 1) / OM;
+    const int64_t per = std::max<int64_t>(1, std::min<int64_t>(rtn, (int64_t(1) << 30) / (KB * OA_ST)));
+    Temp t(s);
+    uint8_t *At = nullptr, *Bt = nullptr;
+    int* ex = nullptr;
+    OZ(t.take(&At, (size_t)(per * KB * OA_ST)));
+    OZ(t.take(&Bt, (size_t)(ctn * KB * OB_ST)));
+    OZ(t.take(&ex, sizeof(int) * N));
+    k_row_exp<<<(unsigned)N, 256, 0, s>>>(Ginv, N, N, ex);
+    note_launch();
+    OZ(tab_b(Mat{Ginv, N, N, N, 0, 0, ex}, KB, Bt, s));
+    for (int64_t r0 = 0; r0 < rtn; r0 += per) {
+        const int64_t j0 = r0 * OM, rows = std::min(per * OM, M - j0);
+        OZ(tab_a(EncRow{e, j0, rows, N, eexp}, KB, At, s));
+        const ReconOz p{R, M, j0, rows, N, KB, ctn};
+        OZ(run(p, (rows + OM - 1) / OM * ctn, Args{At, Bt, KB, nullptr, ex, eexp}, st, s));
+    }
+    return cudaSuccess;
+}
+
+// Ginv = W^H W
+cudaError_t launch_lauum64_oz(const double2* W, int64_t N, double2* Ginv, DevStatus* st, cudaStream_t s) {
+    using namespace oz;
+    const int64_t KB = (N + OKC - 1) / OKC, ctn = (N + ON - 1) / ON, rtn = (N + OM - 1) / OM;
+    Temp t(s);
+    uint8_t *At = nullptr, *Bt = nullptr;
+    int* ex = nullptr;
+    OZ(t.take(&At, (size_t)(rtn * KB * OA_ST)));
+    OZ(t.take(&Bt, (size_t)(ctn * KB * OB_ST)));
+    OZ(t.take(&ex, sizeof(int) * N));
+    k_col_exp<<<(unsigned)((N + 31) / 32), 256, 0, s>>>(W, N, N, N, ex);
+    note_launch();
+    OZ(tab_a(Mat{W, N, N, N, 1, 1, ex}, KB, At, s));
+    OZ(tab_b(Mat{W, N, N, N, 1, 0, ex}, KB, Bt, s));
+    const LauumOz p{Ginv, N, KB, ctn};
+    return run(p, rtn * ctn, Args{At, Bt, KB, ex, ex, 0}, st, s);
+}
+
+// tables of one panel's update: A and B tiles and exponents of up to N rows each
+namespace oz {
+struct PanelWork {
+    uint8_t *At, *Bt;
+    int *ea, *eb;
+};
+static size_t panel_layout(int64_t N, void* base, PanelWork* w) {
+    const size_t a = (size_t)((N + OM - 1) / OM) * PKB * OA_ST, b = (size_t)((N + ON - 1) / ON) * PKB * OB_ST;
+    const size_t x = (sizeof(int) * (size_t)N + 255) & ~(size_t)255;
+    if (w) {
+        uint8_t* q = (uint8_t*)base;
+        *w = PanelWork{q, q + a, (int*)(q + a + b), (int*)(q + a + b + x)};
+    }
+    return a + b + 2 * x;
+}
+}  // namespace oz
+
+size_t oz_panel_bytes(int64_t N) { return oz::panel_layout(N, nullptr, nullptr); }
+
+// G[i][j] -= sum_k L[i][p0+k] conj(L[j][p0+k]), k < kw <= 64, j <= i, rows and columns from p0 + kw
+cudaError_t oz_herk64(double2* G, int64_t N, int64_t p0, int64_t kw, void* work, DevStatus* st, cudaStream_t s) {
+    using namespace oz;
+    PanelWork w;
+    panel_layout(N, work, &w);
+    const int64_t t0 = p0 + kw, n = N - t0, ctn = (n + ON - 1) / ON;
+    // rows past the last in the last 128-row tile keep what the table held: their results are not stored
+    k_oz_panel<<<(unsigned)ctn, 256, 0, s>>>(G + t0 * N + p0, N, 0, n, (int)kw, 1, w.ea, w.At, w.Bt);
+    note_launch();
+    OZ(cudaGetLastError());
+    const UpdateOz p{G, N, N, t0, t0, n, ctn, 1};
+    return run(p, (n + OM - 1) / OM * ctn, Args{w.At, w.Bt, PKB, w.ea, w.ea, 0}, st, s);
+}
+
+// W[i][j] -= sum_k L[i][p0+k] W[p0+k][j], k < kw <= 64, rows i >= p0 + kw, columns j < p0 + kw
+cudaError_t oz_trtri64(double2* W, const double2* L, int64_t N, int64_t p0, int64_t kw, void* work, DevStatus* st,
+                       cudaStream_t s) {
+    using namespace oz;
+    PanelWork w;
+    panel_layout(N, work, &w);
+    const int64_t t0 = p0 + kw, n = N - t0, ctn = (t0 + ON - 1) / ON;
+    k_oz_panel<<<(unsigned)((n + 31) / 32), 256, 0, s>>>(L + t0 * N + p0, N, 0, n, (int)kw, 0, w.ea, w.At, nullptr);
+    k_oz_panel<<<(unsigned)ctn, 256, 0, s>>>(W + p0 * N, N, 1, t0, (int)kw, 0, w.eb, nullptr, w.Bt);
+    note_launch(2);
+    OZ(cudaGetLastError());
+    const UpdateOz p{W, N, N, t0, 0, t0, ctn, 0};
+    return run(p, (n + OM - 1) / OM * ctn, Args{w.At, w.Bt, PKB, w.ea, w.eb, 0}, st, s);
+}
+
+}  // namespace pinv

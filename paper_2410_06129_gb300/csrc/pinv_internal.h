@@ -168,6 +168,24 @@ cudaError_t launch_df_finish(float4* W, int64_t N, int64_t ld, int64_t blk, floa
 
 // Gram G = (A^H A) o (S^H S) + lambda I, lower tiles, FP64.
 cudaError_t launch_gram64(const EncodeDev& e, double lambda, double2* G, int64_t ld, cudaStream_t s);
+// The same without B0 from the table of grid offsets (where gram64_table_ok).
+bool gram64_table_ok(const EncodeDev& e);
+cudaError_t launch_gram64_table(const EncodeDev& e, double lambda, double2* G, int64_t ld, cudaStream_t s);
+// FP64 products on the tensor cores through exact digits (oz.cu; GPUs with tc_available()):
+// Recon, Ginv = W^H W, and the factorisation and inverse whose trailing updates they form
+// (T: N x 32 scratch, work: oz_panel_bytes(N), Dinv: 32 x 32 block inverses). They take
+// their tables from the pool and return cudaErrorMemoryAllocation without room.
+cudaError_t launch_recon64_oz(const EncodeDev& e, int eexp, const double2* Ginv, double2* R, DevStatus* st,
+                              cudaStream_t s);
+cudaError_t launch_lauum64_oz(const double2* W, int64_t N, double2* Ginv, DevStatus* st, cudaStream_t s);
+size_t oz_panel_bytes(int64_t N);
+cudaError_t oz_herk64(double2* G, int64_t N, int64_t p0, int64_t kw, void* work, DevStatus* st, cudaStream_t s);
+cudaError_t oz_trtri64(double2* W, const double2* L, int64_t N, int64_t p0, int64_t kw, void* work, DevStatus* st,
+                       cudaStream_t s);
+cudaError_t launch_potrf64_oz(double2* G, int64_t N, double2* Dinv, double2* T, void* work, DevStatus* st,
+                              cudaStream_t s);
+cudaError_t launch_trtri64_oz(const double2* L, int64_t N, const double2* Dinv, double2* W, void* work, DevStatus* st,
+                              cudaStream_t s);
 // Cholesky in place on the lower triangle of G (FP64, blocked, nb = 64).
 cudaError_t launch_potrf64(double2* G, int64_t N, int64_t ld, double2* Dinv, DevStatus* st,
                            cudaStream_t s);

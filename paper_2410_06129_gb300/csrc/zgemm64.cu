@@ -125,6 +125,110 @@ cudaError_t launch_gram64(const EncodeDev& e, double lambda, double2* G, int64_t
 }
 
 // ---------------------------------------------------------------------------
+// The same Gram without B0: (A^H A)[i][j] depends only on the difference of the two
+// voxels' grid indices (the phases of Eq. 2 on a grid), so it is read from a table
+//   T[dz][dy][dx] = sum_m q_x(m, dx) q_y(m, dy) q_z(m, dz),
+//   q(m, d) = exp(+i 2 pi k_m d fov / n) = conj(e[m][d]) e[m][0] (d >= 0) or its mirror,
+// of (2 n - 1) offsets per axis, half of them by T[-d] = conj(T[d]). Both kernels are bound
+// by the FP64 pipe: at 37 x 37 voxels, 4 coils and 2701 samples the tile kernel above took
+// 23.8 ms for 2.5e9 complex MACs, the table has 7e6 and the coil sums 4e6.
+// ---------------------------------------------------------------------------
+__device__ inline double2 toep_q64(const double2* tab, int n, int64_t m, int d) {
+    if (n == 1) return make_double2(1.0, 0.0);
+    const double2* row = tab + m * n;
+    return d >= 0 ? zmul(zconj(row[d]), row[0]) : zmul(zconj(row[0]), row[-d]);
+}
+struct ToepP {
+    static constexpr bool A_KFAST = false, B_KFAST = false;
+    EncodeDev e;
+    double2* part;                // [splits][F][Tx]
+    int64_t Tx, Ty, F, jm, chunk;  // columns jm .. jm + F - 1 of T[d_yz][d_x]
+    __device__ bool tile(int64_t& i0, int64_t& j0, int64_t& kb, int64_t& ke) const {
+        i0 = (int64_t)blockIdx.x * 16;
+        j0 = (int64_t)blockIdx.y * 16;
+        kb = (int64_t)blockIdx.z * chunk;
+        ke = kb + chunk < e.Mk ? kb + chunk : e.Mk;
+        return true;
+    }
+    __device__ bool a_ok(int64_t i) const { return i < Tx; }
+    __device__ bool b_ok(int64_t j) const { return j < F; }
+    __device__ double2 a(int64_t i, int64_t m) const { return toep_q64(e.ex, e.nx, m, (int)i - (e.nx - 1)); }
+    __device__ double2 b(int64_t m, int64_t j) const {
+        const int64_t jj = j + jm;
+        const double2 qy = toep_q64(e.ey, e.ny, m, (int)(jj % Ty) - (e.ny - 1));
+        return e.nz > 1 ? zmul(qy, toep_q64(e.ez, e.nz, m, (int)(jj / Ty) - (e.nz - 1))) : qy;
+    }
+    __device__ void store(int64_t i, int64_t j, double2 v) const {
+        part[((int64_t)blockIdx.z * F + j) * Tx + i] = v;
+    }
+};
+// T from its partial tables, added in order; canonical entries (d_yz > 0, or d_yz = 0 and
+// d_x >= 0) and their mirrors
+__global__ void k_toep64_sum(const double2* part, int splits, int64_t Tx, int64_t F, int64_t Tyz, double2* T) {
+    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= Tx * F) return;
+    const int64_t i = idx % Tx, j = idx / Tx, jj = j + (Tyz - 1) / 2;
+    if (j == 0 && i < (Tx - 1) / 2) return;
+    double2 v = part[idx];
+    for (int z = 1; z < splits; ++z) v = zadd(v, part[(int64_t)z * Tx * F + idx]);
+    T[jj * Tx + i] = v;
+    const int64_t mi = Tx - 1 - i, mj = Tyz - 1 - jj;
+    if (mi != i || mj != jj) T[mj * Tx + mi] = zconj(v);
+}
+// G[i][j], j <= i
+__global__ void __launch_bounds__(256) k_gram_table64(EncodeDev e, const double2* __restrict__ T, double lam,
+                                                     double2* G, int64_t ld) {
+    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, i = blockIdx.y;
+    if (j > i) return;
+    const int* gi = e.vox_ijk + 3 * i;
+    const int* gj = e.vox_ijk + 3 * j;
+    const int64_t Tx = 2 * e.nx - 1, Ty = 2 * e.ny - 1;
+    double2 v = T[((int64_t)(gi[2] - gj[2] + e.nz - 1) * Ty + (gi[1] - gj[1] + e.ny - 1)) * Tx +
+                  (gi[0] - gj[0] + e.nx - 1)];
+    if (e.coils) {
+        double2 sc = make_double2(0.0, 0.0);
+        for (int c = 0; c < e.C; ++c)
+            zfma(sc, zconj(e.coils[(int64_t)c * e.N + i]), e.coils[(int64_t)c * e.N + j]);
+        v = zmul(v, sc);
+    }
+    if (i == j) v.x += lam;
+    G[i * ld + j] = v;
+}
+
+// Worth it (and its table small beside G) where the offsets are at most a quarter of N^2;
+// a voxel list scattered over a large grid keeps the tile kernel.
+bool gram64_table_ok(const EncodeDev& e) {
+    const double offs = (2.0 * e.nx - 1) * (2.0 * e.ny - 1) * (2.0 * e.nz - 1);
+    return !e.b0tab && offs <= 0.25 * (double)e.N * (double)e.N;
+}
+
+cudaError_t launch_gram64_table(const EncodeDev& e, double lambda, double2* G, int64_t ld, cudaStream_t s) {
+    const int64_t Tx = 2 * e.nx - 1, Ty = 2 * e.ny - 1, Tyz = Ty * (2 * e.nz - 1), jm = (Tyz - 1) / 2, F = Tyz - jm;
+    const int64_t tiles = ((Tx + 15) / 16) * ((F + 15) / 16);
+    // about four CTAs per SM, chunks of at least 64 samples
+    int64_t sp = std::min<int64_t>((600 + tiles - 1) / tiles, (e.Mk + 63) / 64);
+    sp = std::max<int64_t>(1, std::min<int64_t>(sp, 64));
+    const int64_t chunk = (e.Mk + sp - 1) / sp;
+    sp = (e.Mk + chunk - 1) / chunk;
+    double2 *part = nullptr, *T = nullptr;
+    cudaError_t err = work_alloc((void**)&part, sizeof(double2) * (size_t)(sp * Tx * F), s);
+    if (err != cudaSuccess) return err;
+    err = work_alloc((void**)&T, sizeof(double2) * (size_t)(Tx * Tyz), s);
+    if (err == cudaSuccess) {
+        ToepP p{e, part, Tx, Ty, F, jm, chunk};
+        k_ztile<16, 16, 1, 1>
+            <<<dim3((unsigned)((Tx + 15) / 16), (unsigned)((F + 15) / 16), (unsigned)sp), 256, 0, s>>>(p);
+        k_toep64_sum<<<(unsigned)((Tx * F + 255) / 256), 256, 0, s>>>(part, (int)sp, Tx, F, Tyz, T);
+        k_gram_table64<<<dim3((unsigned)((e.N + 255) / 256), (unsigned)e.N), 256, 0, s>>>(e, T, lambda, G, ld);
+        note_launch(3);
+        err = cudaGetLastError();
+        cudaFreeAsync(T, s);
+    }
+    cudaFreeAsync(part, s);
+    return err;
+}
+
+// ---------------------------------------------------------------------------
 // Blocked Cholesky pieces
 // ---------------------------------------------------------------------------
 // panel solve: L[i][k0+j] = sum_k G[i][k0+k] conj(Dinv[j][k]) for rows i >= k0+NB
@@ -296,6 +400,232 @@ cudaError_t launch_potrf64(double2* G, int64_t N, int64_t ld, double2* Dinv, Dev
         note_launch();
     }
     return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------------------
+// The same factorisation with the trailing updates on the tensor cores (oz.cu), for GPUs
+// that have them: 32-wide diagonal blocks inside 64-wide panels. The FP64 pipe (2 DFMA per
+// clock and SM) keeps only work of a few microseconds: the diagonal blocks, and the solve
+// and the update inside a panel in 16 x 16 tiles, so that all SMs share them (a 64 x 64 tile
+// of K = 64 takes one SM 260 us). At N = 1369 the steps of a 64-wide block took 915 us
+// (diagonal block 319, solve 266, update 330).
+// ---------------------------------------------------------------------------
+constexpr int NBS = 32;  // diagonal blocks
+constexpr int NBO = 64;  // panels
+
+// One 32 x 32 diagonal block and its inverse. Right-looking with unscaled columns, one
+// barrier per column: every thread forms 1 / d_j itself and updates its (at most three)
+// entries by A_ij conj(A_kj) / d_j; columns are scaled by 1 / sqrt(d_j) at the end. The
+// inverse by forward substitution, eight lanes a column.
+__global__ void __launch_bounds__(256) k_potrf_diag32(double2* G, int64_t ld, int64_t N, int64_t k0, double2* Dinv,
+                                                      DevStatus* st) {
+    __shared__ double2 A[NBS][NBS + 1], X[NBS][NBS + 1];
+    __shared__ double rd[NBS];  // 1 / L_jj
+    const int tid = threadIdx.x;
+    const int nb = (int)((N - k0) < NBS ? (N - k0) : NBS);
+    for (int e = tid; e < NBS * NBS; e += 256) {
+        const int i = e / NBS, j = e % NBS;
+        A[i][j] = i < nb && j <= i ? G[(k0 + i) * ld + k0 + j] : make_double2(i == j ? 1.0 : 0.0, 0.0);
+    }
+    // entries (i, k), 1 <= k <= i: numbered from the last column, so the threads that still
+    // have work stay together
+    constexpr int NE = (NBS - 1) * NBS / 2;  // 496
+    int ei[2], ek[2];
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+        const int e = tid + 256 * t;
+        ei[t] = -1;
+        ek[t] = 0;
+        if (e < NE) {
+            int r = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
+            while (r * (r + 1) / 2 > e) --r;
+            while ((r + 1) * (r + 2) / 2 <= e) ++r;
+            ek[t] = NBS - 1 - r;
+            ei[t] = ek[t] + (e - r * (r + 1) / 2);
+        }
+    }
+    __syncthreads();
+    for (int j = 0; j < NBS; ++j) {
+        double d = A[j][j].x;
+        const bool fail = !(d > 0.0) || !isfinite(d);
+        if (fail) {
+            d = 1.0;
+            if (tid == 0) atomicMin(&st->not_pd_pivot, (int)(k0 + j));
+        }
+        const double inv = 1.0 / d;
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            if (ei[t] >= 0 && ek[t] > j) {
+                const double2 a = A[ei[t]][j];
+                double2 v = A[ei[t]][ek[t]];
+                zfma(v, make_double2(-a.x * inv, -a.y * inv), zconj(A[ek[t]][j]));
+                A[ei[t]][ek[t]] = v;
+            }
+        }
+        if (tid == 0) rd[j] = rsqrt(d);
+        __syncthreads();
+    }
+    for (int e = tid; e < NBS * NBS; e += 256) {
+        const int i = e / NBS, j = e % NBS;
+        if (j > i) continue;
+        const double r = rd[j];
+        double2 v = A[i][j];
+        // the pivot d r = sqrt(d); a failed pivot counts as 1
+        v = i == j ? make_double2((v.x > 0.0 && isfinite(v.x) ? v.x : 1.0) * r, 0.0) : make_double2(v.x * r, v.y * r);
+        A[i][j] = v;
+        if (i < nb && j < nb) G[(k0 + i) * ld + k0 + j] = v;
+    }
+    __syncthreads();
+    const int c = tid >> 3, q = tid & 7;
+    for (int i = 0; i < NBS; ++i) {
+        double2 part = make_double2(0.0, 0.0);
+        for (int k = c + q; k < i; k += 8) zfma(part, A[i][k], X[k][c]);
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) {
+            part.x += __shfl_xor_sync(0xffffffffu, part.x, o);
+            part.y += __shfl_xor_sync(0xffffffffu, part.y, o);
+        }
+        if (q == 0) {
+            const double r = rd[i];
+            X[i][c] = i >= c ? make_double2(((i == c ? 1.0 : 0.0) - part.x) * r, -part.y * r) : make_double2(0.0, 0.0);
+        }
+        __syncwarp();
+    }
+    __syncthreads();
+    for (int e = tid; e < NBS * NBS; e += 256) Dinv[e] = X[e / NBS][e % NBS];
+}
+
+// 16 x 16 tiles of the panel's products, K = nbk <= 32
+// TrsmS: G[i][k0+j] = sum_k G[i][k0+k] conj(Dinv[j][k]), rows i >= k0 + nbk; the result goes
+// to T [rows][NBS] first (its columns are also its inputs), then back (k_put_cols)
+struct TrsmS {
+    static constexpr bool A_KFAST = true, B_KFAST = true;
+    const double2* G;
+    double2* T;
+    int64_t ld, N, k0, nbk;
+    const double2* Dinv;
+    __device__ bool tile(int64_t& i0, int64_t& j0, int64_t& kb, int64_t& ke) const {
+        i0 = k0 + nbk + (int64_t)blockIdx.x * 16;
+        j0 = (int64_t)blockIdx.y * 16;
+        kb = 0;
+        ke = nbk;
+        return j0 < nbk;
+    }
+    __device__ bool a_ok(int64_t i) const { return i < N; }
+    __device__ bool b_ok(int64_t j) const { return j < nbk; }
+    __device__ double2 a(int64_t i, int64_t k) const { return G[i * ld + k0 + k]; }
+    __device__ double2 b(int64_t k, int64_t j) const { return zconj(Dinv[j * NBS + k]); }
+    __device__ void store(int64_t i, int64_t j, double2 v) const { T[(i - k0 - nbk) * NBS + j] = v; }
+};
+__global__ void k_put_cols(const double2* T, int64_t rows, int64_t w, double2* G, int64_t ld) {
+    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t i = idx / NBS, j = idx % NBS;
+    if (i < rows && j < w) G[i * ld + j] = T[idx];
+}
+// G[i][j] -= sum_k L[i][k0+k] conj(L[j][k0+k]), columns k0 + nbk <= j < jmax, rows j <= i
+struct HerkS {
+    static constexpr bool A_KFAST = true, B_KFAST = true;
+    double2* G;
+    int64_t ld, N, k0, nbk, jmax;
+    __device__ bool tile(int64_t& i0, int64_t& j0, int64_t& kb, int64_t& ke) const {
+        i0 = k0 + nbk + (int64_t)blockIdx.x * 16;
+        j0 = k0 + nbk + (int64_t)blockIdx.y * 16;
+        kb = 0;
+        ke = nbk;
+        return j0 <= i0;
+    }
+    __device__ bool a_ok(int64_t i) const { return i < N; }
+    __device__ bool b_ok(int64_t j) const { return j < jmax; }
+    __device__ double2 a(int64_t i, int64_t k) const { return G[i * ld + k0 + k]; }
+    __device__ double2 b(int64_t k, int64_t j) const { return zconj(G[j * ld + k0 + k]); }
+    __device__ void store(int64_t i, int64_t j, double2 v) const {
+        if (j <= i) G[i * ld + j] = zsub(G[i * ld + j], v);
+    }
+};
+// W[k0+i][j] = sum_k Dinv[i][k] W[k0+k][j], j < k0 + nbk: 32 rows x 8 columns per CTA (each
+// thread one output), the inputs staged before any is overwritten
+__global__ void __launch_bounds__(256) k_trtri_diag32(const double2* __restrict__ Dinv, double2* W, int64_t ld,
+                                                      int64_t k0, int nbk, int64_t ncol) {
+    __shared__ double2 D[NBS][NBS + 1], B[NBS][9];
+    const int tid = threadIdx.x, c = tid & 7, i = tid >> 3;
+    const int64_t j = (int64_t)blockIdx.x * 8 + c;
+    for (int e = tid; e < NBS * NBS; e += 256) D[e / NBS][e % NBS] = Dinv[e];
+    B[i][c] = i < nbk && j < ncol ? W[(k0 + i) * ld + j] : make_double2(0.0, 0.0);
+    __syncthreads();
+    double2 v = make_double2(0.0, 0.0);
+    for (int k = 0; k <= i; ++k) zfma(v, D[i][k], B[k][c]);  // Dinv is lower triangular
+    if (i < nbk && j < ncol) W[(k0 + i) * ld + j] = v;
+}
+// W[i][j] -= sum_k L[i][k0+k] W[k0+k][j], rows k0 + nbk <= i < imax, j < k0 + nbk
+struct TrtriS {
+    static constexpr bool A_KFAST = true, B_KFAST = false;
+    double2* W;
+    const double2* L;
+    int64_t ld, k0, nbk, imax;
+    __device__ bool tile(int64_t& i0, int64_t& j0, int64_t& kb, int64_t& ke) const {
+        i0 = k0 + nbk + (int64_t)blockIdx.y * 16;
+        j0 = (int64_t)blockIdx.x * 16;
+        kb = 0;
+        ke = nbk;
+        return true;
+    }
+    __device__ bool a_ok(int64_t i) const { return i < imax; }
+    __device__ bool b_ok(int64_t j) const { return j < k0 + nbk; }
+    __device__ double2 a(int64_t i, int64_t k) const { return L[i * ld + k0 + k]; }
+    __device__ double2 b(int64_t k, int64_t j) const { return W[(k0 + k) * ld + j]; }
+    __device__ void store(int64_t i, int64_t j, double2 v) const { W[i * ld + j] = zsub(W[i * ld + j], v); }
+};
+
+static unsigned cdivu(int64_t a, int64_t b) { return (unsigned)((a + b - 1) / b); }
+
+// work: oz_panel_bytes(N) (tables of the trailing updates); T: N x 32 scratch
+cudaError_t launch_potrf64_oz(double2* G, int64_t N, double2* Dinv, double2* T, void* work, DevStatus* st,
+                              cudaStream_t s) {
+    const int64_t ld = N;
+    cudaError_t e;
+    for (int64_t p0 = 0; p0 < N; p0 += NBO) {
+        const int64_t pend = std::min<int64_t>(N, p0 + NBO);
+        for (int64_t k0 = p0; k0 < pend; k0 += NBS) {
+            const int64_t nbk = std::min<int64_t>(NBS, N - k0), rest = N - k0 - nbk;
+            double2* Dk = Dinv + (k0 / NBS) * NBS * NBS;
+            k_potrf_diag32<<<1, 256, 0, s>>>(G, ld, N, k0, Dk, st);
+            note_launch();
+            if (rest <= 0) break;
+            k_ztile<16, 16, 1, 1><<<dim3(cdivu(rest, 16), 2), 256, 0, s>>>(TrsmS{G, T, ld, N, k0, nbk, Dk});
+            k_put_cols<<<cdivu(rest * NBS, 256), 256, 0, s>>>(T, rest, nbk, G + (k0 + nbk) * ld + k0, ld);
+            note_launch(2);
+            if (k0 + nbk < pend) {
+                k_ztile<16, 16, 1, 1>
+                    <<<dim3(cdivu(rest, 16), cdivu(pend - k0 - nbk, 16)), 256, 0, s>>>(HerkS{G, ld, N, k0, nbk, pend});
+                note_launch();
+            }
+        }
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if (pend < N && (e = oz_herk64(G, N, p0, pend - p0, work, st, s)) != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+cudaError_t launch_trtri64_oz(const double2* L, int64_t N, const double2* Dinv, double2* W, void* work, DevStatus* st,
+                              cudaStream_t s) {
+    const int64_t ld = N;
+    cudaError_t e = launch_fill_identity(W, N, ld, s);
+    for (int64_t p0 = 0; p0 < N && e == cudaSuccess; p0 += NBO) {
+        const int64_t pend = std::min<int64_t>(N, p0 + NBO);
+        for (int64_t k0 = p0; k0 < pend; k0 += NBS) {
+            const int64_t nbk = std::min<int64_t>(NBS, N - k0), ncol = k0 + nbk;
+            k_trtri_diag32<<<cdivu(ncol, 8), 256, 0, s>>>(Dinv + (k0 / NBS) * NBS * NBS, W, ld, k0, (int)nbk, ncol);
+            note_launch();
+            if (ncol < pend) {
+                k_ztile<16, 16, 1, 1>
+                    <<<dim3(cdivu(ncol, 16), cdivu(pend - ncol, 16)), 256, 0, s>>>(TrtriS{W, L, ld, k0, nbk, pend});
+                note_launch();
+            }
+        }
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if (pend < N) e = oz_trtri64(W, L, N, p0, pend - p0, work, st, s);
+    }
+    return e;
 }
 
 // ---------------------------------------------------------------------------

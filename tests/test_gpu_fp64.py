@@ -155,3 +155,35 @@ def test_zero_frames_and_rebuild():
     pl.build()
     x2 = pl.apply(torch.from_numpy(p.data).cuda()).cpu().numpy()
     assert np.array_equal(x1, x2)
+
+
+# N around the 32-wide blocks, 64-wide panels, 128-row and 32-column tiles of the digit
+# products; one, two and three drain groups of 31 stages of 8 (N = 248, 500, 600); coil maps of
+# very small and very large scale (exponents of the fixed-point operands)
+@pytest.mark.parametrize("dims,coils,samples,scale", [
+    ((1,), 1, 3, 1.0), ((31,), 2, 40, 1.0), ((32,), 1, 70, 1.0), ((33,), 3, 50, 1e-40), ((64,), 1, 128, 1.0),
+    ((65,), 2, 90, 1e40), ((127,), 1, 300, 1.0), ((16, 8), 2, 129, 1.0), ((43, 3), 1, 400, 1.0),
+    ((31, 8), 3, 200, 1.0), ((25, 20), 1, 700, 1e-3), ((6, 10, 10), 1, 640, 1.0)])
+def test_digit_products_at_tile_edges(dims, coils, samples, scale):
+    """Every stage against NumPy in FP64 with lambda = mean diag (kappa small): backward-stable
+    stages differ by a multiple of N kappa 2^-53."""
+    from paper_2410_06129_gb300.plan import Plan
+    rng = np.random.default_rng(1903)
+    N, D = int(np.prod(dims)), len(dims)
+    k = rng.uniform(-0.5 * max(dims), 0.5 * max(dims), size=(samples, D))
+    maps = scale * (rng.standard_normal((coils, N)) + 1j * rng.standard_normal((coils, N)))
+    E = O.encode(k, O.voxel_positions(dims), maps, None, None)
+    lam = O.lambda_abs(E, 1.0)
+    G = E.conj().T @ E + lam * np.eye(N)
+    kappa = np.linalg.cond(G)
+    Gi = np.linalg.inv(G)
+    Rm = Gi @ E.conj().T
+    d = rng.standard_normal((2, coils, samples)) + 1j * rng.standard_normal((2, coils, samples))
+    want = (Rm @ d.reshape(2, -1).T).T
+    tol = (64 + 8 * N) * kappa * 2.0 ** -53
+    pl = Plan(dims, k, maps, lam=1.0, precision=L.FP64, keep_gram=True).build()
+    assert rel(np.tril(pl.export(L.EXPORT_GRAM).cpu().numpy()), np.tril(G)) < tol
+    assert rel(pl.export(L.EXPORT_CHOL).cpu().numpy(), np.linalg.cholesky(G)) < tol
+    assert rel(pl.export(L.EXPORT_GINV).cpu().numpy(), Gi) < tol
+    assert rel(pl.export(L.EXPORT_RECON).cpu().numpy(), Rm) < tol
+    assert rel(pl.apply(torch.from_numpy(d).cuda()).cpu().numpy(), want) < tol
