@@ -61,7 +61,7 @@ static ApplyModes apply_modes(const pinv_plan* p) {
     return m;
 }
 
-size_t apply_scratch_layout(const pinv_plan* p, int64_t F, int dtype, void* base, ApplyScratch* sc) {
+size_t apply_scratch_layout(const pinv_plan* p, int64_t F, int dtype, void* base, ApplyScratch* sc, bool oz) {
     const int64_t N = p->N, M = p->M;
     const ApplyModes md = apply_modes(p);
     // FP64 copy of c64 data (every path but the mixed Recon-only apply reads
@@ -113,6 +113,15 @@ size_t apply_scratch_layout(const pinv_plan* p, int64_t F, int dtype, void* base
         s.xfwd = xfwd;
         s.dfw = w ? (float4*)cv.take<uint8_t>(w) : nullptr;
     }
+    if (oz && (!md.mixed || md.fpres) && tc_available()) {
+        // one FP64 product after another: the largest
+        size_t w = 0;
+        if (md.mixed || !p->recon || md.refine) w = std::max(w, oz_adjoint_bytes(p->enc, F));
+        if (md.refine) w = std::max(w, oz_forward_bytes(p->enc, F));
+        if (!md.mixed && p->recon) w = std::max(w, oz_mat_bytes(N, M, F));
+        if (!md.mixed && (!p->recon || md.refine)) w = std::max(w, oz_mat_bytes(N, N, F));
+        s.oz = w ? cv.take<uint8_t>(w) : nullptr;
+    }
     if (sc) *sc = s;
     return cv.used;
 }
@@ -153,6 +162,16 @@ pinv_status apply_impl(pinv_plan* p, const void* d_data, void* d_image, int64_t 
         return launch_correct32(p->W32, N, r, F, sc.x64, X, s);
     };
 
+    // the FP64 products: exact digits on the tensor cores, or the FP64 pipe
+    auto adj64 = [&](const double2* U, double lam, const double2* Xs, double2* Y) -> cudaError_t {
+        return sc.oz ? launch_adjoint64_oz(p->enc, U, F, lam, Xs, Y, sc.oz, p->st, s)
+                     : launch_adjoint64(p->enc, U, F, lam, Xs, Y, s);
+    };
+    auto ginv64 = [&](const double2* r, const double2* add) -> cudaError_t {
+        return sc.oz ? launch_mat64_oz(p->Ginv, N, N, r, F, add, X, sc.oz, p->st, s)
+                     : launch_hemv64(p->Ginv, N, N, r, F, add, X, s);
+    };
+
     if (md.need_b) {  // b = E^H d, exactly on the tensor cores where possible
         if (sc.xadj && sc.d32)
             CKA(launch_adjoint_exact32(p->enc, (const float2*)d_data, F, sc.fexp, sc.dfw, sc.b128, p->st, s, p->Ad));
@@ -161,10 +180,11 @@ pinv_status apply_impl(pinv_plan* p, const void* d_data, void* d_image, int64_t 
     }
     if (!md.mixed) {
         if (p->recon) {
-            CKA(launch_apply64((const double2*)p->R, N, M, D, F, X, s));
+            if (sc.oz) CKA(launch_mat64_oz((const double2*)p->R, N, M, D, F, nullptr, X, sc.oz, p->st, s));
+            else CKA(launch_apply64((const double2*)p->R, N, M, D, F, X, s));
         } else {
-            CKA(launch_adjoint64(p->enc, D, F, 0.0, nullptr, sc.r128, s));
-            CKA(launch_hemv64(p->Ginv, N, N, sc.r128, F, nullptr, X, s));
+            CKA(adj64(D, 0.0, nullptr, sc.r128));
+            CKA(ginv64(sc.r128, nullptr));
         }
     } else if (md.use_recon) {
         // initial image from the mixed-precision Recon
@@ -181,7 +201,7 @@ pinv_status apply_impl(pinv_plan* p, const void* d_data, void* d_image, int64_t 
         CKA(launch_c64_to_c128(sc.x64, X, F * N, s));
     } else if (md.fpres) {
         // factor-only, FP64 throughout: x = W^H (W (E^H d))
-        CKA(launch_adjoint64(p->enc, D, F, 0.0, nullptr, sc.r128, s));
+        CKA(adj64(D, 0.0, nullptr, sc.r128));
         CKA(launch_trmv64(p->W, N, sc.r128, F, sc.u128, s));
         CKA(launch_trmv_h64(p->W, N, sc.u128, F, nullptr, X, s));
     } else {
@@ -199,7 +219,7 @@ pinv_status apply_impl(pinv_plan* p, const void* d_data, void* d_image, int64_t 
             if (md.need_b) {
                 CKA(launch_frame_norms(sc.b128, F, N, sc.norms + F, s));
             } else {
-                CKA(launch_adjoint64(p->enc, D, F, 0.0, nullptr, sc.r128, s));  // b = E^H d
+                CKA(adj64(D, 0.0, nullptr, sc.r128));  // b = E^H d
                 CKA(launch_frame_norms(sc.r128, F, N, sc.norms + F, s));
             }
         }
@@ -222,8 +242,9 @@ pinv_status apply_impl(pinv_plan* p, const void* d_data, void* d_image, int64_t 
                 if ((e = launch_forward_df(p->enc, X, F, D, sc.u128, s, sc.dfw)) != cudaSuccess) return e;  // u = d - E x
                 return launch_adjoint_df(p->enc, sc.u128, F, p->lambda_abs, X, sc.r128, s, sc.dfw);
             }
-            if ((e = launch_forward64(p->enc, X, F, D, sc.u128, s)) != cudaSuccess) return e;
-            return launch_adjoint64(p->enc, sc.u128, F, p->lambda_abs, X, sc.r128, s);
+            e = sc.oz ? launch_forward64_oz(p->enc, X, F, D, sc.u128, sc.oz, p->st, s)
+                      : launch_forward64(p->enc, X, F, D, sc.u128, s);
+            return e != cudaSuccess ? e : adj64(sc.u128, p->lambda_abs, X, sc.r128);
         };
         // stopping rule: per-frame ||r|| / ||E^H d|| read back in fixed-size chunks (no
         // allocation); with `bound`, also the certified error bound of x (below)
@@ -277,7 +298,7 @@ pinv_status apply_impl(pinv_plan* p, const void* d_data, void* d_image, int64_t 
                 CKA(launch_trmv64(p->W, N, sc.r128, F, sc.u128, s));
                 CKA(launch_trmv_h64(p->W, N, sc.u128, F, X, X, s));
             } else {
-                CKA(launch_hemv64(p->Ginv, N, N, sc.r128, F, X, X, s));
+                CKA(ginv64(sc.r128, X));
             }
             p->last_refine_iters = it + 1;
         }
@@ -303,7 +324,7 @@ extern "C" pinv_status pinv_apply(pinv_plan* p, const void* d_data, void* d_imag
                                   void* stream) {
     pinv_status st = apply_check(p, d_data, d_image, F, dtype);
     if (st != PINV_OK || F == 0) return st;
-    const size_t need = apply_scratch_layout(p, F, dtype, nullptr, nullptr);
+    size_t need = apply_scratch_layout(p, F, dtype, nullptr, nullptr, !p->scratch_small);
     if (need > p->scratch_bytes) {
         // grow the plan-owned scratch, from the library's pool: the old region after
         // every earlier apply (on any stream) is done, the new one complete before
@@ -316,6 +337,13 @@ extern "C" pinv_status pinv_apply(pinv_plan* p, const void* d_data, void* d_imag
             if (e != cudaSuccess) return cuda_err(e, "free(apply scratch)");
         }
         cudaError_t e = work_alloc(&p->scratch_buf, need, 0);
+        if (e == cudaErrorMemoryAllocation && !p->scratch_small) {
+            // no room for the FP64 products' tables: the FP64 pipe needs none
+            cudaGetLastError();
+            p->scratch_small = true;
+            need = apply_scratch_layout(p, F, dtype, nullptr, nullptr, false);
+            e = work_alloc(&p->scratch_buf, need, 0);
+        }
         if (e == cudaSuccess) e = cudaStreamSynchronize(0);
         if (e != cudaSuccess) {
             p->scratch_buf = nullptr;
@@ -324,6 +352,6 @@ extern "C" pinv_status pinv_apply(pinv_plan* p, const void* d_data, void* d_imag
         p->scratch_bytes = need;
     }
     ApplyScratch sc;
-    apply_scratch_layout(p, F, dtype, p->scratch_buf, &sc);
+    apply_scratch_layout(p, F, dtype, p->scratch_buf, &sc, !p->scratch_small);
     return apply_impl(p, d_data, d_image, F, dtype, (cudaStream_t)stream, sc);
 }

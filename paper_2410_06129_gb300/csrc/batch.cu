@@ -46,6 +46,7 @@ struct pinv_batch {
     unsigned long long apply_launches = 0;
     std::vector<void*> scratch;
     std::vector<size_t> scratch_bytes;
+    std::vector<char> small;  // per plan: no room for the FP64 products' tables (apply_scratch_layout)
     ~pinv_batch();
 };
 
@@ -144,7 +145,7 @@ pinv_status apply_sequence(pinv_batch* b, const void* const* data, void* const* 
     for (size_t i = 0; i < b->plans.size(); ++i) {
         pinv_plan* p = b->plans[i];
         ApplyScratch sc;
-        apply_scratch_layout(p, frames[i], dtype, b->scratch[i], &sc);
+        apply_scratch_layout(p, frames[i], dtype, b->scratch[i], &sc, !b->small[i]);
         STB(apply_impl(p, data[i], image[i], frames[i], dtype, b->side[i], sc));
     }
     return join_all(b, s);
@@ -214,6 +215,7 @@ pinv_status pinv_batch_create(pinv_plan* const* plans, int n, int flags, pinv_ba
     b->join.assign(n, nullptr);
     b->scratch.assign(n, nullptr);
     b->scratch_bytes.assign(n, 0);
+    b->small.assign(n, 0);
     for (int i = 0; i < n; ++i)
         if (cudaStreamCreateWithFlags(&b->side[i], cudaStreamNonBlocking) != cudaSuccess ||
             cudaEventCreateWithFlags(&b->join[i], cudaEventDisableTiming) != cudaSuccess)
@@ -288,13 +290,20 @@ pinv_status pinv_batch_apply(pinv_batch* b, const void* const* d_data, void* con
     bool grown = false;
     for (size_t i = 0; i < n; ++i) {
         STB(apply_check(b->plans[i], d_data[i], d_image[i], n_frames[i], dtype));
-        const size_t need = apply_scratch_layout(b->plans[i], n_frames[i], dtype, nullptr, nullptr);
+        size_t need = apply_scratch_layout(b->plans[i], n_frames[i], dtype, nullptr, nullptr, !b->small[i]);
         if (need > b->scratch_bytes[i]) {
             // grow outside any capture; a replayed graph would hold the old buffer
             if (b->scratch[i]) CKB(cudaFree(b->scratch[i]));
             b->scratch[i] = nullptr;
             b->scratch_bytes[i] = 0;
-            CKB(cudaMalloc(&b->scratch[i], need));
+            cudaError_t e = cudaMalloc(&b->scratch[i], need);
+            if (e == cudaErrorMemoryAllocation && !b->small[i]) {
+                cudaGetLastError();
+                b->small[i] = 1;
+                need = apply_scratch_layout(b->plans[i], n_frames[i], dtype, nullptr, nullptr, false);
+                e = cudaMalloc(&b->scratch[i], need);
+            }
+            CKB(e);
             b->scratch_bytes[i] = need;
             grown = true;
         }

@@ -1021,8 +1021,9 @@ extern "C" pinv_status pinv_tsvd_apply(pinv_plan* p, const double* d_mu, const v
     double* w = nullptr;
     int* dev_rank = nullptr;
     double* dev_kappa = nullptr;
+    void* oz = nullptr;
     auto release = [&]() {
-        for (void* ptr : {(void*)D, (void*)b, (void*)c, (void*)Ph, (void*)X, (void*)w, (void*)dev_rank, (void*)dev_kappa})
+        for (void* ptr : {(void*)D, (void*)b, (void*)c, (void*)Ph, (void*)X, (void*)w, (void*)dev_rank, (void*)dev_kappa, oz})
             if (ptr) cudaFreeAsync(ptr, s);
     };
 #define CKT(call)                                        \
@@ -1054,15 +1055,26 @@ extern "C" pinv_status pinv_tsvd_apply(pinv_plan* p, const double* d_mu, const v
         CKT(work_alloc((void**)&b, sizeof(double2) * F * N, s));
         CKT(work_alloc((void**)&c, sizeof(double2) * F * N, s));
         CKT(work_alloc((void**)&Ph, sizeof(double2) * N * N, s));
-        CKT(launch_adjoint64(p->enc, Dd, F, 0.0, nullptr, b, s));  // b = E^H d
+        // the products as exact digits on the tensor cores, or (other GPUs, no room for their
+        // tables) on the FP64 pipe
+        const size_t ob = std::max(oz_adjoint_bytes(p->enc, F), oz_mat_bytes(N, N, F));
+        if (!(tc_available() && work_alloc(&oz, ob, s) == cudaSuccess)) {
+            cudaGetLastError();
+            oz = nullptr;
+        }
+        auto mat = [&](const double2* R, const double2* x, double2* y) -> cudaError_t {
+            return oz ? launch_mat64_oz(R, N, N, x, F, nullptr, y, oz, p->st, s) : launch_apply64(R, N, N, x, F, y, s);
+        };
+        CKT(oz ? launch_adjoint64_oz(p->enc, Dd, F, 0.0, nullptr, b, oz, p->st, s)
+               : launch_adjoint64(p->enc, Dd, F, 0.0, nullptr, b, s));  // b = E^H d
         k_conj_transpose<<<blocks(N * N), 256, 0, s>>>((const double2*)d_P, (int)N, Ph);  // Ph = P^H
         note_launch();
         CKT(cudaGetLastError());
-        CKT(launch_apply64(Ph, N, N, b, F, c, s));  // c = P^H b
+        CKT(mat(Ph, b, c));  // c = P^H b
         k_scale_rows<<<blocks(F * N), 256, 0, s>>>(c, F, (int)N, w);
         note_launch();
         CKT(cudaGetLastError());
-        CKT(launch_apply64((const double2*)d_P, N, N, c, F, Xd, s));  // x = P c
+        CKT(mat((const double2*)d_P, c, Xd));  // x = P c
         if (dtype == PINV_C64) CKT(launch_c128_to_c64(Xd, (float2*)d_image, F * N, s));
     }
     if (rank_out || kappa_out) {

@@ -85,22 +85,6 @@ __device__ inline int bits_exp(unsigned long long b) {
     if (eb == 0) return (64 - __clzll((long long)mf)) - 1074 - ((mf & (mf - 1ull)) == 0ull ? 1 : 0);
     return eb - 1023 + (mf != 0ull ? 1 : 0);
 }
-// exponents of the rows of a [rows][K] matrix, one CTA per row
-__global__ void __launch_bounds__(256) k_row_exp(const double2* __restrict__ A, int64_t ld, int64_t K, int* ex) {
-    __shared__ unsigned long long red[8];
-    const double2* row = A + (int64_t)blockIdx.x * ld;
-    unsigned long long m = 0ull;
-#pragma unroll 4
-    for (int64_t k = threadIdx.x; k < K; k += 256) m = max(m, max_bits(row[k]));
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < 8; ++w) m = max(m, red[w]);
-        ex[blockIdx.x] = bits_exp(m);
-    }
-}
 // exponents of the columns of a [K][cols] matrix: 32 columns per CTA, its 8 warps take the rows
 __global__ void __launch_bounds__(256) k_col_exp(const double2* __restrict__ A, int64_t ld, int64_t K, int64_t cols,
                                                  int* ex) {
@@ -171,6 +155,51 @@ struct EncRow {
     }
 };
 
+// conj(A[m][n]) (rows n, k = samples) and A[m][n] (rows m, k = voxels) without the coil
+// factor, |A| = 1
+struct AdjRow {
+    EncodeDev e;
+    int64_t n, K;
+    __device__ int exponent(int64_t) const { return 0; }
+    __device__ double2 get(int64_t i, int64_t k) const { return zconj(gen_a64(e, k, i)); }
+};
+struct FwdRow {
+    EncodeDev e;
+    int64_t n, K;
+    __device__ int exponent(int64_t) const { return 0; }
+    __device__ double2 get(int64_t i, int64_t k) const { return gen_a64(e, i, k); }
+};
+// s_c(k) x[f][k], column q = f C + c
+struct CoilCol {
+    EncodeDev e;
+    const double2* X;
+    int64_t n, K;
+    const int* ex;
+    __device__ int exponent(int64_t q) const { return ex[q]; }
+    __device__ double2 get(int64_t q, int64_t k) const {
+        const int64_t f = q / e.C, c = q - f * e.C;
+        const double2 x = X[f * e.N + k];
+        return e.coils ? zmul(e.coils[c * e.N + k], x) : x;
+    }
+};
+// exponents of p's rows (columns), one CTA each
+template <class P>
+__global__ void __launch_bounds__(256) k_row_exp(P p, int* ex) {
+    __shared__ unsigned long long red[8];
+    const int64_t i = blockIdx.x;
+    unsigned long long m = 0ull;
+#pragma unroll 4
+    for (int64_t k = threadIdx.x; k < p.K; k += 256) m = max(m, max_bits(p.get(i, k)));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) m = max(m, red[w]);
+        ex[i] = bits_exp(m);
+    }
+}
+
 // the 8 values k0 .. k0 + 7 of row i as fixed-point integers (zeros out of range, and for a
 // row that is not finite, whose results the product replaces by NaN)
 template <class P>
@@ -184,13 +213,14 @@ __device__ inline void load_fix(const P& p, int64_t i, int64_t k0, Fix8& re, Fix
         im.set(t, v.y, in ? e : 0);
     }
 }
-// A tiles [row tile][k block][digit]: rows [re | im]; CTA per (k block, row tile)
+// A tiles [row tile][k block][digit] of the k blocks from kb0: rows [re | im]; CTA per
+// (k block, row tile)
 template <class P>
-__global__ void __launch_bounds__(OM) k_oz_a(P p, int64_t KB, uint8_t* At) {
+__global__ void __launch_bounds__(OM) k_oz_a(P p, int64_t kb0, int64_t KB, uint8_t* At) {
     const int64_t kb = blockIdx.x, rt = blockIdx.y;
     const int r = threadIdx.x;
     Fix8 re, im;
-    load_fix(p, rt * OM + r, kb * OKC, re, im);
+    load_fix(p, rt * OM + r, (kb0 + kb) * OKC, re, im);
     uint8_t* blk = At + (rt * KB + kb) * (int64_t)OA_ST;
 #pragma unroll
     for (int dg = OD - 1; dg >= 0; --dg) {
@@ -228,7 +258,7 @@ __global__ void __launch_bounds__(4 * ON) k_oz_b(P p, int64_t KB, uint8_t* Bt) {
 // ------------------------------------------------------------------ the product
 struct Args {
     const uint8_t *At, *Bt;
-    int64_t KB;          // k blocks of the tables
+    int64_t KB, KBb, kb0;  // k blocks of the tables of A and of B, B's k block of A's first
     const int *ra, *cb;  // exponents of the rows (null: ea) and of the columns
     int ea;
 };
@@ -324,7 +354,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_oz(P p, Args a, DevStatus* st) 
                 uint8_t* base = smem + s * OSTAGE;
                 mbar_arrive_expect_tx(&abar[s], (uint32_t)OSTAGE);
                 bulk_g2s(base, a.At + (rt * a.KB + kb + kt) * (int64_t)OA_ST, (uint32_t)OA_ST, &abar[s]);
-                bulk_g2s(base + OA_ST, a.Bt + (ct * a.KB + kb + kt) * (int64_t)OB_ST, (uint32_t)OB_ST, &abar[s]);
+                bulk_g2s(base + OA_ST, a.Bt + (ct * a.KBb + a.kb0 + kb + kt) * (int64_t)OB_ST, (uint32_t)OB_ST, &abar[s]);
                 issued = kt + 1;
             }
             // a group is drained once the stages after it are in flight: its last
@@ -512,6 +542,55 @@ __global__ void __launch_bounds__(256) k_oz_panel(const double2* __restrict__ p,
     }
 }
 
+// A product with frames: splits of a k chunk side by side, chunks one after another
+// (add: onto the earlier chunks' sums). P [split][column][row].
+struct PartOz {
+    double2* P;
+    int64_t nrows, ncols, rtn, ctn, kbs, KB;
+    int add;
+    __device__ int64_t rows() const { return nrows; }
+    __device__ int64_t cols() const { return ncols; }
+    __device__ bool tile(int64_t b, int64_t& rt, int64_t& ct, int64_t& kb, int64_t& ke) const {
+        ct = b % ctn;
+        rt = b / ctn % rtn;
+        kb = b / (ctn * rtn) * kbs;
+        ke = kb + kbs < KB ? kb + kbs : KB;
+        return true;
+    }
+    __device__ void store(int64_t b, int64_t i, int64_t j, double2 v) const {
+        double2* q = P + (b / (ctn * rtn) * ncols + j) * nrows + i;
+        *q = add ? zadd(*q, v) : v;
+    }
+};
+// Y[f][n] = sum_c conj(s_c(n)) sum_z P[z][f C + c][n] - lam X[f][n] (X may be null)
+__global__ void k_adj_sum(EncodeDev e, const double2* P, int sub, int64_t F, double lam, const double2* X, double2* Y) {
+    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= F * e.N) return;
+    const int64_t n = idx % e.N, f = idx / e.N, Q = F * e.C;
+    double2 y = make_double2(0.0, 0.0);
+    for (int c = 0; c < e.C; ++c) {
+        double2 a = P[(f * e.C + c) * e.N + n];
+        for (int z = 1; z < sub; ++z) a = zadd(a, P[((int64_t)z * Q + f * e.C + c) * e.N + n]);
+        if (e.coils) zfma(y, zconj(e.coils[(int64_t)c * e.N + n]), a);
+        else y = zadd(y, a);
+    }
+    if (X) {
+        const double2 x = X[idx];
+        y.x -= lam * x.x;
+        y.y -= lam * x.y;
+    }
+    Y[idx] = y;
+}
+// Y = B +- sum_z P[z] over n entries (B may be null); Y may be B
+__global__ void k_part_add(const double2* P, int sub, int64_t n, int minus, const double2* B, double2* Y) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    double2 a = P[i];
+    for (int z = 1; z < sub; ++z) a = zadd(a, P[(int64_t)z * n + i]);
+    const double2 b = B ? B[i] : make_double2(0.0, 0.0);
+    Y[i] = minus ? zsub(b, a) : zadd(b, a);
+}
+
 template <class P>
 cudaError_t run(const P& p, int64_t tiles, const Args& a, DevStatus* st, cudaStream_t s) {
     static bool attr = false;
@@ -525,8 +604,8 @@ cudaError_t run(const P& p, int64_t tiles, const Args& a, DevStatus* st, cudaStr
     return cudaGetLastError();
 }
 template <class P>
-cudaError_t tab_a(const P& p, int64_t KB, uint8_t* At, cudaStream_t s) {
-    k_oz_a<P><<<dim3((unsigned)KB, (unsigned)((p.n + OM - 1) / OM)), OM, 0, s>>>(p, KB, At);
+cudaError_t tab_a(const P& p, int64_t kb0, int64_t KB, uint8_t* At, cudaStream_t s) {
+    k_oz_a<P><<<dim3((unsigned)KB, (unsigned)((p.n + OM - 1) / OM)), OM, 0, s>>>(p, kb0, KB, At);
     note_launch();
     return cudaGetLastError();
 }
@@ -575,14 +654,15 @@ cudaError_t launch_recon64_oz(const EncodeDev& e, int eexp, const double2* Ginv,
     OZ(t.take(&At, (size_t)(per * KB * OA_ST)));
     OZ(t.take(&Bt, (size_t)(ctn * KB * OB_ST)));
     OZ(t.take(&ex, sizeof(int) * N));
-    k_row_exp<<<(unsigned)N, 256, 0, s>>>(Ginv, N, N, ex);
+    const Mat gm{Ginv, N, N, N, 0, 0, ex};
+    k_row_exp<<<(unsigned)N, 256, 0, s>>>(gm, ex);
     note_launch();
-    OZ(tab_b(Mat{Ginv, N, N, N, 0, 0, ex}, KB, Bt, s));
+    OZ(tab_b(gm, KB, Bt, s));
     for (int64_t r0 = 0; r0 < rtn; r0 += per) {
         const int64_t j0 = r0 * OM, rows = std::min(per * OM, M - j0);
-        OZ(tab_a(EncRow{e, j0, rows, N, eexp}, KB, At, s));
+        OZ(tab_a(EncRow{e, j0, rows, N, eexp}, 0, KB, At, s));
         const ReconOz p{R, M, j0, rows, N, KB, ctn};
-        OZ(run(p, (rows + OM - 1) / OM * ctn, Args{At, Bt, KB, nullptr, ex, eexp}, st, s));
+        OZ(run(p, (rows + OM - 1) / OM * ctn, Args{At, Bt, KB, KB, 0, nullptr, ex, eexp}, st, s));
     }
     return cudaSuccess;
 }
@@ -599,10 +679,131 @@ cudaError_t launch_lauum64_oz(const double2* W, int64_t N, double2* Ginv, DevSta
     OZ(t.take(&ex, sizeof(int) * N));
     k_col_exp<<<(unsigned)((N + 31) / 32), 256, 0, s>>>(W, N, N, N, ex);
     note_launch();
-    OZ(tab_a(Mat{W, N, N, N, 1, 1, ex}, KB, At, s));
+    OZ(tab_a(Mat{W, N, N, N, 1, 1, ex}, 0, KB, At, s));
     OZ(tab_b(Mat{W, N, N, N, 1, 0, ex}, KB, Bt, s));
     const LauumOz p{Ginv, N, KB, ctn};
-    return run(p, rtn * ctn, Args{At, Bt, KB, ex, ex, 0}, st, s);
+    return run(p, rtn * ctn, Args{At, Bt, KB, KB, 0, ex, ex, 0}, st, s);
+}
+
+// ------------------------------------------------------------------ products with frames
+// rows x K times K x Q, Q columns in all, in groups of qg columns: the A tables of one k
+// chunk (at most 128 MiB), the B tables of one group (at most 256 MiB), the partials of
+// as many splits as give every SM a tile, and the exponents, in one region of scratch.
+namespace oz {
+struct FrameShape {
+    int64_t rtn, KB, kc, qg;   // row tiles, k blocks, k blocks per chunk, columns per group
+    int64_t sub, kbs;          // splits per chunk, their k blocks
+    size_t at, bt, pt, xr, xc;  // bytes
+    size_t bytes() const { return at + bt + pt + xr + xc; }
+};
+static FrameShape frame_shape(int64_t rows, int64_t K, int64_t Q, int64_t unit) {
+    auto up = [](size_t n) { return (n + 255) & ~(size_t)255; };
+    FrameShape f;
+    f.rtn = (rows + OM - 1) / OM;
+    f.KB = (K + OKC - 1) / OKC;
+    f.kc = std::max<int64_t>(1, std::min<int64_t>(f.KB, (int64_t(128) << 20) / (f.rtn * OA_ST)));
+    // columns of one group: whole multiples of unit (the coils of a frame)
+    int64_t g = std::max<int64_t>(1, (int64_t(256) << 20) / (f.KB * OB_ST)) * ON;
+    g = std::max<int64_t>(unit, g / unit * unit);
+    f.qg = std::min<int64_t>(Q, g);
+    const int64_t ctn = (f.qg + ON - 1) / ON;
+    // splits of at least 16 k blocks that fill the SMs once
+    f.sub = std::max<int64_t>(1, std::min<int64_t>(f.kc / 16, tc::sm_count() / std::max<int64_t>(1, f.rtn * ctn)));
+    f.kbs = (f.kc + f.sub - 1) / f.sub;
+    f.at = (size_t)(f.rtn * f.kc * OA_ST);
+    f.bt = (size_t)(ctn * f.KB * OB_ST);
+    f.pt = up(sizeof(double2) * (size_t)(f.sub * f.qg * rows));
+    f.xr = up(sizeof(int) * (size_t)rows);
+    f.xc = up(sizeof(int) * (size_t)f.qg);
+    return f;
+}
+struct FrameWork {
+    uint8_t *At, *Bt;
+    double2* P;
+    int *xr, *xc;
+};
+static FrameWork frame_work(const FrameShape& f, void* base) {
+    uint8_t* q = (uint8_t*)base;
+    return {q, q + f.at, (double2*)(q + f.at + f.bt), (int*)(q + f.at + f.bt + f.pt),
+            (int*)(q + f.at + f.bt + f.pt + f.xr)};
+}
+// the partials of one group of columns (b.n of them); ra: exponents of A's rows or null (0)
+template <class PA, class PB>
+static cudaError_t frame_group(const FrameShape& f, const FrameWork& w, const PA& a, const PB& b, const int* ra,
+                               DevStatus* st, cudaStream_t s) {
+    k_row_exp<PB><<<(unsigned)b.n, 256, 0, s>>>(b, w.xc);
+    note_launch();
+    OZ(tab_b(b, f.KB, w.Bt, s));
+    const int64_t ctn = (b.n + ON - 1) / ON;
+    for (int64_t k0 = 0; k0 < f.KB; k0 += f.kc) {
+        const int64_t kn = std::min(f.kc, f.KB - k0);
+        OZ(tab_a(a, k0, kn, w.At, s));
+        const PartOz p{w.P, a.n, b.n, f.rtn, ctn, f.kbs, kn, k0 > 0 ? 1 : 0};
+        OZ(run(p, f.rtn * ctn * f.sub, Args{w.At, w.Bt, kn, f.KB, k0, ra, w.xc, 0}, st, s));
+    }
+    return cudaSuccess;
+}
+}  // namespace oz
+
+size_t oz_adjoint_bytes(const EncodeDev& e, int64_t F) { return oz::frame_shape(e.N, e.Mk, F * e.C, e.C).bytes(); }
+size_t oz_forward_bytes(const EncodeDev& e, int64_t F) { return oz::frame_shape(e.Mk, e.N, F * e.C, e.C).bytes(); }
+size_t oz_mat_bytes(int64_t N, int64_t K, int64_t F) { return oz::frame_shape(N, K, F, 1).bytes(); }
+
+// Y[f][n] = sum_{c,m} conj(s_c(n) A[m][n]) D[f][c][m] - lam X[f][n] (X may be null)
+cudaError_t launch_adjoint64_oz(const EncodeDev& e, const double2* D, int64_t F, double lam, const double2* X,
+                                double2* Y, void* scratch, DevStatus* st, cudaStream_t s) {
+    using namespace oz;
+    if (F == 0) return cudaSuccess;
+    const FrameShape f = frame_shape(e.N, e.Mk, F * e.C, e.C);
+    const FrameWork w = frame_work(f, scratch);
+    for (int64_t q0 = 0; q0 < F * e.C; q0 += f.qg) {
+        const int64_t q = std::min(f.qg, F * e.C - q0), f0 = q0 / e.C, Fn = q / e.C;
+        OZ(frame_group(f, w, AdjRow{e, e.N, e.Mk}, Mat{D + q0 * e.Mk, e.Mk, q, e.Mk, 0, 0, w.xc}, nullptr, st, s));
+        k_adj_sum<<<(unsigned)((Fn * e.N + 255) / 256), 256, 0, s>>>(e, w.P, (int)f.sub, Fn, lam,
+                                                                     X ? X + f0 * e.N : nullptr, Y + f0 * e.N);
+        note_launch();
+        OZ(cudaGetLastError());
+    }
+    return cudaSuccess;
+}
+
+// U[f][c][m] = D[f][c][m] - sum_n s_c(n) A[m][n] X[f][n] (D may be null: U = -E X)
+cudaError_t launch_forward64_oz(const EncodeDev& e, const double2* X, int64_t F, const double2* D, double2* U,
+                                void* scratch, DevStatus* st, cudaStream_t s) {
+    using namespace oz;
+    if (F == 0) return cudaSuccess;
+    const FrameShape f = frame_shape(e.Mk, e.N, F * e.C, e.C);
+    const FrameWork w = frame_work(f, scratch);
+    for (int64_t q0 = 0; q0 < F * e.C; q0 += f.qg) {
+        const int64_t q = std::min(f.qg, F * e.C - q0), f0 = q0 / e.C;
+        OZ(frame_group(f, w, FwdRow{e, e.Mk, e.N}, CoilCol{e, X + f0 * e.N, q, e.N, w.xc}, nullptr, st, s));
+        k_part_add<<<(unsigned)((q * e.Mk + 255) / 256), 256, 0, s>>>(w.P, (int)f.sub, q * e.Mk, 1,
+                                                                      D ? D + q0 * e.Mk : nullptr, U + q0 * e.Mk);
+        note_launch();
+        OZ(cudaGetLastError());
+    }
+    return cudaSuccess;
+}
+
+// Y[f][n] = B[f][n] + sum_k R[n][k] X[f][k] (R row-major, ld K; B may be null, or Y)
+cudaError_t launch_mat64_oz(const double2* R, int64_t N, int64_t K, const double2* X, int64_t F, const double2* B,
+                            double2* Y, void* scratch, DevStatus* st, cudaStream_t s) {
+    using namespace oz;
+    if (F == 0) return cudaSuccess;
+    const FrameShape f = frame_shape(N, K, F, 1);
+    const FrameWork w = frame_work(f, scratch);
+    const Mat a{R, K, N, K, 0, 0, w.xr};
+    k_row_exp<<<(unsigned)N, 256, 0, s>>>(a, w.xr);
+    note_launch();
+    for (int64_t f0 = 0; f0 < F; f0 += f.qg) {
+        const int64_t q = std::min(f.qg, F - f0);
+        OZ(frame_group(f, w, a, Mat{X + f0 * K, K, q, K, 0, 0, w.xc}, w.xr, st, s));
+        k_part_add<<<(unsigned)((q * N + 255) / 256), 256, 0, s>>>(w.P, (int)f.sub, q * N, 0, B ? B + f0 * N : nullptr,
+                                                                   Y + f0 * N);
+        note_launch();
+        OZ(cudaGetLastError());
+    }
+    return cudaSuccess;
 }
 
 // tables of one panel's update: A and B tiles and exponents of up to N rows each
@@ -635,7 +836,7 @@ cudaError_t oz_herk64(double2* G, int64_t N, int64_t p0, int64_t kw, void* work,
     note_launch();
     OZ(cudaGetLastError());
     const UpdateOz p{G, N, N, t0, t0, n, ctn, 1};
-    return run(p, (n + OM - 1) / OM * ctn, Args{w.At, w.Bt, PKB, w.ea, w.ea, 0}, st, s);
+    return run(p, (n + OM - 1) / OM * ctn, Args{w.At, w.Bt, PKB, PKB, 0, w.ea, w.ea, 0}, st, s);
 }
 
 // W[i][j] -= sum_k L[i][p0+k] W[p0+k][j], k < kw <= 64, rows i >= p0 + kw, columns j < p0 + kw
@@ -650,7 +851,7 @@ cudaError_t oz_trtri64(double2* W, const double2* L, int64_t N, int64_t p0, int6
     note_launch(2);
     OZ(cudaGetLastError());
     const UpdateOz p{W, N, N, t0, 0, t0, ctn, 0};
-    return run(p, (n + OM - 1) / OM * ctn, Args{w.At, w.Bt, PKB, w.ea, w.eb, 0}, st, s);
+    return run(p, (n + OM - 1) / OM * ctn, Args{w.At, w.Bt, PKB, PKB, 0, w.ea, w.eb, 0}, st, s);
 }
 
 }  // namespace pinv

@@ -187,3 +187,36 @@ def test_digit_products_at_tile_edges(dims, coils, samples, scale):
     assert rel(pl.export(L.EXPORT_GINV).cpu().numpy(), Gi) < tol
     assert rel(pl.export(L.EXPORT_RECON).cpu().numpy(), Rm) < tol
     assert rel(pl.apply(torch.from_numpy(d).cuda()).cpu().numpy(), want) < tol
+
+
+# frames around the 32-column tiles; one and several splits of k; Recon's k in two chunks of 4096
+@pytest.mark.parametrize("dims,coils,samples,frames,recon", [
+    ((33,), 1, 50, 1, True), ((33,), 3, 50, 31, False), ((16, 8), 2, 129, 33, False), ((43, 3), 1, 400, 70, True),
+    ((32, 32), 4, 1100, 5, True)])
+def test_apply_digit_products_frames(dims, coils, samples, frames, recon):
+    """Frames of very different scale, an empty one and one that is not finite: each frame's
+    image against NumPy in FP64 (lambda = mean diag, tolerance as above)."""
+    from paper_2410_06129_gb300.plan import Plan
+    rng = np.random.default_rng(1904)
+    N, D = int(np.prod(dims)), len(dims)
+    k = rng.uniform(-0.5 * max(dims), 0.5 * max(dims), size=(samples, D))
+    maps = rng.standard_normal((coils, N)) + 1j * rng.standard_normal((coils, N))
+    E = O.encode(k, O.voxel_positions(dims), maps, None, None)
+    G = E.conj().T @ E + O.lambda_abs(E, 1.0) * np.eye(N)
+    d = rng.standard_normal((frames, coils, samples)) + 1j * rng.standard_normal((frames, coils, samples))
+    d *= 10.0 ** rng.integers(-30, 30, size=(frames, 1, 1))
+    want = np.linalg.solve(G, E.conj().T @ d.reshape(frames, -1).T).T
+    if frames > 2:
+        d[1], want[1] = 0, 0
+        d[2, 0, 0] = np.nan
+    tol = (64 + 8 * N) * np.linalg.cond(G) * 2.0 ** -53
+    pl = Plan(dims, k, maps, lam=1.0, precision=L.FP64,
+              recon_mode=L.RECON_STORE if recon else L.RECON_NONE).build()
+    x = pl.apply(torch.from_numpy(d).cuda()).cpu().numpy()
+    for f in range(frames):
+        if frames > 2 and f == 1:
+            assert not x[f].any()
+        elif frames > 2 and f == 2:
+            assert not np.isfinite(x[f]).any()
+        else:
+            assert rel(x[f], want[f]) < tol
