@@ -413,86 +413,73 @@ cudaError_t launch_potrf64(double2* G, int64_t N, int64_t ld, double2* Dinv, Dev
 constexpr int NBS = 32;  // diagonal blocks
 constexpr int NBO = 64;  // panels
 
-// One 32 x 32 diagonal block and its inverse. Right-looking with unscaled columns, one
-// barrier per column: every thread forms 1 / d_j itself and updates its (at most three)
-// entries by A_ij conj(A_kj) / d_j; columns are scaled by 1 / sqrt(d_j) at the end. The
-// inverse by forward substitution, eight lanes a column.
+// One 32 x 32 diagonal block and its inverse, right-looking together. A warp instruction on
+// the FP64 pipe takes 16 cycles of the whole SM, so what counts is how many of them there
+// are: step j has one warp form S_i = A_ij / d_j (the only division), and every entry
+// (i, c) of the rows below takes one complex FMA, A_ic -= S_i conj(A_cj) right of column j
+// and Y_ic -= S_i Y_jc up to it (Y, the inverse, unscaled). Warp w holds rows w + 8 t, lane
+// c column c, in registers; an entry of A is published before its column's step, a row of
+// Y before its row's. Columns and rows are scaled by 1 / sqrt(d_j) at the end. (All warps
+// dividing, and the inverse by shuffled dot products, took 72 us.)
 __global__ void __launch_bounds__(256) k_potrf_diag32(double2* G, int64_t ld, int64_t N, int64_t k0, double2* Dinv,
                                                       DevStatus* st) {
-    __shared__ double2 A[NBS][NBS + 1], X[NBS][NBS + 1];
-    __shared__ double rd[NBS];  // 1 / L_jj
-    const int tid = threadIdx.x;
+    __shared__ double2 At[NBS][NBS];  // At[j][i] = A_ij once column j is final
+    __shared__ double2 Ys[NBS][NBS];  // Ys[i][c] once row i is final
+    __shared__ double2 S[NBS];
+    __shared__ double dj[NBS], rd[NBS];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nb = (int)((N - k0) < NBS ? (N - k0) : NBS);
-    for (int e = tid; e < NBS * NBS; e += 256) {
-        const int i = e / NBS, j = e % NBS;
-        A[i][j] = i < nb && j <= i ? G[(k0 + i) * ld + k0 + j] : make_double2(i == j ? 1.0 : 0.0, 0.0);
-    }
-    // entries (i, k), 1 <= k <= i: numbered from the last column, so the threads that still
-    // have work stay together
-    constexpr int NE = (NBS - 1) * NBS / 2;  // 496
-    int ei[2], ek[2];
+    double2 v[4], y[4];
 #pragma unroll
-    for (int t = 0; t < 2; ++t) {
-        const int e = tid + 256 * t;
-        ei[t] = -1;
-        ek[t] = 0;
-        if (e < NE) {
-            int r = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
-            while (r * (r + 1) / 2 > e) --r;
-            while ((r + 1) * (r + 2) / 2 <= e) ++r;
-            ek[t] = NBS - 1 - r;
-            ei[t] = ek[t] + (e - r * (r + 1) / 2);
-        }
+    for (int t = 0; t < 4; ++t) {
+        const int i = warp + 8 * t;
+        v[t] = i < nb && lane <= i ? G[(k0 + i) * ld + k0 + lane] : make_double2(i == lane ? 1.0 : 0.0, 0.0);
+        y[t] = make_double2(i == lane ? 1.0 : 0.0, 0.0);
+        if (lane == 0) At[0][i] = v[t];
+        if (i == 0) Ys[0][lane] = y[t];
     }
     __syncthreads();
     for (int j = 0; j < NBS; ++j) {
-        double d = A[j][j].x;
-        const bool fail = !(d > 0.0) || !isfinite(d);
-        if (fail) {
-            d = 1.0;
-            if (tid == 0) atomicMin(&st->not_pd_pivot, (int)(k0 + j));
+        if (warp == 0) {
+            double d = At[j][j].x;
+            const bool fail = !(d > 0.0) || !isfinite(d);
+            if (fail) {
+                d = 1.0;
+                if (lane == 0) atomicMin(&st->not_pd_pivot, (int)(k0 + j));
+            }
+            const double inv = 1.0 / d;
+            const double2 a = At[j][lane];
+            S[lane] = make_double2(-a.x * inv, -a.y * inv);
+            if (lane == 0) dj[j] = d;
         }
-        const double inv = 1.0 / d;
+        __syncthreads();
 #pragma unroll
-        for (int t = 0; t < 2; ++t) {
-            if (ei[t] >= 0 && ek[t] > j) {
-                const double2 a = A[ei[t]][j];
-                double2 v = A[ei[t]][ek[t]];
-                zfma(v, make_double2(-a.x * inv, -a.y * inv), zconj(A[ek[t]][j]));
-                A[ei[t]][ek[t]] = v;
+        for (int t = 0; t < 4; ++t) {
+            const int i = warp + 8 * t;
+            if (i > j && lane <= i) {
+                const double2 s = S[i];
+                if (lane > j) {
+                    zfma(v[t], s, zconj(At[j][lane]));
+                    if (lane == j + 1) At[j + 1][i] = v[t];
+                } else {
+                    zfma(y[t], s, Ys[j][lane]);
+                }
+                if (i == j + 1) Ys[i][lane] = y[t];
             }
         }
-        if (tid == 0) rd[j] = rsqrt(d);
         __syncthreads();
     }
-    for (int e = tid; e < NBS * NBS; e += 256) {
-        const int i = e / NBS, j = e % NBS;
-        if (j > i) continue;
-        const double r = rd[j];
-        double2 v = A[i][j];
-        // the pivot d r = sqrt(d); a failed pivot counts as 1
-        v = i == j ? make_double2((v.x > 0.0 && isfinite(v.x) ? v.x : 1.0) * r, 0.0) : make_double2(v.x * r, v.y * r);
-        A[i][j] = v;
-        if (i < nb && j < nb) G[(k0 + i) * ld + k0 + j] = v;
-    }
+    if (warp == 0) rd[lane] = rsqrt(dj[lane]);
     __syncthreads();
-    const int c = tid >> 3, q = tid & 7;
-    for (int i = 0; i < NBS; ++i) {
-        double2 part = make_double2(0.0, 0.0);
-        for (int k = c + q; k < i; k += 8) zfma(part, A[i][k], X[k][c]);
 #pragma unroll
-        for (int o = 1; o < 8; o <<= 1) {
-            part.x += __shfl_xor_sync(0xffffffffu, part.x, o);
-            part.y += __shfl_xor_sync(0xffffffffu, part.y, o);
-        }
-        if (q == 0) {
-            const double r = rd[i];
-            X[i][c] = i >= c ? make_double2(((i == c ? 1.0 : 0.0) - part.x) * r, -part.y * r) : make_double2(0.0, 0.0);
-        }
-        __syncwarp();
+    for (int t = 0; t < 4; ++t) {
+        const int i = warp + 8 * t;
+        const double ri = rd[i], rc = rd[lane];
+        Dinv[i * NBS + lane] = lane <= i ? make_double2(y[t].x * ri, y[t].y * ri) : make_double2(0.0, 0.0);
+        if (i < nb && lane <= i)
+            G[(k0 + i) * ld + k0 + lane] =
+                lane == i ? make_double2(dj[i] * ri, 0.0) : make_double2(v[t].x * rc, v[t].y * rc);
     }
-    __syncthreads();
-    for (int e = tid; e < NBS * NBS; e += 256) Dinv[e] = X[e / NBS][e % NBS];
 }
 
 // 16 x 16 tiles of the panel's products, K = nbk <= 32
