@@ -6,7 +6,7 @@
 //  1. Householder reduction to a real symmetric tridiagonal T (the reflectors kept);
 //  2. the eigenvalues of T alone by bisection with Sturm counts, or with eigenvectors by
 //     divide and conquer (J. J. M. Cuppen, Numer. Math. 36, 1981): T is torn into leaves of
-//     at most 32 rows (each solved by one warp with cyclic Jacobi), and neighbours are
+//     at most 32 rows (each solved by one warp with implicit QR steps), and neighbours are
 //     merged level by level. A merge is a rank-one update D + rho z z^T: entries of z that
 //     vanish and poles that coincide are deflated, the other eigenvalues are the roots of
 //     the secular equation, each found by one warp as an offset from its nearest pole, and
@@ -177,7 +177,8 @@ __global__ void __launch_bounds__(HH_THREADS) k_hh_reduce(double2* A, int n, dou
     double2* w = hsm + n;
     double2* vn = hsm + 2 * n;  // v of this step
     const int tid = threadIdx.x, lane = tid & 31;
-    const int gw = blockIdx.x * (HH_THREADS / 32) + (tid >> 5), nw = gridDim.x * (HH_THREADS / 32);
+    // rows spread over the CTAs first: the FP64 pipes of all SMs share them
+    const int gw = (tid >> 5) * gridDim.x + blockIdx.x, nw = gridDim.x * (HH_THREADS / 32);
     double2 tau = make_double2(0.0, 0.0);
     for (int k = 0;; ++k) {
         if (k > 0) {  // w of step k - 1
@@ -406,6 +407,7 @@ __global__ void k_tridiag_bisect(const double* __restrict__ d, const double* __r
 // node t joins leaves 2 w t .. 2 w t + w - 1 with the next w. Q holds the eigenvectors of
 // the blocks formed so far (block diagonal, row-major n x n), D their eigenvalues.
 constexpr int DC_LEAF = 32;
+constexpr int DC_WARPS = 2;  // roots per CTA: few, so that the roots spread over the SMs' FP64 pipes
 constexpr double DC_EPS = 2.220446049250313e-16;
 __host__ __device__ inline int dc_bound(int i, int n, int nl) { return (int)((int64_t)i * n / nl); }
 struct DcNode {
@@ -427,109 +429,76 @@ struct DcWork {
     int* failed;
 };
 
-// The leaf's tridiagonal (its corners less |e| of the torn couplings) by cyclic Jacobi, one
-// warp: the pairs of a round are disjoint, lane l mixes row l's columns, then column l's rows.
+// The leaf's tridiagonal (its corners less |e| of the torn couplings) by the implicit QR
+// iteration with Wilkinson's shift, one warp: every lane follows the same rotations of
+// (a, b), which lane 0 stores, and lane l mixes row l of the eigenvectors.
 __global__ void __launch_bounds__(32) k_dc_leaf(const double* __restrict__ d, const double* __restrict__ e, int n,
                                                int nl, double* D, double* Q, int* failed) {
-    __shared__ double A[DC_LEAF][DC_LEAF + 1], Z[DC_LEAF][DC_LEAF + 1];
-    __shared__ double cs[DC_LEAF / 2], sn[DC_LEAF / 2];
+    __shared__ double a[DC_LEAF], b[DC_LEAF], Z[DC_LEAF][DC_LEAF + 1];
     const int lane = threadIdx.x;
-    const int lo = dc_bound(blockIdx.x, n, nl), hi = dc_bound(blockIdx.x + 1, n, nl), m = hi - lo;
-    const int mp = m + (m & 1);
-    for (int j = 0; j < m; ++j) {
-        if (lane < m) {
-            double a = 0.0;
-            if (lane == j) {
-                a = d[lo + j];
-                if (j == 0 && lo > 0) a -= fabs(e[lo - 1]);
-                if (j == m - 1 && hi < n) a -= fabs(e[hi - 1]);
-            } else if (lane == j + 1) {
-                a = e[lo + j];
-            } else if (lane == j - 1) {
-                a = e[lo + j - 1];
-            }
-            A[lane][j] = a;
-            Z[lane][j] = lane == j ? 1.0 : 0.0;
-        }
-    }
-    __syncwarp();
+    const int lo0 = dc_bound(blockIdx.x, n, nl), m = dc_bound(blockIdx.x + 1, n, nl) - lo0;
     double nrm = 0.0;
-    if (lane < m)
-        for (int j = 0; j < m; ++j) nrm = fmax(nrm, fabs(A[lane][j]));
+    if (lane < m) {
+        double x = d[lo0 + lane];
+        if (lane == 0 && lo0 > 0) x -= fabs(e[lo0 - 1]);
+        if (lane == m - 1 && lo0 + m < n) x -= fabs(e[lo0 + m - 1]);
+        a[lane] = x;
+        b[lane] = lane < m - 1 ? e[lo0 + lane] : 0.0;
+        nrm = fmax(fabs(x), fabs(b[lane]));
+        for (int j = 0; j < m; ++j) Z[lane][j] = lane == j ? 1.0 : 0.0;
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) nrm = fmax(nrm, __shfl_xor_sync(0xffffffffu, nrm, o));
-    const double tiny = nrm * (DC_EPS / 16.0);  // an off-diagonal entry below it changes no eigenvalue
-    bool again = m > 1;
-    int sweep = 0;
-    for (; again && sweep < 40; ++sweep) {
-        again = false;
-        for (int r = 0; r < mp - 1; ++r) {
-            // circle method: pair 0 is (mp - 1, r), pair k is (r + k, r - k) mod (mp - 1)
-            if (lane < mp / 2) {
-                int p = lane ? (r + lane) % (mp - 1) : r, q = lane ? (r - lane + mp - 1) % (mp - 1) : mp - 1;
-                if (p > q) {
-                    const int t = p;
-                    p = q;
-                    q = t;
-                }
-                double c = 1.0, s = 0.0;
-                if (q < m) {
-                    const double b = A[p][q];
-                    if (fabs(b) > tiny) {
-                        const double th = (A[q][q] - A[p][p]) / (2.0 * b);
-                        const double t = fabs(th) > 1e150 ? 0.5 / th
-                                                          : (th >= 0.0 ? 1.0 : -1.0) / (fabs(th) + sqrt(1.0 + th * th));
-                        c = 1.0 / sqrt(1.0 + t * t);
-                        s = c * t;
-                    }
-                }
-                cs[lane] = c;
-                sn[lane] = s;
-            }
-            __syncwarp();
-            bool any = false;
-            for (int k = 0; k < mp / 2; ++k) {
-                const double c = cs[k], s = sn[k];
-                if (s == 0.0) continue;
-                any = true;
-                int p = k ? (r + k) % (mp - 1) : r, q = k ? (r - k + mp - 1) % (mp - 1) : mp - 1;
-                if (p > q) {
-                    const int t = p;
-                    p = q;
-                    q = t;
-                }
-                if (lane < m) {
-                    const double x = A[lane][p], y = A[lane][q], u = Z[lane][p], v = Z[lane][q];
-                    A[lane][p] = c * x - s * y;
-                    A[lane][q] = s * x + c * y;
-                    Z[lane][p] = c * u - s * v;
-                    Z[lane][q] = s * u + c * v;
-                }
-            }
-            __syncwarp();
-            for (int k = 0; k < mp / 2; ++k) {
-                const double c = cs[k], s = sn[k];
-                if (s == 0.0) continue;
-                int p = k ? (r + k) % (mp - 1) : r, q = k ? (r - k + mp - 1) % (mp - 1) : mp - 1;
-                if (p > q) {
-                    const int t = p;
-                    p = q;
-                    q = t;
-                }
-                if (lane < m) {
-                    const double x = A[p][lane], y = A[q][lane];
-                    A[p][lane] = c * x - s * y;
-                    A[q][lane] = s * x + c * y;
-                }
-            }
-            __syncwarp();
-            again = again || any;
+    __syncwarp();
+    const double tiny = nrm * (DC_EPS / 16.0);  // a coupling below it changes no eigenvalue
+    auto negligible = [&](int k) { return fabs(b[k]) <= tiny || fabs(b[k]) <= 0.5 * DC_EPS * (fabs(a[k]) + fabs(a[k + 1])); };
+    int hi = m - 1, it = 0;
+    bool ok = true;
+    while (hi > 0 && ok) {
+        if (negligible(hi - 1)) {
+            --hi;
+            it = 0;
+            continue;
         }
+        if (++it > 60) {
+            ok = false;
+            break;
+        }
+        int lo = hi - 1;
+        while (lo > 0 && !negligible(lo - 1)) --lo;
+        const double h = 0.5 * (a[hi - 1] - a[hi]), t = b[hi - 1];
+        const double mu = a[hi] - t * t / (h + copysign(sqrt(h * h + t * t), h));
+        double ak = a[lo], bk = b[lo], x = ak - mu, z = bk;
+        for (int k = lo; k < hi; ++k) {
+            const double an = a[k + 1], bn = k < hi - 1 ? b[k + 1] : 0.0;
+            __syncwarp();  // every lane has read before lane 0 writes
+            // [c s; -s c]^T (x, z) = (r, 0)
+            const double q = x * x + z * z;
+            const double ri = q > 0.0 ? rsqrt(q) : 0.0;
+            const double c = q > 0.0 ? x * ri : 1.0, sn = -z * ri;
+            const double dk = ak - an, zz = (2.0 * c * bk + dk * sn) * sn;
+            x = dk * c * sn + (c * c - sn * sn) * bk;
+            if (lane == 0) {
+                if (k > lo) b[k - 1] = q * ri;
+                a[k] = ak - zz;
+                b[k] = x;
+                if (k == hi - 1) a[hi] = an + zz;
+            }
+            ak = an + zz;  // of k + 1, before its rotation
+            z = -sn * bn;
+            bk = c * bn;
+            if (lane < m) {
+                const double u = Z[lane][k], w = Z[lane][k + 1];
+                Z[lane][k] = c * u - sn * w;
+                Z[lane][k + 1] = sn * u + c * w;
+            }
+        }
+        __syncwarp();
     }
-    if (again && lane == 0) atomicExch(failed, 1);
+    if (!ok && lane == 0) atomicExch(failed, 1);
     if (lane < m) {
-        D[lo + lane] = A[lane][lane];
-        for (int j = 0; j < m; ++j) Q[(size_t)(lo + lane) * n + lo + j] = Z[lane][j];
+        D[lo0 + lane] = a[lane];
+        for (int j = 0; j < m; ++j) Q[(size_t)(lo0 + lane) * n + lo0 + j] = Z[lane][j];
     }
 }
 
@@ -590,9 +559,11 @@ __global__ void __launch_bounds__(512) k_dc_setup(const double* __restrict__ D, 
             pj = j;
             continue;
         }
-        const double gap = ds[j] - ds[pj], tau = hypot(zs[j], zs[pj]);
-        const double c = zs[j] / tau, s = zs[pj] / tau;
-        if (fabs(gap * c * s) <= tol) {
+        // gap c s with c = z_j / tau, s = z_pj / tau, tau^2 = z_j^2 + z_pj^2 (no root or division
+        // where nothing deflates: this scan is one thread's)
+        const double zj = zs[j], zp = zs[pj], tau2 = zj * zj + zp * zp;
+        if (fabs((ds[j] - ds[pj]) * zj * zp) <= tol * tau2) {
+            const double tau = sqrt(tau2), c = zj / tau, s = zp / tau;
             // columns (pj, j) <- (c pj - s j, s pj + c j)
             k.rcol[nd.lo + nr] = make_int2(pm[pj], pm[j]);
             k.rc[nd.lo + nr] = c;
@@ -640,9 +611,9 @@ __device__ inline double warp_sum_d(double v) {
 // midpoint tells). Each step fits psi and phi (the sums left and right of the root) by
 // one pole each with their values and slopes matched, and falls back to shrinking the
 // bracket, so it always ends; it stops when the sum is rounding, or the bracket a last place.
-__global__ void __launch_bounds__(256) k_dc_secular(int n, int nl, int wd, DcWork k, double* Dn) {
+__global__ void __launch_bounds__(32 * DC_WARPS) k_dc_secular(int n, int nl, int wd, DcWork k, double* Dn) {
     const DcNode nd = dc_node(blockIdx.y, wd, n, nl);
-    const int K = k.K[blockIdx.y], i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const int K = k.K[blockIdx.y], i = blockIdx.x * DC_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (i >= K) return;
     const double rho = k.rho[blockIdx.y];
     const double* d = k.kd + nd.lo;
@@ -719,9 +690,9 @@ __global__ void __launch_bounds__(256) k_dc_secular(int n, int nl, int wd, DcWor
 }
 
 // z_j^2 = prod_k (lambda_k - d_j) / (the poles other than d_j, and rho), with z's sign; one warp per j
-__global__ void __launch_bounds__(256) k_dc_zhat(int n, int nl, int wd, DcWork k) {
+__global__ void __launch_bounds__(32 * DC_WARPS) k_dc_zhat(int n, int nl, int wd, DcWork k) {
     const DcNode nd = dc_node(blockIdx.y, wd, n, nl);
-    const int K = k.K[blockIdx.y], j = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const int K = k.K[blockIdx.y], j = blockIdx.x * DC_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (j >= K) return;
     const double* d = k.kd + nd.lo;
     const double dj = d[j];
@@ -738,9 +709,9 @@ __global__ void __launch_bounds__(256) k_dc_zhat(int n, int nl, int wd, DcWork k
 
 // U[lo + i][lo + j] = z_j / (d_j - lambda_i), normalised: eigenvector i of D + rho z z^T in
 // row i; one warp per eigenvector
-__global__ void __launch_bounds__(256) k_dc_vectors(int n, int nl, int wd, DcWork k, double* U) {
+__global__ void __launch_bounds__(32 * DC_WARPS) k_dc_vectors(int n, int nl, int wd, DcWork k, double* U) {
     const DcNode nd = dc_node(blockIdx.y, wd, n, nl);
-    const int K = k.K[blockIdx.y], i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const int K = k.K[blockIdx.y], i = blockIdx.x * DC_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (i >= K) return;
     const double* d = k.kd + nd.lo;
     const double base = d[k.org[nd.lo + i]], mu = k.mu[nd.lo + i];
@@ -906,8 +877,8 @@ extern "C" pinv_status pinv_plan_eig(pinv_plan* p, double* d_mu, void* d_P, int*
         CKE(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         CKE(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_hh_reduce, HH_THREADS, smem));
         if (per < 1) return done(set_error(PINV_ERR_INTERNAL, "the reduction does not fit an SM"));
-        // a warp per row of the first columns, at most one CTA per SM
-        const unsigned grid = std::max(1u, std::min((unsigned)sms, blocks(n, HH_THREADS / 32)));
+        // at least two rows a CTA, at most one CTA per SM
+        const unsigned grid = std::max(1u, std::min((unsigned)sms, blocks(n, 2)));
         int nv = n;
         GridBar* gb = &fl->bar;
         void* args[] = {&A, &nv, &V, &taus, &dd, &ee, &ph, &pb, &gb};
@@ -975,12 +946,12 @@ extern "C" pinv_status pinv_plan_eig(pinv_plan* p, double* d_mu, void* d_P, int*
                 for (unsigned t = 0; t < nodes; ++t)
                     mm = std::max(mm, dc_bound(2 * wd * (int)(t + 1), n, nl) - dc_bound(2 * wd * (int)t, n, nl));
                 const size_t sm = (2 * sizeof(double) + sizeof(int)) * (size_t)mm;
-                const dim3 wg(blocks(mm, 8), nodes);
+                const dim3 wg(blocks(mm, DC_WARPS), nodes);
                 k_dc_setup<<<nodes, 512, sm, s>>>(D, ee, Q, n, nl, wd, w);
                 k_dc_rotate<<<dim3(blocks(mm, 128), nodes), 128, 0, s>>>(Q, n, nl, wd, w);
-                k_dc_secular<<<wg, 256, 0, s>>>(n, nl, wd, w, Dn);
-                k_dc_zhat<<<wg, 256, 0, s>>>(n, nl, wd, w);
-                k_dc_vectors<<<wg, 256, 0, s>>>(n, nl, wd, w, U);
+                k_dc_secular<<<wg, 32 * DC_WARPS, 0, s>>>(n, nl, wd, w, Dn);
+                k_dc_zhat<<<wg, 32 * DC_WARPS, 0, s>>>(n, nl, wd, w);
+                k_dc_vectors<<<wg, 32 * DC_WARPS, 0, s>>>(n, nl, wd, w, U);
                 k_dc_update<<<dim3(blocks(mm, 32), blocks(mm, 32), nodes), 256, 0, s>>>(Q, U, n, nl, wd, w, Qn, Dn);
                 note_launch(6);
                 CKE(cudaGetLastError());
@@ -989,8 +960,10 @@ extern "C" pinv_status pinv_plan_eig(pinv_plan* p, double* d_mu, void* d_P, int*
             }
         }
         k_dc_order<<<blocks(n, 128), 128, 0, s>>>(D, n, p->lambda_abs, d_mu, order);
-        // a warp per column, as many warps as hold their column in shared memory
-        const int wpb = (int)std::max<int64_t>(1, std::min<int64_t>(8, (int64_t)(200 << 10) / (16 * (int64_t)n)));
+        // a warp per column: two CTAs per SM before more warps per CTA, and as many as hold
+        // their columns in shared memory
+        const int64_t fit = (int64_t)(200 << 10) / (16 * (int64_t)n), want = (n + 303) / 304;
+        const int wpb = (int)std::max<int64_t>(1, std::min<int64_t>(8, std::min(fit, want)));
         const size_t bsm = sizeof(double2) * (size_t)n * wpb;
         CKE(cudaFuncSetAttribute(k_hh_back, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bsm));
         k_hh_back<<<blocks(n, wpb), wpb * 32, bsm, s>>>(V, taus, ph, Q, n, order, (double2*)d_P);
@@ -1002,7 +975,7 @@ extern "C" pinv_status pinv_plan_eig(pinv_plan* p, double* d_mu, void* d_P, int*
     CKE(cudaStreamSynchronize(s));
     if (sweeps_out) *sweeps_out = d_P ? levels + 1 : 0;
     if (hf.bar.failed) return done(set_error(PINV_ERR_TIMEOUT, "a bounded device wait gave up (tridiagonal reduction)"));
-    if (hf.leaf_failed) return done(set_error(PINV_ERR_INTERNAL, "a leaf's Jacobi sweeps did not converge"));
+    if (hf.leaf_failed) return done(set_error(PINV_ERR_INTERNAL, "a leaf's QR iteration did not converge"));
 #undef CKE
     return done(PINV_OK);
 }
