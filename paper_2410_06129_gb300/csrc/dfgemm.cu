@@ -455,17 +455,19 @@ __device__ inline float4 df_norm(float4 a) {  // renormalise both (hi, lo) pairs
 }
 }  // namespace
 
-// 1 / sqrt(d) for a positive double-float d: FP32 estimate and one Newton
-// step in double-float (error about the square of the estimate's, ~2^-44)
+// 1 / sqrt(d) for a positive double-float d: FP32 estimate r and the first two terms
+// of (1 - u)^(-1/2), u = 1 - d r^2: r + r u (1/2 + 3/8 u). The residual cancels, so
+// FP32 holds it: r^2 as an exact pair, d r^2 by FMA. These operations are on the
+// serial chain of the Cholesky.
 __device__ inline float2 df_rsqrt(float dh, float dl) {
     const float r0 = rsqrtf(dh);
-    float sh, sl, th, tl, uh, ul;
-    df_mul(r0, 0.f, r0, 0.f, sh, sl);          // r0^2
-    df_mul(dh, dl, sh, sl, th, tl);            // d r0^2
-    df_add(1.f, 0.f, -th, -tl, uh, ul);        // 1 - d r0^2
-    df_mul(uh, ul, 0.5f * r0, 0.f, th, tl);    // r0 (1 - d r0^2) / 2
-    df_add(r0, 0.f, th, tl, uh, ul);
-    return make_float2(uh, ul);
+    const float sh = r0 * r0, sl = fmaf(r0, r0, -sh);
+    float u = fmaf(-dh, sh, 1.f);
+    u = fmaf(-dh, sl, u);
+    u = fmaf(-dl, sh, u);
+    float h, l;
+    fast_two_sum(r0, r0 * u * fmaf(0.375f, u, 0.5f), h, l);
+    return make_float2(h, l);
 }
 
 // Column sweep over the 64 x 64 block, factor and inverse together (both
@@ -566,45 +568,51 @@ __global__ void __launch_bounds__(DIAG_THREADS) k_potrf_diag_df(float4* G, int64
     }
 }
 
-// The same block on a cluster of two CTAs with a one-column lookahead: rank 0
-// factors, rank 1 forms the inverse X = L^-1 behind it. Each rank splits its
-// 32 warps: the first two finish the next column (rank 0) or row (rank 1), the
-// critical path; the next 28 apply the current column's term to everything
-// beyond it, each thread to the two or three entries it keeps in registers;
-// on rank 0 the last two warps take turns to raise rank 1's flags after the
-// barriers (a release at cluster scope takes about 450 cycles, which the
-// barrier would otherwise wait for). One block barrier per column.
+// The same block on a cluster of three CTAs, four columns (a panel) at a time: rank
+// 0 factors, ranks 1 and 2 form the even and the odd columns of the inverse X =
+// L^-1 behind it. All keep the entries beyond the current panel in registers.
 //
-// Rank 0, step j (columns 0..j of L final, column j + 1 holding the terms of
-// columns 0..j-1): every thread i of the first two warps forms the pivot
-// d = A_{j+1,j+1} - |L_{j+1,j}|^2 and r = 1 / sqrt(d) (the same value in each,
-// so no barrier), and thread i > j + 1 finishes its entry of column j + 1,
-// L_{i,j+1} = r (A_{i,j+1} - L_ij conj(L_{j+1,j})), and stores it also into rank
-// 1's shared memory (posted remote stores; thread j + 1 stores r). Meanwhile
-// the other warps subtract column j's term from the entries (i, c), c >= j + 2,
-// and store an entry to shared memory after its last such term (c = j + 2),
-// where step c - 1 reads it. After the barrier one of the last two warps raises
-// a flag in rank 1 (release at cluster scope): columns 0..j+1 have arrived.
+// Rank 0, panel b (columns b..b+3; the columns before it are final):
+//  (a) the owners of the panel's entries apply the previous panel's four terms and
+//      put them into shared memory; barrier among all warps but the publisher;
+//  (b) two warps (three for the first panel) factor the panel: lanes 0-3 of each
+//      hold its pivot rows, the other 28 one row below it each, four entries to a
+//      lane. Column by column the pivot goes round by shuffle, every lane forms
+//      r = 1 / sqrt(pivot) and scales its entry, and the pivot rows' entries go
+//      round by shuffle for the update of the panel's later columns. Meanwhile the
+//      update warps apply the previous panel's four terms to everything beyond
+//      this panel, and the publisher's warp copies the previous panel into ranks
+//      1 and 2 (remote stores, then a flag there with release at cluster scope:
+//      about 450 cycles that the barriers would otherwise wait for). Block barrier.
 //
-// Rank 1, step j (rows 0..j of X final): thread c <= j + 1 of the first two
-// warps waits for column j + 1 (acquire; bounded, about 2 s, past the limit it
-// records timeout site DIAG_SITE and the rank stops, still meeting rank 0 at the
-// final cluster barrier) and forms X_{j+1,c} = r_{j+1} (Y_{j+1,c} - L_{j+1,j}
-// X_jc), Y = I minus the terms applied so far; the other warps subtract row j's
-// term from the rows below row j + 1, Y_ic -= L_ij X_jc.
+// Ranks 1 and 2, panel b (rows b..b+3 of X, half the columns): (a) the owners of
+// the four rows' entries left of the panel apply the previous four rows' terms;
+// (b) the first warp waits for the panel of L (acquire; bounded, about 2 s, past
+// the limit it records timeout site DIAG_SITE and the rank stops, still meeting
+// the others at the final cluster barrier) and each lane substitutes down its
+// column of the four rows, Y_ic -= L_ik X_kc, X_ic = r_i Y_ic; the other warps
+// apply the previous four rows' terms to the rows below and write the finished
+// rows of X, and rank 2 the panel of L, to global memory.
 //
 // Every entry takes the same operations in the same order as in the one-CTA
 // sweep above (right-looking, one term per column, renormalised after each),
-// only spread differently over threads.
+// only spread differently over threads. The block is a serial chain: with one
+// column at a time, on two CTAs (a barrier, a trip through shared memory and a
+// square root for each column), it took 49 us; with panels of four, set-up
+// and stores beside the chain and the inverse on two CTAs it takes 33 us,
+// of which the 16 panels' chains are about 12, the trailing updates that do not
+// hide behind them 10 and launch, load and cluster set-up 7.
 constexpr int DIAG_SITE = 20;
 constexpr long long DIAG_WAIT_LIMIT = 4000000000LL;
-constexpr int DCW = 64;                          // critical threads: the first two warps
-constexpr int DUT = DIAG_THREADS - DCW - 64;     // update threads: the next 28 warps (896)
-constexpr int DSIG = DIAG_THREADS - 64;          // rank 0: flag raisers, DSIG (even counts), DSIG + 32 (odd)
-constexpr int DUE = 3;                           // entries per update thread
-constexpr int DNE = (NBD - 2) * (NBD - 1) / 2;   // 1953 entries updated off the critical path
-static_assert(DNE <= DUE * DUT, "update entries per thread");
-// A (rank 0) or X (rank 1); Lb[j][i] = L_ij and r_j received by rank 1; L_jj on rank 0
+constexpr int DPW = 4;                                   // panel width
+constexpr int DUE = 2;                                   // rank 0: entries per update thread
+constexpr int DU0 = 96;                                  // rank 0: first update thread (29 update warps)
+constexpr int DU1 = 64;                                  // ranks 1, 2: first update thread (30 update warps)
+constexpr int DNE0 = (NBD - DPW) * (NBD - DPW + 1) / 2;  // 1830 entries (i, c), DPW <= c <= i
+constexpr int DNE1 = NBD * (NBD - DPW) / 4;              // 960 entries left of their row's panel, a rank's columns
+constexpr int DIS = DPW * NBD / 2;                       // threads that write a panel of X: the last DIS
+static_assert(DNE0 <= DUE * (DIAG_THREADS - DU0) && DNE1 <= DIAG_THREADS - DU1, "update entries per thread");
+// A (rank 0) or X (ranks 1, 2); Lb[j][i] = L_ij as received; r_j; L_jj on rank 0
 constexpr size_t DIAG2_SMEM = (size_t)(NBD * NBDP + NBD * NBD) * sizeof(float4) + 2 * NBD * sizeof(float2);
 
 __device__ inline void st_release_cluster(unsigned* p, unsigned v) {
@@ -615,16 +623,12 @@ __device__ inline unsigned ld_acquire_cluster(const unsigned* p) {
     asm volatile("ld.acquire.cluster.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
-// rank 1: wait until rank 0 has published `need` columns (the larger of the two
-// flags; `seen` keeps the count this thread has acquired, so most steps need no
-// load); false on timeout
-__device__ inline bool diag_wait(const unsigned* flag, unsigned need, unsigned& seen, DevStatus* st) {
-    if (seen >= need) return true;
+// ranks 1, 2: wait until rank 0 has published `need` panels; false on timeout
+__device__ inline bool diag_wait(const unsigned* flag, unsigned need, DevStatus* st) {
+    if (ld_acquire_cluster(flag) >= need) return true;
     const long long t0 = clock64();
     for (;;) {
-        const unsigned a = ld_acquire_cluster(flag), b = ld_acquire_cluster(flag + 1);
-        seen = a > b ? a : b;
-        if (seen >= need) return true;
+        if (ld_acquire_cluster(flag) >= need) return true;
         if (clock64() - t0 > DIAG_WAIT_LIMIT) {
             atomicMax(&st->timeout_site, DIAG_SITE);
             return false;
@@ -639,29 +643,146 @@ __device__ inline void tri_index(int e, int& r, int& q) {
     q = e - r * (r + 1) / 2;
 }
 __device__ inline float4 cdf_neg(float4 a) { return make_float4(-a.x, -a.y, -a.z, -a.w); }
+__device__ inline float4 shfl4(float4 v, int src) {
+    return make_float4(__shfl_sync(~0u, v.x, src), __shfl_sync(~0u, v.y, src), __shfl_sync(~0u, v.z, src),
+                       __shfl_sync(~0u, v.w, src));
+}
+template <int ID, int COUNT>
+__device__ inline void bar_named() {
+    asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(COUNT) : "memory");
+}
 
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(DIAG_THREADS)
+// rank 0, threads of the first two warps (three if b = 0): factor the panel of columns b..b+3
+__device__ inline void diag_panel(float4* A, float2* Ld, float2* rb, int b, int64_t k0, DevStatus* st) {
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const bool pivot = lane < DPW;
+    const int i = pivot ? b + lane : b + 28 * w + lane;
+    const bool row = i < NBD;
+    float4 v[DPW];
+#pragma unroll
+    for (int t = 0; t < DPW; ++t) v[t] = row ? A[i * NBDP + b + t] : make_float4(0.f, 0.f, 0.f, 0.f);
+    if (b)  // every warp has its copy of the pivot rows before the first one overwrites them
+        bar_named<2, 64>();
+    else
+        bar_named<2, 96>();
+#pragma unroll
+    for (int t = 0; t < DPW; ++t) {
+        float dh = __shfl_sync(~0u, v[t].x, t), dl = __shfl_sync(~0u, v[t].y, t);
+        const bool fail = !(dh > 0.f) || !isfinite(dh);  // a normalised pair has the sign of dh
+        if (fail) {
+            dh = 1.f;
+            dl = 0.f;
+        }
+        const float2 r = df_rsqrt(dh, dl);
+        const float4 l = df_scale(v[t], r.x, r.y);
+#pragma unroll
+        for (int q = t + 1; q < DPW; ++q) {  // above the diagonal (lanes q' < q) unused values
+            cacc(v[q], cdf_neg(l), cdf_conj(shfl4(l, q)));
+            v[q] = df_norm(v[q]);
+        }
+        if (row && (!pivot || (w == 0 && lane > t))) {
+            A[i * NBDP + b + t] = l;
+        }
+        if (w == 0 && lane == t) {
+            if (fail) atomicMin(&st->not_pd_pivot, (int)(k0 + b + t));
+            float lh, ll;
+            df_mul(dh, dl, r.x, r.y, lh, ll);  // L_jj = d / sqrt(d)
+            Ld[b + t] = make_float2(lh, ll);
+            rb[b + t] = r;
+        }
+    }
+}
+
+// rank 0, one warp: columns b..b+3 of L below the diagonal, their r and L_jj to the shared
+// memory of ranks 1 and 2, then their flags
+__device__ inline void diag_publish(const float4* A, const float2* rb, int b, float4* Lb1, float4* Lb2, float2* rb1,
+                                    float2* rb2, unsigned* flag1, unsigned* flag2) {
+    const int lane = threadIdx.x & 31;
+    for (int i = b + 1 + lane; i < NBD; i += 32) {
+        float4 v[DPW];
+#pragma unroll
+        for (int t = 0; t < DPW; ++t) v[t] = A[i * NBDP + b + t];
+#pragma unroll
+        for (int t = 0; t < DPW; ++t) {  // on and above the diagonal: not read
+            Lb1[(b + t) * NBD + i] = v[t];
+            Lb2[(b + t) * NBD + i] = v[t];
+        }
+    }
+    if (lane < 2 * DPW) {
+        const int e = (lane & (DPW - 1)) + b + (lane < DPW ? 0 : NBD);  // r, then L_jj
+        const float2 r = rb[e];
+        rb1[e] = r;
+        rb2[e] = r;
+    }
+    __syncwarp();
+    if (lane < 2) st_release_cluster(lane == 0 ? flag1 : flag2, (unsigned)(b / DPW + 1));
+}
+// rank 2, 256 threads (e): columns b..b+3 of L as received, to G and L32
+__device__ inline void diag_store(const float4* Lb, const float2* Ld, int b, int e, int nb, float4* G, int64_t ld,
+                                  float2* L32, int64_t ldl) {
+    const int i = e / DPW, j = b + e % DPW;
+    if (i >= nb || j > i) return;
+    const float4 a = i == j ? make_float4(Ld[j].x, Ld[j].y, 0.f, 0.f) : Lb[j * NBD + i];
+    G[i * ld + j] = a;
+    if (L32) L32[i * ldl + j] = df_to_f32(a);
+}
+// ranks 1, 2, the last DIS threads: the rank's columns of rows b..b+3 of X, one entry each
+__device__ inline void diag_store_inv(const float4* X, int par, int b, double2* Dinv, float2* Dinv32) {
+    const int e = threadIdx.x - (DIAG_THREADS - DIS), i = b + e / (NBD / 2), j = 2 * (e % (NBD / 2)) + par;
+    if (j > i) return;
+    const float4 x = X[i * NBDP + j];
+    if (Dinv) Dinv[i * NBD + j] = make_double2(join_f64(x.x, x.y), join_f64(x.z, x.w));
+    if (Dinv32) Dinv32[i * NBD + j] = make_float2(x.x + x.y, x.z + x.w);
+}
+
+__global__ void __cluster_dims__(3, 1, 1) __launch_bounds__(DIAG_THREADS)
     k_potrf_diag_df2(float4* G, int64_t ld, int64_t N, int64_t k0, double2* Dinv, float2* Dinv32, float2* L32,
                      int64_t ldl, DevStatus* st) {
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
     extern __shared__ float4 smd[];
-    float4* A = smd;                                        // rank 0: the block, then L; rank 1: Y, then X
-    float4* Lb = smd + NBD * NBDP;                          // rank 1: Lb[j][i] = L_ij
-    float2* rb = reinterpret_cast<float2*>(Lb + NBD * NBD);  // rank 1: r_j
-    float2* Ld = rb + NBD;                                  // rank 0: L_jj
-    __shared__ unsigned flag[2];  // rank 1: columns of L published by rank 0 (even, odd counts)
+    float4* A = smd;                                        // rank 0: the block, then L; others: Y, then X
+    float4* Lb = smd + NBD * NBDP;                          // others: Lb[j][i] = L_ij
+    float2* rb = reinterpret_cast<float2*>(Lb + NBD * NBD);  // r_j
+    float2* Ld = rb + NBD;                                  // L_jj
+    __shared__ unsigned flag;  // ranks 1, 2: panels of L published by rank 0
     __shared__ int stop;
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, wid = tid >> 5;
     const unsigned rank = cl.block_rank();
+    const int par = (int)rank - 1;  // ranks 1, 2: columns 2 n + par of X
     const int nb = (int)((N - k0) < NBD ? (N - k0) : NBD);
-    griddep_wait();    // the block's updates have landed
-    griddep_launch();  // the next kernel's CTAs may take their SMs and wait for this one
     if (tid == 0) {
-        flag[0] = flag[1] = 0;
+        flag = 0;
         stop = 0;
     }
-    {  // the block's lower triangle (rank 0) or I (rank 1); all loads issued before the stores
+    // the entries this thread keeps: rank 0 (i, c), 4 <= c <= i, numbered from the last
+    // column, so a panel's entries lie on neighbouring warps; ranks 1, 2 one entry (i, c),
+    // c left of row i's panel, numbered by panel of rows and there by column
+    int ui[DUE], uc[DUE];
+#pragma unroll
+    for (int k = 0; k < DUE; ++k) {
+        ui[k] = uc[k] = -1;
+        if (rank == 0) {
+            const int e = tid - DU0 + k * (DIAG_THREADS - DU0);
+            if (tid >= DU0 && e < DNE0) {
+                int r, q;
+                tri_index(e, r, q);
+                uc[k] = NBD - 1 - r;
+                ui[k] = uc[k] + q;
+            }
+        } else if (k == 0 && tid >= DU1) {
+            const int e = tid - DU1;  // < DNE1; panel p = r + 1 holds entries 4 p (p - 1) .. 4 p (p + 1) - 1
+            int r, q;
+            tri_index(e / 8, r, q);
+            q = e - 4 * r * (r + 1);
+            ui[k] = DPW * (r + 1) + (q & 3);
+            uc[k] = 2 * (q >> 2) + par;
+        }
+    }
+    cl.sync();         // the flags are zero before rank 0 may raise it
+    griddep_wait();    // the block's updates have landed
+    griddep_launch();  // the next kernel's CTAs may take their SMs and wait for this one
+    {  // the block's lower triangle (rank 0) or I; all loads issued before the stores
         constexpr int PER = NBD * NBD / DIAG_THREADS;
         float4 g[PER];
 #pragma unroll
@@ -674,167 +795,119 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(DIAG_THREADS)
         for (int t = 0; t < PER; ++t) {
             const int e = tid + t * DIAG_THREADS, i = e / NBD, j = e % NBD;
             A[i * NBDP + j] = g[t];
-        }
-    }
-    // the entries this thread updates off the critical path; rank 0: (i, c), 2 <= c <= i,
-    // numbered from the last column; rank 1: (i, c), c <= i - 2, numbered by row from row 2
-    const int u = tid - DCW;
-    int ui[DUE], uc[DUE];
-#pragma unroll
-    for (int k = 0; k < DUE; ++k) {
-        const int e = u + k * DUT;
-        ui[k] = -1;
-        uc[k] = -1;
-        if (u >= 0 && u < DUT && e < DNE) {
-            int r, q;
-            tri_index(e, r, q);
+            // above the diagonal: zeros
             if (rank == 0) {
-                uc[k] = NBD - 1 - r;
-                ui[k] = uc[k] + q;
-            } else {
-                ui[k] = r + 2;
-                uc[k] = q;
+                if (j > i && L32 && i < nb && j < nb) L32[(k0 + i) * ldl + k0 + j] = make_float2(0.f, 0.f);
+            } else if (rank == 1 && j > i) {
+                if (Dinv) Dinv[e] = make_double2(0.0, 0.0);
+                if (Dinv32) Dinv32[e] = make_float2(0.f, 0.f);
             }
         }
     }
-    cl.sync();  // the blocks are loaded and rank 1's flag is zero before rank 0 may raise it
+    __syncthreads();
     float4 uv[DUE];
 #pragma unroll
     for (int k = 0; k < DUE; ++k) uv[k] = ui[k] >= 0 ? A[ui[k] * NBDP + uc[k]] : make_float4(0.f, 0.f, 0.f, 0.f);
     if (rank == 0) {
-        unsigned* rflag = cl.map_shared_rank(flag, 1);
-        float4* rLb = cl.map_shared_rank(Lb, 1);
-        float2* rrb = cl.map_shared_rank(rb, 1);
-        // column 0
-        if (tid < DCW) {
-            const float4 a = A[0];
-            float dh = a.x, dl = a.y;
-            const bool fail = !(dh > 0.f) || !isfinite(dh);  // a normalised pair has the sign of dh
-            if (fail) {
-                dh = 1.f;
-                dl = 0.f;
-            }
-            const float2 r = df_rsqrt(dh, dl);
-            if (tid > 0) {
-                const float4 l = df_norm(df_scale(A[tid * NBDP], r.x, r.y));
-                A[tid * NBDP] = l;
-                rLb[tid] = l;
-            } else {
-                if (fail) atomicMin(&st->not_pd_pivot, (int)k0);
-                float lh, ll;
-                df_mul(dh, dl, r.x, r.y, lh, ll);
-                Ld[0] = make_float2(lh, ll);
-                rrb[0] = r;
-            }
-        }
-        __syncthreads();
-        if (tid == DSIG + 32) st_release_cluster(rflag + 1, 1u);
-        for (int j = 0; j + 1 < NBD; ++j) {
-            if (tid < DCW) {
-                if (tid > j) {  // rows j + 1 .. 63 of column j + 1
-                    // the entry's update first: it does not wait for the pivot, and the
-                    // two chains interleave (thread j + 1's entry is the pivot itself)
-                    const float4 lj = A[(j + 1) * NBDP + j];  // L_{j+1,j}
-                    float4 v = A[tid * NBDP + j + 1];
-                    float4 dd = A[(j + 1) * NBDP + j + 1];
-                    cacc(v, cdf_neg(A[tid * NBDP + j]), cdf_conj(lj));
-                    cacc(dd, cdf_neg(lj), cdf_conj(lj));
-                    v = df_norm(v);
-                    dd = df_norm(dd);
-                    float dh = dd.x, dl = dd.y;
-                    const bool fail = !(dh > 0.f) || !isfinite(dh);
-                    if (fail) {
-                        dh = 1.f;
-                        dl = 0.f;
-                    }
-                    const float2 r = df_rsqrt(dh, dl);
-                    if (tid > j + 1) {
-                        const float4 l = df_norm(df_scale(v, r.x, r.y));
-                        A[tid * NBDP + j + 1] = l;
-                        rLb[(j + 1) * NBD + tid] = l;
-                    } else {
-                        if (fail) atomicMin(&st->not_pd_pivot, (int)(k0 + j + 1));
-                        float lh, ll;
-                        df_mul(dh, dl, r.x, r.y, lh, ll);
-                        Ld[j + 1] = make_float2(lh, ll);
-                        rrb[j + 1] = r;
-                    }
-                }
-            } else {
+        unsigned *flag1 = cl.map_shared_rank(&flag, 1), *flag2 = cl.map_shared_rank(&flag, 2);
+        float4 *Lb1 = cl.map_shared_rank(Lb, 1), *Lb2 = cl.map_shared_rank(Lb, 2);
+        float2 *rb1 = cl.map_shared_rank(rb, 1), *rb2 = cl.map_shared_rank(rb, 2);
+        for (int b = 0; b < NBD; b += DPW) {
+            if (b > 0 && wid == 2) {
+                diag_publish(A, rb, b - DPW, Lb1, Lb2, rb1, rb2, flag1, flag2);
+            } else if (wid < 3) {
+                if (b > 0) bar_named<1, DIAG_THREADS - 32>();
+                diag_panel(A, Ld, rb, b, k0, st);
+            } else if (b > 0) {
 #pragma unroll
                 for (int k = 0; k < DUE; ++k) {
-                    if (uc[k] >= j + 2) {
-                        cacc(uv[k], cdf_neg(A[ui[k] * NBDP + j]), cdf_conj(A[uc[k] * NBDP + j]));
-                        uv[k] = df_norm(uv[k]);
-                        if (uc[k] == j + 2) A[ui[k] * NBDP + uc[k]] = uv[k];
+                    if (uc[k] >= b && uc[k] < b + DPW) {
+#pragma unroll
+                        for (int t = b - DPW; t < b; ++t) {
+                            cacc(uv[k], cdf_neg(A[ui[k] * NBDP + t]), cdf_conj(A[uc[k] * NBDP + t]));
+                            uv[k] = df_norm(uv[k]);
+                        }
+                        A[ui[k] * NBDP + uc[k]] = uv[k];
+                    }
+                }
+                bar_named<1, DIAG_THREADS - 32>();
+#pragma unroll
+                for (int k = 0; k < DUE; ++k) {
+                    if (uc[k] >= b + DPW) {
+#pragma unroll
+                        for (int t = b - DPW; t < b; ++t) {
+                            cacc(uv[k], cdf_neg(A[ui[k] * NBDP + t]), cdf_conj(A[uc[k] * NBDP + t]));
+                            uv[k] = df_norm(uv[k]);
+                        }
                     }
                 }
             }
             __syncthreads();
-            // columns 0..j+1; each raiser has two steps for its release
-            if (tid == DSIG + 32 * (j & 1)) st_release_cluster(rflag + (j & 1), (unsigned)(j + 2));
         }
-        for (int e = tid; e < NBD * NBD; e += DIAG_THREADS) {
-            const int i = e / NBD, j = e % NBD;
-            if (i < nb && j < nb && j <= i) {
-                const float4 a = i == j ? make_float4(Ld[j].x, Ld[j].y, 0.f, 0.f) : A[i * NBDP + j];
-                G[(k0 + i) * ld + k0 + j] = a;
-                if (L32) L32[(k0 + i) * ldl + k0 + j] = df_to_f32(a);
-            } else if (L32 && i < nb && j < nb) {
-                L32[(k0 + i) * ldl + k0 + j] = make_float2(0.f, 0.f);
-            }
-        }
-        cl.sync();
+        if (wid == 2) diag_publish(A, rb, NBD - DPW, Lb1, Lb2, rb1, rb2, flag1, flag2);
+        cl.sync();  // no remote store after ranks 1 and 2 are gone
     } else {
         float4* X = A;
-        float4 xp = make_float4(0.f, 0.f, 0.f, 0.f);  // thread c < 64: X_jc of the current step
-        unsigned seen = 0;
-        if (tid < DCW) {
-            if (!diag_wait(flag, 1u, seen, st)) {
-                stop = 1;
-            } else if (tid == 0) {
-                const float2 r = rb[0];
-                xp = df_norm(df_scale(X[0], r.x, r.y));
-                X[0] = xp;
-            }
-        }
-        __syncthreads();
-        for (int j = 0; j + 1 < NBD; ++j) {
-            if (stop) break;  // set before the last barrier: the same in every thread
-            if (tid < DCW) {
-                if (tid <= j + 1) {  // row j + 1, columns 0 .. j + 1
-                    if (!diag_wait(flag, (unsigned)(j + 2), seen, st)) {
-                        stop = 1;
-                    } else {
-                        const float2 r = rb[j + 1];
-                        float4 y = X[(j + 1) * NBDP + tid];
-                        if (tid <= j) {
-                            cacc(y, cdf_neg(Lb[j * NBD + j + 1]), xp);
-                            y = df_norm(y);
-                        }
-                        xp = df_norm(df_scale(y, r.x, r.y));
-                        X[(j + 1) * NBDP + tid] = xp;
-                    }
-                }
-            } else {
+        const int i = ui[0], c = uc[0];
+        float4 y = uv[0];
+        float4* Gk = G + k0 * ld + k0;
+        float2* Lk = L32 ? L32 + k0 * ldl + k0 : nullptr;
+        for (int b = 0; b < NBD; b += DPW) {
+            if (wid == 0) {
+                int ok = 1;
+                if (tid == 0) ok = diag_wait(&flag, (unsigned)(b / DPW + 1), st);
+                ok = __shfl_sync(~0u, ok, 0);
+                if (b > 0) bar_named<1, DIAG_THREADS>();
+                const int cc = 2 * tid + par;
+                if (!ok) {
+                    stop = 1;
+                } else if (cc < b + DPW) {  // columns up to b + 3 of rows b .. b + 3
+                    float4 x[DPW];
 #pragma unroll
-                for (int k = 0; k < DUE; ++k) {
-                    if (uc[k] >= 0 && uc[k] <= j && ui[k] >= j + 2) {
-                        cacc(uv[k], cdf_neg(Lb[j * NBD + ui[k]]), X[j * NBDP + uc[k]]);
-                        uv[k] = df_norm(uv[k]);
-                        if (ui[k] == j + 2) X[ui[k] * NBDP + uc[k]] = uv[k];
+                    for (int t = 0; t < DPW; ++t) {
+                        float4 v = X[(b + t) * NBDP + cc];
+#pragma unroll
+                        for (int q = 0; q < t; ++q) {  // x_q = 0 for cc > b + q
+                            cacc(v, cdf_neg(Lb[(b + q) * NBD + b + t]), x[q]);
+                            v = df_norm(v);
+                        }
+                        const float2 r = rb[b + t];
+                        x[t] = df_scale(v, r.x, r.y);
+                        if (cc <= b + t) X[(b + t) * NBDP + cc] = x[t];
                     }
                 }
+            } else if (b > 0) {
+                if (i >= b && i < b + DPW) {
+#pragma unroll
+                    for (int t = b - DPW; t < b; ++t) {  // X_tc = 0 for c > t
+                        cacc(y, cdf_neg(Lb[t * NBD + i]), X[t * NBDP + c]);
+                        y = df_norm(y);
+                    }
+                    X[i * NBDP + c] = y;
+                }
+                bar_named<1, DIAG_THREADS>();
+                if (i >= b + DPW && c < b) {
+#pragma unroll
+                    for (int t = b - DPW; t < b; ++t) {
+                        cacc(y, cdf_neg(Lb[t * NBD + i]), X[t * NBDP + c]);
+                        y = df_norm(y);
+                    }
+                }
+                if (tid >= DIAG_THREADS - DIS)
+                    diag_store_inv(X, par, b - DPW, Dinv, Dinv32);
+                else if (par == 1 && tid >= DIAG_THREADS - DIS - DPW * NBD)
+                    diag_store(Lb, Ld, b - DPW, tid - (DIAG_THREADS - DIS - DPW * NBD), nb, Gk, ld, Lk, ldl);
             }
             __syncthreads();
+            if (stop) break;  // set before the barrier: the same in every thread
         }
-        cl.sync();  // rank 0 has published everything and may exit
-        for (int e = tid; e < NBD * NBD; e += DIAG_THREADS) {
-            const int i = e / NBD, j = e % NBD;
-            const float4 x = j <= i ? X[i * NBDP + j] : make_float4(0.f, 0.f, 0.f, 0.f);
-            if (Dinv) Dinv[e] = make_double2(join_f64(x.x, x.y), join_f64(x.z, x.w));
-            if (Dinv32) Dinv32[e] = make_float2(x.x + x.y, x.z + x.w);
+        if (!stop) {
+            if (tid >= DIAG_THREADS - DIS)
+                diag_store_inv(X, par, NBD - DPW, Dinv, Dinv32);
+            else if (par == 1 && tid >= DIAG_THREADS - DIS - DPW * NBD)
+                diag_store(Lb, Ld, NBD - DPW, tid - (DIAG_THREADS - DIS - DPW * NBD), nb, Gk, ld, Lk, ldl);
         }
+        cl.sync();
     }
 }
 
@@ -852,7 +925,7 @@ cudaError_t launch_potrf_diag_df(float4* G, int64_t ld, int64_t N, int64_t k0, d
             if (err != cudaSuccess) return err;
             attr2 = true;
         }
-        cudaError_t err = launch_pdl(k_potrf_diag_df2, dim3(2), dim3(DIAG_THREADS), smem2, s, G, ld, N, k0, Dinv,
+        cudaError_t err = launch_pdl(k_potrf_diag_df2, dim3(3), dim3(DIAG_THREADS), smem2, s, G, ld, N, k0, Dinv,
                                      Dinv32, L32, ldl, st);
         return err != cudaSuccess ? err : cudaGetLastError();
     }
