@@ -295,10 +295,9 @@ size_t factor_table_bytes(int64_t N, int slices);
 // ev_panel (or nullptr): one event per 256-wide panel, recorded by the Cholesky once
 // the panel's columns of L32 and its diagonal inverses are final, and waited on by
 // the inverse before that panel
-// la (or nullptr): a second stream with its own status block and two events, on
-// which all but the next panel's columns of each trailing update run (lookahead);
-// and (s2 non-null) a third stream with two events for the solves and updates inside
-// a panel beyond the next diagonal block (block lookahead)
+// la (or nullptr): streams and events of the lookahead. s, with its own status block:
+// the part of each trailing update beyond the next panel's columns; s2: the solves and
+// updates beyond what the next diagonal block needs
 struct TrailLookahead {
     cudaStream_t s;
     DevStatus* st;

@@ -602,7 +602,7 @@ struct HerkBulk {
         j0 = r0 + jt * BN;
         kb = 0;
         ke = kcn * KC;
-        return jt <= it;
+        return jt <= it && it > 0;  // the first tile is updated block by block (launch_potrf_tc)
     }
     __device__ const uint8_t* bulk_a(int64_t i0, int64_t kc, int sl) const {
         return tab + ((((i0 - r0) / BM) * kcn + kc) * S + sl) * B_SL;
@@ -668,7 +668,7 @@ struct HerkTC {
         j0 = t0 + bx * BN;
         kb = 0;
         ke = nbk;
-        return i0 < N && j0 < jmax && j0 <= i0 + BM - 1;
+        return i0 > t0 && i0 < N && j0 < jmax && j0 <= i0 + BM - 1;  // without the first tile, as HerkBulk
     }
     __device__ RowPtr row_a(int64_t i) const { return RowPtr{P + (i < N ? i : 0) * ldp, i < N}; }
     __device__ RowPtr row_b(int64_t j) const { return RowPtr{P + (j < N ? j : 0) * ldp, j < N}; }
@@ -959,11 +959,12 @@ __global__ void __launch_bounds__(256) k_trsm_panel(float2* P, int64_t ldp, cons
 }
 
 // G[i][j] -= sum_k P[i][k] conj(P[j][k]) for t0 <= j < jmax, j <= i, rows r0 <= i < N
-// (K = nbk <= 64; jmax - t0 <= 32 CB; r0 >= t0). Dynamic shared memory: herk_panel_smem(CB).
+// (jmax - t0 <= 32 CB; r0 >= t0), one term after the other for nch blocks of 64 columns
+// of P. Dynamic shared memory: herk_panel_smem(CB).
 constexpr size_t herk_panel_smem(int cb) { return sizeof(float2) * (PNL_ROWS * 64 + 64 * (32 * cb + 1)); }
 template <int CB>
 __global__ void __launch_bounds__(256) k_herk_panel(const float2* __restrict__ P, int64_t ldp, float4* G,
-                                                  int64_t ldg, int nbk, int64_t t0, int64_t jmax, int64_t r0,
+                                                  int64_t ldg, int nch, int64_t t0, int64_t jmax, int64_t r0,
                                                   int64_t N) {
     constexpr int WP = 32 * CB + 1;  // padded row of Bt: transposed stores spread over the banks
     extern __shared__ float2 pnl_smem[];
@@ -974,48 +975,65 @@ __global__ void __launch_bounds__(256) k_herk_panel(const float2* __restrict__ P
     const int64_t i0 = r0 + (int64_t)blockIdx.x * PNL_ROWS;
     griddep_wait();
     griddep_launch();
-    {
-        float2 u[4];
+    float4 g[2][CB];
+    for (int ch = 0; ch < nch; ++ch, P += 64) {
+        if (ch) __syncthreads();
+        {
+            float2 u[4];
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            const int e = tid + 256 * t, r = e / 64, k = e % 64;
-            const int64_t i = i0 + r;
-            u[t] = (i < N && k < nbk) ? P[i * ldp + k] : make_float2(0.f, 0.f);
-        }
+            for (int t = 0; t < 4; ++t) {
+                const int e = tid + 256 * t, r = e / 64, k = e % 64;
+                const int64_t i = i0 + r;
+                u[t] = i < N ? P[i * ldp + k] : make_float2(0.f, 0.f);
+            }
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            const int e = tid + 256 * t;
-            Ai[e / 64][e % 64] = u[t];
+            for (int t = 0; t < 4; ++t) {
+                const int e = tid + 256 * t;
+                Ai[e / 64][e % 64] = u[t];
+            }
         }
-    }
 #pragma unroll 1
-    for (int t0b = 0; t0b < 8 * CB; t0b += 16) {  // 8 CB loads per thread, 16 at a time
-        float2 v[16];
+        for (int t0b = 0; t0b < 8 * CB; t0b += 16) {  // 8 CB loads per thread, 16 at a time
+            float2 v[16];
 #pragma unroll
-        for (int t = 0; t < 16; ++t) {
-            const int e = tid + 256 * (t0b + t), c = e / 64, k = e % 64;
-            const int64_t j = t0 + c;
-            v[t] = (t0b + t < 8 * CB && c < W && j < N && k < nbk) ? P[j * ldp + k] : make_float2(0.f, 0.f);
+            for (int t = 0; t < 16; ++t) {
+                const int e = tid + 256 * (t0b + t), c = e / 64, k = e % 64;
+                const int64_t j = t0 + c;
+                v[t] = (t0b + t < 8 * CB && c < W && j < N) ? P[j * ldp + k] : make_float2(0.f, 0.f);
+            }
+#pragma unroll
+            for (int t = 0; t < 16; ++t) {
+                const int e = tid + 256 * (t0b + t);
+                if (t0b + t < 8 * CB) Bt[e % 64][e / 64] = v[t];
+            }
         }
+        if (ch == 0) {  // the old entries arrive while the products run
 #pragma unroll
-        for (int t = 0; t < 16; ++t) {
-            const int e = tid + 256 * (t0b + t);
-            if (t0b + t < 8 * CB) Bt[e % 64][e / 64] = v[t];
+            for (int ra = 0; ra < 2; ++ra)
+#pragma unroll
+                for (int b = 0; b < CB; ++b) {
+                    const int64_t i = i0 + w + 8 * ra, j = t0 + lane + 32 * b;
+                    g[ra][b] = (i < N && lane + 32 * b < W && j <= i) ? G[i * ldg + j] : make_float4(0.f, 0.f, 0.f, 0.f);
+                }
         }
-    }
-    __syncthreads();
-    float2 acc[2][CB];
+        __syncthreads();
+        float2 acc[2][CB];
 #pragma unroll
-    for (int b = 0; b < CB; ++b) acc[0][b] = acc[1][b] = make_float2(0.f, 0.f);
+        for (int b = 0; b < CB; ++b) acc[0][b] = acc[1][b] = make_float2(0.f, 0.f);
 #pragma unroll 4
-    for (int k = 0; k < 64; ++k) {
-        const float2 a0 = Ai[w][k], a1 = Ai[w + 8][k];
+        for (int k = 0; k < 64; ++k) {
+            const float2 a0 = Ai[w][k], a1 = Ai[w + 8][k];
 #pragma unroll
-        for (int b = 0; b < CB; ++b) {
-            const float2 bv = Bt[k][lane + 32 * b];
-            cmac_conj(acc[0][b], a0, bv);
-            cmac_conj(acc[1][b], a1, bv);
+            for (int b = 0; b < CB; ++b) {
+                const float2 bv = Bt[k][lane + 32 * b];
+                cmac_conj(acc[0][b], a0, bv);
+                cmac_conj(acc[1][b], a1, bv);
+            }
         }
+#pragma unroll
+        for (int ra = 0; ra < 2; ++ra)
+#pragma unroll
+            for (int b = 0; b < CB; ++b) g[ra][b] = df_sub_f32(g[ra][b], acc[ra][b]);
     }
 #pragma unroll
     for (int ra = 0; ra < 2; ++ra) {
@@ -1024,13 +1042,13 @@ __global__ void __launch_bounds__(256) k_herk_panel(const float2* __restrict__ P
         for (int b = 0; b < CB; ++b) {
             const int c = lane + 32 * b;
             const int64_t j = t0 + c;
-            if (i < N && c < W && j <= i) G[i * ldg + j] = df_sub_f32(G[i * ldg + j], acc[ra][b]);
+            if (i < N && c < W && j <= i) G[i * ldg + j] = g[ra][b];
         }
     }
 }
 
 template <int CB>
-static cudaError_t launch_herk_panel(const float2* P, int64_t ldp, float4* G, int64_t ldg, int nbk, int64_t t0,
+static cudaError_t launch_herk_panel(const float2* P, int64_t ldp, float4* G, int64_t ldg, int nch, int64_t t0,
                                      int64_t jmax, int64_t r0, int64_t N, cudaStream_t s) {
     static bool attr = false;
     if (!attr) {
@@ -1041,17 +1059,17 @@ static cudaError_t launch_herk_panel(const float2* P, int64_t ldp, float4* G, in
     }
     const int64_t rows = N - r0;
     cudaError_t e = launch_pdl(k_herk_panel<CB>, dim3((unsigned)((rows + PNL_ROWS - 1) / PNL_ROWS)), dim3(256),
-                               herk_panel_smem(CB), s, P, ldp, G, ldg, nbk, t0, jmax, r0, N);
+                               herk_panel_smem(CB), s, P, ldp, G, ldg, nch, t0, jmax, r0, N);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 // G[i][j] -= sum_k P[i][k] conj(P[j][k]) for columns t0 <= j < jmax (at most 192), rows r0 <= i < N
-static cudaError_t herk_panel(const float2* P, int64_t ldp, float4* G, int64_t ldg, int nbk, int64_t t0,
+static cudaError_t herk_panel(const float2* P, int64_t ldp, float4* G, int64_t ldg, int nch, int64_t t0,
                               int64_t jmax, int64_t r0, int64_t N, cudaStream_t s) {
     const int64_t w = jmax - t0;
-    return w <= 64    ? launch_herk_panel<2>(P, ldp, G, ldg, nbk, t0, jmax, r0, N, s)
-           : w <= 128 ? launch_herk_panel<4>(P, ldp, G, ldg, nbk, t0, jmax, r0, N, s)
-                      : launch_herk_panel<6>(P, ldp, G, ldg, nbk, t0, jmax, r0, N, s);
+    return w <= 64    ? launch_herk_panel<2>(P, ldp, G, ldg, nch, t0, jmax, r0, N, s)
+           : w <= 128 ? launch_herk_panel<4>(P, ldp, G, ldg, nch, t0, jmax, r0, N, s)
+                      : launch_herk_panel<6>(P, ldp, G, ldg, nch, t0, jmax, r0, N, s);
 }
 static cudaError_t trsm_panel(float2* P, int64_t ldp, const float2* Dinv32, float4* G, int64_t ldg, int64_t k0,
                               int nbk, int64_t row0, int64_t N, cudaStream_t s) {
@@ -1080,116 +1098,155 @@ static cudaError_t panel_table(const float2* L32, int64_t N, int64_t p0, int64_t
 // panel each step updates only the panel's remaining columns (K = 64); the
 // trailing matrix gets one update per panel with K = 256, so its tiles run
 // 16 tensor-core stages instead of 4 and G is read and written a quarter as
-// often. G is in double-float storage (float4 per entry) for the whole
-// factorisation, and L is left there in the same form.
+// often. The trailing matrix's first 128 x 128 tile holds the next panel's first
+// two diagonal blocks and takes its update block by block (K = 64, FP32) instead,
+// so that the next diagonal block need not wait for the panel's last solves, the
+// operand table and the tensor-core update. G is in double-float storage (float4
+// per entry) for the whole factorisation, and L is left there in the same form.
+//
+// With lookahead (streams of la) only this runs on the chain's stream: a diagonal
+// block, the solve of the next block's 64 rows and their update of that block. A
+// second stream takes, for each block, first the rows that the chain's next step
+// needs and then the rest of the panel's work; the far part of the trailing update
+// runs on a third. Every entry is computed as without the lookahead
+// (PINV_CHOL_LOOKAHEAD=0: all on the chain's stream), so the factor is the same bit
+// for bit. Where the chain waited for each panel's solves, table and update of the
+// next panel's columns, a panel of four blocks took 268 us at N = 4096; so it takes
+// 243 us: the diagonal blocks 4 x 33, their small solves and updates 4 x 13, the rest
+// waits for the second stream's work and for free SMs.
 constexpr int NBK = 64, NBP = 256;
+
+// SMs that a persistent launch beside the Cholesky chain takes (the far trailing updates;
+// the inverse's updates): the chain's small launches find the others free. Above N = 16384
+// all work is throughput-bound and each launch takes every SM. Build at 2/5 and 1/2 of
+// the SMs (updates, inverse) / 3/5 / 3/4 / all: 64 x 64 5.19 / 5.17 / 5.23 / 5.62 ms,
+// 80 x 80 11.65 / 11.26 / 11.18 / 11.91, 96 x 96 26.1 / 24.4 / 23.8 / 24.9, 128 x 128
+// 114.9 / 100.1 / 95.0 / 96.2.
+static int side_sms(int64_t N) {
+    const int n = tc::sm_count();
+    return N <= 5632 ? std::max(1, 3 * n / 5) : N <= 16384 ? std::max(1, 3 * n / 4) : 0;
+}
 
 cudaError_t launch_potrf_tc(float4* G, int64_t N, int64_t ld, double2* Dinv, float2* Dinv32, float2* L32,
                             int slices, DevStatus* st, cudaStream_t s, void* tab, const cudaEvent_t* ev_panel,
                             const TrailLookahead* la) {
-    // lookahead: after each panel only the next panel's columns (two column tiles)
-    // are updated on the chain's stream; the rest of the trailing matrix on la->s,
-    // beside the next panel's steps, and before the next panel's update
-    // (PINV_CHOL_LOOKAHEAD=0: all of it on the chain's stream). Every tile is
-    // computed the same way either way, so the factor is the same bit for bit.
     const char* lenv = std::getenv("PINV_CHOL_LOOKAHEAD");
-    const bool ahead = la && la->s && tab && !(lenv && std::strcmp(lenv, "0") == 0);
+    const bool ahead = la && la->s && la->s2 && tab && !(lenv && std::strcmp(lenv, "0") == 0);
     int cap = 0;
     if (ahead) {
         const char* cenv = std::getenv("PINV_TRAIL_SMS");
-        cap = cenv ? std::atoi(cenv) : (N <= 16384 ? std::max(1, 2 * tc::sm_count() / 5) : 0);
+        cap = cenv ? std::atoi(cenv) : side_sms(N);
     }
-    bool pending = false;  // a side update of the previous panel may still run
-    // block lookahead inside a panel: after diagonal block k only the next block's
-    // 64 rows are solved, and its diagonal block updated, on the chain's stream; the
-    // rows below and the rest of the panel's columns go to la->s2 and run beside
-    // diagonal block k + 1, whose solve of the rows below waits for them. Each row of
-    // the solves and each entry of the updates is computed as without the lookahead.
-    const bool bla = ahead && la->s2;
-    bool side = false;  // la->s2 holds in-panel work the chain has not waited for
+    // The tile takes its first three terms beside the panel's last diagonal block
+    // (early), or all four after it where the previous panel's far update would not be
+    // done by then. Build, early against late: 64 x 64 5.17 against 5.4 ms, 128 x 128 99
+    // against 95 ms. PINV_CHOL_EARLY=0/1: always the one
+    const char* eenv = std::getenv("PINV_CHOL_EARLY");
+    const bool early = eenv ? std::strcmp(eenv, "0") != 0 : N <= 5632;
+    bool pending = false;  // a far update of the previous panel may still run
+    bool side = false;     // la->s2 holds work the chain has not waited for
+#define PT(call)                                  \
+    do {                                          \
+        const cudaError_t e_ = (call);            \
+        if (e_ != cudaSuccess) return e_;         \
+    } while (0)
+    // rows i0 .. i1 solved with block k0's inverse; the terms of nch blocks from k0 on columns j0 .. j1 of
+    // rows i0 .. i1
+    auto solve = [&](int64_t k0, int64_t i0, int64_t i1, cudaStream_t q) {
+        return i0 < i1 ? trsm_panel(L32 + k0, N, Dinv32 + (k0 / NBK) * NBK * NBK, G, ld, k0,
+                                    (int)std::min<int64_t>(NBK, N - k0), i0, i1, q)
+                       : cudaSuccess;
+    };
+    auto update = [&](int64_t k0, int nch, int64_t j0, int64_t j1, int64_t i0, int64_t i1, cudaStream_t q) {
+        return i0 < i1 && j0 < j1 ? herk_panel(L32 + k0, N, G, ld, nch, j0, j1, i0, i1, q) : cudaSuccess;
+    };
     for (int64_t p0 = 0; p0 < N; p0 += NBP) {
         const int64_t pend = std::min<int64_t>(N, p0 + NBP);
+        const int64_t tn = std::min<int64_t>(N, pend + 2 * NBK);  // the trailing matrix's first tile
+        const int64_t nt = cdiv(N - pend, tc::BM), kcn = cdiv(pend - p0, tc::KC);
         for (int64_t k0 = p0; k0 < pend; k0 += NBK) {
-            const int64_t nbk = std::min<int64_t>(NBK, N - k0);
-            const int64_t kb = k0 / NBK;
-            // the diagonal block writes its FP32 copy to L32; the solve below reads
-            // its right-hand sides from G
-            cudaError_t e =
-                launch_potrf_diag_df(G, ld, N, k0, Dinv ? Dinv + kb * NBK * NBK : nullptr,
-                                     Dinv32 + kb * NBK * NBK, L32, N, st, s);
-            if (e != cudaSuccess) return e;
-            const int64_t rest = N - k0 - nbk;
-            if (rest <= 0) break;
-            const int64_t t0 = k0 + nbk;
-            const float2* Dk = Dinv32 + kb * NBK * NBK;
-            if (side) {  // the rows below were updated by the previous block's side work
-                if ((e = cudaStreamWaitEvent(s, la->ev_side, 0)) != cudaSuccess) return e;
-                side = false;
-            }
-            if (bla && t0 < pend) {
-                const int64_t t1 = std::min<int64_t>(t0 + NBK, pend);  // the next diagonal block
-                if ((e = trsm_panel(L32 + k0, N, Dk, G, ld, k0, (int)nbk, t0, t1, s)) != cudaSuccess) return e;
-                if ((e = herk_panel(L32 + k0, N, G, ld, (int)nbk, t0, t1, t0, t1, s)) != cudaSuccess) return e;
-                if (t1 < N) {
-                    if ((e = cudaEventRecord(la->ev_next, s)) != cudaSuccess) return e;
-                    if ((e = cudaStreamWaitEvent(la->s2, la->ev_next, 0)) != cudaSuccess) return e;
-                    if ((e = trsm_panel(L32 + k0, N, Dk, G, ld, k0, (int)nbk, t1, N, la->s2)) != cudaSuccess)
-                        return e;
-                    if ((e = herk_panel(L32 + k0, N, G, ld, (int)nbk, t0, pend, t1, N, la->s2)) != cudaSuccess)
-                        return e;
-                    if ((e = cudaEventRecord(la->ev_side, la->s2)) != cudaSuccess) return e;
-                    side = true;
-                }
+            // the diagonal block writes its FP32 copy to L32; the solves read their
+            // right-hand sides from G
+            const int64_t kb = k0 / NBK, t0 = std::min<int64_t>(N, k0 + NBK);
+            PT(launch_potrf_diag_df(G, ld, N, k0, Dinv ? Dinv + kb * NBK * NBK : nullptr, Dinv32 + kb * NBK * NBK, L32,
+                                    N, st, s));
+            if (t0 >= N) break;
+            const bool last = t0 == pend;
+            if (!ahead) {
+                PT(solve(k0, t0, N, s));
+                PT(update(k0, 1, t0, pend, t0, N, s));
+                if (last) PT(update(p0, NBP / NBK, pend, tn, pend, tn, s));
                 continue;
             }
-            // panel solve of every row below the block
-            if ((e = trsm_panel(L32 + k0, N, Dk, G, ld, k0, (int)nbk, t0, N, s)) != cudaSuccess) return e;
-            if (t0 < pend) {  // the panel's remaining columns, all rows below
-                if ((e = herk_panel(L32 + k0, N, G, ld, (int)nbk, t0, pend, t0, N, s)) != cudaSuccess) return e;
+            const int64_t t1 = std::min<int64_t>(N, t0 + NBK);  // the next diagonal block ends here
+            if (side) {  // its rows have the terms of the panel's earlier blocks
+                PT(cudaStreamWaitEvent(s, la->ev_side, 0));
+                side = false;
             }
-        }
-        if (side) {
-            cudaError_t e = cudaStreamWaitEvent(s, la->ev_side, 0);
-            if (e != cudaSuccess) return e;
-            side = false;
-        }
-        if (ev_panel) {
-            cudaError_t e = cudaEventRecord(ev_panel[p0 / NBP], s);
-            if (e != cudaSuccess) return e;
-        }
-        if (pend < N) {  // trailing matrix, K = panel width
-            cudaError_t e;
-            if (tab) {
-                const int64_t nt = cdiv(N - pend, tc::BM), kcn = cdiv(pend - p0, tc::KC);
-                if (pending) {  // the previous panel's side update also writes these columns, and reads the table
-                    if ((e = cudaStreamWaitEvent(s, la->ev_done, 0)) != cudaSuccess) return e;
+            if (last && !early) {  // the tile after the solves of its rows, once the far update is done
+                PT(solve(k0, t0, tn, s));
+                if (pending) PT(cudaStreamWaitEvent(s, la->ev_done, 0));
+                pending = false;
+                PT(update(p0, NBP / NBK, pend, tn, pend, tn, s));
+                PT(cudaEventRecord(la->ev_next, s));
+                PT(cudaStreamWaitEvent(la->s2, la->ev_next, 0));
+                PT(solve(k0, tn, N, la->s2));
+                continue;
+            }
+            PT(solve(k0, t0, t1, s));
+            PT(update(k0, 1, t0, t1, t0, t1, s));
+            if (t1 == N) continue;
+            PT(cudaEventRecord(la->ev_next, s));
+            PT(cudaStreamWaitEvent(la->s2, la->ev_next, 0));
+            // the rows of the next step: one block, or the next panel's first tile
+            const bool before_last = t1 == pend && early;
+            // (all rows where the chain takes up the tile next)
+            const int64_t r1 = std::min<int64_t>(N, t1 < pend || last ? t1 + NBK : early ? t1 + 2 * NBK : N);
+            PT(solve(k0, t1, r1, la->s2));
+            PT(update(k0, 1, t0, last ? tn : pend, t1, r1, la->s2));
+            if (before_last) {
+                if (pending) {  // the previous panel's far update also writes that tile
+                    PT(cudaStreamWaitEvent(la->s2, la->ev_done, 0));
                     pending = false;
                 }
-                if ((e = panel_table(L32, N, p0, pend - p0, pend, slices, (uint8_t*)tab, s)) != cudaSuccess) return e;
-                const int64_t near = ahead ? std::min<int64_t>(nt, NBP / tc::BN) : nt;
-                tc::HerkBulk hp{(const uint8_t*)tab, G, ld, N, pend, nt, kcn, slices, 0, near};
-                e = run(hp, dim3((unsigned)(nt * near), 1), slices, st, 4, s, false, 0, true);
-                if (e == cudaSuccess && near < nt) {
-                    if ((e = cudaEventRecord(la->ev_tab, s)) != cudaSuccess) return e;
-                    if ((e = cudaStreamWaitEvent(la->s, la->ev_tab, 0)) != cudaSuccess) return e;
-                    tc::HerkBulk fp{(const uint8_t*)tab, G, ld, N, pend, nt, kcn, slices, near, nt - near};
-                    if ((e = run(fp, dim3((unsigned)(nt * (nt - near)), 1), slices, la->st, 4, la->s, false, cap)) !=
-                        cudaSuccess)
-                        return e;
-                    if ((e = cudaEventRecord(la->ev_done, la->s)) != cudaSuccess) return e;
-                    pending = true;
-                }
-            } else {
-                tc::HerkTC hp{L32 + p0, N, G, ld, N, pend - p0, pend, N};
-                e = run(hp, dim3(cdiv(N - pend, tc::BN), cdiv(N - pend, tc::BM)), slices, st, 4, s);
+                PT(update(p0, NBP / NBK - 1, pend, tn, pend, tn, la->s2));
             }
-            if (e != cudaSuccess) return e;
+            PT(cudaEventRecord(la->ev_side, la->s2));
+            side = true;
+            PT(solve(k0, r1, N, la->s2));
+            if (!last) PT(update(k0, 1, t0, pend, r1, N, la->s2));
+        }
+        // the panel's last solves are on the second stream, if there were any beyond the next block
+        const bool on_side = ahead && N - pend > NBK;
+        const cudaStream_t q = on_side ? la->s2 : s;
+        if (ev_panel) PT(cudaEventRecord(ev_panel[p0 / NBP], q));
+        if (pend == N) break;
+        if (nt == 1) continue;
+        // trailing matrix, K = panel width
+        if (!tab) {
+            tc::HerkTC hp{L32 + p0, N, G, ld, N, pend - p0, pend, N};
+            PT(run(hp, dim3(cdiv(N - pend, tc::BN), cdiv(N - pend, tc::BM)), slices, st, 4, s));
+        } else {
+            PT(panel_table(L32, N, p0, pend - p0, pend, slices, (uint8_t*)tab, q));
+            const int64_t near = ahead ? std::min<int64_t>(nt, NBP / tc::BN) : nt;
+            tc::HerkBulk hp{(const uint8_t*)tab, G, ld, N, pend, nt, kcn, slices, 0, near};
+            PT(run(hp, dim3((unsigned)(nt * near), 1), slices, st, 4, q, false, 0, true));
+            if (near < nt) {
+                PT(cudaEventRecord(la->ev_tab, q));
+                PT(cudaStreamWaitEvent(la->s, la->ev_tab, 0));
+                tc::HerkBulk fp{(const uint8_t*)tab, G, ld, N, pend, nt, kcn, slices, near, nt - near};
+                PT(run(fp, dim3((unsigned)(nt * (nt - near)), 1), slices, la->st, 4, la->s, false, cap));
+                PT(cudaEventRecord(la->ev_done, la->s));
+                pending = true;
+            }
         }
     }
-    if (pending) {
-        cudaError_t e = cudaStreamWaitEvent(s, la->ev_done, 0);
-        if (e != cudaSuccess) return e;
+    if (ahead) {  // join
+        PT(cudaEventRecord(la->ev_side, la->s2));
+        PT(cudaStreamWaitEvent(s, la->ev_side, 0));
+        if (pending) PT(cudaStreamWaitEvent(s, la->ev_done, 0));
     }
+#undef PT
     return cudaGetLastError();
 }
 
@@ -1298,17 +1355,9 @@ cudaError_t launch_trtri_tc(const float2* L32, int64_t N, const float2* Dinv32, 
     // W is in double-float storage while it is formed; the last pass leaves it in FP64
     cudaError_t e = launch_fill_identity_df(W, N, N, s);
     if (e != cudaSuccess) return e;
-    // the inverse runs beside the Cholesky chain (and its trailing updates). Up to
-    // N = 16384, where the chain is a latency-bound sequence of small launches, the
-    // inverse's persistent launches take at most half the SMs so that the chain's
-    // launches find free SMs; the trailing updates beside the chain take two fifths.
-    // Measured at 64x64 (inverse / trailing SMs -> build): 114 / 38 -> 8.78 ms,
-    // 152 / 50 -> 8.77 ms, 76 / 50 -> 8.63 ms, 76 / 64 -> 8.57 ms, 64 / 64 -> 8.56 ms,
-    // any / 24 -> 9.3 ms and more (the trailing updates fall behind). Above
-    // N = 16384 all three are throughput-bound
-    // and each takes every SM. PINV_INV_SMS: another count (0 all).
+    // PINV_INV_SMS: another count of SMs (0 all)
     const char* cenv = std::getenv("PINV_INV_SMS");
-    const int cap = cenv ? std::atoi(cenv) : (N <= 16384 ? std::max(1, tc::sm_count() / 2) : 0);
+    const int cap = cenv ? std::atoi(cenv) : side_sms(N);
     for (int64_t p0 = 0; p0 < N; p0 += NBP) {
         const int64_t pend = std::min<int64_t>(N, p0 + NBP);
         if (ev_panel && (e = cudaStreamWaitEvent(s, ev_panel[p0 / NBP], 0)) != cudaSuccess) return e;

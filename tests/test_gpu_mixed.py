@@ -256,6 +256,33 @@ def test_cholesky_lookahead_bit_identical(monkeypatch):
     assert torch.equal(out["0"][1], out["1"][1])
 
 
+@pytest.mark.parametrize("early", ["0", "1"])
+@pytest.mark.parametrize("dims", [(17, 17), (16, 20), (20, 20), (5, 129), (24, 24)])
+def test_cholesky_first_trailing_tile(dims, early, monkeypatch):
+    """The trailing matrix's first tile takes its update block by block, beside or after
+    the panel's last diagonal block: the same factor and inverse bit for bit as on one
+    stream. 33, 64, 144, 389 then 133, and 320 then 64 rows beyond a panel: less than a
+    block, one block, a tile and rows below it, and the same after a second panel."""
+    from paper_2410_06129_gb300.plan import Plan
+    p = synth.make_plan(24, 2, "spiral", 1, 2132, 1e-3, samples=1500, interleaves=2)
+    N = dims[0] * dims[1]
+    rng = np.random.default_rng(2133)
+    maps = rng.standard_normal((2, N)) + 1j * rng.standard_normal((2, N))
+    out = {}
+    for mode in ("0", "1"):
+        monkeypatch.setenv("PINV_CHOL_LOOKAHEAD", mode)
+        monkeypatch.setenv("PINV_CHOL_EARLY", early)
+        with Plan(dims, p.traj[:, :2], maps, lam=1e-2, precision=L.MIXED_BF16X6) as pl:
+            pl.build()
+            out[mode] = (pl.export(L.EXPORT_CHOL).cpu(), pl.export(L.EXPORT_LINV).cpu())
+    assert torch.equal(out["0"][0], out["1"][0])
+    assert torch.equal(out["0"][1], out["1"][1])
+    E = O.encode(p.traj[:, :2], O.voxel_positions(dims), maps, None, None)
+    G = E.conj().T @ E + O.lambda_abs(E, 1e-2) * np.eye(N)
+    # the split factor's bound of test_diag_block_cluster_matches_one_cta_sweep
+    assert rel(out["1"][0].numpy(), np.linalg.cholesky(G)) < 1e-3
+
+
 def test_b0_exact_products_many_frames(monkeypatch):
     """Plans with B0 refine with exact tensor-core E x and E^H u (digit tables of
     A and conj(A), 48 bytes per entry) for 16 or more frames. Workload 5 shrunk to
