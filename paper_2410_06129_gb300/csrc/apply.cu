@@ -61,7 +61,7 @@ static ApplyModes apply_modes(const pinv_plan* p) {
     return m;
 }
 
-size_t apply_scratch_layout(const pinv_plan* p, int64_t F, int dtype, void* base, ApplyScratch* sc, bool oz) {
+size_t apply_scratch_layout(const pinv_plan* p, int64_t F, int dtype, void* base, ApplyScratch* sc, bool roomy) {
     const int64_t N = p->N, M = p->M;
     const ApplyModes md = apply_modes(p);
     // FP64 copy of c64 data (every path but the mixed Recon-only apply reads
@@ -77,7 +77,10 @@ size_t apply_scratch_layout(const pinv_plan* p, int64_t F, int dtype, void* base
     const bool need_u128 = (md.refine && !md.toep) || (md.fpres && !p->recon);
     const bool need_r128 = md.refine || !p->recon;
     const bool need_d64 = md.use_recon && dtype == PINV_C128;
-    const bool need_x64 = md.mixed && (p->recon || md.dfres || md.toep);
+    const bool corr = md.mixed && (md.dfres || md.toep || !p->recon) && correct_tc_ok(F);
+    const bool crows = corr && correct_rows_ok(N, F), ctc = corr && !crows && roomy;
+    // FP32 image of the Recon apply; W r of the corrections but the tensor cores'
+    const bool need_x64 = md.mixed && (p->recon || md.dfres || md.toep) && (md.use_recon || !ctc);
     Carver cv{static_cast<unsigned char*>(base)};
     ApplyScratch s{};
     s.d128 = need_d128 ? cv.take<double2>((size_t)(F * M)) : nullptr;
@@ -89,12 +92,10 @@ size_t apply_scratch_layout(const pinv_plan* p, int64_t F, int dtype, void* base
     s.x64 = need_x64 ? cv.take<float2>((size_t)(F * N)) : nullptr;
     s.norms = md.stop_rule ? cv.take<double>((size_t)(3 * F)) : nullptr;
     const bool atc = md.use_recon && apply_tc_ok(F);
-    const bool corr = md.mixed && (md.dfres || md.toep || !p->recon) && correct_tc_ok(F);
-    const bool crows = corr && correct_rows_ok(N, F), ctc = corr && !crows;
     if (atc) s.apw = cv.take<float2>(apply_tc_work_elems(N, M, F));
-    if (ctc) s.cw = cv.take<float2>(correct_tc_work_elems(N, F));
+    if (ctc) s.cw = cv.take<uint8_t>(correct_tc_work_bytes(N, F, p->slices()));
     if (crows) s.r32 = cv.take<float2>((size_t)(F * N));
-    if (atc || ctc) s.sched = cv.take<DevStatus>(1);
+    if (atc) s.sched = cv.take<DevStatus>(1);
     if (md.dfres || md.toep || md.need_b) {
         // E^H u (rows N, length M), E x (rows M, length N), G x (rows N, length N) one
         // after another: the largest scratch of any
@@ -113,7 +114,7 @@ size_t apply_scratch_layout(const pinv_plan* p, int64_t F, int dtype, void* base
         s.xfwd = xfwd;
         s.dfw = w ? (float4*)cv.take<uint8_t>(w) : nullptr;
     }
-    if (oz && (!md.mixed || md.fpres) && tc_available()) {
+    if (roomy && (!md.mixed || md.fpres) && tc_available()) {
         // one FP64 product after another: the largest
         size_t w = 0;
         if (md.mixed || !p->recon || md.refine) w = std::max(w, oz_adjoint_bytes(p->enc, F));
@@ -158,7 +159,7 @@ pinv_status apply_impl(pinv_plan* p, const void* d_data, void* d_image, int64_t 
     // (correct_rows_ok), else on the tensor cores (correct_tc_ok), else SIMT
     auto correct = [&](const double2* r) -> cudaError_t {
         if (sc.r32) return launch_correct_rows(p->W32, N, r, F, sc.x64, X, sc.r32, s);
-        if (sc.cw) return launch_correct_tc(p->W32, N, r, F, sc.x64, X, sc.cw, p->slices(), sc.sched, s);
+        if (sc.cw) return launch_correct_tc(p->W32, N, r, F, X, sc.cw, p->slices(), p->st, s);
         return launch_correct32(p->W32, N, r, F, sc.x64, X, s);
     };
 
@@ -338,7 +339,7 @@ extern "C" pinv_status pinv_apply(pinv_plan* p, const void* d_data, void* d_imag
         }
         cudaError_t e = work_alloc(&p->scratch_buf, need, 0);
         if (e == cudaErrorMemoryAllocation && !p->scratch_small) {
-            // no room for the FP64 products' tables: the FP64 pipe needs none
+            // no room for the tensor-core tables: the SIMT products need none
             cudaGetLastError();
             p->scratch_small = true;
             need = apply_scratch_layout(p, F, dtype, nullptr, nullptr, false);

@@ -46,7 +46,7 @@ struct pinv_batch {
     unsigned long long apply_launches = 0;
     std::vector<void*> scratch;
     std::vector<size_t> scratch_bytes;
-    std::vector<char> small;  // per plan: no room for the FP64 products' tables (apply_scratch_layout)
+    std::vector<char> small;  // per plan: no room for the tensor-core tables (apply_scratch_layout)
     ~pinv_batch();
 };
 

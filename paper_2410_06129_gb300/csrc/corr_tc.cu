@@ -1,0 +1,475 @@
+// The refinement's correction x += W^H (W r) for many frames, on the tensor cores:
+// W the FP32 lower-triangular L^-1 of a mixed plan, split into bf16 slices as in
+// tc_engine.cuh, up to 64 frames in a pass.
+//
+// Two products of the same form: C[i][f] = sum_k a(i, k) b(k, f) over 128-row tiles,
+// a = W or W^H, 16 k to a stage. Only the stages on one side of the diagonal exist;
+// they are numbered row tile by row tile and cut into equal runs, one CTA each, so
+// every SM has the same work whatever the triangle's shape. A run covers parts of one
+// or more row tiles and leaves one FP32 partial sum for each; run c's part of row tile
+// t is slot c + t. The next kernel adds a tile's slots in order.
+//
+// In a CTA eight warps read W from memory (two or three stages ahead), split it and write the
+// A tiles; the B tiles come from a table of the frames' slices (one bulk copy a
+// stage); one thread issues the MMAs, N = 2 x 64 or 2 x 32 columns. Accumulation as in
+// tc_engine.cuh: at most DRAIN stages in tensor memory, then added to a running total
+// in registers with round to nearest, two buffers taking turns.
+//
+// Bound by the conversion of W and the latency of its loads. Per correction (N = 4096,
+// 64 frames): two products on the generating engine, 128 columns wide with the frames'
+// FP64 values split again in every tile, 192 us; this 104 us (44 and 36 for the
+// products; without the loads of W 31 each, without its split and the MMAs either, 20).
+#include <algorithm>
+#include <cstdlib>
+
+#include "tc_engine.cuh"
+
+namespace pinv {
+namespace tc {
+namespace {
+
+constexpr int CT_THREADS = NTHREADS + 32;  // 8 producer / drain warps, MMA issuer, table loader
+constexpr int CT_SITE = 22;
+
+template <int S, int NF>
+struct CtCfg {
+    static constexpr int BSL = 2 * NF * ROWB;  // one slice of a stage's B tile
+    static constexpr int STAGE = S * (A_SL + BSL);
+    static constexpr int STAGES = (int)(200 * 1024) / STAGE;
+    static constexpr int SMEM = STAGES * STAGE + 1024;
+    static constexpr int NPAIRS = S == 3 ? 6 : 3;
+    static constexpr uint32_t COLS = 4 * NF;  // two buffers of real and imaginary columns
+    // kind::f16: D f32, A/B bf16, K-major, M = 128, N = 2 NF
+    static constexpr uint32_t IDESC_N =
+        (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)((2 * NF) >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+};
+
+// stages before row tile t, of nt, with kcn chunks of 16 k; T: the transposed product
+__host__ __device__ inline int64_t ct_prefix(bool T, int64_t t, int64_t nt, int64_t kcn) {
+    if (T) return t * kcn - 4 * t * (t - 1);       // tile t: chunks 8 t .. kcn - 1
+    return t < nt ? 4 * t * (t + 1) : 4 * (nt - 1) * nt + kcn;  // tile t: the first 8 (t + 1) chunks
+}
+
+// 8 consecutive values of a row of W: whole 32-byte sectors to a thread and instruction where the
+// row is aligned to them (with 200 KB of shared memory the L1 holds no lines for a second touch:
+// product W r 46 us with 16-byte loads, 44 us so, at N = 4096 and 64 frames)
+__device__ inline void load8row(const float2* p, int avail, float2 (&v)[8]) {
+    if (avail >= 8 && ((uintptr_t)p & 31) == 0) {
+#pragma unroll
+        for (int u = 0; u < 8; u += 4)
+            asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                         : "=f"(v[u].x), "=f"(v[u].y), "=f"(v[u + 1].x), "=f"(v[u + 1].y), "=f"(v[u + 2].x),
+                           "=f"(v[u + 2].y), "=f"(v[u + 3].x), "=f"(v[u + 3].y)
+                         : "l"(p + u));
+        return;
+    }
+    load8f(p, avail, v);
+}
+
+// 8 k of frame f into the stage's B tile (rows f: [Br | -Bi], rows NF + f: [Bi | Br])
+template <int S, int NF>
+__device__ inline void ct_put_b(uint8_t* blk, int f, int g, const float2 (&v)[8]) {
+    float re[8], im[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        re[u] = v[u].x;
+        im[u] = v[u].y;
+    }
+    uint32_t wr[S][4], wi[S][4];
+    split8<S>(re, wr);
+    split8<S>(im, wi);
+    auto put = [&](int off, const uint32_t(&w)[4], uint32_t flip) {
+        *reinterpret_cast<uint4*>(blk + off) = make_uint4(w[0] ^ flip, w[1] ^ flip, w[2] ^ flip, w[3] ^ flip);
+    };
+#pragma unroll
+    for (int s = 0; s < S; ++s) {
+        const int o = s * CtCfg<S, NF>::BSL;
+        put(o + koff(f, g), wr[s], 0u);
+        put(o + koff(f, g + 2), wi[s], 0x80008000u);
+        put(o + koff(NF + f, g), wi[s], 0u);
+        put(o + koff(NF + f, g + 2), wr[s], 0u);
+    }
+}
+
+// the table of r [F][N] (rounded to FP32): one CTA per chunk of 16 k, 2 NF threads
+template <int S, int NF>
+__global__ void __launch_bounds__(2 * NF) k_corr_tab(const double2* __restrict__ R, int64_t N, int F, uint8_t* tab) {
+    const int f = threadIdx.x >> 1, g = threadIdx.x & 1;
+    const int64_t k = (int64_t)blockIdx.x * KC + 8 * g;
+    griddep_wait();
+    griddep_launch();
+    float2 v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        const double2 a = f < F && k + u < N ? R[f * N + k + u] : make_double2(0.0, 0.0);
+        v[u] = make_float2(f64_to_f32_rn(a.x), f64_to_f32_rn(a.y));
+    }
+    ct_put_b<S, NF>(tab + (int64_t)blockIdx.x * S * CtCfg<S, NF>::BSL, f, g, v);
+}
+
+// the table of W r from its partial sums
+template <int S, int NF>
+__global__ void __launch_bounds__(2 * NF) k_corr_sum_tab(const float2* __restrict__ part, int64_t nt, int64_t kcn,
+                                                         int F, int64_t per, uint8_t* tab) {
+    const int f = threadIdx.x >> 1, g = threadIdx.x & 1;
+    const int64_t k = (int64_t)blockIdx.x * KC + 8 * g, t = k / BM;
+    const int r = (int)(k % BM);
+    griddep_wait();
+    griddep_launch();
+    float2 v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = make_float2(0.f, 0.f);
+    if (f < F) {
+        const int64_t c1 = (ct_prefix(false, t + 1, nt, kcn) - 1) / per;
+        for (int64_t c = ct_prefix(false, t, nt, kcn) / per; c <= c1; ++c) {
+            const float4* p = reinterpret_cast<const float4*>(part + ((c + t) * F + f) * BM + r);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const float4 a = p[u];
+                v[2 * u].x += a.x;
+                v[2 * u].y += a.y;
+                v[2 * u + 1].x += a.z;
+                v[2 * u + 1].y += a.w;
+            }
+        }
+    }
+    ct_put_b<S, NF>(tab + (int64_t)blockIdx.x * S * CtCfg<S, NF>::BSL, f, g, v);
+}
+
+// X[f][n] += the partial sums of W^H (W r) in double-float (FP64 issues at 1/64 of the FP32 rate)
+__global__ void __launch_bounds__(256) k_corr_sum_x(const float2* __restrict__ part, int64_t N, int64_t nt,
+                                                    int64_t kcn, int F, int64_t per, double2* __restrict__ X) {
+    const int64_t n = (int64_t)blockIdx.x * 256 + threadIdx.x, f = blockIdx.y;
+    griddep_wait();
+    griddep_launch();
+    if (n >= N) return;
+    const int64_t t = n / BM, c1 = (ct_prefix(true, t + 1, nt, kcn) - 1) / per;
+    float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
+    for (int64_t c = ct_prefix(true, t, nt, kcn) / per; c <= c1; ++c) {
+        const float2 a = part[((c + t) * F + f) * BM + n % BM];
+        df_add(rh, rl, a.x, 0.f, rh, rl);
+        df_add(ih, il, a.y, 0.f, ih, il);
+    }
+    const double2 x = X[f * N + n];
+    X[f * N + n] = make_double2(x.x + ((double)rh + (double)rl), x.y + ((double)ih + (double)il));
+}
+
+// part: slots of row tiles' partial sums, [slot][F][128]
+template <int S, int NF, bool T>
+__global__ void __launch_bounds__(CT_THREADS, 1)
+    k_corr_tc(const float2* __restrict__ W, int64_t N, int F, const uint8_t* __restrict__ tab, float2* part,
+              int64_t per, DevStatus* st) {
+    using CF = CtCfg<S, NF>;
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ uint64_t full_bar[CF::STAGES], tab_bar[CF::STAGES], empty_bar[CF::STAGES];
+    __shared__ uint64_t tfull[2], tempty[2], done_bar;
+    __shared__ uint32_t tmem_base_sh;
+    __shared__ int abort_flag;
+    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t nt = (N + BM - 1) / BM, kcn = (N + KC - 1) / KC;
+    const int64_t total = ct_prefix(T, nt, nt, kcn);
+    const int64_t s0 = (int64_t)blockIdx.x * per, s1 = s0 + per < total ? s0 + per : total;
+    int64_t t0 = 0;  // the run's first row tile
+    while (ct_prefix(T, t0 + 1, nt, kcn) <= s0) ++t0;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < CF::STAGES; ++s) {
+            mbar_init(&full_bar[s], NPW);  // A: one arrival a producer warp
+            mbar_init(&tab_bar[s], 1);     // B: the loader and its bytes
+            mbar_init(&empty_bar[s], 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&tfull[b], 1);
+            mbar_init(&tempty[b], NPW);
+        }
+        mbar_init(&done_bar, 1);
+        abort_flag = 0;
+        fence_barrier_init();
+    }
+    if (warp == NPW) tmem_alloc(&tmem_base_sh, CF::COLS);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tmem_base_sh;
+    griddep_wait();
+    griddep_launch();
+    const long long wlim = st->wait_limit > 0 ? st->wait_limit : WAIT_LIMIT;
+
+    uint32_t kq = 0, gq = 0;  // stages and accumulation groups of the row tiles before
+    uint32_t issued = 0;      // stages the loader has started
+    if (warp < NPW) {
+        const int q = warp & 3, h = warp >> 2;
+        const int r = threadIdx.x & (BM - 1), g8 = threadIdx.x >> 7;  // this thread's row and half of the 16 k
+        const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(h * NF / 2);
+        // the loads run PRE stages ahead of the splitting, across row tiles, each into the
+        // registers of its turn (a copy between registers would wait for the load)
+        constexpr int PRE = NF == 32 ? 3 : 2;
+        int left = (int)(s1 - s0), lt = (int)t0, k = 0, lrem = 0;
+        const float2* ptr = W;
+        bool row = false;
+        auto tile = [&](int64_t first) {  // row tile lt from its stage `first` on
+            const int64_t b = ct_prefix(T, lt, nt, kcn), i = (int64_t)lt * BM + r;
+            lrem = (int)(ct_prefix(T, lt + 1, nt, kcn) - first);
+            k = (int)(first - b) * KC + (T ? lt * BM : 0) + 8 * g8;
+            row = i < N;
+            ptr = T ? W + (int64_t)k * N + i : W + i * N + k;
+        };
+        tile(s0);
+        auto fetch = [&](float2(&v)[8]) {
+            if (left == 0) return;
+            const int avail = row ? (int)N - k : 0;
+            if (T)
+                load8col(ptr, N, avail, v);
+            else
+                load8row(ptr, avail, v);
+            --left;
+            k += KC;
+            ptr += T ? KC * N : KC;
+            if (--lrem == 0 && left) {
+                ++lt;
+                tile(ct_prefix(T, lt, nt, kcn));
+            }
+        };
+        float2 p[PRE][8];
+#pragma unroll
+        for (int u = 0; u < PRE; ++u) fetch(p[u]);
+        int turn = 0;
+        bool ok = true;
+        int64_t t = t0;
+        for (int64_t s = s0; s < s1 && ok; ++t) {
+            const int64_t end = ct_prefix(T, t + 1, nt, kcn), e = end < s1 ? end : s1;
+            const int nk = (int)(e - s), ngroups = (nk + DRAIN - 1) / DRAIN;
+            float tot[NF];
+#pragma unroll
+            for (int u = 0; u < NF; ++u) tot[u] = 0.f;
+            int drained = 0;
+            auto drain = [&]() -> bool {
+                const uint32_t G = gq + (uint32_t)drained, b = G & 1u;
+                if (!mbar_wait(&tfull[b], (G >> 1) & 1u, &abort_flag, wlim)) return false;
+                tc_fence_after();
+#pragma unroll
+                for (int pt = 0; pt < NF / 16; ++pt) {
+                    uint32_t v[16];
+                    tmem_ld16(taddr + 2u * NF * b + (uint32_t)(pt < NF / 32 ? 16 * pt : NF + 16 * (pt - NF / 32)), v);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int u = 0; u < 16; ++u) tot[16 * pt + u] += __uint_as_float(v[u]);
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&tempty[b]);
+                ++drained;
+                return true;
+            };
+            for (int kt = 0; kt < nk; ++kt) {
+                // the MMAs of group g + 2 wait for the drain of group g: drain before the ring
+                // can only advance past them
+                if (drained < ngroups && (drained + 1) * DRAIN + CF::STAGES - 1 <= kt && !(ok = drain())) break;
+                const uint32_t kg = kq + (uint32_t)kt;
+                const int sl = (int)(kg % CF::STAGES);
+                if (kg >= CF::STAGES && !(ok = mbar_wait(&empty_bar[sl], ((kg / CF::STAGES) & 1u) ^ 1u, &abort_flag, wlim)))
+                    break;
+                uint8_t* base = smem + sl * CF::STAGE + koff(r, g8);
+                auto split = [&](float2(&v)[8]) {
+                    float x[8], y[8];
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        x[u] = v[u].x;
+                        y[u] = T ? -v[u].y : v[u].y;
+                    }
+                    fetch(v);
+                    uint32_t w[S][4];
+                    split8<S>(x, w);
+#pragma unroll
+                    for (int z = 0; z < S; ++z)
+                        *reinterpret_cast<uint4*>(base + z * A_SL) = make_uint4(w[z][0], w[z][1], w[z][2], w[z][3]);
+                    split8<S>(y, w);
+#pragma unroll
+                    for (int z = 0; z < S; ++z)
+                        *reinterpret_cast<uint4*>(base + z * A_SL + (koff(0, 2) - koff(0, 0))) =
+                            make_uint4(w[z][0], w[z][1], w[z][2], w[z][3]);
+                };
+                if (turn == 0)
+                    split(p[0]);
+                else if (PRE == 2 || turn == 1)
+                    split(p[1]);
+                else
+                    split(p[PRE - 1]);
+                turn = turn == PRE - 1 ? 0 : turn + 1;
+                fence_proxy_async();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&full_bar[sl]);
+            }
+            while (ok && drained < ngroups) ok = drain();
+            if (ok && !abort_flag) {
+                float2* o = part + ((int64_t)blockIdx.x + t) * F * BM + q * 32 + lane;
+#pragma unroll
+                for (int u = 0; u < NF / 2; ++u) {
+                    const int f = h * (NF / 2) + u;
+                    if (f < F) o[(int64_t)f * BM] = make_float2(tot[u], tot[NF / 2 + u]);
+                }
+            }
+            kq += (uint32_t)nk;
+            gq += (uint32_t)ngroups;
+            s = e;
+        }
+    } else if (warp == NPW && lane == 0) {
+        // ---------------- MMA issuer
+        bool ok = true;
+        int64_t t = t0;
+        for (int64_t s = s0; s < s1 && ok; ++t) {
+            const int64_t end = ct_prefix(T, t + 1, nt, kcn), e = end < s1 ? end : s1;
+            const int nk = (int)(e - s);
+            for (int kt = 0; kt < nk; ++kt) {
+                const uint32_t G = gq + (uint32_t)(kt / DRAIN), b = G & 1u;
+                const bool first = kt % DRAIN == 0;
+                if (first && G >= 2 && !(ok = mbar_wait(&tempty[b], ((G >> 1) - 1u) & 1u, &abort_flag, wlim))) break;
+                const uint32_t kg = kq + (uint32_t)kt;
+                const int sl = (int)(kg % CF::STAGES);
+                const uint32_t ph = (kg / CF::STAGES) & 1u;
+                if (!(ok = mbar_wait(&full_bar[sl], ph, &abort_flag, wlim) && mbar_wait(&tab_bar[sl], ph, &abort_flag, wlim)))
+                    break;
+                tc_fence_after();
+                const uint32_t sa = smem_u32(smem + sl * CF::STAGE), sb = sa + S * A_SL;
+#pragma unroll
+                for (int pq = 0; pq < CF::NPAIRS; ++pq)
+#pragma unroll
+                    for (int kk = 0; kk < 2; ++kk)
+                        mma_bf16(tmem + 2u * NF * b, sdesc(sa + pair_a(pq) * A_SL + kk * 256, 128, 512),
+                                 sdesc(sb + pair_b(pq) * CF::BSL + kk * 256, 128, 512), CF::IDESC_N,
+                                 (first && pq == 0 && kk == 0) ? 0u : 1u);
+                mma_commit(&empty_bar[sl]);
+                if (kt % DRAIN == DRAIN - 1 || kt == nk - 1) mma_commit(&tfull[b]);
+            }
+            kq += (uint32_t)nk;
+            gq += (uint32_t)((nk + DRAIN - 1) / DRAIN);
+            s = e;
+        }
+        mma_commit(&done_bar);  // completes when every issued MMA has finished
+    } else if (warp == NPW + 1 && lane == 0) {
+        // ---------------- table loader
+        int64_t t = t0, end = ct_prefix(T, t0 + 1, nt, kcn);
+        for (int64_t s = s0; s < s1; ++s) {
+            if (s == end) end = ct_prefix(T, ++t + 1, nt, kcn);
+            const int64_t kc = s - ct_prefix(T, t, nt, kcn) + (T ? 8 * t : 0);
+            const uint32_t kg = (uint32_t)(s - s0);
+            const int sl = (int)(kg % CF::STAGES);
+            if (kg >= CF::STAGES && !mbar_wait(&empty_bar[sl], ((kg / CF::STAGES) & 1u) ^ 1u, &abort_flag, wlim)) break;
+            mbar_arrive_expect_tx(&tab_bar[sl], (uint32_t)(S * CF::BSL));
+            bulk_g2s(smem + sl * CF::STAGE + S * A_SL, tab + kc * S * CF::BSL, (uint32_t)(S * CF::BSL), &tab_bar[sl]);
+            issued = kg + 1;
+        }
+        // copies still in flight (only after an abort): wait, bounded, for their bytes
+        for (uint32_t kg = issued > (uint32_t)CF::STAGES ? issued - CF::STAGES : 0u; kg < issued; ++kg)
+            mbar_wait(&tab_bar[kg % CF::STAGES], (kg / CF::STAGES) & 1u, nullptr);
+    }
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
+    if (warp == NPW) {
+        mbar_wait(&done_bar, 0, nullptr);  // no MMA may still write TMEM when it is released
+        tc_fence_after();
+        tmem_dealloc(tmem, CF::COLS);
+    }
+    if (threadIdx.x == 0 && abort_flag) atomicMax(&st->timeout_site, CT_SITE);
+}
+
+struct Shape {
+    int nf;                       // frames of a tile
+    int64_t nt, kcn, pw, ph;      // row tiles, chunks of k, stages of a run (W, W^H)
+    int64_t gw, gh;               // runs
+    size_t tab, part;             // bytes
+};
+// Runs fill the SMs once and hold at least DRAIN stages.
+Shape shape(int64_t N, int64_t F, int slices) {
+    Shape h{};
+    const int64_t Fc = std::min<int64_t>(F, 64);
+    h.nf = Fc <= 32 ? 32 : 64;
+    h.nt = (N + BM - 1) / BM;
+    h.kcn = (N + KC - 1) / KC;
+    h.tab = (size_t)(h.kcn * slices * 2 * h.nf * ROWB);
+    const size_t slot = sizeof(float2) * (size_t)(Fc * BM);
+    const int64_t runs = sm_count();
+    auto cut = [&](bool T, int64_t& per, int64_t& n) {
+        const int64_t total = ct_prefix(T, h.nt, h.nt, h.kcn);
+        per = std::max<int64_t>(DRAIN, (total + runs - 1) / runs);
+        n = (total + per - 1) / per;
+    };
+    cut(false, h.pw, h.gw);
+    cut(true, h.ph, h.gh);
+    h.part = slot * (size_t)(std::max(h.gw, h.gh) + h.nt);
+    return h;
+}
+
+template <int S, int NF, bool T>
+cudaError_t product(const float2* W, int64_t N, int F, const uint8_t* tab, float2* part, int64_t per, int64_t runs,
+                    DevStatus* st, cudaStream_t s) {
+    using CF = CtCfg<S, NF>;
+    static bool attr = false;
+    if (!attr) {
+        cudaError_t e = cudaFuncSetAttribute(k_corr_tc<S, NF, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, CF::SMEM);
+        if (e != cudaSuccess) return e;
+        attr = true;
+    }
+    return launch_pdl(k_corr_tc<S, NF, T>, dim3((unsigned)runs), dim3(CT_THREADS), (size_t)CF::SMEM, s, W, N, F, tab,
+                      part, per, st);
+}
+
+template <int S, int NF>
+cudaError_t correct_pass(const Shape& h, const float2* W, int64_t N, const double2* R, int F, double2* X, uint8_t* tab,
+                         float2* part, DevStatus* st, cudaStream_t s) {
+    cudaError_t e;
+    const uint8_t* ct = tab;
+    const float2* pc = part;
+    if ((e = launch_pdl(k_corr_tab<S, NF>, dim3((unsigned)h.kcn), dim3(2 * NF), 0, s, R, N, F, tab)) != cudaSuccess ||
+        (e = product<S, NF, false>(W, N, F, ct, part, h.pw, h.gw, st, s)) != cudaSuccess ||
+        (e = launch_pdl(k_corr_sum_tab<S, NF>, dim3((unsigned)h.kcn), dim3(2 * NF), 0, s, pc, h.nt, h.kcn, F, h.pw,
+                        tab)) != cudaSuccess ||
+        (e = product<S, NF, true>(W, N, F, ct, part, h.ph, h.gh, st, s)) != cudaSuccess ||
+        (e = launch_pdl(k_corr_sum_x, dim3((unsigned)((N + 255) / 256), (unsigned)F), dim3(256), 0, s, pc, N, h.nt,
+                        h.kcn, F, h.ph, X)) != cudaSuccess)
+        return e;
+    return cudaGetLastError();
+}
+
+}  // namespace
+}  // namespace tc
+
+// the fewest frames for which the correction runs on the tensor cores: every count
+// beyond correct_rows_ok. PINV_CORR_TC_MIN_FRAMES: another count.
+static int64_t correct_tc_min_frames() {
+    static const int64_t v = [] {
+        const char* e = std::getenv("PINV_CORR_TC_MIN_FRAMES");
+        return e ? std::max<int64_t>(1, std::atoll(e)) : (int64_t)1;
+    }();
+    return v;
+}
+bool correct_tc_ok(int64_t F) { return F >= correct_tc_min_frames() && tc_available(); }
+
+size_t correct_tc_work_bytes(int64_t N, int64_t F, int slices) {
+    const tc::Shape h = tc::shape(N, F, slices);
+    return h.tab + h.part;
+}
+
+cudaError_t launch_correct_tc(const float2* W32, int64_t N, const double2* R, int64_t F, double2* X, void* work,
+                              int slices, DevStatus* st, cudaStream_t s) {
+    const tc::Shape h = tc::shape(N, F, slices);
+    uint8_t* tab = (uint8_t*)work;
+    float2* part = (float2*)(tab + h.tab);
+    for (int64_t f0 = 0; f0 < F; f0 += 64) {
+        const int Fc = (int)std::min<int64_t>(64, F - f0);
+        const double2* r = R + f0 * N;
+        double2* x = X + f0 * N;
+        cudaError_t e;
+        if (h.nf == 32)
+            e = slices == 3 ? tc::correct_pass<3, 32>(h, W32, N, r, Fc, x, tab, part, st, s)
+                            : tc::correct_pass<2, 32>(h, W32, N, r, Fc, x, tab, part, st, s);
+        else
+            e = slices == 3 ? tc::correct_pass<3, 64>(h, W32, N, r, Fc, x, tab, part, st, s)
+                            : tc::correct_pass<2, 64>(h, W32, N, r, Fc, x, tab, part, st, s);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+}  // namespace pinv

@@ -64,10 +64,10 @@ extern "C" pinv_status pinv_apply_noalloc(pinv_plan* p, const void* d_data, void
                                           void* stream) {
     pinv_status st = apply_check(p, d_data, d_image, F, dtype);
     if (st != PINV_OK || F == 0) return st;
-    // FP64 plans: with the tables of the products on the tensor cores where they fit
+    // with the tables of the tensor-core products where they fit
     size_t need = apply_scratch_layout(p, F, dtype, nullptr, nullptr);
-    const bool oz = need <= (size_t)PINV_NOALLOC_SCRATCH_BYTES;
-    if (!oz) need = apply_scratch_layout(p, F, dtype, nullptr, nullptr, false);
+    const bool roomy = need <= (size_t)PINV_NOALLOC_SCRATCH_BYTES;
+    if (!roomy) need = apply_scratch_layout(p, F, dtype, nullptr, nullptr, false);
     if (need > (size_t)PINV_NOALLOC_SCRATCH_BYTES)
         return set_error(PINV_ERR_INVALID_ARG,
                          "pinv_apply_noalloc needs " + std::to_string(need) + " B of scratch for " +
@@ -76,6 +76,6 @@ extern "C" pinv_status pinv_apply_noalloc(pinv_plan* p, const void* d_data, void
     unsigned char* base = nullptr;
     if ((st = scratch_address(&base)) != PINV_OK) return st;
     ApplyScratch sc;
-    apply_scratch_layout(p, F, dtype, base, &sc, oz);
+    apply_scratch_layout(p, F, dtype, base, &sc, roomy);
     return apply_impl(p, d_data, d_image, F, dtype, (cudaStream_t)stream, sc);
 }

@@ -435,11 +435,11 @@ cudaError_t launch_correct32(const float2* W32, int64_t N, const double2* R, int
 bool correct_rows_ok(int64_t N, int64_t F);
 cudaError_t launch_correct_rows(const float2* W32, int64_t N, const double2* R, int64_t F, float2* T, double2* X,
                                 float2* r32, cudaStream_t s);
-// The same on the tensor cores (split-BF16, split-K with ordered partial sums; `work` of
-// correct_tc_work_elems() float2).
+// The same on the tensor cores (corr_tc.cu; split-BF16, partial sums in order); work of
+// correct_tc_work_bytes(), 256-byte aligned
 bool correct_tc_ok(int64_t F);
-size_t correct_tc_work_elems(int64_t N, int64_t F);
-cudaError_t launch_correct_tc(const float2* W32, int64_t N, const double2* R, int64_t F, float2* T, double2* X,
-                              float2* work, int slices, DevStatus* sched, cudaStream_t s);
+size_t correct_tc_work_bytes(int64_t N, int64_t F, int slices);
+cudaError_t launch_correct_tc(const float2* W32, int64_t N, const double2* R, int64_t F, double2* X, void* work,
+                              int slices, DevStatus* st, cudaStream_t s);
 
 }  // namespace pinv

@@ -31,7 +31,7 @@ struct ApplyScratch {
     bool xfwd;      // the residual's E x and E^H u by the exact tensor-core kernels (plans with B0)
     double2* y128;  // s_c o x [F][C][N] for the exact E x
     float2* apw;    // partials of the tensor-core Recon x data
-    float2* cw;     // partials of the tensor-core correction x += W^H (W r)
+    void* cw;       // table and partials of the tensor-core correction x += W^H (W r), or null: SIMT
     float2* r32;    // FP32 copy of r for the correction of few frames [F][N]
     void* oz;       // tables and partials of the FP64 products on the tensor cores (oz.cu), or
                     // null: on the FP64 pipe
@@ -39,9 +39,10 @@ struct ApplyScratch {
                        // applies of one plan may run concurrently on several streams
 };
 // Bytes an apply of F frames of `dtype` needs; with base != nullptr also
-// carves the region at base into *sc. oz = false: without the tables of the FP64
-// products on the tensor cores (for callers whose scratch cannot hold them).
-size_t apply_scratch_layout(const pinv_plan* p, int64_t F, int dtype, void* base, ApplyScratch* sc, bool oz = true);
+// carves the region at base into *sc. roomy = false: without the tables of the FP64
+// products and of the correction on the tensor cores (for callers whose scratch cannot
+// hold them).
+size_t apply_scratch_layout(const pinv_plan* p, int64_t F, int dtype, void* base, ApplyScratch* sc, bool roomy = true);
 // Argument checks shared by the apply entry points.
 pinv_status apply_check(const pinv_plan* p, const void* d_data, void* d_image, int64_t F, int dtype);
 // image = Recon x data (or G^-1 E^H data) plus refinement on stream s, using
@@ -130,7 +131,7 @@ struct pinv_plan {
     // pinv_apply's scratch region, grown on demand
     void* scratch_buf = nullptr;
     size_t scratch_bytes = 0;
-    bool scratch_small = false;  // the region with the FP64 products' tables could not be had
+    bool scratch_small = false;  // the region with the tensor-core tables could not be had
 
     cudaEvent_t ev[10] = {};  // build stages 0-5; 6-7 around the Gram kernels; 8-9 around the condition estimate
     int last_refine_iters = 0;

@@ -329,8 +329,8 @@ bool pinv_server::dispatch_one(std::unique_lock<std::mutex>& lk) {
     if (st == PINV_OK && F > 0) {
         const size_t es = q.dtype == PINV_C128 ? 16 : 8;
         const int64_t rows = r.plan->M, n = r.plan->N;
-        // FP64 plans: with the tables of the products on the tensor cores where there is room
-        bool oz = true;
+        // with the tables of the tensor-core products where there is room
+        bool roomy = true;
         size_t base = (apply_scratch_layout(r.plan, F, q.dtype, nullptr, nullptr) + 255) & ~(size_t)255;
         const size_t dbytes = more.empty() ? 0 : (((size_t)F * rows * es + 255) & ~(size_t)255);
         const size_t tail = dbytes + (more.empty() ? 0 : (size_t)F * n * es);
@@ -341,7 +341,7 @@ bool pinv_server::dispatch_one(std::unique_lock<std::mutex>& lk) {
             slot->scratch_bytes = 0;
             if (cudaMalloc(&slot->scratch, need) != cudaSuccess) {
                 cudaGetLastError();
-                oz = false;
+                roomy = false;
                 base = (apply_scratch_layout(r.plan, F, q.dtype, nullptr, nullptr, false) + 255) & ~(size_t)255;
                 need = base + tail;
                 if (cudaMalloc(&slot->scratch, need) != cudaSuccess) st = set_error(PINV_ERR_OOM, "slot scratch");
@@ -350,7 +350,7 @@ bool pinv_server::dispatch_one(std::unique_lock<std::mutex>& lk) {
         }
         if (st == PINV_OK) {
             ApplyScratch sc;
-            apply_scratch_layout(r.plan, F, q.dtype, slot->scratch, &sc, oz);
+            apply_scratch_layout(r.plan, F, q.dtype, slot->scratch, &sc, roomy);
             uint8_t* dbuf = (uint8_t*)slot->scratch + base;  // merged: frames gathered here
             uint8_t* ibuf = dbuf + dbytes;                   // and their images
             const void* data = q.data;

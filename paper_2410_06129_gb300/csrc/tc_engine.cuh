@@ -276,6 +276,33 @@ __device__ inline void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.alig
 // byte offset of (row r, 8-wide k' group g in 0..3) in a [R][32] K-major no-swizzle tile
 __device__ inline uint32_t koff(int r, int g) { return (uint32_t)((r >> 3) * 512 + g * 128 + (r & 7) * 16); }
 
+// 8 consecutive values from a 16-byte aligned address
+__device__ inline void ld8a(const float2* p, float2 (&v)[8]) {
+    const float4* q = reinterpret_cast<const float4*>(p);
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+        const float4 w = __ldg(q + t);
+        v[2 * t] = make_float2(w.x, w.y);
+        v[2 * t + 1] = make_float2(w.z, w.w);
+    }
+}
+
+// 8 consecutive FP32 complex values p[0..7] (zero past `avail`)
+__device__ inline void load8f(const float2* p, int avail, float2 (&v)[8]) {
+    if (avail >= 8 && (((uintptr_t)p) & 15) == 0) {
+        ld8a(p, v);
+        return;
+    }
+#pragma unroll
+    for (int t = 0; t < 8; ++t) v[t] = t < avail ? __ldg(p + t) : make_float2(0.f, 0.f);
+}
+
+// 8 values down a column: p[0], p[ld], ..., p[7 ld] (zero past `avail`)
+__device__ inline void load8col(const float2* p, int64_t ld, int avail, float2 (&v)[8]) {
+#pragma unroll
+    for (int t = 0; t < 8; ++t) v[t] = t < avail ? __ldg(p + t * ld) : make_float2(0.f, 0.f);
+}
+
 // split 8 floats into S bf16 slices, packed 2 per word: w[s][0..3]
 template <int S>
 __device__ inline void split8(float (&x)[8], uint32_t (&w)[S][4]) {

@@ -24,33 +24,6 @@ __device__ inline float2 cmulf(float2 a, float2 b) {
 }
 __device__ inline float2 conjf2(float2 a) { return make_float2(a.x, -a.y); }
 
-// 8 consecutive values from a 16-byte aligned address
-__device__ inline void ld8a(const float2* p, float2 (&v)[8]) {
-    const float4* q = reinterpret_cast<const float4*>(p);
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-        const float4 w = __ldg(q + t);
-        v[2 * t] = make_float2(w.x, w.y);
-        v[2 * t + 1] = make_float2(w.z, w.w);
-    }
-}
-
-// 8 consecutive FP32 complex values p[0..7] (zero past `avail`)
-__device__ inline void load8f(const float2* p, int avail, float2 (&v)[8]) {
-    if (avail >= 8 && (((uintptr_t)p) & 15) == 0) {
-        ld8a(p, v);
-        return;
-    }
-#pragma unroll
-    for (int t = 0; t < 8; ++t) v[t] = t < avail ? __ldg(p + t) : make_float2(0.f, 0.f);
-}
-
-// 8 values down a column: p[0], p[ld], ..., p[7 ld] (zero past `avail`)
-__device__ inline void load8col(const float2* p, int64_t ld, int avail, float2 (&v)[8]) {
-#pragma unroll
-    for (int t = 0; t < 8; ++t) v[t] = t < avail ? __ldg(p + t * ld) : make_float2(0.f, 0.f);
-}
-
 // A row of a memory operand: pointer to its first element and a validity flag.
 struct RowPtr {
     const float2* p;
@@ -367,75 +340,6 @@ struct GramBulk {
     __device__ bool row_ok(int64_t i) const { return i % (nt * BM) < e.N; }
     __device__ bool col_ok(int64_t j) const { return j < e.N; }
     __device__ void store(int64_t, int64_t, float2) const {}
-};
-
-// ------------------------------------------------------------------ refinement correction
-// x += W^H (W r) for a block of frames (F <= BN), in two split-K products whose
-// partial sums (one per range of k, `chunk` wide) are added in order afterwards:
-//   CorrW   T[f][i]  = sum_{k <= i} W[i][k] r[f][k]
-//   CorrWH  X[f][n] += sum_{k >= n} conj(W[k][n]) T[f][k]
-// The column coordinate carries the k range: column j is frame j % BN of split j / BN.
-__device__ inline void load8d(const double2* p, int avail, float2 (&v)[8]) {
-#pragma unroll
-    for (int t = 0; t < 8; ++t) {
-        const double2 a = t < avail ? p[t] : make_double2(0.0, 0.0);
-        v[t] = make_float2((float)a.x, (float)a.y);
-    }
-}
-struct CorrW {
-    static constexpr bool kPrefetch = true;  // W streams from HBM
-    const float2* W;
-    const double2* R;  // [F][N]
-    float2* part;      // [splits][F][N]
-    int64_t N, F, chunk;
-    __device__ bool tile(int64_t bx, int64_t by, int64_t& i0, int64_t& j0, int64_t& kb, int64_t& ke) const {
-        i0 = by * BM;
-        j0 = bx * BN;
-        kb = bx * chunk;
-        ke = kb + chunk;
-        const int64_t kmax = i0 + BM < N ? i0 + BM : N;  // W is lower triangular
-        if (ke > kmax) ke = kmax;
-        return kb < ke;
-    }
-    __device__ RowPtr row_a(int64_t i) const { return RowPtr{W + (i < N ? i : 0) * N, i < N}; }
-    __device__ int64_t row_b(int64_t j) const { return j % BN; }
-    __device__ void a8(const RowPtr& r, int64_t k, int64_t ke, float2 (&v)[8]) const {
-        load8f(r.p + k, r.ok ? (int)(ke - k) : 0, v);
-    }
-    __device__ void b8(int64_t f, int64_t k, int64_t ke, float2 (&v)[8]) const {
-        load8d(R + (f < F ? f : 0) * N + k, f < F ? (int)(ke - k) : 0, v);
-    }
-    __device__ bool row_ok(int64_t i) const { return i < N; }
-    __device__ bool col_ok(int64_t j) const { return j % BN < F; }
-    __device__ void store(int64_t i, int64_t j, float2 v) const { part[((j / BN) * F + j % BN) * N + i] = v; }
-};
-struct CorrWH {
-    static constexpr bool kPrefetch = true;  // W streams from HBM
-    const float2* W;
-    const float2* T;  // [F][N]
-    float2* part;     // [splits][F][N]
-    int64_t N, F, chunk;
-    __device__ bool tile(int64_t bx, int64_t by, int64_t& i0, int64_t& j0, int64_t& kb, int64_t& ke) const {
-        i0 = by * BM;
-        j0 = bx * BN;
-        kb = bx * chunk;
-        if (kb < i0) kb = i0;  // W is lower triangular: k >= n
-        ke = (bx + 1) * chunk < N ? (bx + 1) * chunk : N;
-        return kb < ke;
-    }
-    __device__ int64_t row_a(int64_t i) const { return i; }
-    __device__ int64_t row_b(int64_t j) const { return j % BN; }
-    __device__ void a8(int64_t n, int64_t k, int64_t ke, float2 (&v)[8]) const {
-        load8col(W + k * N + (n < N ? n : 0), N, n < N ? (int)(ke - k) : 0, v);
-#pragma unroll
-        for (int t = 0; t < 8; ++t) v[t].y = -v[t].y;
-    }
-    __device__ void b8(int64_t f, int64_t k, int64_t ke, float2 (&v)[8]) const {
-        load8f(T + (f < F ? f : 0) * N + k, f < F ? (int)(ke - k) : 0, v);
-    }
-    __device__ bool row_ok(int64_t i) const { return i < N; }
-    __device__ bool col_ok(int64_t j) const { return j % BN < F; }
-    __device__ void store(int64_t i, int64_t j, float2 v) const { part[((j / BN) * F + j % BN) * N + i] = v; }
 };
 
 // ------------------------------------------------------------------ Recon, bulk-fed
@@ -1512,102 +1416,6 @@ cudaError_t launch_recon_bulk(const EncodeDev& e, const float2* W32, int slices,
         if ((err = run(p1, dim3((unsigned)items, 1), slices, st, 2, s)) != cudaSuccess) return err;
         const tc::ReconB2 p2 = recon_b2_problem(e, slices, R, work, c, &items);
         if ((err = run(p2, dim3((unsigned)items, 1), slices, st, 8, s)) != cudaSuccess) return err;
-    }
-    return cudaSuccess;
-}
-
-// ------------------------------------------------------------------ refinement correction (host)
-namespace {
-// k ranges of the correction: about two tiles per SM, at least 256 wide
-// k chunk of the correction's triangular products: row tile r holds the
-// nonempty chunks below min((r + 1) BM, N); the chunk that minimises whole waves of
-// those tiles x (chunk + per-tile overhead), at least 256 columns
-int64_t correct_tc_chunk(int64_t N) {
-    const int64_t rows = (N + tc::BM - 1) / tc::BM, sms = tc::sm_count();
-    const int64_t hi = std::max<int64_t>(1, std::min<int64_t>(64, N / 256));
-    int64_t best = 0;
-    double bt = 0.0;
-    for (int64_t sp = 1; sp <= hi; ++sp) {
-        const int64_t chunk = ((N + sp - 1) / sp + tc::KC - 1) / tc::KC * tc::KC;
-        int64_t tiles = 0;
-        for (int64_t r = 0; r < rows; ++r) tiles += (std::min<int64_t>((r + 1) * tc::BM, N) + chunk - 1) / chunk;
-        const double t = (double)((tiles + sms - 1) / sms) * (double)(chunk + 256);
-        if (best == 0 || t < bt * (1.0 - 1e-9)) {
-            bt = t;
-            best = chunk;
-        }
-    }
-    return best;
-}
-}  // namespace
-
-// T[f][i] = sum of the nonempty splits (k range below the end of i's row tile), in order
-__global__ void k_corr_reduce_w(const float2* __restrict__ part, int64_t N, int64_t F, int64_t chunk,
-                                float2* __restrict__ T) {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= N * F) return;
-    const int64_t f = idx / N, i = idx - f * N;
-    const int64_t kend = (i / tc::BM + 1) * tc::BM, kmax = kend < N ? kend : N;
-    float2 a = make_float2(0.f, 0.f);
-    for (int64_t sp = 0; sp * chunk < kmax; ++sp) {
-        const float2 b = part[(sp * F + f) * N + i];
-        a.x += b.x;
-        a.y += b.y;
-    }
-    T[f * N + i] = a;
-}
-// X[f][n] += sum of the nonempty splits (k range reaching n's row tile), in order
-__global__ void k_corr_reduce_wh(const float2* __restrict__ part, int64_t N, int64_t F, int64_t chunk,
-                                 double2* __restrict__ X) {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= N * F) return;
-    const int64_t f = idx / N, n = idx - f * N;
-    const int64_t n0 = n / tc::BM * tc::BM;
-    double2 a = make_double2(0.0, 0.0);
-    for (int64_t sp = n0 / chunk; sp * chunk < N; ++sp) {
-        const float2 b = part[(sp * F + f) * N + n];
-        a.x += (double)b.x;
-        a.y += (double)b.y;
-    }
-    double2 x = X[f * N + n];
-    X[f * N + n] = make_double2(x.x + a.x, x.y + a.y);
-}
-
-// the fewest frames for which the refinement's correction runs on the tensor cores:
-// every count (a 64x64 apply of 1-6 frames: 5.4 ms with the SIMT W products, 1.8 ms
-// here). PINV_CORR_TC_MIN_FRAMES: another count.
-static int64_t correct_tc_min_frames() {
-    static const int64_t v = [] {
-        const char* e = std::getenv("PINV_CORR_TC_MIN_FRAMES");
-        return e ? std::max<int64_t>(1, std::atoll(e)) : (int64_t)1;
-    }();
-    return v;
-}
-bool correct_tc_ok(int64_t F) { return F >= correct_tc_min_frames() && tc_available(); }
-
-size_t correct_tc_work_elems(int64_t N, int64_t F) {
-    const int64_t chunk = correct_tc_chunk(N), sp = (N + chunk - 1) / chunk;
-    return (size_t)(sp * std::min<int64_t>(F, tc::BN) * N);
-}
-
-cudaError_t launch_correct_tc(const float2* W32, int64_t N, const double2* R, int64_t F, float2* T, double2* X,
-                              float2* work, int slices, DevStatus* sched, cudaStream_t s) {
-    const int64_t chunk = correct_tc_chunk(N), sp = (N + chunk - 1) / chunk;
-    for (int64_t f0 = 0; f0 < F; f0 += tc::BN) {
-        const int64_t Fc = std::min<int64_t>(tc::BN, F - f0);
-        const int64_t n = N * Fc;
-        const unsigned rb = (unsigned)((n + 255) / 256);
-        tc::CorrW p1{W32, R + f0 * N, work, N, Fc, chunk};
-        cudaError_t e = run(p1, dim3((unsigned)sp, cdiv(N, tc::BM)), slices, sched, 10, s);
-        if (e != cudaSuccess) return e;
-        k_corr_reduce_w<<<rb, 256, 0, s>>>(work, N, Fc, chunk, T + f0 * N);
-        note_launch();
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        tc::CorrWH p2{W32, T + f0 * N, work, N, Fc, chunk};
-        if ((e = run(p2, dim3((unsigned)sp, cdiv(N, tc::BM)), slices, sched, 11, s)) != cudaSuccess) return e;
-        k_corr_reduce_wh<<<rb, 256, 0, s>>>(work, N, Fc, chunk, X + f0 * N);
-        note_launch();
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     return cudaSuccess;
 }

@@ -124,3 +124,28 @@ def test_correction_of_few_frames(dims, frames):
     amp = np.linalg.norm(np.abs(W).T @ (np.abs(W) @ np.abs(b))) / np.linalg.norm(want)
     # two FP32 passes, and W and b rounded to FP32
     assert rel(x, want) < (2 * 4 * np.sqrt(N) + 4) * 2.0 ** -24 * amp
+
+
+# the correction of many frames: one row tile, ragged last tiles and stages, odd N (rows off 16
+# bytes), one and two passes of 64, both tile widths; x = W^H (W b) as the factor-only apply
+@pytest.mark.parametrize("prec,ulp", [(L.MIXED_BF16X6, 2.0 ** -24), (L.MIXED_BF16X3, 2.0 ** -16)])
+@pytest.mark.parametrize("dims,frames", [((37,), 49), ((128,), 64), ((129,), 65), ((255,), 130), ((33, 17), 17),
+                                         ((24, 24), 32), ((31, 33), 33), ((40, 41), 64)])
+def test_correction_many_frames(dims, frames, prec, ulp):
+    """lambda = mean diag: W^H (W b) is off by a few kappa ulp (FP32 or two-slice products and
+    FP32 sums), and one refinement step by the square of that or the FP32 output."""
+    from paper_2410_06129_gb300.plan import Plan
+    rng = np.random.default_rng(2207)
+    N, D = int(np.prod(dims)), len(dims)
+    k = rng.uniform(-0.5 * max(dims), 0.5 * max(dims), size=(2 * N, D))
+    maps = np.exp(2j * np.pi * rng.random((2, N)))
+    E = O.encode(k, O.voxel_positions(dims), maps, None, None)
+    G = E.conj().T @ E + O.lambda_abs(E, 1.0) * np.eye(N)
+    kappa = np.linalg.cond(G)
+    d = rng.standard_normal((frames, 2, 2 * N)) + 1j * rng.standard_normal((frames, 2, 2 * N))
+    want = np.linalg.solve(G, E.conj().T @ d.reshape(frames, -1).T).T
+    for iters, tol in ((0, 64 * kappa * ulp), (2, 64 * kappa * 2.0 ** -40 + (64 * kappa * ulp) ** 2)):
+        with Plan(dims, k, maps, lam=1.0, precision=prec, recon_mode=L.RECON_NONE, refine_max_iters=iters) as pl:
+            x = pl.build().apply(torch.from_numpy(d).cuda()).cpu().numpy()
+        for f in (0, frames // 2, frames - 1):
+            assert rel(x[f], want[f]) < tol
