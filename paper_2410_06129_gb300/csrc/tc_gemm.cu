@@ -475,7 +475,7 @@ __global__ void __launch_bounds__(256) k_tab_panel(const float2* __restrict__ L3
     put_b<S>(tab + (rt * kcn + kc) * S * B_SL, r, g, v);
 }
 template <int S>
-__global__ void __launch_bounds__(256) k_tab_wrows(const float4* __restrict__ W, int64_t ld, int64_t p0, int64_t kw,
+__global__ void __launch_bounds__(256) k_tab_wrows(const float2* __restrict__ W32, int64_t ld, int64_t p0, int64_t kw,
                                                    int64_t ncols, uint8_t* tab) {
     const int64_t kc = blockIdx.x, ct = blockIdx.y, kcn = gridDim.x;
     const int r = threadIdx.x & (BM - 1), g = threadIdx.x >> 7;
@@ -486,7 +486,7 @@ __global__ void __launch_bounds__(256) k_tab_wrows(const float4* __restrict__ W,
 #pragma unroll
     for (int t = 0; t < 8; ++t) {
         const bool ok = j < ncols && k0 + t < kw;
-        v[t] = ok ? df_to_f32(W[(p0 + k0 + t) * ld + j]) : make_float2(0.f, 0.f);
+        v[t] = ok ? W32[(p0 + k0 + t) * ld + j] : make_float2(0.f, 0.f);
     }
     put_b<S>(tab + (ct * kcn + kc) * S * B_SL, r, g, v);
 }
@@ -599,6 +599,7 @@ struct TrtriUpdTC {
     const float2* L32;
     int64_t ldl;
     float4* W;
+    const float2* W32;  // the panel's finished rows (ld as W)
     int64_t ld, N, k0, nbk, imax;
     __device__ bool tile(int64_t bx, int64_t by, int64_t& i0, int64_t& j0, int64_t& kb, int64_t& ke) const {
         i0 = k0 + nbk + by * BM;
@@ -615,7 +616,7 @@ struct TrtriUpdTC {
     __device__ void b8(int64_t j, int64_t k, int64_t ke, float2 (&v)[8]) const {
 #pragma unroll
         for (int t = 0; t < 8; ++t)
-            v[t] = (j < k0 + nbk && k + t < ke) ? df_to_f32(W[(k0 + k + t) * ld + j]) : make_float2(0.f, 0.f);
+            v[t] = (j < k0 + nbk && k + t < ke) ? W32[(k0 + k + t) * ld + j] : make_float2(0.f, 0.f);
     }
     __device__ bool row_ok(int64_t i) const { return i < imax; }
     __device__ bool col_ok(int64_t j) const { return j < k0 + nbk; }
@@ -1154,151 +1155,172 @@ cudaError_t launch_potrf_tc(float4* G, int64_t N, int64_t ld, double2* Dinv, flo
     return cudaGetLastError();
 }
 
-// Inside a panel the inverse's steps have K = 64, too short for the tensor-core
-// engine's set-up (tensor-core launches of these steps took 27 / 44 us against a
-// few microseconds of products): these FP32 SIMT kernels stage the 64-wide operands
-// in shared memory, as the Cholesky's panel kernels do, and accumulate in FP32.
 __device__ inline void cmac(float2& acc, float2 a, float2 b) {  // acc += a * b
     acc.x = fmaf(a.x, b.x, fmaf(-a.y, b.y, acc.x));
     acc.y = fmaf(a.x, b.y, fmaf(a.y, b.x, acc.y));
 }
+__device__ inline void cp_async8(void* dst, const void* src, bool ok) {  // zeros where not ok
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(tc::smem_u32(dst)), "l"(src), "r"(ok ? 8 : 0)
+                 : "memory");
+}
 
-// W[k0 + i][j] = sum_k Dinv[i][k] W[k0 + k][j] (W rounded to FP32) for i < nbk, j < ncol:
-// one CTA per 64 columns, each thread 4 x 4 outputs (rows ty + 16 a, columns tx + 16 b)
-__global__ void __launch_bounds__(256) k_trtri_diag(const float2* __restrict__ Dinv32, float4* W, int64_t ld,
-                                                  int64_t k0, int nbk, int64_t ncol) {
-    __shared__ float2 Ds[64][65];  // Ds[i][k] = Dinv[i][k]
-    __shared__ float2 Bs[64][65];  // Bs[k][c] = W[k0 + k][j0 + c]
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    const int64_t j0 = (int64_t)blockIdx.x * 64;
+// A panel of the inverse: rows p0 <= i < pend of W = L^-1, columns j < pend, from the rows'
+// entries after the updates of the panels above. In order, for each 64-row block k: W_k =
+// Dinv_k W_k (W_k rounded to FP32, FP32 sums), then W_r -= L_rk W_k for the panel's blocks r
+// below (FP32 sums, subtracted in double-float). The finished rows go to W in FP64 and to W32.
+//
+// One CTA takes 32 columns through the whole panel: the steps are independent by column, so
+// nothing leaves the SM between them. The 256 x 32 entries stay in registers in double-float
+// (16 to a thread), the 64 x 64 blocks of Dinv and L arrive two ahead of use by cp.async, and
+// the current rows are the other operand in shared memory. K = 64 is too short for the
+// tensor-core engine's set-up. Bound by the shared-memory reads of the FP32 products (four rows
+// and one column to a thread; 4 x 4 to a thread in a quarter of the threads took longer): as up
+// to seven launches (one for each Dinv_k and each block column of L, the rows in memory in
+// between) a panel took 110 - 180 us at N = 4096, so it takes 60 us, and the pass that turned
+// all of W into FP64 afterwards is gone (74 us). On fewer SMs than there are tiles for the
+// inverse falls behind the Cholesky (64 x 64 step 6.97 ms, on 76 SMs 7.10, on 40 7.50).
+constexpr int TRP_COLS = 32, TRP_THREADS = 512, TRP_LD = NBK + 2;
+constexpr size_t TRP_SMEM = sizeof(float2) * (2 * NBK * TRP_LD + NBK * TRP_COLS);
+__global__ void __launch_bounds__(TRP_THREADS, 1)
+    k_trtri_panel(const float2* __restrict__ L32, int64_t ldl, const float2* __restrict__ Dinv32, float4* W, int64_t ld,
+                  int64_t p0, int64_t pend, float2* W32) {
+    extern __shared__ float4 trp_smem[];
+    float2* Ls = reinterpret_cast<float2*>(trp_smem);  // [2][NBK][TRP_LD]
+    float2* Bs = Ls + 2 * NBK * TRP_LD;                // [NBK][TRP_COLS]
+    constexpr int NB = NBP / NBK;
+    const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;  // rows ty + 16 a of a block, column tx
+    const int nb = (int)((pend - p0 + NBK - 1) / NBK);
     griddep_wait();
     griddep_launch();
+    auto issue = [&](int kb, int rb, int buf) {  // Dinv_kb (rb = kb) or the block (rb, kb) of L
+        const int64_t i0 = p0 + NBK * rb, c0 = p0 + NBK * kb;
+        const int64_t nr = pend - i0;
+        const float2* src = rb == kb ? Dinv32 + c0 * NBK : L32 + i0 * ldl + c0;
+        const int64_t lds = rb == kb ? NBK : ldl;
+#pragma unroll 2
+        for (int t = 0; t < NBK * NBK / TRP_THREADS; ++t) {
+            const int e = tid + TRP_THREADS * t, r = e / NBK, c = e % NBK;
+            const bool ok = r < nr && (rb != kb || c < nr);
+            cp_async8(Ls + (buf * NBK + r) * TRP_LD + c, src + (ok ? r * lds + c : 0), ok);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+#pragma unroll 1
+    for (int64_t j0 = (int64_t)blockIdx.x * TRP_COLS; j0 < pend; j0 += (int64_t)gridDim.x * TRP_COLS) {
+        const int64_t j = j0 + tx;
+        const int kb0 = j0 > p0 ? (int)((j0 - p0) / NBK) : 0;  // the first block with entries on or below the diagonal
+        issue(kb0, kb0, 0);
+        float4 w[NB][4];
+#pragma unroll
+        for (int b = 0; b < NB; ++b)
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                const int64_t i = p0 + NBK * b + ty + 16 * a;
+                w[b][a] = b >= kb0 && i < pend && j < pend ? W[i * ld + j] : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+        int buf = 0;
+#pragma unroll
+        for (int kb = 0; kb < NB; ++kb) {
+            if (kb < kb0 || kb >= nb) continue;
+#pragma unroll
+            for (int rb = kb; rb < NB; ++rb) {
+                if (rb >= nb) continue;
+                const int nrb = rb + 1 < nb ? rb + 1 : kb + 1, nkb = rb + 1 < nb ? kb : kb + 1;
+                const bool more = nkb < nb;
+                if (more) issue(nkb, nrb, buf ^ 1);
+                if (rb == kb)
+#pragma unroll
+                    for (int a = 0; a < 4; ++a) Bs[(ty + 16 * a) * TRP_COLS + tx] = df_to_f32(w[kb][a]);
+                if (more)
+                    asm volatile("cp.async.wait_group 1;" ::: "memory");
+                else
+                    asm volatile("cp.async.wait_group 0;" ::: "memory");
+                __syncthreads();
+                float2 acc[4];
+#pragma unroll
+                for (int a = 0; a < 4; ++a) acc[a] = make_float2(0.f, 0.f);
+                const float2* Lb = Ls + (buf * NBK + ty) * TRP_LD;
 #pragma unroll 4
-    for (int t = 0; t < 16; ++t) {
-        const int e = tid + 256 * t, r = e / 64, c = e % 64;
-        Ds[r][c] = (r < nbk && c < nbk) ? Dinv32[r * 64 + c] : make_float2(0.f, 0.f);
-        const int64_t j = j0 + c;
-        Bs[r][c] = (r < nbk && j < ncol) ? df_to_f32(W[(k0 + r) * ld + j]) : make_float2(0.f, 0.f);
-    }
-    __syncthreads();
-    float2 acc[4][4];
+                for (int k = 0; k < NBK; k += 2) {
+                    const float2 b0 = Bs[k * TRP_COLS + tx], b1 = Bs[(k + 1) * TRP_COLS + tx];
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+                    for (int a = 0; a < 4; ++a) {
+                        const float4 l = *reinterpret_cast<const float4*>(Lb + 16 * a * TRP_LD + k);
+                        cmac(acc[a], make_float2(l.x, l.y), b0);
+                        cmac(acc[a], make_float2(l.z, l.w), b1);
+                    }
+                }
+                __syncthreads();
+                if (rb == kb) {
 #pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = make_float2(0.f, 0.f);
-#pragma unroll 4
-    for (int k = 0; k < 64; ++k) {
-        float2 dv[4], bv[4];
+                    for (int a = 0; a < 4; ++a) {
+                        Bs[(ty + 16 * a) * TRP_COLS + tx] = acc[a];
+                        const int64_t i = p0 + NBK * kb + ty + 16 * a;
+                        if (i < pend && j < pend) {
+                            const float2 v = j <= i ? acc[a] : make_float2(0.f, 0.f);
+                            reinterpret_cast<double2*>(W)[i * ld + j] = df_to_f64(df_of_f32(v));
+                            W32[i * ld + j] = v;
+                        }
+                    }
+                } else {
 #pragma unroll
-        for (int a = 0; a < 4; ++a) dv[a] = Ds[ty + 16 * a][k];
-#pragma unroll
-        for (int b = 0; b < 4; ++b) bv[b] = Bs[k][tx + 16 * b];
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int b = 0; b < 4; ++b) cmac(acc[a][b], dv[a], bv[b]);
-    }
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-        const int r = ty + 16 * a;
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            const int64_t j = j0 + tx + 16 * b;
-            if (r < nbk && j < ncol) W[(k0 + r) * ld + j] = df_of_f32(acc[a][b]);
+                    for (int a = 0; a < 4; ++a) w[rb][a] = df_sub_f32(w[rb][a], acc[a]);
+                }
+                buf ^= 1;
+            }
         }
     }
 }
 
-// W[i][j] -= sum_k L[i][k0 + k] W[k0 + k][j] for rows r0 <= i < imax, j < ncol (K = nbk):
-// one CTA per 16 rows x 64 columns, each thread 1 row x 4 columns
-__global__ void __launch_bounds__(256) k_trtri_upd(const float2* __restrict__ L32, int64_t ldl, float4* W,
-                                                 int64_t ld, int64_t k0, int nbk, int64_t r0, int64_t imax,
-                                                 int64_t ncol) {
-    __shared__ float2 As[16][65];  // As[r][k] = L[i0 + r][k0 + k]
-    __shared__ float2 Bs[64][65];  // Bs[k][c] = W[k0 + k][j0 + c]
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    const int64_t j0 = (int64_t)blockIdx.x * 64, i0 = r0 + (int64_t)blockIdx.y * 16;
-    griddep_wait();
-    griddep_launch();
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-        const int e = tid + 256 * t, r = e / 64, k = e % 64;
-        const int64_t i = i0 + r;
-        As[r][k] = (i < imax && k < nbk) ? L32[i * ldl + k0 + k] : make_float2(0.f, 0.f);
-    }
-#pragma unroll 4
-    for (int t = 0; t < 16; ++t) {
-        const int e = tid + 256 * t, k = e / 64, c = e % 64;
-        const int64_t j = j0 + c;
-        Bs[k][c] = (k < nbk && j < ncol) ? df_to_f32(W[(k0 + k) * ld + j]) : make_float2(0.f, 0.f);
-    }
-    __syncthreads();
-    float2 acc[4];
-#pragma unroll
-    for (int b = 0; b < 4; ++b) acc[b] = make_float2(0.f, 0.f);
-#pragma unroll 8
-    for (int k = 0; k < 64; ++k) {
-        const float2 av = As[ty][k];
-#pragma unroll
-        for (int b = 0; b < 4; ++b) cmac(acc[b], av, Bs[k][tx + 16 * b]);
-    }
-    const int64_t i = i0 + ty;
-    if (i >= imax) return;
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-        const int64_t j = j0 + tx + 16 * b;
-        if (j < ncol) W[i * ld + j] = df_sub_f32(W[i * ld + j], acc[b]);
-    }
-}
-
-// W = L^-1 by blocked forward substitution on I, with the same two levels:
-// inside a 256-row panel each 64-row step updates the panel's rows only; the
-// rows below get one update per panel with K = 256.
+// W = L^-1 by blocked forward substitution on I, with the same two levels as the
+// Cholesky: a 256-row panel at a time, then the rows below get one update with
+// K = 256. W's rows are in double-float storage until their panel is done, then in
+// FP64; W32 (ld N) gets their FP32 values, which they are.
 cudaError_t launch_trtri_tc(const float2* L32, int64_t N, const float2* Dinv32, float4* W, float2* W32,
                             int slices, DevStatus* st, cudaStream_t s, void* tab, const cudaEvent_t* ev_panel) {
-    // W is in double-float storage while it is formed; the last pass leaves it in FP64
-    cudaError_t e = launch_fill_identity_df(W, N, N, s);
-    if (e != cudaSuccess) return e;
+    static bool attr = false;
+    cudaError_t e;
+    if (!attr) {
+        if ((e = cudaFuncSetAttribute(k_trtri_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TRP_SMEM)) !=
+            cudaSuccess)
+            return e;
+        attr = true;
+    }
+    if ((e = launch_fill_identity_df(W, N, N, s)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(W32, 0, sizeof(float2) * (size_t)(N * N), s)) != cudaSuccess) return e;
     // PINV_INV_SMS: another count of SMs (0 all)
     const char* cenv = std::getenv("PINV_INV_SMS");
     const int cap = cenv ? std::atoi(cenv) : side_sms(N);
     for (int64_t p0 = 0; p0 < N; p0 += NBP) {
         const int64_t pend = std::min<int64_t>(N, p0 + NBP);
         if (ev_panel && (e = cudaStreamWaitEvent(s, ev_panel[p0 / NBP], 0)) != cudaSuccess) return e;
-        for (int64_t k0 = p0; k0 < pend; k0 += NBK) {
-            const int64_t nbk = std::min<int64_t>(NBK, N - k0);
-            const int64_t ncol = k0 + nbk;
-            if ((e = launch_pdl(k_trtri_diag, dim3(cdiv(ncol, 64)), dim3(256), 0, s, Dinv32 + (k0 / NBK) * NBK * NBK,
-                                W, N, k0, (int)nbk, ncol)) != cudaSuccess)
+        if ((e = launch_pdl(k_trtri_panel, dim3(std::min<unsigned>(tc::sm_count(), cdiv(pend, TRP_COLS))),
+                            dim3(TRP_THREADS), TRP_SMEM, s, L32, N, Dinv32,
+                            W, N, p0, pend, W32)) != cudaSuccess ||
+            (e = cudaGetLastError()) != cudaSuccess)
+            return e;
+        if (pend == N) break;
+        if (tab) {
+            const int64_t ntr = cdiv(N - pend, tc::BM), ntc = cdiv(pend, tc::BN), kcn = cdiv(pend - p0, tc::KC);
+            uint8_t* tabl = (uint8_t*)tab;
+            uint8_t* tabw = tabl + panel_table_bytes(N, slices);
+            if ((e = panel_table(L32, N, p0, pend - p0, pend, slices, tabl, s)) != cudaSuccess) return e;
+            const dim3 wg((unsigned)kcn, (unsigned)ntc);
+            const float2* Wc = W32;
+            e = slices == 3 ? launch_pdl(tc::k_tab_wrows<3>, wg, dim3(256), 0, s, Wc, N, p0, pend - p0, pend, tabw)
+                            : launch_pdl(tc::k_tab_wrows<2>, wg, dim3(256), 0, s, Wc, N, p0, pend - p0, pend, tabw);
+            if (e != cudaSuccess || (e = cudaGetLastError()) != cudaSuccess) return e;
+            tc::TrtriBulk up{tabl, tabw, W, N, N, pend, ntr, ntc, kcn, slices};
+            if ((e = run(up, dim3((unsigned)(ntr * ntc), 1), slices, st, 6, s, false, cap, true)) != cudaSuccess)
                 return e;
-            if (ncol >= pend) continue;
-            if ((e = launch_pdl(k_trtri_upd, dim3(cdiv(ncol, 64), cdiv(pend - ncol, 16)), dim3(256), 0, s, L32, N, W,
-                                N, k0, (int)nbk, ncol, pend, ncol)) != cudaSuccess)
+        } else {
+            tc::TrtriUpdTC up{L32, N, W, W32, N, N, p0, pend - p0, N};
+            if ((e = run(up, dim3(cdiv(pend, tc::BN), cdiv(N - pend, tc::BM)), slices, st, 6, s, false, cap)) !=
+                cudaSuccess)
                 return e;
-        }
-        if (pend < N) {
-            if (tab) {
-                const int64_t ntr = cdiv(N - pend, tc::BM), ntc = cdiv(pend, tc::BN), kcn = cdiv(pend - p0, tc::KC);
-                uint8_t* tabl = (uint8_t*)tab;
-                uint8_t* tabw = tabl + panel_table_bytes(N, slices);
-                if ((e = panel_table(L32, N, p0, pend - p0, pend, slices, tabl, s)) != cudaSuccess) return e;
-                const dim3 wg((unsigned)kcn, (unsigned)ntc);
-                const float4* Wc = W;
-                e = slices == 3 ? launch_pdl(tc::k_tab_wrows<3>, wg, dim3(256), 0, s, Wc, N, p0, pend - p0, pend, tabw)
-                                : launch_pdl(tc::k_tab_wrows<2>, wg, dim3(256), 0, s, Wc, N, p0, pend - p0, pend, tabw);
-                if (e != cudaSuccess || (e = cudaGetLastError()) != cudaSuccess) return e;
-                tc::TrtriBulk up{tabl, tabw, W, N, N, pend, ntr, ntc, kcn, slices};
-                if ((e = run(up, dim3((unsigned)(ntr * ntc), 1), slices, st, 6, s, false, cap, true)) != cudaSuccess)
-                    return e;
-            } else {
-                tc::TrtriUpdTC up{L32, N, W, N, N, p0, pend - p0, N};
-                if ((e = run(up, dim3(cdiv(pend, tc::BN), cdiv(N - pend, tc::BM)), slices, st, 6, s, false, cap)) !=
-                    cudaSuccess)
-                    return e;
-            }
         }
     }
-    return launch_df_finish(W, N, N, NBK, W32, s);  // above the diagonal only k_trtri_diag writes
+    return cudaSuccess;
 }
 
 cudaError_t launch_recon_tc(const EncodeDev& e, const float2* W32, const float2* WT32, float2* T, int slices,
