@@ -23,10 +23,11 @@
 // E^H E y + lambda y generated in double-float or FP64). The estimate therefore
 // stays below kappa_1(G) up to the rounding of the sums.
 //
-// Everything runs on the device with no host synchronisation: single-block
-// kernels keep the iteration's state in device memory, and once it has
-// converged the remaining kernels of the fixed launch sequence return at once.
+// Everything runs on the device with no host synchronisation: the iteration's state
+// is in device memory, and once it has converged the remaining kernels of the fixed
+// launch sequence return at once.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <string>
 #include <type_traits>
@@ -52,13 +53,22 @@ pinv_status cuda_err(cudaError_t e, const char* where) {
     } while (0)
 
 struct HagerState {
-    double est;       // best ||G^-1 v||_1 / ||v||_1 so far (v = the start vector or some e_j)
-    double est_alt;   // the same for the alternating-sign vector
-    int j, jlast;     // current and previous unit-vector index
-    int done;         // the iteration has finished
-    int rounds;       // unit-vector rounds taken
-    int best_j;       // start vector of the best estimate: -1 = uniform, else e_best_j
+    double est;      // best ||G^-1 v||_1 / ||v||_1 so far (v = the start vector or some e_j)
+    double est_alt;  // the same for the alternating-sign vector
+    int j;           // the current unit vector
+    int done;        // the iteration has finished
+    int rounds;      // unit vectors taken
+    int best_j;      // start vector of the best estimate: -1 = uniform, else e_best_j
+    int best_buf;    // which of Y's first two vectors holds its y
+    unsigned arrived;  // CTAs of the running kernel that have left their part
 };
+// what a CTA leaves of its entries of y (or z)
+struct HgPart {
+    double sum[2];  // sums of |y| (start: of both vectors)
+    float vmax;     // largest |z_i| ...
+    int imax;       // ... and its lowest index
+};
+enum { HG_START, HG_ALT, HG_PICK, HG_UNIT, HG_ADD };
 
 // |a + ib| in FP32 from FP64 parts, without the FP64 pipe
 __device__ inline float abs_f(double2 g) {
@@ -145,111 +155,6 @@ __global__ void __launch_bounds__(CB) k_norm1_finish(const float2* rs, const flo
     if (threadIdx.x == 0) *out = red[0];
 }
 
-// -------------------------------------------------------------------- solves
-// Products with the FP32 W = L^-1 for F <= 2 vectors at once, FP32 arithmetic
-// (the search only needs the estimate's order; the final candidates are refined
-// and certified against G).
-constexpr int FMAX = 2;
-
-// u[f] = W x[f], W lower FP32 [N][N] row-major; one warp per row
-__global__ void k_w_mv(const float2* W, int64_t N, int F, const float2* x, float2* u, const int* skip) {
-    if (skip && *skip) return;
-    const int lane = threadIdx.x & 31;
-    const int64_t i = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (i >= N) return;
-    const float2* row = W + i * N;
-    float re[FMAX] = {0.f, 0.f}, im[FMAX] = {0.f, 0.f};
-    auto mac = [&](float2 w, int64_t j) {
-#pragma unroll
-        for (int f = 0; f < FMAX; ++f) {
-            if (f < F) {
-                const float2 v = x[(int64_t)f * N + j];
-                re[f] = fmaf(w.x, v.x, fmaf(-w.y, v.y, re[f]));
-                im[f] = fmaf(w.x, v.y, fmaf(w.y, v.x, im[f]));
-            }
-        }
-    };
-    if ((N & 1) == 0) {  // rows start on 16-byte boundaries: two entries per load
-        const float4* row4 = reinterpret_cast<const float4*>(row);
-#pragma unroll 4
-        for (int64_t q = lane; 2 * q <= i; q += 32) {
-            const float4 w = row4[q];
-            mac(make_float2(w.x, w.y), 2 * q);
-            if (2 * q + 1 <= i) mac(make_float2(w.z, w.w), 2 * q + 1);
-        }
-    } else {
-#pragma unroll 4
-        for (int64_t j = lane; j <= i; j += 32) mac(row[j], j);
-    }
-#pragma unroll
-    for (int f = 0; f < FMAX; ++f) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            re[f] += __shfl_xor_sync(0xffffffffu, re[f], o);
-            im[f] += __shfl_xor_sync(0xffffffffu, im[f], o);
-        }
-        if (lane == 0 && f < F) u[(int64_t)f * N + i] = make_float2(re[f], im[f]);
-    }
-}
-
-// part[s][f][j] = sum over rows i of chunk s with i >= j of conj(W[i][j]) u[f][i]
-__global__ void k_wh_part(const float2* W, int64_t N, int F, const float2* u, int64_t rows_per_chunk, float2* part,
-                          const int* skip) {
-    if (skip && *skip) return;
-    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t i0 = (int64_t)blockIdx.y * rows_per_chunk;
-    const int64_t i1 = N < i0 + rows_per_chunk ? N : i0 + rows_per_chunk;
-    if (j >= N) return;
-    float re[FMAX] = {0.f, 0.f}, im[FMAX] = {0.f, 0.f};
-#pragma unroll 4
-    for (int64_t i = i0 > j ? i0 : j; i < i1; ++i) {
-        const float2 w = W[i * N + j];
-#pragma unroll
-        for (int f = 0; f < FMAX; ++f) {
-            if (f < F) {
-                const float2 v = u[(int64_t)f * N + i];
-                re[f] = fmaf(w.x, v.x, fmaf(w.y, v.y, re[f]));
-                im[f] = fmaf(w.x, v.y, fmaf(-w.y, v.x, im[f]));
-            }
-        }
-    }
-    for (int f = 0; f < F; ++f) part[((int64_t)blockIdx.y * F + f) * N + j] = make_float2(re[f], im[f]);
-}
-
-// y[f][j] (+)= sum_s part[s][f][j]
-__global__ void k_part_sum(const float2* part, int chunks, int64_t N, int F, double2* y, int accumulate,
-                           const int* skip) {
-    if (skip && *skip) return;
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= N * F) return;
-    float re = 0.f, im = 0.f;
-    for (int s = 0; s < chunks; ++s) {
-        const float2 p = part[(int64_t)s * N * F + idx];
-        re += p.x;
-        im += p.y;
-    }
-    double2 v = make_double2((double)re, (double)im);
-    if (accumulate) v = zadd(y[idx], v);
-    y[idx] = v;
-}
-
-// y = H x with the full Hermitian FP64 H (G^-1 of FP64 plans); one warp per row
-__global__ void k_hemv_full(const double2* H, int64_t N, const float2* xf, double2* y, const int* skip) {
-    if (skip && *skip) return;
-    const int lane = threadIdx.x & 31;
-    const int64_t i = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (i >= N) return;
-    const double2* row = H + i * N;
-    double2 acc = make_double2(0.0, 0.0);
-    for (int64_t j = lane; j < N; j += 32) zfma(acc, row[j], make_double2(xf[j].x, xf[j].y));
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
-        acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
-    }
-    if (lane == 0) y[i] = acc;
-}
-
 // FP64 -> FP32 vector copy on the integer pipe
 __global__ void k_vec_f32(const double2* a, float2* b, int64_t n) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -257,144 +162,305 @@ __global__ void k_vec_f32(const double2* a, float2* b, int64_t n) {
 }
 
 // -------------------------------------------------------------------- Hager's iteration
-// |v| in FP32 from FP64 parts, without the FP64 pipe
-__device__ inline float mag(double2 v) { return abs_f(v); }
+// One kernel for each product: u = W x (k_hg_wx), then y = W^H u (k_hg_wtu), or y = G^-1 x
+// at once with the FP64 G^-1 (k_hg_gx). Arithmetic with W is FP32 (the search only needs
+// the estimate's order; the final candidates are refined and certified against G). The
+// kernel that forms y also takes the iteration's step: its CTAs leave sums of |y| and the
+// largest entry, and the last one to arrive decides. The unit vector's W e_j is a column of
+// W, read in place, and the alternating vector goes with the start vector, so a run of
+// two unit vectors reads W seven times; as separate kernels with single-block steps
+// (ten reads, 45 launches, the ones of rounds not needed at 4 us each) the estimate took
+// 0.52 ms at N = 2304 and 0.66 at N = 4096, so it takes 0.31 and 0.50, a third of it the
+// two exact residuals of the refinement and the certificate.
 
-// block sum of |v[i]| (FP32 magnitudes, double-float sums), result in every thread
-__device__ double block_abs_sum(const double2* v, int64_t N, float2* red) {
-    float h = 0.f, l = 0.f;
-    for (int64_t i = threadIdx.x; i < N; i += CB) acc_df(h, l, mag(v[i]));
-    const float2 w = warp_sum_df(h, l);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = w;
+// y = the entry of index i, for the threads with `own`: stored, and its part of the step
+struct HgStep {
+    int kind;
+    double2* Y;   // [3][N]: the iteration's two vectors, the alternating vector's
+    double2* z;   // [N]
+    const float2* alt;  // the alternating vector
+    float2* xi;         // y / |y| (1 where y vanishes); no product that writes it reads it
+    HgPart* part;
+    HagerState* h;
+};
+struct HgAcc {  // a thread's part, reduced over the CTA by hg_finish
+    float sh[2], sl[2];
+    float vmax;
+    int imax;
+    __device__ void larger(float v, int i) {
+        if (v > vmax || (v == vmax && i < imax)) {
+            vmax = v;
+            imax = i;
+        }
+    }
+};
+__device__ inline HgAcc hg_none() { return HgAcc{{0.f, 0.f}, {0.f, 0.f}, -1.f, INT_MAX}; }
+__device__ inline void hg_entry(const HgStep& st, HgAcc& a, int f, int64_t i, int64_t N, double2 y, int buf) {
+    const float re = f64_to_f32_rn(y.x), im = f64_to_f32_rn(y.y);
+    const float m = sqrtf(fmaf(re, re, im * im));
+    if (st.kind == HG_ADD) {
+        st.Y[f * N + i] = zadd(st.Y[f * N + i], y);
+        return;
+    }
+    if (st.kind == HG_PICK) {
+        st.z[i] = y;
+        a.larger(m, (int)i);
+        return;
+    }
+    acc_df(a.sh[f], a.sl[f], m);
+    const bool alt = f == 1 || st.kind == HG_ALT;
+    st.Y[(alt ? 2 : buf) * N + i] = y;
+    if (!alt) st.xi[i] = m > 0.f ? make_float2(re / m, im / m) : make_float2(1.f, 0.f);
+}
+// every thread of the CTA; the last CTA to arrive takes the step
+__device__ inline void hg_finish(const HgStep& st, HgAcc a, int64_t N, int buf) {
+    __shared__ HgAcc red[32];
+    __shared__ HgPart fin[32];
+    __shared__ int last;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, nw = blockDim.x >> 5;
+    if (st.kind == HG_ADD) return;
+    for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+        for (int f = 0; f < 2; ++f) {
+            const float oh = __shfl_xor_sync(~0u, a.sh[f], o), ol = __shfl_xor_sync(~0u, a.sl[f], o);
+            df_add(a.sh[f], a.sl[f], oh, ol, a.sh[f], a.sl[f]);
+        }
+        const float ov = __shfl_xor_sync(~0u, a.vmax, o);
+        a.larger(ov, __shfl_xor_sync(~0u, a.imax, o));
+    }
+    if (lane == 0) red[w] = a;
+    __threadfence();  // this thread's entries before its CTA's arrival
     __syncthreads();
-    float2 t = threadIdx.x < CB / 32 ? red[threadIdx.x] : make_float2(0.f, 0.f);
-    if (threadIdx.x < 32) t = warp_sum_df(t.x, t.y);
-    if (threadIdx.x == 0) red[0] = t;
+    if (tid == 0) {
+        for (int i = 1; i < nw; ++i) {
+#pragma unroll
+            for (int f = 0; f < 2; ++f) df_add(a.sh[f], a.sl[f], red[i].sh[f], red[i].sl[f], a.sh[f], a.sl[f]);
+            a.larger(red[i].vmax, red[i].imax);
+        }
+        st.part[blockIdx.x] = HgPart{{(double)a.sh[0] + (double)a.sl[0], (double)a.sh[1] + (double)a.sl[1]}, a.vmax, a.imax};
+        __threadfence();
+        last = atomicAdd(&st.h->arrived, 1u) == gridDim.x - 1;
+    }
     __syncthreads();
-    const double r = (double)red[0].x + (double)red[0].y;
+    if (!last) return;
+    __threadfence();
+    HgAcc t = hg_none();
+    double s0 = 0.0, s1 = 0.0, xa = 0.0;
+    for (int i = tid; i < (int)gridDim.x; i += blockDim.x) {
+        const HgPart q = st.part[i];
+        s0 += q.sum[0];
+        s1 += q.sum[1];
+        t.larger(q.vmax, q.imax);
+    }
+    if (st.kind == HG_START || st.kind == HG_ALT) {  // ||v||_1 of the alternating vector as rounded
+        float h = 0.f, l = 0.f;
+        for (int64_t i = tid; i < N; i += blockDim.x) acc_df(h, l, fabsf(st.alt[i].x));
+        xa = (double)h + (double)l;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        s0 += __shfl_xor_sync(~0u, s0, o);
+        s1 += __shfl_xor_sync(~0u, s1, o);
+        xa += __shfl_xor_sync(~0u, xa, o);
+        const float ov = __shfl_xor_sync(~0u, t.vmax, o);
+        t.larger(ov, __shfl_xor_sync(~0u, t.imax, o));
+    }
+    if (lane == 0) {
+        fin[w] = HgPart{{s0, s1}, t.vmax, t.imax};
+        red[w].sh[0] = __double2float_rn(xa);  // near 1
+        red[w].sl[0] = (float)(xa - (double)red[w].sh[0]);
+    }
     __syncthreads();
-    return r;
+    if (tid) return;
+    for (int i = 1; i < nw; ++i) {
+        s0 += fin[i].sum[0];
+        s1 += fin[i].sum[1];
+        xa += (double)red[i].sh[0] + (double)red[i].sl[0];
+        t.larger(fin[i].vmax, fin[i].imax);
+    }
+    HagerState* h = st.h;
+    if (st.kind == HG_START) {
+        h->est = s0;
+        h->best_j = -1;
+        h->best_buf = 0;
+        h->est_alt = s1 / xa;
+    } else if (st.kind == HG_ALT) {
+        h->est_alt = s0 / xa;
+    } else if (st.kind == HG_UNIT) {
+        if (s0 <= h->est) {
+            h->done = 1;  // no growth: the iteration has converged
+        } else {
+            h->est = s0;
+            h->best_j = h->j;
+            h->best_buf = buf;
+        }
+    } else {  // HG_PICK: stop when the current unit vector's index attains the maximum again
+        if (h->j >= 0 && (abs_f(st.z[h->j]) >= t.vmax || h->rounds >= HAGER_ROUNDS)) h->done = 1;
+        h->j = t.imax == INT_MAX ? 0 : t.imax;  // no finite entry: any
+        h->rounds += 1;
+    }
+    h->arrived = 0;
 }
 
+// x = (1/N, ...) and x_i = (-1)^i (1 + i / (N - 1)), scaled to ||x||_1 = 1
 __global__ void k_hg_init(float2* x, int64_t N, HagerState* h) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < N) x[i] = make_float2((float)(1.0 / (double)N), 0.f);
-    if (i == 0) *h = HagerState{0.0, 0.0, -1, -1, 0, 0, -1};
+    griddep_wait();
+    griddep_launch();
+    if (i < N) {
+        x[i] = make_float2((float)(1.0 / (double)N), 0.f);
+        const double v = N > 1 ? (1.0 + (double)i / (double)(N - 1)) / (1.5 * (double)N) : 1.0;
+        x[N + i] = make_float2((float)((i & 1) ? -v : v), 0.f);
+    }
+    if (i == 0) *h = HagerState{0.0, 0.0, -1, 0, 0, -1, 0, 0u};
 }
 
-// After y = G^-1 v with v the start vector (first = 1) or e_j: record the
-// estimate ||y||_1 (||v||_1 = 1), stop when it no longer grows, keep the best y
-// in ybest, and write xi = y / |y| (1 where y vanishes) for the next solve.
-__global__ void __launch_bounds__(CB) k_hg_sign(const double2* y, float2* xi, double2* ybest, int64_t N,
-                                                HagerState* h, int first) {
-    __shared__ float2 red[CB / 32];
-    __shared__ int stop;
-    if (h->done) return;
-    const double s = block_abs_sum(y, N, red);
-    if (threadIdx.x == 0) {
-        stop = 0;
-        if (!first && s <= h->est) {
-            h->done = 1;  // no growth: the iteration has converged
-            stop = 1;
-        } else {
-            h->est = s;
-            h->best_j = first ? -1 : h->j;
+// u[f] = W x[f], W lower FP32 [N][N] row-major; one warp per row
+template <int F>
+__global__ void __launch_bounds__(256) k_hg_wx(const float2* __restrict__ W, int64_t N, const float2* __restrict__ x,
+                                               float2* u, const HagerState* h) {
+    const int lane = threadIdx.x & 31;
+    const int64_t i = N - 1 - ((int64_t)blockIdx.x * 8 + (threadIdx.x >> 5));  // the longest rows first
+    griddep_wait();
+    griddep_launch();
+    if ((h && h->done) || i < 0) return;
+    const float2* row = W + i * N;
+    float re[F], im[F];
+#pragma unroll
+    for (int f = 0; f < F; ++f) re[f] = im[f] = 0.f;
+    auto mac = [&](float2 w, float2 v, int f) {
+        re[f] = fmaf(w.x, v.x, fmaf(-w.y, v.y, re[f]));
+        im[f] = fmaf(w.x, v.y, fmaf(w.y, v.x, im[f]));
+    };
+    if ((N & 1) == 0) {  // rows start on 16-byte boundaries: two entries per load (W is zero right of the diagonal)
+        const float4* row4 = reinterpret_cast<const float4*>(row);
+#pragma unroll 8
+        for (int64_t q = lane; 2 * q <= i; q += 32) {
+            const float4 w = row4[q];
+#pragma unroll
+            for (int f = 0; f < F; ++f) {
+                const float4 v = reinterpret_cast<const float4*>(x + f * N)[q];
+                mac(make_float2(w.x, w.y), make_float2(v.x, v.y), f);
+                mac(make_float2(w.z, w.w), make_float2(v.z, v.w), f);
+            }
+        }
+    } else {
+#pragma unroll 8
+        for (int64_t j = lane; j <= i; j += 32) {
+            const float2 w = row[j];
+#pragma unroll
+            for (int f = 0; f < F; ++f) mac(w, x[f * N + j], f);
         }
     }
-    __syncthreads();
-    if (stop) return;
-    for (int64_t i = threadIdx.x; i < N; i += CB) {
-        const double2 v = y[i];
-        ybest[i] = v;
-        const float re = f64_to_f32_rn(v.x), im = f64_to_f32_rn(v.y);
-        const float a = sqrtf(fmaf(re, re, im * im));
-        xi[i] = a > 0.f ? make_float2(re / a, im / a) : make_float2(1.f, 0.f);
+#pragma unroll
+    for (int f = 0; f < F; ++f) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            re[f] += __shfl_xor_sync(~0u, re[f], o);
+            im[f] += __shfl_xor_sync(~0u, im[f], o);
+        }
+        if (lane == 0) u[f * N + i] = make_float2(re[f], im[f]);
     }
 }
 
-// After z = G^-1 xi: j = the first index of the largest |z_j|. Stop when the
-// previous index attains the same maximum or after HAGER_ROUNDS rounds;
-// otherwise x = e_j.
-__global__ void __launch_bounds__(CB) k_hg_pick(const double2* z, float2* x, int64_t N, HagerState* h) {
-    __shared__ float rv[CB];
-    __shared__ int ri[CB];
-    __shared__ int stop, jn;
-    if (h->done) return;
-    float best = -1.f;
-    int bi = 0;
-    for (int64_t i = threadIdx.x; i < N; i += CB) {
-        const float a = mag(z[i]);
-        if (a > best) {
-            best = a;
-            bi = (int)i;
-        }
+// y[f] = W^H u[f] and the step; kind HG_UNIT: u is column h->j of W. A CTA takes four columns
+// (one sector of a row) from the left and four from the right, so that all read as many rows,
+// 128 rows at a time: wider tiles leave too few CTAs at a few thousand voxels (estimate at
+// N = 4096 0.58 ms with 16 columns, 0.51 with 8, 0.50 with 4; at N = 16384 4.8 - 4.9 with any).
+constexpr int HGC = 4, HGT = 512;
+template <int F>
+__global__ void __launch_bounds__(HGT) k_hg_wtu(const float2* __restrict__ W, int64_t N, const float2* __restrict__ u,
+                                                HgStep st, const HagerState* skip) {
+    __shared__ float2 red[F][HGT / HGC][HGC];
+    const int c = threadIdx.x % HGC, g = threadIdx.x / HGC;
+    griddep_wait();
+    griddep_launch();
+    if (skip && skip->done) return;
+    const int64_t nb = (N + HGC - 1) / HGC;
+    const int buf = st.kind == HG_UNIT ? 1 - st.h->best_buf : 0;
+    int64_t su = 1;
+    if (st.kind == HG_UNIT) {
+        u = W + st.h->j;
+        su = N;
     }
-    rv[threadIdx.x] = best;
-    ri[threadIdx.x] = bi;
-    __syncthreads();
-    for (int w = CB / 2; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) {
-            const float o = rv[threadIdx.x + w];
-            const int oi = ri[threadIdx.x + w];
-            if (o > rv[threadIdx.x] || (o == rv[threadIdx.x] && oi < ri[threadIdx.x])) {
-                rv[threadIdx.x] = o;
-                ri[threadIdx.x] = oi;
+    HgAcc acc = hg_none();
+    for (int side = 0; side < 2; ++side) {
+        const int64_t cb = side ? nb - 1 - blockIdx.x : blockIdx.x;
+        if (side && cb == blockIdx.x) break;
+        const int64_t j = cb * HGC + c;
+        float re[F], im[F];
+#pragma unroll
+        for (int f = 0; f < F; ++f) re[f] = im[f] = 0.f;
+        if (j < N) {
+#pragma unroll 8
+            for (int64_t i = cb * HGC + g; i < N; i += HGT / HGC) {  // W is zero above the diagonal
+                const float2 w = W[i * N + j];
+#pragma unroll
+                for (int f = 0; f < F; ++f) {
+                    const float2 v = u[f * N + i * su];
+                    re[f] = fmaf(w.x, v.x, fmaf(w.y, v.y, re[f]));
+                    im[f] = fmaf(w.x, v.y, fmaf(-w.y, v.x, im[f]));
+                }
             }
         }
         __syncthreads();
+#pragma unroll
+        for (int f = 0; f < F; ++f) red[f][g][c] = make_float2(re[f], im[f]);
+        __syncthreads();
+        if (threadIdx.x < F * HGC) {  // thread f * 16 + c
+            const int f = threadIdx.x / HGC;
+            if (j < N) {
+                float a = 0.f, b = 0.f;
+#pragma unroll 8
+                for (int q = 0; q < HGT / HGC; ++q) {
+                    a += red[f][q][c].x;
+                    b += red[f][q][c].y;
+                }
+                hg_entry(st, acc, f, j, N, make_double2((double)a, (double)b), buf);
+            }
+        }
     }
-    if (threadIdx.x == 0) {
-        const int j = ri[0];
-        stop = 0;
-        if (h->j >= 0 && (mag(z[h->j]) >= rv[0] || h->rounds >= HAGER_ROUNDS)) stop = 1;
-        if (stop) h->done = 1;
-        h->jlast = h->j;
-        h->j = j;
-        h->rounds += 1;
-        jn = j;
-    }
-    __syncthreads();
-    if (stop) return;
-    for (int64_t i = threadIdx.x; i < N; i += CB) x[i] = make_float2(i == jn ? 1.f : 0.f, 0.f);
+    hg_finish(st, acc, N, buf);
 }
 
-// x_i = (-1)^i (1 + i / (N - 1)), scaled to ||x||_1 = 1
-__global__ void k_hg_alt(float2* x, int64_t N) {
+// y = H x with the full Hermitian FP64 H (G^-1 of FP64 plans) and the step; one warp per row;
+// kind HG_UNIT: column h->j of H
+__global__ void __launch_bounds__(256) k_hg_gx(const double2* __restrict__ H, int64_t N, const float2* __restrict__ x,
+                                               HgStep st, const HagerState* skip) {
+    const int lane = threadIdx.x & 31;
+    const int64_t i = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    griddep_wait();
+    griddep_launch();
+    if (skip && skip->done) return;
+    const int buf = st.kind == HG_UNIT ? 1 - st.h->best_buf : 0;
+    HgAcc acc = hg_none();
+    if (i < N) {
+        double2 a = make_double2(0.0, 0.0);
+        if (st.kind == HG_UNIT) {
+            if (lane == 0) a = H[i * N + st.h->j];
+        } else {
+            for (int64_t j = lane; j < N; j += 32) zfma(a, H[i * N + j], make_double2(x[j].x, x[j].y));
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                a.x += __shfl_xor_sync(~0u, a.x, o);
+                a.y += __shfl_xor_sync(~0u, a.y, o);
+            }
+        }
+        if (lane == 0) hg_entry(st, acc, 0, i, N, a, buf);
+    }
+    hg_finish(st, acc, N, buf);
+}
+
+// the two final candidates: V the vectors v in FP64 (the best iterate's start vector, uniform
+// or e_j; the alternating-sign vector), Y2 their y
+__global__ void k_hg_vecs(const HagerState* h, const float2* x, const double2* Y, double2* V, double2* Y2, int64_t N) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    const double v = N > 1 ? (1.0 + (double)i / (double)(N - 1)) / (1.5 * (double)N) : 1.0;
-    x[i] = make_float2((float)((i & 1) ? -v : v), 0.f);
-}
-
-// est_alt = ||y||_1 / ||x||_1 for the rounded alternating vector; y kept in yalt
-__global__ void __launch_bounds__(CB) k_hg_alt_finish(const double2* y, const float2* x, double2* yalt, int64_t N,
-                                                      HagerState* h) {
-    __shared__ float2 red[CB / 32];
-    const double s = block_abs_sum(y, N, red);
-    float th = 0.f, tl = 0.f;
-    for (int64_t i = threadIdx.x; i < N; i += CB) {
-        acc_df(th, tl, fabsf(x[i].x));
-        yalt[i] = y[i];
-    }
-    const float2 w = warp_sum_df(th, tl);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = w;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        float2 t = threadIdx.x < CB / 32 ? red[threadIdx.x] : make_float2(0.f, 0.f);
-        t = warp_sum_df(t.x, t.y);
-        if (threadIdx.x == 0) h->est_alt = s / ((double)t.x + (double)t.y);
-    }
-}
-
-// the two final candidate vectors v in FP64: V[0] = the best iterate's start
-// vector (uniform or e_j), V[1] = the alternating-sign vector (x)
-__global__ void k_hg_vecs(const HagerState* h, const float2* x, double2* V, int64_t N) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    griddep_wait();
     if (i >= N) return;
     const int bj = h->best_j;
     V[i] = make_double2(bj < 0 ? 1.0 / (double)N : (i == bj ? 1.0 : 0.0), 0.0);
-    V[N + i] = make_double2(x[i].x, x[i].y);
+    V[N + i] = make_double2(x[N + i].x, x[N + i].y);
+    Y2[i] = Y[h->best_buf * N + i];
+    Y2[N + i] = Y[2 * N + i];
 }
 
 // FP64 plans: kappa = ||G||_1 max(est, est_alt) (their G^-1 is accurate)
@@ -402,16 +468,33 @@ __global__ void k_hg_final(const HagerState* h, DevStatus* st) {
     st->kappa_est = st->norm1_g * fmax(h->est, h->est_alt);
 }
 
-// Mixed plans: kappa = ||G||_1 max_f ||Y[f]||_1 / ||R[f]||_1 with R = -G Y
+// Mixed plans: kappa = ||G||_1 max_f ||Y[f]||_1 / ||R[f]||_1 with R = -G Y; FP32
+// magnitudes, double-float sums, the four of them together
 __global__ void __launch_bounds__(CB) k_hg_certify(const double2* Y, const double2* R, int64_t N, DevStatus* st) {
-    __shared__ float2 red[CB / 32];
-    double best = 0.0;
-    for (int f = 0; f < 2; ++f) {
-        const double ny = block_abs_sum(Y + (int64_t)f * N, N, red);
-        const double nr = block_abs_sum(R + (int64_t)f * N, N, red);
-        if (nr > 0.0) best = fmax(best, ny / nr);
+    __shared__ float2 red[4][CB / 32];
+    float h[4] = {0.f, 0.f, 0.f, 0.f}, l[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+    for (int64_t i = threadIdx.x; i < N; i += CB)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc_df(h[q], l[q], abs_f((q < 2 ? Y : R)[(q & 1) * N + i]));
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const float2 w = warp_sum_df(h[q], l[q]);
+        if ((threadIdx.x & 31) == 0) red[q][threadIdx.x >> 5] = w;
     }
-    if (threadIdx.x == 0) st->kappa_est = st->norm1_g * best;
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    double v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const float2 w = red[q][threadIdx.x], t = warp_sum_df(w.x, w.y);
+        v[q] = (double)t.x + (double)t.y;
+    }
+    if (threadIdx.x) return;
+    double best = 0.0;
+    for (int f = 0; f < 2; ++f)
+        if (v[2 + f] > 0.0) best = fmax(best, v[f] / v[2 + f]);
+    st->kappa_est = st->norm1_g * best;
 }
 
 // row chunks of the column-sum kernels: at least 128 rows, at most 64 chunks
@@ -455,8 +538,6 @@ cudaError_t launch_gram_norm1(const double2* G, const float4* Gdf, const float4*
 pinv_status build_condition(pinv_plan* p, cudaStream_t s) {
     const int64_t N = p->N, M = p->M;
     const bool mixed = p->precision != PINV_FP64;
-    const int chunks = chunks_for(N);
-    const int64_t rpc = rows_per_chunk(N);
     // every buffer goes back to the pool in stream order when this returns, on
     // every path (the kernels enqueued before it still see it)
     struct Release {
@@ -472,55 +553,46 @@ pinv_status build_condition(pinv_plan* p, cudaStream_t s) {
         return e;
     };
     HagerState* h = nullptr;
-    float2 *x = nullptr, *u = nullptr, *part = nullptr;
-    double2 *y = nullptr, *z = nullptr, *Y2 = nullptr, *V2 = nullptr, *R2 = nullptr, *zero = nullptr, *U2 = nullptr;
+    HgPart* part = nullptr;
+    float2 *x = nullptr, *u = nullptr;
+    double2 *Y = nullptr, *z = nullptr, *Y2 = nullptr, *V2 = nullptr, *R2 = nullptr, *zero = nullptr, *U2 = nullptr;
+    const unsigned vb = (unsigned)((N + 255) / 256), rb = (unsigned)((N + 7) / 8);
+    const unsigned cb = (unsigned)(((N + HGC - 1) / HGC + 1) / 2);  // k_hg_wtu
     CKC(take((void**)&h, sizeof(HagerState)));
-    CKC(take((void**)&x, sizeof(float2) * FMAX * N));
-    CKC(take((void**)&y, sizeof(double2) * N));
+    CKC(take((void**)&x, sizeof(float2) * 3 * N));  // uniform, alternating, xi
+    CKC(take((void**)&Y, sizeof(double2) * 3 * N));
     CKC(take((void**)&z, sizeof(double2) * N));
-    CKC(take((void**)&Y2, sizeof(double2) * 2 * N));
-    if (mixed) {
-        CKC(take((void**)&u, sizeof(float2) * FMAX * N));
-        CKC(take((void**)&part, sizeof(float2) * FMAX * N * chunks));
-    }
-    const unsigned vb = (unsigned)((N + 255) / 256), wb = (unsigned)((N + 7) / 8);
-    const int* skip = &h->done;
-    // out (+)= G^-1 x for F vectors in x (float2 [F][N]); skip_on: return at once
-    // once the iteration is done
-    auto solve = [&](double2* out, int F, bool skip_on, int accumulate) -> cudaError_t {
-        const int* sk = skip_on ? skip : nullptr;
-        if (mixed) {
-            k_w_mv<<<wb, 256, 0, s>>>(p->W32, N, F, x, u, sk);
-            k_wh_part<<<dim3(vb, (unsigned)chunks), 256, 0, s>>>(p->W32, N, F, u, rpc, part, sk);
-            k_part_sum<<<(unsigned)((N * F + 255) / 256), 256, 0, s>>>(part, chunks, N, F, out, accumulate, sk);
-            note_launch(3);
-        } else {
-            k_hemv_full<<<wb, 256, 0, s>>>(p->Ginv, N, x, out, sk);
-            note_launch();
-        }
-        return cudaGetLastError();
+    CKC(take((void**)&part, sizeof(HgPart) * std::max(rb, cb)));
+    if (mixed) CKC(take((void**)&u, sizeof(float2) * 2 * N));
+    const HagerState* hc = h;
+    const float2 *xc = x, *uc = u, *W = p->W32;
+    const double2* Gi = p->Ginv;
+    // y = G^-1 x and the iteration's step; skip: nothing once the iteration is done
+    auto wtu = [&](int f, const HgStep& st, const HagerState* skip) -> cudaError_t {
+        auto k = f == 2 ? k_hg_wtu<2> : k_hg_wtu<1>;
+        return launch_pdl(k, dim3(cb), dim3(HGT), 0, s, W, N, uc, st, skip);
     };
-    k_hg_init<<<vb, 256, 0, s>>>(x, N, h);
-    note_launch();
-    CKC(solve(y, 1, false, 0));
-    k_hg_sign<<<1, CB, 0, s>>>(y, x, Y2, N, h, 1);
-    note_launch();
-    CKC(solve(z, 1, true, 0));
-    k_hg_pick<<<1, CB, 0, s>>>(z, x, N, h);
-    note_launch();
+    auto solve = [&](int kind, const float2* v, const HagerState* skip) -> cudaError_t {
+        const HgStep st{kind, Y, z, x + N, x + 2 * N, part, h};
+        if (!mixed) return launch_pdl(k_hg_gx, dim3(rb), dim3(256), 0, s, Gi, N, v, st, skip);
+        if (kind == HG_START) {  // with the alternating vector
+            const cudaError_t e = launch_pdl(k_hg_wx<2>, dim3(rb), dim3(256), 0, s, W, N, v, u, skip);
+            return e != cudaSuccess ? e : wtu(2, st, skip);
+        }
+        if (kind != HG_UNIT) {
+            const cudaError_t e = launch_pdl(k_hg_wx<1>, dim3(rb), dim3(256), 0, s, W, N, v, u, skip);
+            if (e != cudaSuccess) return e;
+        }
+        return wtu(1, st, skip);
+    };
+    CKC(launch_pdl(k_hg_init, dim3(vb), dim3(256), 0, s, x, N, h));
+    CKC(solve(HG_START, xc, nullptr));
+    if (!mixed) CKC(solve(HG_ALT, xc + N, nullptr));
+    CKC(solve(HG_PICK, xc + 2 * N, hc));
     for (int r = 1; r < HAGER_ROUNDS; ++r) {
-        CKC(solve(y, 1, true, 0));
-        k_hg_sign<<<1, CB, 0, s>>>(y, x, Y2, N, h, 0);
-        note_launch();
-        CKC(solve(z, 1, true, 0));
-        k_hg_pick<<<1, CB, 0, s>>>(z, x, N, h);
-        note_launch();
+        CKC(solve(HG_UNIT, nullptr, hc));
+        CKC(solve(HG_PICK, xc + 2 * N, hc));
     }
-    k_hg_alt<<<vb, 256, 0, s>>>(x, N);
-    note_launch();
-    CKC(solve(y, 1, false, 0));
-    k_hg_alt_finish<<<1, CB, 0, s>>>(y, x, Y2 + N, N, h);
-    note_launch();
     CKC(cudaGetLastError());
     if (!mixed) {
         k_hg_final<<<1, 1, 0, s>>>(h, p->st);
@@ -530,9 +602,10 @@ pinv_status build_condition(pinv_plan* p, cudaStream_t s) {
     // Mixed plans: the two candidates v (V2) and their solves y (Y2), refined
     // (r = v - G y, y += W^H W r), then certified with R2 = -G Y2
     CKC(take((void**)&V2, sizeof(double2) * 2 * N));
+    CKC(take((void**)&Y2, sizeof(double2) * 2 * N));
     CKC(take((void**)&R2, sizeof(double2) * 2 * N));
-    k_hg_vecs<<<vb, 256, 0, s>>>(h, x, V2, N);
-    note_launch();
+    const double2* Yc = Y;
+    CKC(launch_pdl(k_hg_vecs, dim3(vb), dim3(256), 0, s, hc, xc, Yc, V2, Y2, N));
     const bool toep = p->refine_residual == PINV_RESIDUAL_TOEPLITZ;
     // plans with B0 and the digit tables of A and conj(A): E y and E^H u exactly on
     // the tensor cores (two frames in one 32-frame tile), far cheaper here than the
@@ -587,7 +660,9 @@ pinv_status build_condition(pinv_plan* p, cudaStream_t s) {
         CKC(resid(V2, Y2, R2));
         k_vec_f32<<<(unsigned)((2 * N + 255) / 256), 256, 0, s>>>(R2, x, 2 * N);
         note_launch();
-        CKC(solve(Y2, 2, false, 1));
+        const HgStep add{HG_ADD, Y2, nullptr, nullptr, nullptr, nullptr, h};
+        CKC(launch_pdl(k_hg_wx<2>, dim3(rb), dim3(256), 0, s, W, N, xc, u, (const HagerState*)nullptr));
+        CKC(wtu(2, add, nullptr));
     }
     CKC(resid(nullptr, Y2, R2));
     k_hg_certify<<<1, CB, 0, s>>>(Y2, R2, N, p->st);

@@ -69,6 +69,27 @@ def test_kappa_estimate_against_oracle(side, coils, traj, b0, lam, prec, res, sl
     assert k >= k1 / 3, (k, k1)
 
 
+@pytest.mark.parametrize("prec", [L.FP64, L.MIXED_BF16X6])
+@pytest.mark.parametrize("dims", [(1,), (3,), (4,), (5,), (8,), (9,), (65,), (33, 31), (37, 37)])
+def test_kappa_estimate_tile_edges(dims, prec):
+    """N below, at and past the four columns and eight rows of a CTA, odd N, and several
+    CTAs a product: a lower bound of kappa_1 and at least a third of it."""
+    from paper_2410_06129_gb300.plan import Plan
+    if prec != L.FP64 and not _mixed_ok():
+        pytest.skip("tcgen05 kernels need sm_103a")
+    rng = np.random.default_rng(2750)
+    N = int(np.prod(dims))
+    k = rng.uniform(-0.5 * max(dims), 0.5 * max(dims), size=(N + 3, len(dims)))
+    maps = rng.standard_normal((2, N)) + 1j * rng.standard_normal((2, N))
+    E = O.encode(k, O.voxel_positions(dims), maps, None, None)
+    G = E.conj().T @ E + O.lambda_abs(E, 1e-3) * np.eye(N)
+    k1 = np.linalg.cond(G, 1)
+    with Plan(dims, k, maps, lam=1e-3, precision=prec) as pl:
+        pl.build()
+        est = pl.info()["kappa_est"]
+    assert k1 / 3 <= est <= k1 * (1 + 1e-6), (est, k1)
+
+
 def test_kappa_estimate_lean_plan_and_rebuild():
     """A lean mixed plan (G, L and the FP64 W are build temporaries) gives the same
     estimate as a full one, and a second build the same value again."""
