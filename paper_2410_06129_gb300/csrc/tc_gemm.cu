@@ -380,6 +380,94 @@ __global__ void __launch_bounds__(256) k_tab_w(const float2* __restrict__ W32, i
     put_b<S>(tab + (ct * kcn + kc) * S * B_SL, r, g, v);
 }
 
+// Step 1 over mirror pairs of voxels (plans without B0): with X = conj(s_c) W[i] at a pair's two
+// voxels, theta = the phase of conj(A[m]) at the first,
+//   T^T[(c, m)][i] = sum_pairs cos(theta) (X_a + X_b) + i sin(theta) (X_a - X_b),
+// four real MACs a pair where the voxels one by one take four each (45 x 51, 5 coils, 5003 samples a
+// coil: step 1 1.68 -> 1.30 ms, ET 0.23 ms -> 0.03). ET holds (cos, sin), which is every coil's, and WB1 one block
+// of tiles for each coil: rows [Re+ | -Im-] for the real part and [Im+ | Re-] for the imaginary
+// part. Pairs are ordered by their first voxel, so row i needs those whose first is at most i.
+__global__ void k_pair_kend(EncodeDev e, int64_t nt, int* kend) {
+    const int64_t ct = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (ct >= nt) return;
+    int64_t lo = 0, hi = e.U;  // pairs with a first voxel below (ct + 1) BN
+    while (lo < hi) {
+        const int64_t m = (lo + hi) / 2;
+        if (e.pair[m].x < (ct + 1) * BN)
+            lo = m + 1;
+        else
+            hi = m;
+    }
+    kend[ct] = (int)((lo + KC - 1) / KC * KC);
+}
+template <int S>
+__global__ void __launch_bounds__(256) k_tab_etp(EncodeDev e, int64_t kc1, uint8_t* tab) {
+    const int64_t kc = blockIdx.x, rt = blockIdx.y;
+    const int r = threadIdx.x & (BM - 1), g = threadIdx.x >> 7;
+    const int64_t m = rt * BM + r, p0 = kc * KC + 8 * g;
+    float2 v[8];
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+        v[t] = make_float2(0.f, 0.f);
+        if (m < e.Mk && p0 + t < e.U) {
+            const int* q = e.vox_ijk + 3 * (int64_t)e.pair[p0 + t].x;
+            float2 a = __ldg(e.ex32 + m * e.nx + q[0]);
+            if (e.ny > 1) a = cmulf(a, __ldg(e.ey32 + m * e.ny + q[1]));
+            if (e.nz > 1) a = cmulf(a, __ldg(e.ez32 + m * e.nz + q[2]));
+            v[t] = conjf2(a);
+        }
+    }
+    put_a<S>(tab + (rt * kc1 + kc) * S * A_SL, r, g, v);
+}
+template <int S>
+__global__ void __launch_bounds__(256) k_tab_wp(EncodeDev e, const float2* __restrict__ W32, int64_t nt, int64_t kc1,
+                                                const int* __restrict__ kend, uint8_t* tab) {
+    const int64_t kc = blockIdx.x, ct = blockIdx.y;
+    if (kc * KC >= kend[ct]) return;
+    const int r = threadIdx.x & (BM - 1), g = threadIdx.x >> 7;
+    const int64_t i = ct * BN + r, p0 = kc * KC + 8 * g;
+    float2 wa[8], wb[8];
+    int na[8], nb[8];
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+        const int2 pr = p0 + t < e.U ? e.pair[p0 + t] : make_int2(-1, -1);
+        na[t] = pr.x;
+        nb[t] = pr.y;
+        wa[t] = i < e.N && pr.x >= 0 ? W32[i * e.N + pr.x] : make_float2(0.f, 0.f);
+        wb[t] = i < e.N && pr.y >= 0 ? W32[i * e.N + pr.y] : make_float2(0.f, 0.f);
+    }
+    for (int c = 0; c < e.C; ++c) {
+        float xr[8], xi[8], yr[8], yi[8];  // X_a + X_b, X_a - X_b
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            float2 a = wa[t], b = wb[t];
+            if (e.coils32) {
+                const float2* sc = e.coils32 + (int64_t)c * e.N;
+                a = cmulf(a, conjf2(na[t] >= 0 ? __ldg(sc + na[t]) : make_float2(0.f, 0.f)));
+                b = cmulf(b, conjf2(nb[t] >= 0 ? __ldg(sc + nb[t]) : make_float2(0.f, 0.f)));
+            }
+            xr[t] = a.x + b.x;
+            xi[t] = a.y + b.y;
+            yr[t] = a.x - b.x;
+            yi[t] = a.y - b.y;
+        }
+        uint32_t pr[S][4], pi[S][4], qr[S][4], qi[S][4];
+        split8<S>(xr, pr);
+        split8<S>(xi, pi);
+        split8<S>(yr, qr);
+        split8<S>(yi, qi);
+        uint8_t* blk = tab + ((c * nt + ct) * kc1 + kc) * S * B_SL;
+#pragma unroll
+        for (int sl = 0; sl < S; ++sl) {
+            uint8_t* b = blk + sl * B_SL;
+            st16(b + koff(r, g), pr[sl], 0u);
+            st16(b + koff(r, g + 2), qi[sl], 0x80008000u);
+            st16(b + A_SL + koff(r, g), pi[sl], 0u);
+            st16(b + A_SL + koff(r, g + 2), qr[sl], 0u);
+        }
+    }
+}
+
 struct ReconB1 {
     static constexpr bool kBulk = true;
     static constexpr bool kHintB = true;
@@ -388,25 +476,31 @@ struct ReconB1 {
     uint8_t* tt;
     int64_t rows, nt, kcn;  // sample tiles in the chunk, voxel tiles, voxel chunks
     int S;
+    // mirror pairs (kend not null): k runs over kc1 chunks of pairs, those of voxel tile ct end
+    // at kend[ct]; the tk sample tiles of a coil share ET, WB1 is one coil's after another
+    // (column c nt BN + i), and the chunk starts at sample tile row0. Else kc1 = kcn, one "coil".
+    int64_t kc1, tk, row0;
+    const int* kend;
     __device__ bool tile(int64_t bx, int64_t, int64_t& i0, int64_t& j0, int64_t& kb, int64_t& ke) const {
         int64_t rt, ct;
         band_tile(bx, rows, nt, rt, ct);
         ct = nt - 1 - ct;  // the longest tiles of a band first
         i0 = rt * BM;
-        j0 = ct * BN;
+        j0 = ((row0 + rt) / tk * nt + ct) * BN;
         kb = 0;
-        ke = (ct + 1) * BN;
+        ke = kend ? kend[ct] : (ct + 1) * BN;
         return true;
     }
     __device__ const uint8_t* bulk_a(int64_t i0, int64_t kc, int sl) const {
-        return et + (((i0 / BM) * kcn + kc) * S + sl) * A_SL;
+        const int64_t rt = kend ? (row0 + i0 / BM) % tk : i0 / BM;
+        return et + ((rt * kc1 + kc) * S + sl) * A_SL;
     }
     __device__ const uint8_t* bulk_b(int64_t j0, int64_t kc, int sl) const {
-        return wb + (((j0 / BN) * kcn + kc) * S + sl) * B_SL;
+        return wb + (((j0 / BN) * kc1 + kc) * S + sl) * B_SL;
     }
     // row i of T^T, voxels j0 .. j0 + 15 (one chunk of TT), split into S slices
     __device__ void store16(int64_t i, int64_t j0, const float (&re)[16], const float (&im)[16]) const {
-        uint8_t* blk = tt + ((i / BM) * kcn + j0 / KC) * S * A_SL;
+        uint8_t* blk = tt + ((i / BM) * kcn + (j0 / KC) % kcn) * S * A_SL;
         const int r = (int)(i % BM);
 #pragma unroll
         for (int g = 0; g < 2; ++g) {
@@ -431,7 +525,7 @@ struct ReconB2 {
     const uint8_t* wb;
     float2* R;
     int64_t rows, nt, kcn;
-    int64_t N, M, j_off, mvalid;  // Recon is [N][M]; this chunk holds samples j_off .. j_off + mvalid - 1
+    int64_t N, M, tk, mrow, row0;  // Recon is [N][M]; the chunk starts at sample tile row0; tk tiles hold mrow samples
     int S;
     __device__ bool tile(int64_t bx, int64_t, int64_t& i0, int64_t& j0, int64_t& kb, int64_t& ke) const {
         int64_t rt, ct;
@@ -442,15 +536,20 @@ struct ReconB2 {
         ke = nt * BN;
         return true;
     }
+    __device__ int64_t sample(int64_t i) const {  // of its coil's
+        return (int64_t)((unsigned)(row0 + i / BM) % (unsigned)tk) * BM + i % BM;
+    }
     __device__ const uint8_t* bulk_a(int64_t i0, int64_t kc, int sl) const {
         return tt + (((i0 / BM) * kcn + kc) * S + sl) * A_SL;
     }
     __device__ const uint8_t* bulk_b(int64_t j0, int64_t kc, int sl) const {
         return wb + (((j0 / BN) * kcn + kc) * S + sl) * B_SL;
     }
-    __device__ bool row_ok(int64_t i) const { return i < mvalid; }
+    __device__ bool row_ok(int64_t i) const { return sample(i) < mrow; }
     __device__ bool col_ok(int64_t j) const { return j < N; }
-    __device__ void store(int64_t i, int64_t j, float2 v) const { R[j * M + j_off + i] = v; }
+    __device__ void store(int64_t i, int64_t j, float2 v) const {
+        R[j * M + (int64_t)((unsigned)(row0 + i / BM) / (unsigned)tk) * mrow + sample(i)] = v;
+    }
 };
 
 // ------------------------------------------------------------------ panel trailing updates, bulk-fed
@@ -1337,7 +1436,9 @@ cudaError_t launch_recon_tc(const EncodeDev& e, const float2* W32, const float2*
 namespace {
 struct ReconBulkShape {
     int64_t nt, kcn, mt, rows, chunks;  // voxel tiles, voxel chunks, sample tiles, sample tiles per chunk
-    size_t wb_bytes, et_bytes;
+    bool pairs;                         // step 1 over mirror pairs
+    int64_t kc1, tk, mrow;              // its chunks of k; sample tiles of a coil, which hold mrow samples
+    size_t wb1_bytes, wb2_bytes, et_bytes, tt_bytes, kend_bytes;
 };
 // ET + TT of one chunk of samples: 4 GiB, or PINV_RECON_CHUNK_MB
 size_t recon_chunk_bytes() {
@@ -1345,29 +1446,58 @@ size_t recon_chunk_bytes() {
     const long mb = v ? std::atol(v) : 0;
     return mb > 0 ? (size_t)mb << 20 : size_t(4) << 30;
 }
+// Step 1 runs over mirror pairs where their tables take no more memory than those of single
+// voxels (a block of WB1 for each coil against ET for each coil: as many samples as half the
+// voxels and more). PINV_RECON_PAIRS=0: never.
 ReconBulkShape recon_bulk_shape(const EncodeDev& e, int slices) {
     ReconBulkShape r;
+    const int64_t M = e.Mk * e.C;
     r.nt = (e.N + tc::BM - 1) / tc::BM;
-    r.kcn = r.nt * (tc::BM / tc::KC);
-    r.mt = (e.Mk * e.C + tc::BM - 1) / tc::BM;
-    const size_t per_tile = 2 * (size_t)r.kcn * slices * tc::A_SL;
-    int64_t cap = (int64_t)(recon_chunk_bytes() / per_tile);
-    if (cap < 1) cap = 1;
-    r.chunks = (r.mt + cap - 1) / cap;
-    r.rows = (r.mt + r.chunks - 1) / r.chunks;
-    r.wb_bytes = (size_t)r.nt * r.kcn * slices * tc::B_SL;
-    r.et_bytes = (size_t)r.rows * r.kcn * slices * tc::A_SL;
+    r.kcn = r.kc1 = r.nt * (tc::BM / tc::KC);
+    r.mt = r.tk = (M + tc::BM - 1) / tc::BM;
+    r.mrow = M;
+    const size_t tile = (size_t)r.kcn * slices * tc::A_SL;
+    const int64_t cap = std::max<int64_t>(1, (int64_t)(recon_chunk_bytes() / (2 * tile)));
+    auto cut = [&] {
+        r.chunks = (r.mt + cap - 1) / cap;
+        r.rows = (r.mt + r.chunks - 1) / r.chunks;
+        r.tt_bytes = (size_t)r.rows * tile;
+    };
+    cut();
+    r.pairs = false;
+    r.kend_bytes = 0;
+    r.wb1_bytes = r.wb2_bytes = (size_t)r.nt * r.kcn * slices * tc::B_SL;
+    r.et_bytes = r.tt_bytes;
+    const char* env = std::getenv("PINV_RECON_PAIRS");
+    if (e.pair && !e.b0tab && !(env && std::strcmp(env, "0") == 0)) {
+        const int64_t kc1 = (e.U + tc::KC - 1) / tc::KC, tk = (e.Mk + tc::BM - 1) / tc::BM;
+        const size_t wb1 = (size_t)(e.C * r.nt * kc1) * slices * tc::B_SL;
+        const size_t et = (size_t)(tk * kc1) * slices * tc::A_SL;
+        if (wb1 + et <= r.wb1_bytes + std::min((size_t)r.mt * tile, size_t(2) << 30)) {  // not by the chunk asked for
+            r.pairs = true;
+            r.kc1 = kc1;
+            r.tk = tk;
+            r.mrow = e.Mk;
+            r.mt = tk * e.C;
+            cut();
+            r.wb1_bytes = wb1;
+            r.et_bytes = et;
+            r.kend_bytes = sizeof(int) * (size_t)r.nt;
+        }
+    }
     return r;
 }
 struct ReconWork {
     uint8_t *wb1, *wb2, *et, *tt;
+    int* kend;
 };
 ReconWork recon_work(const ReconBulkShape& r, void* work) {
     ReconWork w;
     w.wb1 = (uint8_t*)work;
-    w.wb2 = w.wb1 + r.wb_bytes;
-    w.et = w.wb2 + r.wb_bytes;
+    w.wb2 = w.wb1 + r.wb1_bytes;
+    w.et = w.wb2 + r.wb2_bytes;
     w.tt = w.et + r.et_bytes;
+    w.kend = r.pairs ? (int*)(w.tt + r.tt_bytes) : nullptr;
     return w;
 }
 int64_t chunk_rows(const ReconBulkShape& r, int64_t c) {
@@ -1379,20 +1509,20 @@ tc::ReconB1 recon_b1_problem(const EncodeDev& e, int slices, void* work, int64_t
     const ReconWork w = recon_work(r, work);
     const int64_t rows = chunk_rows(r, c);
     *items = rows * r.nt;
-    return tc::ReconB1{w.et, w.wb1, w.tt, rows, r.nt, r.kcn, slices};
+    return tc::ReconB1{w.et, w.wb1, w.tt, rows, r.nt, r.kcn, slices, r.kc1, r.tk, c * r.rows, w.kend};
 }
 tc::ReconB2 recon_b2_problem(const EncodeDev& e, int slices, float2* R, void* work, int64_t c, int64_t* items) {
     const ReconBulkShape r = recon_bulk_shape(e, slices);
     const ReconWork w = recon_work(r, work);
-    const int64_t rows = chunk_rows(r, c), M = e.Mk * e.C, j_off = c * r.rows * tc::BM;
+    const int64_t rows = chunk_rows(r, c);
     *items = rows * r.nt;
-    return tc::ReconB2{w.tt, w.wb2, R, rows, r.nt, r.kcn, e.N, M, j_off, std::min(rows * tc::BM, M - j_off), slices};
+    return tc::ReconB2{w.tt, w.wb2, R, rows, r.nt, r.kcn, e.N, e.Mk * e.C, r.tk, r.mrow, c * r.rows, slices};
 }
 }  // namespace
 
 size_t recon_bulk_bytes(const EncodeDev& e, int slices) {
     const ReconBulkShape r = recon_bulk_shape(e, slices);
-    return 2 * r.wb_bytes + 2 * r.et_bytes;
+    return r.wb1_bytes + r.wb2_bytes + r.et_bytes + r.tt_bytes + r.kend_bytes;
 }
 
 int64_t recon_bulk_chunks(const EncodeDev& e, int slices) { return recon_bulk_shape(e, slices).chunks; }
@@ -1401,7 +1531,16 @@ cudaError_t recon_bulk_wtables(const EncodeDev& e, const float2* W32, int slices
     const ReconBulkShape r = recon_bulk_shape(e, slices);
     const ReconWork w = recon_work(r, work);
     const dim3 wg((unsigned)r.kcn, (unsigned)r.nt);
-    for (int lower = 1; lower >= 0; --lower) {
+    if (r.pairs) {
+        const dim3 pg((unsigned)r.kc1, (unsigned)r.nt);
+        tc::k_pair_kend<<<(unsigned)((r.nt + 127) / 128), 128, 0, s>>>(e, r.nt, w.kend);
+        if (slices == 3)
+            tc::k_tab_wp<3><<<pg, 256, 0, s>>>(e, W32, r.nt, r.kc1, w.kend, w.wb1);
+        else
+            tc::k_tab_wp<2><<<pg, 256, 0, s>>>(e, W32, r.nt, r.kc1, w.kend, w.wb1);
+        note_launch(2);
+    }
+    for (int lower = r.pairs ? 0 : 1; lower >= 0; --lower) {
         if (slices == 3)
             tc::k_tab_w<3><<<wg, 256, 0, s>>>(W32, e.N, r.kcn, lower, lower ? w.wb1 : w.wb2);
         else
@@ -1416,6 +1555,16 @@ cudaError_t recon_bulk_et(const EncodeDev& e, int slices, void* work, int64_t c,
     const ReconWork w = recon_work(r, work);
     const int64_t rows = chunk_rows(r, c);
     if (rows <= 0) return cudaSuccess;
+    if (r.pairs) {  // one for all chunks and coils
+        if (c > 0) return cudaSuccess;
+        const dim3 pg((unsigned)r.kc1, (unsigned)r.tk);
+        if (slices == 3)
+            tc::k_tab_etp<3><<<pg, 256, 0, s>>>(e, r.kc1, w.et);
+        else
+            tc::k_tab_etp<2><<<pg, 256, 0, s>>>(e, r.kc1, w.et);
+        note_launch();
+        return cudaGetLastError();
+    }
     const dim3 eg((unsigned)r.kcn, (unsigned)rows);
     const int64_t j_off = c * r.rows * tc::BM;
     if (slices == 3)

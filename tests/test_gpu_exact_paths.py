@@ -149,3 +149,35 @@ def test_correction_many_frames(dims, frames, prec, ulp):
             x = pl.build().apply(torch.from_numpy(d).cuda()).cpu().numpy()
         for f in (0, frames // 2, frames - 1):
             assert rel(x[f], want[f]) < tol
+
+
+# Recon's first product over mirror pairs: even and odd axes (voxels without a partner), three
+# dimensions, a ragged voxel list, one coil, several voxel and sample tiles, chunks of samples
+@pytest.mark.parametrize("prec,tol", [(L.MIXED_BF16X6, 2e-6), (L.MIXED_BF16X3, 1e-4)])
+@pytest.mark.parametrize("dims,coils,samples,drop,chunk", [
+    ((16, 8), 1, 129, 0, ""), ((15, 9), 3, 200, 0, ""), ((5, 6, 7), 2, 257, 0, ""), ((20, 13), 2, 300, 61, ""),
+    ((31, 17), 3, 900, 0, "1"), ((24, 24), 2, 640, 5, "1")])
+def test_recon_over_mirror_pairs(dims, coils, samples, drop, chunk, prec, tol, monkeypatch):
+    """Both forms of T = W E^H against NumPy with the plan's own W: each of the two products
+    is off by the split arithmetic's tolerance on its inputs' magnitudes."""
+    if chunk:
+        monkeypatch.setenv("PINV_RECON_CHUNK_MB", chunk)
+    rng = np.random.default_rng(2309)
+    n, D = int(np.prod(dims)), len(dims)
+    vox = None if not drop else np.sort(rng.choice(n, n - drop, replace=False)).astype(np.int32)
+    k = rng.uniform(-0.5 * max(dims), 0.5 * max(dims), size=(samples, D))
+    maps = rng.standard_normal((coils, n)) + 1j * rng.standard_normal((coils, n))
+    pos = O.voxel_positions(dims)
+    if drop:
+        pos, maps = pos[vox], maps[:, vox]
+    E = O.encode(k, pos, maps, None, None)
+    for pairs in ("1", "0"):
+        monkeypatch.setenv("PINV_RECON_PAIRS", pairs)
+        with _plan(dims, k, maps, lam=1e-2, precision=prec, recon_mode=L.RECON_STORE, voxel_index=vox) as pl:
+            pl.build()
+            W = pl.export(L.EXPORT_LINV).cpu().numpy()
+            R = pl.export(L.EXPORT_RECON).cpu().numpy()
+        T = W @ E.conj().T
+        want = W.conj().T @ T
+        amp = np.linalg.norm(W) * np.linalg.norm(T) / np.linalg.norm(want)
+        assert rel(R, want) < tol * max(1.0, amp), pairs
