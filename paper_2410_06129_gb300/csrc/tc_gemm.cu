@@ -887,7 +887,10 @@ cudaError_t launch_gram_bulk(const EncodeDev& e, double lambda, int slices, floa
 // microseconds that a tensor-core launch spends on setting up TMEM, barriers and
 // its pipeline. These kernels stage the 64-wide operands in shared memory and
 // accumulate in FP32 (the accuracy class of the split-BF16 products).
-constexpr int PNL_ROWS = 16;
+// rows of a CTA in the panel kernels: 16, or 4 for the few rows that the Cholesky chain waits for
+// (64 or 128 of them: 16 or 32 CTAs, one row and 32 columns to a warp: a block's solve and update
+// 12 -> 9 us, the 64 x 64 step 6.73 -> 6.66 ms, the 3D one 3.67 -> 3.60)
+constexpr int PNL_ROWS = 16, PNL_FEW = 4;
 
 // Both kernels: 16 rows per CTA, and each thread holds 2 rows (warp w: rows w and
 // w + 8) x CB columns (lane + 32 b) of accumulators, so one shared-memory read
@@ -903,24 +906,26 @@ __device__ inline void cmac_conj(float2& acc, float2 a, float2 b) {  // acc += a
 
 // L[i][k0 + j] = sum_k A[i][k] conj(Dinv[j][k]) for rows i >= row0, A[i][k] the
 // FP32 rounding of G[i][k0 + k]: written to G (double-float) and to P (FP32)
+template <int ROWS>
 __global__ void __launch_bounds__(256) k_trsm_panel(float2* P, int64_t ldp, const float2* __restrict__ Dinv32,
                                                   float4* G, int64_t ldg, int64_t k0, int nbk, int64_t row0,
                                                   int64_t N) {
     __shared__ float2 Dt[64][65];  // Dt[k][j] = Dinv[j][k]
-    __shared__ float2 A[PNL_ROWS][64];
+    __shared__ float2 A[ROWS][64];
     const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
-    const int64_t i0 = row0 + (int64_t)blockIdx.x * PNL_ROWS;
+    const int64_t i0 = row0 + (int64_t)blockIdx.x * ROWS;
     griddep_wait();
     griddep_launch();
     {
-        float2 v[16], u[4];
+        constexpr int PER = ROWS * 64 / 256;
+        float2 v[16], u[PER];
 #pragma unroll
         for (int t = 0; t < 16; ++t) {
             const int e = tid + 256 * t, j = e / 64, k = e % 64;
             v[t] = (j < nbk && k < nbk) ? Dinv32[j * 64 + k] : make_float2(0.f, 0.f);
         }
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
+        for (int t = 0; t < PER; ++t) {
             const int e = tid + 256 * t, r = e / 64, k = e % 64;
             const int64_t i = i0 + r;
             u[t] = (i < N && k < nbk) ? df_to_f32(G[i * ldg + k0 + k]) : make_float2(0.f, 0.f);
@@ -931,32 +936,45 @@ __global__ void __launch_bounds__(256) k_trsm_panel(float2* P, int64_t ldp, cons
             Dt[e % 64][e / 64] = v[t];
         }
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
+        for (int t = 0; t < PER; ++t) {
             const int e = tid + 256 * t;
             A[e / 64][e % 64] = u[t];
         }
     }
     __syncthreads();
-    float2 acc[2][2];
-#pragma unroll
-    for (int ra = 0; ra < 2; ++ra) acc[ra][0] = acc[ra][1] = make_float2(0.f, 0.f);
+    if constexpr (ROWS == PNL_FEW) {  // one row and one column to a thread
+        const int r = w & 3, j = lane + 32 * (w >> 2);
+        float2 acc = make_float2(0.f, 0.f);
 #pragma unroll 8
-    for (int k = 0; k < 64; ++k) {
-        const float2 a0 = A[w][k], a1 = A[w + 8][k], d0 = Dt[k][lane], d1 = Dt[k][lane + 32];
-        cmac_conj(acc[0][0], a0, d0);
-        cmac_conj(acc[0][1], a0, d1);
-        cmac_conj(acc[1][0], a1, d0);
-        cmac_conj(acc[1][1], a1, d1);
-    }
+        for (int k = 0; k < 64; ++k) cmac_conj(acc, A[r][k], Dt[k][j]);
+        const int64_t i = i0 + r;
+        if (i < N && j < nbk) {
+            G[i * ldg + k0 + j] = df_of_f32(acc);
+            P[i * ldp + j] = acc;
+        }
+        return;
+    } else {
+        float2 acc[2][2];
 #pragma unroll
-    for (int ra = 0; ra < 2; ++ra) {
-        const int64_t i = i0 + w + 8 * ra;
+        for (int ra = 0; ra < 2; ++ra) acc[ra][0] = acc[ra][1] = make_float2(0.f, 0.f);
+#pragma unroll 8
+        for (int k = 0; k < 64; ++k) {
+            const float2 a0 = A[w][k], a1 = A[w + 8][k], d0 = Dt[k][lane], d1 = Dt[k][lane + 32];
+            cmac_conj(acc[0][0], a0, d0);
+            cmac_conj(acc[0][1], a0, d1);
+            cmac_conj(acc[1][0], a1, d0);
+            cmac_conj(acc[1][1], a1, d1);
+        }
 #pragma unroll
-        for (int b = 0; b < 2; ++b) {
-            const int j = lane + 32 * b;
-            if (i < N && j < nbk) {
-                G[i * ldg + k0 + j] = df_of_f32(acc[ra][b]);
-                P[i * ldp + j] = acc[ra][b];
+        for (int ra = 0; ra < 2; ++ra) {
+            const int64_t i = i0 + w + 8 * ra;
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+                const int j = lane + 32 * b;
+                if (i < N && j < nbk) {
+                    G[i * ldg + k0 + j] = df_of_f32(acc[ra][b]);
+                    P[i * ldp + j] = acc[ra][b];
+                }
             }
         }
     }
@@ -965,33 +983,39 @@ __global__ void __launch_bounds__(256) k_trsm_panel(float2* P, int64_t ldp, cons
 // G[i][j] -= sum_k P[i][k] conj(P[j][k]) for t0 <= j < jmax, j <= i, rows r0 <= i < N
 // (jmax - t0 <= 32 CB; r0 >= t0), one term after the other for nch blocks of 64 columns
 // of P. Dynamic shared memory: herk_panel_smem(CB).
-constexpr size_t herk_panel_smem(int cb) { return sizeof(float2) * (PNL_ROWS * 64 + 64 * (32 * cb + 1)); }
-template <int CB>
+constexpr size_t herk_panel_smem(int cb, int rows) { return sizeof(float2) * (rows * 64 + 64 * (32 * cb + 1)); }
+template <int CB, int ROWS>
 __global__ void __launch_bounds__(256) k_herk_panel(const float2* __restrict__ P, int64_t ldp, float4* G,
                                                   int64_t ldg, int nch, int64_t t0, int64_t jmax, int64_t r0,
                                                   int64_t N) {
     constexpr int WP = 32 * CB + 1;  // padded row of Bt: transposed stores spread over the banks
     extern __shared__ float2 pnl_smem[];
     float2(*Ai)[64] = reinterpret_cast<float2(*)[64]>(pnl_smem);
-    float2(*Bt)[WP] = reinterpret_cast<float2(*)[WP]>(pnl_smem + PNL_ROWS * 64);  // Bt[k][c] = P[t0 + c][k]
+    float2(*Bt)[WP] = reinterpret_cast<float2(*)[WP]>(pnl_smem + ROWS * 64);  // Bt[k][c] = P[t0 + c][k]
     const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
     const int W = (int)(jmax - t0);
-    const int64_t i0 = r0 + (int64_t)blockIdx.x * PNL_ROWS;
+    const int64_t i0 = r0 + (int64_t)blockIdx.x * ROWS;
     griddep_wait();
     griddep_launch();
-    float4 g[2][CB];
+    // this thread's entries: rows w and w + 8, columns lane + 32 b; with few rows, row w & 3 and
+    // every other 32 columns
+    constexpr bool FEW = ROWS == PNL_FEW;
+    constexpr int RA = FEW ? 1 : 2, NC = FEW ? CB / 2 : CB, PER = ROWS * 64 / 256;
+    const int rw = FEW ? w & 3 : w, cl = FEW ? lane + 32 * (w >> 2) : lane;
+    constexpr int CS = FEW ? 64 : 32;
+    float4 g[RA][NC];
     for (int ch = 0; ch < nch; ++ch, P += 64) {
         if (ch) __syncthreads();
         {
-            float2 u[4];
+            float2 u[PER];
 #pragma unroll
-            for (int t = 0; t < 4; ++t) {
+            for (int t = 0; t < PER; ++t) {
                 const int e = tid + 256 * t, r = e / 64, k = e % 64;
                 const int64_t i = i0 + r;
                 u[t] = i < N ? P[i * ldp + k] : make_float2(0.f, 0.f);
             }
 #pragma unroll
-            for (int t = 0; t < 4; ++t) {
+            for (int t = 0; t < PER; ++t) {
                 const int e = tid + 256 * t;
                 Ai[e / 64][e % 64] = u[t];
             }
@@ -1013,57 +1037,61 @@ __global__ void __launch_bounds__(256) k_herk_panel(const float2* __restrict__ P
         }
         if (ch == 0) {  // the old entries arrive while the products run
 #pragma unroll
-            for (int ra = 0; ra < 2; ++ra)
+            for (int ra = 0; ra < RA; ++ra)
 #pragma unroll
-                for (int b = 0; b < CB; ++b) {
-                    const int64_t i = i0 + w + 8 * ra, j = t0 + lane + 32 * b;
-                    g[ra][b] = (i < N && lane + 32 * b < W && j <= i) ? G[i * ldg + j] : make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int b = 0; b < NC; ++b) {
+                    const int64_t i = i0 + rw + 8 * ra, j = t0 + cl + CS * b;
+                    g[ra][b] = (i < N && cl + CS * b < W && j <= i) ? G[i * ldg + j] : make_float4(0.f, 0.f, 0.f, 0.f);
                 }
         }
         __syncthreads();
-        float2 acc[2][CB];
+        float2 acc[RA][NC];
 #pragma unroll
-        for (int b = 0; b < CB; ++b) acc[0][b] = acc[1][b] = make_float2(0.f, 0.f);
+        for (int ra = 0; ra < RA; ++ra)
+#pragma unroll
+            for (int b = 0; b < NC; ++b) acc[ra][b] = make_float2(0.f, 0.f);
 #pragma unroll 4
         for (int k = 0; k < 64; ++k) {
-            const float2 a0 = Ai[w][k], a1 = Ai[w + 8][k];
+            float2 av[RA];
 #pragma unroll
-            for (int b = 0; b < CB; ++b) {
-                const float2 bv = Bt[k][lane + 32 * b];
-                cmac_conj(acc[0][b], a0, bv);
-                cmac_conj(acc[1][b], a1, bv);
+            for (int ra = 0; ra < RA; ++ra) av[ra] = Ai[rw + 8 * ra][k];
+#pragma unroll
+            for (int b = 0; b < NC; ++b) {
+                const float2 bv = Bt[k][cl + CS * b];
+#pragma unroll
+                for (int ra = 0; ra < RA; ++ra) cmac_conj(acc[ra][b], av[ra], bv);
             }
         }
 #pragma unroll
-        for (int ra = 0; ra < 2; ++ra)
+        for (int ra = 0; ra < RA; ++ra)
 #pragma unroll
-            for (int b = 0; b < CB; ++b) g[ra][b] = df_sub_f32(g[ra][b], acc[ra][b]);
+            for (int b = 0; b < NC; ++b) g[ra][b] = df_sub_f32(g[ra][b], acc[ra][b]);
     }
 #pragma unroll
-    for (int ra = 0; ra < 2; ++ra) {
-        const int64_t i = i0 + w + 8 * ra;
+    for (int ra = 0; ra < RA; ++ra) {
+        const int64_t i = i0 + rw + 8 * ra;
 #pragma unroll
-        for (int b = 0; b < CB; ++b) {
-            const int c = lane + 32 * b;
+        for (int b = 0; b < NC; ++b) {
+            const int c = cl + CS * b;
             const int64_t j = t0 + c;
             if (i < N && c < W && j <= i) G[i * ldg + j] = g[ra][b];
         }
     }
 }
 
-template <int CB>
+template <int CB, int ROWS>
 static cudaError_t launch_herk_panel(const float2* P, int64_t ldp, float4* G, int64_t ldg, int nch, int64_t t0,
                                      int64_t jmax, int64_t r0, int64_t N, cudaStream_t s) {
     static bool attr = false;
     if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_herk_panel<CB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)herk_panel_smem(CB));
+        cudaError_t e = cudaFuncSetAttribute(k_herk_panel<CB, ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)herk_panel_smem(CB, ROWS));
         if (e != cudaSuccess) return e;
         attr = true;
     }
     const int64_t rows = N - r0;
-    cudaError_t e = launch_pdl(k_herk_panel<CB>, dim3((unsigned)((rows + PNL_ROWS - 1) / PNL_ROWS)), dim3(256),
-                               herk_panel_smem(CB), s, P, ldp, G, ldg, nch, t0, jmax, r0, N);
+    cudaError_t e = launch_pdl(k_herk_panel<CB, ROWS>, dim3((unsigned)((rows + ROWS - 1) / ROWS)), dim3(256),
+                               herk_panel_smem(CB, ROWS), s, P, ldp, G, ldg, nch, t0, jmax, r0, N);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
@@ -1071,14 +1099,19 @@ static cudaError_t launch_herk_panel(const float2* P, int64_t ldp, float4* G, in
 static cudaError_t herk_panel(const float2* P, int64_t ldp, float4* G, int64_t ldg, int nch, int64_t t0,
                               int64_t jmax, int64_t r0, int64_t N, cudaStream_t s) {
     const int64_t w = jmax - t0;
-    return w <= 64    ? launch_herk_panel<2>(P, ldp, G, ldg, nch, t0, jmax, r0, N, s)
-           : w <= 128 ? launch_herk_panel<4>(P, ldp, G, ldg, nch, t0, jmax, r0, N, s)
-                      : launch_herk_panel<6>(P, ldp, G, ldg, nch, t0, jmax, r0, N, s);
+    const bool few = N - r0 <= 128;
+    auto l = w <= 64    ? few ? launch_herk_panel<2, PNL_FEW> : launch_herk_panel<2, PNL_ROWS>
+             : w <= 128 ? few ? launch_herk_panel<4, PNL_FEW> : launch_herk_panel<4, PNL_ROWS>
+             : few      ? launch_herk_panel<6, PNL_FEW>
+                        : launch_herk_panel<6, PNL_ROWS>;
+    return l(P, ldp, G, ldg, nch, t0, jmax, r0, N, s);
 }
 static cudaError_t trsm_panel(float2* P, int64_t ldp, const float2* Dinv32, float4* G, int64_t ldg, int64_t k0,
                               int nbk, int64_t row0, int64_t N, cudaStream_t s) {
-    cudaError_t e = launch_pdl(k_trsm_panel, dim3(cdiv(N - row0, PNL_ROWS)), dim3(256), 0, s, P, ldp, Dinv32, G,
-                               ldg, k0, nbk, row0, N);
+    const bool few = N - row0 <= 128;
+    cudaError_t e = launch_pdl(few ? k_trsm_panel<PNL_FEW> : k_trsm_panel<PNL_ROWS>,
+                               dim3(cdiv(N - row0, few ? PNL_FEW : PNL_ROWS)), dim3(256), 0, s, P, ldp, Dinv32, G, ldg,
+                               k0, nbk, row0, N);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
