@@ -594,14 +594,22 @@ __global__ void __launch_bounds__(DIAG_THREADS) k_potrf_diag_df(float4* G, int64
 // apply the previous four rows' terms to the rows below and write the finished
 // rows of X, and rank 2 the panel of L, to global memory.
 //
+// While the inverse has few rows, rank 2 also takes the terms of the first DHP panels
+// for the entries right of column DHC, loaded from G by itself: rank 0's updates bound
+// the early panels. It puts them into rank 0's shared memory, where rank 0 takes them
+// over two panels later with the terms of the panels since (two, so that it need not wait):
+// 32.8 -> 30.2 us a block (other shares, columns from 24, 28, 36 and 40 on: 30.7, 30.3, 30.5
+// and 31.2).
+//
 // Every entry takes the same operations in the same order as in the one-CTA
 // sweep above (right-looking, one term per column, renormalised after each),
 // only spread differently over threads. The block is a serial chain: with one
 // column at a time, on two CTAs (a barrier, a trip through shared memory and a
 // square root for each column), it took 49 us; with panels of four, set-up
-// and stores beside the chain and the inverse on two CTAs it takes 33 us,
-// of which the 16 panels' chains are about 12, the trailing updates that do not
-// hide behind them 10 and launch, load and cluster set-up 7.
+// and stores beside the chain and the inverse on two CTAs it took 33 us, with rank 2's
+// help it takes 30: launch and load 3, 16 panels of 1.2 us (two barriers, the update of
+// the panel's own entries, the chain of four columns) and what the early ones' updates
+// take beyond that, and 2 until the inverse has followed.
 constexpr int DIAG_SITE = 20;
 constexpr long long DIAG_WAIT_LIMIT = 4000000000LL;
 constexpr int DPW = 4;                                   // panel width
@@ -610,6 +618,10 @@ constexpr int DU0 = 96;                                  // rank 0: first update
 constexpr int DU1 = 64;                                  // ranks 1, 2: first update thread (30 update warps)
 constexpr int DNE0 = (NBD - DPW) * (NBD - DPW + 1) / 2;  // 1830 entries (i, c), DPW <= c <= i
 constexpr int DNE1 = NBD * (NBD - DPW) / 4;              // 960 entries left of their row's panel, a rank's columns
+constexpr int DHC = 32, DHP = 5;                         // rank 2's help: first column, panels
+constexpr int DHB = DPW * (DHP + 2);                     // the panel at which rank 0 takes over
+constexpr int DNH = (NBD - DHC) * (NBD - DHC + 1) / 2;   // 528 entries (i, c), DHC <= c <= i
+static_assert(DHB + DPW <= DHC && DNH <= DIAG_THREADS - DU1, "taken over before their panel");
 constexpr int DIS = DPW * NBD / 2;                       // threads that write a panel of X: the last DIS
 static_assert(DNE0 <= DUE * (DIAG_THREADS - DU0) && DNE1 <= DIAG_THREADS - DU1, "update entries per thread");
 // A (rank 0) or X (ranks 1, 2); Lb[j][i] = L_ij as received; r_j; L_jj on rank 0
@@ -745,7 +757,7 @@ __global__ void __cluster_dims__(3, 1, 1) __launch_bounds__(DIAG_THREADS)
     float4* Lb = smd + NBD * NBDP;                          // others: Lb[j][i] = L_ij
     float2* rb = reinterpret_cast<float2*>(Lb + NBD * NBD);  // r_j
     float2* Ld = rb + NBD;                                  // L_jj
-    __shared__ unsigned flag;  // ranks 1, 2: panels of L published by rank 0
+    __shared__ unsigned flag;  // ranks 1, 2: panels of L published by rank 0; rank 0: rank 2's entries are there
     __shared__ int stop;
     const int tid = threadIdx.x, wid = tid >> 5;
     const unsigned rank = cl.block_rank();
@@ -831,15 +843,25 @@ __global__ void __cluster_dims__(3, 1, 1) __launch_bounds__(DIAG_THREADS)
                     }
                 }
                 bar_named<1, DIAG_THREADS - 32>();
+                if (b == DHB) {
+                    if ((tid & 31) == 0) diag_wait(&flag, 1u, st);
+                    __syncwarp();
+                }
 #pragma unroll
                 for (int k = 0; k < DUE; ++k) {
-                    if (uc[k] >= b + DPW) {
+                    if (uc[k] < b + DPW || (uc[k] >= DHC && b < DHB)) continue;
+                    int t0 = b - DPW;
+                    if (uc[k] >= DHC && b == DHB) {
+                        uv[k] = A[ui[k] * NBDP + uc[k]];
+                        t0 = DPW * DHP;
+                    }
+#pragma unroll 1
+                    for (; t0 < b; t0 += DPW)
 #pragma unroll
-                        for (int t = b - DPW; t < b; ++t) {
+                        for (int t = t0; t < t0 + DPW; ++t) {
                             cacc(uv[k], cdf_neg(A[ui[k] * NBDP + t]), cdf_conj(A[uc[k] * NBDP + t]));
                             uv[k] = df_norm(uv[k]);
                         }
-                    }
                 }
             }
             __syncthreads();
@@ -852,7 +874,32 @@ __global__ void __cluster_dims__(3, 1, 1) __launch_bounds__(DIAG_THREADS)
         float4 y = uv[0];
         float4* Gk = G + k0 * ld + k0;
         float2* Lk = L32 ? L32 + k0 * ldl + k0 : nullptr;
+        // rank 2's help
+        int hi = -1, hc = -1;
+        float4 hv = make_float4(0.f, 0.f, 0.f, 0.f);
+        float4* rA = cl.map_shared_rank(A, 0);
+        unsigned* flag0 = cl.map_shared_rank(&flag, 0);
+        if (rank == 2 && tid >= DU1 && tid - DU1 < DNH) {
+            tri_index(tid - DU1, hi, hc);
+            hi += DHC;
+            hc += DHC;
+            hv = hi < nb ? Gk[hi * ld + hc] : make_float4(hi == hc ? 1.f : 0.f, 0.f, 0.f, 0.f);
+        }
         for (int b = 0; b < NBD; b += DPW) {
+            if (rank == 2 && tid >= DU1 && b > 0 && b <= DPW * DHP) {
+                if (hi >= 0) {
+#pragma unroll
+                    for (int t = b - DPW; t < b; ++t) {
+                        cacc(hv, cdf_neg(Lb[t * NBD + hi]), cdf_conj(Lb[t * NBD + hc]));
+                        hv = df_norm(hv);
+                    }
+                    if (b == DPW * DHP) rA[hi * NBDP + hc] = hv;
+                }
+                if (b == DPW * DHP) {
+                    bar_named<3, DIAG_THREADS - DU1>();
+                    if (tid == DU1) st_release_cluster(flag0, 1u);
+                }
+            }
             if (wid == 0) {
                 int ok = 1;
                 if (tid == 0) ok = diag_wait(&flag, (unsigned)(b / DPW + 1), st);

@@ -32,8 +32,9 @@
 // the last drain. A 128-row tile covers 128 voxels and 32 samples a stage where the
 // complex embedding covers 16: half the MMAs, half the digit table and half the data
 // digits. A voxel without a mirror in the plan (grid edge, mask) is a pair of one, which
-// costs what the complex embedding would. Measured with folded columns and the longer
-// drain groups: see k_exact.
+// costs what the complex embedding would. Measured at 64 x 64, 8 coils, 8192 samples
+// with pairs, columns folded over coils and the longer drain groups: E^H d of 64 frames
+// 1.81 -> 0.98 ms, the apply of one frame 1.76 -> 1.06 ms.
 //
 // Tiles are 128 rows x 32 columns (64 output columns, real and imaginary parts side
 // by side, as in the split-BF16 engine), or narrower (16, 8) where there are fewer

@@ -1,8 +1,10 @@
-// FP64 complex tile engine and the FP64 path's contraction kernels.
+// FP64 complex tile engine and the FP64 path's SIMT contraction kernels: the FP64
+// factorisation's steps inside a panel, and, where there are no tensor cores or no room for
+// their tables, every contraction of the FP64 path (else they are exact digit products on
+// the tensor cores, oz.cu).
 //
-// GB300 has few FP64 units (no FP64 tensor-core kind in tcgen05), so every
-// FP64 contraction here is a SIMT DFMA kernel. One engine serves all of them:
-// a CTA of 256 threads computes a BM x BN tile of C[i][j] = sum_k a(i,k) b(k,j)
+// GB300 has few FP64 units and no FP64 tensor-core kind in tcgen05. One engine serves all
+// the contractions: a CTA of 256 threads computes a BM x BN tile of C[i][j] = sum_k a(i,k) b(k,j)
 // where a() and b() are operand functors that either read memory or generate
 // encoding-matrix elements on the fly (the encoding matrix is never stored).
 // Tiles are staged through shared memory BK = 16 at a time; each thread owns a
@@ -420,7 +422,7 @@ constexpr int NBO = 64;  // panels
 // and Y_ic -= S_i Y_jc up to it (Y, the inverse, unscaled). Warp w holds rows w + 8 t, lane
 // c column c, in registers; an entry of A is published before its column's step, a row of
 // Y before its row's. Columns and rows are scaled by 1 / sqrt(d_j) at the end. (All warps
-// dividing, and the inverse by shuffled dot products, took 72 us.)
+// dividing, and the inverse by shuffled dot products, took 72 us, this 53.)
 __global__ void __launch_bounds__(256) k_potrf_diag32(double2* G, int64_t ld, int64_t N, int64_t k0, double2* Dinv,
                                                       DevStatus* st) {
     __shared__ double2 At[NBS][NBS];  // At[j][i] = A_ij once column j is final
