@@ -1,19 +1,18 @@
 // Batched build and apply of several plans of uneven size.
 //
 // A batch groups existing plans (many slices, time series or trajectories).
-// Its build runs the dominant tensor-core work of all plans as shared
-// persistent launches: one launch forms the Gram of every plan that keeps no
-// exact one (those form theirs on their own streams), and per chunk of
-// samples one launch forms every plan's T = W E^H and one every plan's
-// Recon = W^H T (all bulk-fed from per-plan operand tables); the sequential
-// Cholesky and triangular inverse of each plan run concurrently on per-plan
-// streams between them. Its apply runs every plan's apply (Recon x data plus
+// One persistent launch forms the Gram of every plan that keeps no exact one,
+// bulk-fed from per-plan operand tables; then every plan's build runs on its own
+// stream, its Cholesky and inverse, latency-bound chains, beside the others' and
+// beside the Recon products of the plans that are done with theirs. (Shared launches of
+// all plans' Recon after the last chain left most SMs idle until then: batch of six plans
+// 51.2 ms, so 47.6; with the Recon launches on 2/3 of the SMs 48.8.) Its apply runs every plan's apply (Recon x data plus
 // refinement) concurrently on the per-plan streams. With PINV_BATCH_GRAPH the
 // whole sequence is captured once into a CUDA graph and replayed, so a step
 // of hundreds of launches costs one graph launch on the host.
 //
 // Results are bit-identical to building and applying the plans one by one:
-// the shared launches run the same tile code over the same K order.
+// the shared launch runs the same tile code over the same K order.
 #include <algorithm>
 #include <cstring>
 #include <vector>
@@ -33,7 +32,6 @@ struct pinv_batch {
     void* work = nullptr;
     std::vector<void*> pwork;
     TcMulti gram;
-    std::vector<TcMulti> rec1, rec2;  // per chunk of samples
     DevStatus* st = nullptr;
     DevStatus* st_host = nullptr;
     // graphs: the build is captured on its second call (the first runs
@@ -54,8 +52,6 @@ pinv_batch::~pinv_batch() {
     if (build_exec) cudaGraphExecDestroy(build_exec);
     if (apply_exec) cudaGraphExecDestroy(apply_exec);
     tc_multi_free(&gram);
-    for (auto& m : rec1) tc_multi_free(&m);
-    for (auto& m : rec2) tc_multi_free(&m);
     if (work) cudaFree(work);
     for (void* p : scratch)
         if (p) cudaFree(p);
@@ -115,15 +111,10 @@ pinv_status build_sequence(pinv_batch* b, cudaStream_t s) {
                 CKB(gram_bulk_finish(p->enc, p->lambda_abs, b->slices, (float4*)p->G, p->N, b->pwork[i], b->side[i]));
             STB(build_gram(p, b->side[i], p->Gx != nullptr));
             STB(build_factor(p, b->side[i], false));
-            if (p->recon) CKB(recon_bulk_wtables(p->enc, p->W32, b->slices, b->pwork[i], b->side[i]));
+            if (p->recon)
+                CKB(launch_recon_bulk(p->enc, p->W32, b->slices, (float2*)p->R, b->pwork[i], p->st, b->side[i]));
         }
         STB(join_all(b, s));
-        for (size_t c = 0; c < b->rec1.size(); ++c) {
-            for (size_t i = 0; i < n; ++i)
-                if (b->plans[i]->recon) CKB(recon_bulk_et(b->plans[i]->enc, b->slices, b->pwork[i], (int64_t)c, s));
-            CKB(tc_multi_launch(b->rec1[c], b->slices, b->st, s));  // every plan's W E^H over chunk c
-            CKB(tc_multi_launch(b->rec2[c], b->slices, b->st, s));  // every plan's W^H (W E^H)
-        }
     } else {
         STB(fork_all(b, s));
         for (size_t i = 0; i < b->plans.size(); ++i) {
@@ -224,35 +215,22 @@ pinv_status pinv_batch_create(pinv_plan* const* plans, int n, int flags, pinv_ba
         // operand tables of every plan: the Gram's, then (same memory) the Recon's
         size_t bytes = 0;
         std::vector<size_t> off(n, 0);
-        int64_t chunks = 0;
         for (int i = 0; i < n; ++i) {
             const pinv_plan* p = b->plans[i];
             size_t need = p->Gx ? 0 : gram_bulk_bytes(p->enc, b->slices);
-            if (p->recon) {
-                need = std::max(need, recon_bulk_bytes(p->enc, b->slices));
-                chunks = std::max(chunks, recon_bulk_chunks(p->enc, b->slices));
-            }
+            if (p->recon) need = std::max(need, recon_bulk_bytes(p->enc, b->slices));
             off[i] = bytes;
             bytes += (need + 255) & ~(size_t)255;
         }
         cudaError_t e = bytes ? cudaMalloc(&b->work, bytes) : cudaSuccess;
         if (e != cudaSuccess) return bad(cuda_err(e, "batch workspace"));
-        std::vector<TcPlanArgs> all, rec;
+        std::vector<TcPlanArgs> all;
         for (int i = 0; i < n; ++i) {
             pinv_plan* p = b->plans[i];
             b->pwork.push_back((unsigned char*)b->work + off[i]);
-            const TcPlanArgs a{&p->enc, p->lambda_abs, (float4*)p->G, p->W32, (float2*)p->R, b->pwork[i]};
-            if (!p->Gx) all.push_back(a);
-            if (p->recon) rec.push_back(a);
+            if (!p->Gx) all.push_back(TcPlanArgs{&p->enc, p->lambda_abs, (float4*)p->G, b->pwork[i]});
         }
-        e = tc_multi_create(TC_MULTI_GRAM, all.data(), (int)all.size(), b->slices, 0, &b->gram);
-        b->rec1.resize(chunks);
-        b->rec2.resize(chunks);
-        for (int64_t c = 0; c < chunks && e == cudaSuccess; ++c) {
-            e = tc_multi_create(TC_MULTI_RECON1, rec.data(), (int)rec.size(), b->slices, c, &b->rec1[c]);
-            if (e == cudaSuccess)
-                e = tc_multi_create(TC_MULTI_RECON2, rec.data(), (int)rec.size(), b->slices, c, &b->rec2[c]);
-        }
+        e = tc_multi_create(all.data(), (int)all.size(), b->slices, &b->gram);
         if (e != cudaSuccess) return bad(cuda_err(e, "batch descriptors"));
     }
     *out = b;

@@ -318,36 +318,27 @@ cudaError_t launch_to_df(const double2* src, float4* dst, int64_t n, cudaStream_
 cudaError_t launch_reset_status(DevStatus* st, cudaStream_t s);
 cudaError_t launch_merge_timeout(DevStatus* dst, const DevStatus* src, cudaStream_t s);
 
-// Several plans' tensor-core Gram or Recon in one persistent launch. The
+// Several plans' tensor-core Gram in one persistent launch. The
 // problem descriptors are uploaded once (tc_multi_create) and stay valid
 // while the plans and buffers they point to live.
 struct TcPlanArgs {
     const EncodeDev* e;
     double lam;
     float4* G;            // Gram output (lower tiles, double-float), ld = N
-    const float2* W32;    // W = L^-1, FP32 [N][N]
-    float2* R;            // Recon [N][M]
-    void* work;           // operand tables: gram_bulk_bytes() for the Gram, recon_bulk_bytes() for Recon
+    void* work;           // operand tables, gram_bulk_bytes()
 };
-enum TcMultiKind { TC_MULTI_GRAM = 0, TC_MULTI_RECON1 = 1, TC_MULTI_RECON2 = 2 };
 struct TcMulti {
     void* buf = nullptr;
-    int kind = 0, n = 0;
+    int n = 0;
     int64_t items = 0;
     size_t off_start = 0, off_gx = 0;
 };
-// Shared persistent launches of bulk-fed problems over several plans: every
-// plan's Gram, or the two Recon steps over sample chunk `chunk` of every plan
-// that has it. The per-plan stages around them (tables, split sums) are the
-// gram_bulk_* / recon_bulk_* calls.
-cudaError_t tc_multi_create(int kind, const TcPlanArgs* args, int n, int slices, int64_t chunk, TcMulti* out);
+// The per-plan stages around it (tables, split sums) are the gram_bulk_* calls.
+cudaError_t tc_multi_create(const TcPlanArgs* args, int n, int slices, TcMulti* out);
 cudaError_t tc_multi_launch(const TcMulti& m, int slices, DevStatus* st, cudaStream_t s);
 cudaError_t gram_bulk_table(const EncodeDev& e, int slices, void* work, cudaStream_t s);
 cudaError_t gram_bulk_finish(const EncodeDev& e, double lambda, int slices, float4* G, int64_t ld, void* work,
                              cudaStream_t s);
-int64_t recon_bulk_chunks(const EncodeDev& e, int slices);
-cudaError_t recon_bulk_wtables(const EncodeDev& e, const float2* W32, int slices, void* work, cudaStream_t s);
-cudaError_t recon_bulk_et(const EncodeDev& e, int slices, void* work, int64_t chunk, cudaStream_t s);
 void tc_multi_free(TcMulti* m);
 
 // ||G||_1 into st->norm1_g, from the lower triangle of G before the Cholesky

@@ -1558,9 +1558,7 @@ size_t recon_bulk_bytes(const EncodeDev& e, int slices) {
     return r.wb1_bytes + r.wb2_bytes + r.et_bytes + r.tt_bytes + r.kend_bytes;
 }
 
-int64_t recon_bulk_chunks(const EncodeDev& e, int slices) { return recon_bulk_shape(e, slices).chunks; }
-
-cudaError_t recon_bulk_wtables(const EncodeDev& e, const float2* W32, int slices, void* work, cudaStream_t s) {
+static cudaError_t recon_bulk_wtables(const EncodeDev& e, const float2* W32, int slices, void* work, cudaStream_t s) {
     const ReconBulkShape r = recon_bulk_shape(e, slices);
     const ReconWork w = recon_work(r, work);
     const dim3 wg((unsigned)r.kcn, (unsigned)r.nt);
@@ -1583,7 +1581,7 @@ cudaError_t recon_bulk_wtables(const EncodeDev& e, const float2* W32, int slices
     return cudaGetLastError();
 }
 
-cudaError_t recon_bulk_et(const EncodeDev& e, int slices, void* work, int64_t c, cudaStream_t s) {
+static cudaError_t recon_bulk_et(const EncodeDev& e, int slices, void* work, int64_t c, cudaStream_t s) {
     const ReconBulkShape r = recon_bulk_shape(e, slices);
     const ReconWork w = recon_work(r, work);
     const int64_t rows = chunk_rows(r, c);
@@ -1612,7 +1610,7 @@ cudaError_t launch_recon_bulk(const EncodeDev& e, const float2* W32, int slices,
                               DevStatus* st, cudaStream_t s) {
     cudaError_t err = recon_bulk_wtables(e, W32, slices, work, s);
     if (err != cudaSuccess) return err;
-    const int64_t chunks = recon_bulk_chunks(e, slices);
+    const int64_t chunks = recon_bulk_shape(e, slices).chunks;
     for (int64_t c = 0; c < chunks; ++c) {
         if ((err = recon_bulk_et(e, slices, work, c, s)) != cudaSuccess) return err;
         int64_t items = 0;
@@ -1625,36 +1623,20 @@ cudaError_t launch_recon_bulk(const EncodeDev& e, const float2* W32, int slices,
 }
 
 // ------------------------------------------------------------------ batched launches
-cudaError_t tc_multi_create(int kind, const TcPlanArgs* a, int n, int slices, int64_t chunk, TcMulti* out) {
+cudaError_t tc_multi_create(const TcPlanArgs* a, int n, int slices, TcMulti* out) {
     *out = TcMulti{};
-    out->kind = kind;
     std::vector<int64_t> start(1, 0), gx;
     std::vector<unsigned char> probs;  // problem descriptors, stride sizeof(problem)
-    // plans with the longest tiles first (K per tile: M_k for the Gram, up to N for Recon)
+    // plans with the longest tiles (K = M_k) first
     std::vector<int> order(n);
     for (int i = 0; i < n; ++i) order[i] = i;
-    std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
-        const int64_t kx = kind == TC_MULTI_GRAM ? a[x].e->Mk : a[x].e->N;
-        const int64_t ky = kind == TC_MULTI_GRAM ? a[y].e->Mk : a[y].e->N;
-        return kx > ky;
-    });
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return a[x].e->Mk > a[y].e->Mk; });
     for (int ii = 0; ii < n; ++ii) {
         const int i = order[ii];
         const EncodeDev& e = *a[i].e;
         int64_t items = 0;
-        if (kind == TC_MULTI_GRAM) {
-            const tc::GramBulk p = gram_bulk_problem(e, a[i].lam, slices, a[i].G, e.N, a[i].work, &items);
-            probs.insert(probs.end(), (const unsigned char*)&p, (const unsigned char*)&p + sizeof(p));
-        } else {
-            if (chunk >= recon_bulk_chunks(e, slices)) continue;
-            if (kind == TC_MULTI_RECON1) {
-                const tc::ReconB1 p = recon_b1_problem(e, slices, a[i].work, chunk, &items);
-                probs.insert(probs.end(), (const unsigned char*)&p, (const unsigned char*)&p + sizeof(p));
-            } else {
-                const tc::ReconB2 p = recon_b2_problem(e, slices, a[i].R, a[i].work, chunk, &items);
-                probs.insert(probs.end(), (const unsigned char*)&p, (const unsigned char*)&p + sizeof(p));
-            }
-        }
+        const tc::GramBulk p = gram_bulk_problem(e, a[i].lam, slices, a[i].G, e.N, a[i].work, &items);
+        probs.insert(probs.end(), (const unsigned char*)&p, (const unsigned char*)&p + sizeof(p));
         gx.push_back(items);  // bulk problems decode their own tile from the item index
         start.push_back(start.back() + items);
     }
@@ -1679,11 +1661,7 @@ static cudaError_t multi_launch_s(const TcMulti& m, DevStatus* st, cudaStream_t 
     const unsigned char* b = (const unsigned char*)m.buf;
     const int64_t* start = (const int64_t*)(b + m.off_start);
     const int64_t* gx = (const int64_t*)(b + m.off_gx);
-    if (m.kind == TC_MULTI_GRAM)
-        return tc::launch_many<S>((const tc::GramBulk*)b, start, gx, m.n, m.items, st, 1, s);
-    if (m.kind == TC_MULTI_RECON1)
-        return tc::launch_many<S>((const tc::ReconB1*)b, start, gx, m.n, m.items, st, 2, s);
-    return tc::launch_many<S>((const tc::ReconB2*)b, start, gx, m.n, m.items, st, 8, s);
+    return tc::launch_many<S>((const tc::GramBulk*)b, start, gx, m.n, m.items, st, 1, s);
 }
 
 cudaError_t tc_multi_launch(const TcMulti& m, int slices, DevStatus* st, cudaStream_t s) {
