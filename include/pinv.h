@@ -72,7 +72,8 @@ typedef enum {
 } pinv_status;
 
 typedef enum {
-    PINV_FP64 = 0,          /* every stage in FP64 (SIMT DFMA) */
+    PINV_FP64 = 0,          /* every stage to FP64 accuracy: contractions as exact integer digit
+                               products on the tensor cores, or on the FP64 units */
     PINV_MIXED_BF16X3 = 1,  /* tensor-core stages in split BF16, 2 slices / 3 products,
                                FP32 accumulation, FP64 panels, FP64-residual refinement */
     PINV_MIXED_BF16X6 = 2   /* as above with 3 slices / 6 products */
@@ -122,15 +123,16 @@ typedef struct {
  * DOUBLE_FLOAT and FP64 generate E twice per step (2 N M F complex MACs).
  * TOEPLITZ uses the identity r = E^H d - G x with the exact Gram G: without B0
  * and with voxels on the grid, (A^H A)[n][n'] depends only on the grid offset
- * between n and n' (Eq. 2), so G is formed in FP64 from a (2n_x-1)(2n_y-1)(2n_z-1)
- * table and the coil products at build time and stored as double-float
- * [N][N] (16 N^2 bytes) plus fixed-point digit tiles (24 N^2 bytes); each
- * apply forms E^H d once and each step costs N^2 F complex MACs. G x runs
- * exactly on the tensor cores (integer digit products); E^H d too with 16 or
- * more frames, otherwise in double-float. Plans with b0_hz reject TOEPLITZ. */
+ * between n and n' (Eq. 2), so G is formed in double-float from a
+ * (2n_x-1)(2n_y-1)(2n_z-1) table and the coil products at build time, factored,
+ * and stored as double-float [N][N] (16 N^2 bytes) plus fixed-point digit tiles
+ * (24 N^2 bytes); each apply forms E^H d once and each step costs N^2 F complex
+ * MACs. G x and E^H d run exactly on the tensor cores (integer digit products);
+ * with an explicit Recon the refinement still starts from the factors. Plans with
+ * b0_hz reject TOEPLITZ. */
 typedef enum {
     PINV_RESIDUAL_DOUBLE_FLOAT = 0, /* r in double-float (hi + lo floats, ~44 bits) on the FP32 units */
-    PINV_RESIDUAL_FP64 = 1,         /* r in FP64 (DFMA); FP64 plans always use this */
+    PINV_RESIDUAL_FP64 = 1,         /* r to FP64 accuracy; FP64 plans always use this */
     PINV_RESIDUAL_TOEPLITZ = 2      /* r = E^H d - G x, exact G from the Toeplitz table, double-float */
 } pinv_residual;
 
@@ -480,7 +482,9 @@ pinv_status pinv_tsvd_apply(pinv_plan* plan, const double* d_mu, const void* d_P
  *   24 F     when the refinement's stopping rule (refine_tol > 0) is on;
  * plus the partial sums and digit tiles of the tensor-core products, and for
  * plans with B0 that hold the exact-product digit tables, 16 F C N for the
- * coil-weighted images (the call computes the exact total).
+ * coil-weighted images (the call computes the exact total). The tables of the
+ * FP64 products and of the correction of many frames are left out where they would
+ * not fit (those then run on the FP64 and FP32 units).
  * A call that needs more fails with PINV_ERR_INVALID_ARG and a message giving
  * the size; split the frames over several calls.
  *

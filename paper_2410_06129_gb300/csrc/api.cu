@@ -358,7 +358,7 @@ pinv_status build_recon(pinv_plan* p, cudaStream_t s) {
             CK(cudaFreeAsync(T, s));
         }
     } else {
-        cudaError_t e = tc_available() ? launch_recon64_oz(p->enc, p->eexp, p->Ginv, (double2*)p->R, p->st, s)
+        cudaError_t e = tc_available() ? launch_recon64_oz(p->enc, p->Ginv, (double2*)p->R, p->st, s)
                                        : cudaErrorMemoryAllocation;
         if (e == cudaErrorMemoryAllocation) {
             cudaGetLastError();
@@ -466,23 +466,14 @@ pinv_status pinv_plan_create(const pinv_plan_desc* d, void* stream, pinv_plan** 
         ijk[3 * n + 2] = (int)(g / ((int64_t)p->dims[0] * p->dims[1]));
     }
     // lambda: trace(E^H E) / N = M_k * mean_n sum_c |s_c(n)|^2 since |A| = 1
-    double sos = (double)p->N, smax = 1.0;
+    double sos = (double)p->N;
     if (d->coil_maps) {
         sos = 0.0;
-        smax = 0.0;
         for (int64_t i = 0; i < 2 * p->N * p->C; ++i) {
             double v = d->coil_maps[i];
             if (!std::isfinite(v)) return cleanup(fail(PINV_ERR_INVALID_ARG, "non-finite coil map"));
             sos += v * v;
         }
-        for (int64_t i = 0; i < p->N * p->C; ++i)
-            smax = std::max(smax, std::hypot(d->coil_maps[2 * i], d->coil_maps[2 * i + 1]));
-    }
-    // |E| = |s_c(n)| (|A| = 1): the exponent bounding every component of E
-    {
-        int ex = 0;
-        const double mant = smax > 0.0 ? std::frexp(smax * (1.0 + 1e-12), &ex) : 0.0;
-        p->eexp = smax > 0.0 ? (mant == 0.5 ? ex - 1 : ex) : 0;
     }
     p->lambda_abs = d->lambda_mode == PINV_LAMBDA_ABS ? d->lambda
                                                       : d->lambda * (double)p->Mk * sos / (double)p->N;
@@ -695,6 +686,14 @@ pinv_status pinv_plan_create(const pinv_plan_desc* d, void* stream, pinv_plan** 
     if (p->recon) {
         size_t rb = (size_t)p->N * p->M * (p->precision == PINV_FP64 ? sizeof(double2) : sizeof(float2));
         AL(p->R, rb, "Recon");
+        if (p->precision == PINV_FP64 && !d->b0_hz) {  // mirror pairs for the FP64 Recon
+            pairs = mirror_pairs(p->dims, ijk, !d->voxel_index);
+            int2* pd;
+            AL(pd, sizeof(int) * pairs.size(), "mirror pairs");
+            CKC(cudaMemcpyAsync(pd, pairs.data(), sizeof(int) * pairs.size(), cudaMemcpyHostToDevice, s));
+            e.pair = pd;
+            e.U = (int64_t)pairs.size() / 2;
+        }
         p->bytes_recon = rb;
     }
     for (auto& ev : p->ev) CKC(cudaEventCreate(&ev));

@@ -22,6 +22,8 @@
 // Roles, waits and aborts follow k_exact: warps 0-7 drain and store (thread 0 also starts
 // the copies), warp 8 issues the MMAs.
 #include <algorithm>
+#include <cstdlib>
+#include <cstring>
 #include <climits>
 
 #include "df.cuh"
@@ -147,8 +149,8 @@ struct Mat {
 struct EncRow {
     EncodeDev e;
     int64_t j_off, n, K;
-    int ex;
-    __device__ int exponent(int64_t) const { return ex; }
+    const int* ex;  // of rows
+    __device__ int exponent(int64_t i) const { return ex[i]; }
     __device__ double2 get(int64_t i, int64_t k) const {
         const int64_t j = j_off + i, c = j / e.Mk;
         return zconj(gen_e64(e, (int)c, j - c * e.Mk, k));
@@ -183,6 +185,43 @@ struct CoilCol {
     }
 };
 // exponents of p's rows (columns), one CTA each
+// Mirror pairs of voxels (plans without B0), the two operands of sum_k E^H[k][(c, m)] G[n][k]: with
+// X = conj(s_c) G[n] at a pair's two voxels and theta the phase of conj(A[m]) at the first,
+// the sum is that over the pairs of cos(theta) (X_a + X_b) + i sin(theta) (X_a - X_b).
+// PairRow: (cos, sin) of row m; PairCol: column n, whose exponent holds for both X.
+struct PairRow {
+    EncodeDev e;
+    int64_t m0, n, K;
+    __device__ int exponent(int64_t) const { return 0; }
+    __device__ double2 get(int64_t i, int64_t k) const { return zconj(gen_a64(e, m0 + i, e.pair[k].x)); }
+};
+struct PairCol {
+    EncodeDev e;
+    const double2* G;  // [N][N]
+    int c;
+    int64_t n, K;
+    const int* ex;
+    __device__ int exponent(int64_t i) const { return ex[i]; }
+    __device__ void both(int64_t i, int64_t k, double2& p, double2& q) const {
+        const int2 v = e.pair[k];
+        double2 a = G[i * e.N + v.x], b = v.y >= 0 ? G[i * e.N + v.y] : make_double2(0.0, 0.0);
+        if (e.coils) {
+            const double2* s = e.coils + (int64_t)c * e.N;
+            a = zmul(a, zconj(s[v.x]));
+            if (v.y >= 0) b = zmul(b, zconj(s[v.y]));
+        }
+        p = make_double2(a.x + b.x, a.y + b.y);
+        q = make_double2(a.x - b.x, a.y - b.y);
+    }
+    __device__ double2 get(int64_t i, int64_t k) const {  // the larger components, for the exponent
+        double2 p, q;
+        both(i, k, p, q);
+        // a NaN or an infinity in either must show
+        const double x = abs_bits(p.x) > abs_bits(q.x) ? p.x : q.x, y = abs_bits(p.y) > abs_bits(q.y) ? p.y : q.y;
+        return make_double2(x, y);
+    }
+};
+
 template <class P>
 __global__ void __launch_bounds__(256) k_row_exp(P p, int* ex) {
     __shared__ unsigned long long red[8];
@@ -198,6 +237,14 @@ __global__ void __launch_bounds__(256) k_row_exp(P p, int* ex) {
         for (int w = 1; w < 8; ++w) m = max(m, red[w]);
         ex[i] = bits_exp(m);
     }
+}
+
+// exponents of the rows j0 .. of conj(E) from those of their coils' maps (|A| = 1), or for s = 1
+__global__ void k_enc_exp(const int* coil, int64_t j0, int64_t rows, int64_t Mk, int* ex) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= rows) return;
+    const int c = coil ? coil[(j0 + i) / Mk] : 0;
+    ex[i] = c == NONFINITE ? c : c + 1;
 }
 
 // the 8 values k0 .. k0 + 7 of row i as fixed-point integers (zeros out of range, and for a
@@ -252,6 +299,43 @@ __global__ void __launch_bounds__(4 * ON) k_oz_b(P p, int64_t KB, uint8_t* Bt) {
             make_uint4(wi[0] ^ 0x80008000u, wi[1] ^ 0x80008000u, wi[2] ^ 0x80008000u, wi[3] ^ 0x80008000u);
         *reinterpret_cast<uint4*>(sl + koff16(ON + c, 0)) = make_uint4(wi[0], wi[1], wi[2], wi[3]);
         *reinterpret_cast<uint4*>(sl + koff16(ON + c, 1)) = make_uint4(wr[0], wr[1], wr[2], wr[3]);
+    }
+}
+
+// ... of pairs: column c owns row c, [Re+ | -Im-], and row ON + c, [Im+ | Re-]
+__global__ void __launch_bounds__(4 * ON) k_oz_bp(PairCol p, int64_t KB, uint8_t* Bt) {
+    const int64_t kb = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5), ct = blockIdx.y;
+    if (kb >= KB) return;
+    const int c = threadIdx.x & 31;
+    const int64_t i = ct * ON + c, k0 = kb * OKC;
+    const int e = i < p.n ? p.exponent(i) : NONFINITE;
+    uint8_t* blk = Bt + (ct * KB + kb) * (int64_t)OB_ST;
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {  // Re+ and Im+, then Re- and Im-
+        Fix8 re, im;
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            const bool in = e != NONFINITE && k0 + t < p.K;
+            double2 a = make_double2(0.0, 0.0), b = a;
+            if (in) p.both(i, k0 + t, a, b);
+            re.set(t, h ? b.x : a.x, in ? e : 0);
+            im.set(t, h ? b.y : a.y, in ? e : 0);
+        }
+#pragma unroll
+        for (int dg = OD - 1; dg >= 0; --dg) {
+            uint32_t wr[4], wi[4];
+            re.next(wr, dg == 0);
+            im.next(wi, dg == 0);
+            uint8_t* sl = blk + dg * OB_SL;
+            if (h == 0) {
+                *reinterpret_cast<uint4*>(sl + koff16(c, 0)) = make_uint4(wr[0], wr[1], wr[2], wr[3]);
+                *reinterpret_cast<uint4*>(sl + koff16(ON + c, 0)) = make_uint4(wi[0], wi[1], wi[2], wi[3]);
+            } else {
+                *reinterpret_cast<uint4*>(sl + koff16(c, 1)) =
+                    make_uint4(wi[0] ^ 0x80008000u, wi[1] ^ 0x80008000u, wi[2] ^ 0x80008000u, wi[3] ^ 0x80008000u);
+                *reinterpret_cast<uint4*>(sl + koff16(ON + c, 1)) = make_uint4(wr[0], wr[1], wr[2], wr[3]);
+            }
+        }
     }
 }
 
@@ -642,7 +726,7 @@ struct Temp {
 
 // Recon[n][j] = sum_k Ginv[n][k] conj(E[j][k]) over chunks of samples whose tables stay
 // within 1 GiB
-cudaError_t launch_recon64_oz(const EncodeDev& e, int eexp, const double2* Ginv, double2* R, DevStatus* st,
+cudaError_t launch_recon64_oz(const EncodeDev& e, const double2* Ginv, double2* R, DevStatus* st,
                               cudaStream_t s) {
     using namespace oz;
     const int64_t N = e.N, M = e.Mk * e.C, KB = (N + OKC - 1) / OKC, ctn = (N + ON - 1) / ON;
@@ -651,6 +735,30 @@ cudaError_t launch_recon64_oz(const EncodeDev& e, int eexp, const double2* Ginv,
     Temp t(s);
     uint8_t *At = nullptr, *Bt = nullptr;
     int* ex = nullptr;
+    const char* env = std::getenv("PINV_RECON_PAIRS");
+    if (e.pair && !e.b0tab && !(env && std::strcmp(env, "0") == 0)) {
+        // over mirror pairs, coil by coil: half the products, one table of A for all coils
+        // (37 x 37, 4 coils, 2701 samples a coil: 4.92 -> 3.22 ms). PINV_RECON_PAIRS=0: voxel by voxel
+        const int64_t KP = (e.U + OKC - 1) / OKC, rtk = (e.Mk + OM - 1) / OM;
+        const int64_t perk = std::max<int64_t>(1, std::min<int64_t>(rtk, (int64_t(1) << 30) / (KP * OA_ST)));
+        OZ(t.take(&At, (size_t)(perk * KP * OA_ST)));
+        OZ(t.take(&Bt, (size_t)(ctn * KP * OB_ST)));
+        OZ(t.take(&ex, sizeof(int) * N));
+        for (int64_t r0 = 0; r0 < rtk; r0 += perk) {
+            const int64_t m0 = r0 * OM, rows = std::min(perk * OM, e.Mk - m0);
+            OZ(tab_a(PairRow{e, m0, rows, e.U}, 0, KP, At, s));
+            for (int c = 0; c < e.C; ++c) {
+                const PairCol pc{e, Ginv, c, N, e.U, ex};
+                k_row_exp<<<(unsigned)N, 256, 0, s>>>(pc, ex);
+                k_oz_bp<<<dim3((unsigned)((KP + 3) / 4), (unsigned)ctn), 4 * ON, 0, s>>>(pc, KP, Bt);
+                note_launch(2);
+                OZ(cudaGetLastError());
+                const ReconOz p{R, M, c * e.Mk + m0, rows, N, KP, ctn};
+                OZ(run(p, (rows + OM - 1) / OM * ctn, Args{At, Bt, KP, KP, 0, nullptr, ex, 0}, st, s));
+            }
+        }
+        return cudaSuccess;
+    }
     OZ(t.take(&At, (size_t)(per * KB * OA_ST)));
     OZ(t.take(&Bt, (size_t)(ctn * KB * OB_ST)));
     OZ(t.take(&ex, sizeof(int) * N));
@@ -658,11 +766,20 @@ cudaError_t launch_recon64_oz(const EncodeDev& e, int eexp, const double2* Ginv,
     k_row_exp<<<(unsigned)N, 256, 0, s>>>(gm, ex);
     note_launch();
     OZ(tab_b(gm, KB, Bt, s));
+    int *cex = nullptr, *rex = nullptr;  // each coil to its own scale
+    OZ(t.take(&rex, sizeof(int) * (size_t)(per * OM)));
+    if (e.coils) {
+        OZ(t.take(&cex, sizeof(int) * (size_t)e.C));
+        k_row_exp<<<(unsigned)e.C, 256, 0, s>>>(Mat{e.coils, N, e.C, N, 0, 0, cex}, cex);
+        note_launch();
+    }
     for (int64_t r0 = 0; r0 < rtn; r0 += per) {
         const int64_t j0 = r0 * OM, rows = std::min(per * OM, M - j0);
-        OZ(tab_a(EncRow{e, j0, rows, N, eexp}, 0, KB, At, s));
+        k_enc_exp<<<(unsigned)((rows + 255) / 256), 256, 0, s>>>(cex, j0, rows, e.Mk, rex);
+        note_launch();
+        OZ(tab_a(EncRow{e, j0, rows, N, rex}, 0, KB, At, s));
         const ReconOz p{R, M, j0, rows, N, KB, ctn};
-        OZ(run(p, (rows + OM - 1) / OM * ctn, Args{At, Bt, KB, KB, 0, nullptr, ex, eexp}, st, s));
+        OZ(run(p, (rows + OM - 1) / OM * ctn, Args{At, Bt, KB, KB, 0, rex, ex, 0}, st, s));
     }
     return cudaSuccess;
 }

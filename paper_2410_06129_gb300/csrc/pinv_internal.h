@@ -170,7 +170,7 @@ cudaError_t launch_gram64_table(const EncodeDev& e, double lambda, double2* G, i
 // Recon, Ginv = W^H W, and the factorisation and inverse whose trailing updates they form
 // (T: N x 32 scratch, work: oz_panel_bytes(N), Dinv: 32 x 32 block inverses). They take
 // their tables from the pool and return cudaErrorMemoryAllocation without room.
-cudaError_t launch_recon64_oz(const EncodeDev& e, int eexp, const double2* Ginv, double2* R, DevStatus* st,
+cudaError_t launch_recon64_oz(const EncodeDev& e, const double2* Ginv, double2* R, DevStatus* st,
                               cudaStream_t s);
 cudaError_t launch_lauum64_oz(const double2* W, int64_t N, double2* Ginv, DevStatus* st, cudaStream_t s);
 // The products of an FP64 apply (scratch: the *_bytes of the same sizes), as

@@ -73,7 +73,6 @@ struct pinv_plan {
     int64_t N = 0, Mk = 0, M = 0;
     int C = 1;
     double lambda_abs = 0;
-    int eexp = 0;  // every component of E is at most 2^eexp in magnitude
     int precision = PINV_FP64;
     int recon = 1;
     int refine_iters = 0;

@@ -220,3 +220,34 @@ def test_apply_digit_products_frames(dims, coils, samples, frames, recon):
             assert not np.isfinite(x[f]).any()
         else:
             assert rel(x[f], want[f]) < tol
+
+
+# even and odd axes (voxels without a mirror), a voxel list, one and several coils and sample
+# tiles, maps of very different scale
+@pytest.mark.parametrize("dims,coils,samples,drop", [((1,), 1, 5, 0), ((16, 8), 1, 129, 0), ((15, 9), 3, 200, 0),
+                                                     ((5, 6, 7), 2, 257, 0), ((20, 13), 2, 300, 61)])
+def test_recon_over_mirror_pairs(dims, coils, samples, drop, monkeypatch):
+    """Recon formed over mirror pairs of voxels and voxel by voxel, against NumPy in FP64
+    (lambda = mean diag, tolerance as test_digit_products_at_tile_edges)."""
+    from paper_2410_06129_gb300.plan import Plan
+    rng = np.random.default_rng(1905)
+    n, D = int(np.prod(dims)), len(dims)
+    vox = np.sort(rng.choice(n, n - drop, replace=False)).astype(np.int64) if drop else None
+    k = rng.uniform(-0.5 * max(dims), 0.5 * max(dims), size=(samples, D))
+    maps = rng.standard_normal((coils, n)) + 1j * rng.standard_normal((coils, n))
+    maps *= 10.0 ** (6 * np.arange(coils))[:, None] if coils == 3 else 1.0
+    pos = O.voxel_positions(dims)
+    if drop:
+        pos, maps = pos[vox], maps[:, vox]
+    E = O.encode(k, pos, maps, None, None)
+    N = n - drop
+    G = E.conj().T @ E + O.lambda_abs(E, 1.0) * np.eye(N)
+    want = np.linalg.solve(G, E.conj().T)
+    tol = (64 + 8 * N) * np.linalg.cond(G) * 2.0 ** -53
+    for pairs in ("1", "0"):
+        monkeypatch.setenv("PINV_RECON_PAIRS", pairs)
+        with Plan(dims, k, maps, lam=1.0, precision=L.FP64, voxel_index=vox) as pl:
+            got = pl.build().export(L.EXPORT_RECON).cpu().numpy()
+        for c in range(coils):  # each coil to its own scale
+            cols = slice(c * samples, (c + 1) * samples)
+            assert rel(got[:, cols], want[:, cols]) < tol, (pairs, c)
